@@ -54,6 +54,9 @@ kmv_status fail(kmv_handle h, kmv_status s, const std::string& msg) {
 
 // Bump allocator over the handle workspace; 256-byte aligned regions.
 constexpr int kMaxPoles = 32;
+// Largest system (rows) whose CG direction one CTA forms: above, its 128 threads take
+// longer than the launch that they spare.
+constexpr int kFusedPRows = 4096;
 
 struct Arena {
   size_t used = 0;
@@ -142,10 +145,21 @@ kmv_status prepare_layout(kmv_handle h, const kmv_points* pts, int32_t chains, c
   const size_t b_inst = sizeof(int32_t) * std::max(1, L.n_items);
   const size_t b_row0 = sizeof(int64_t) * std::max(1, L.n_items);
   const size_t b_ii = sizeof(int32_t) * (n_inst + 1);
+  // first items of the 2- and 4-item tiles, one table after the other
+  std::vector<int32_t> wide;
+  int n_wide[2];
+  for (int w = 0; w < 2; ++w) {
+    const size_t before = wide.size();
+    for (int b = 0; b < n_inst; ++b)
+      for (int32_t it = L.inst_item0[b]; it < L.inst_item0[b + 1]; it += 2 << w) wide.push_back(it);
+    n_wide[w] = (int)(wide.size() - before);
+  }
+  const size_t b_wide = sizeof(int32_t) * std::max<size_t>(1, wide.size());
   const size_t o_off = 0, o_row0 = (b_off + 255) & ~size_t(255);
   const size_t o_inst = o_row0 + ((b_row0 + 255) & ~size_t(255));
   const size_t o_ii = o_inst + ((b_inst + 255) & ~size_t(255));
-  const size_t total = o_ii + b_ii;
+  const size_t o_wide = o_ii + ((b_ii + 255) & ~size_t(255));
+  const size_t total = o_wide + b_wide;
   if (total > h->tables_bytes) {
     if (h->tables) {
       KMV_CUDA(h, cudaDeviceSynchronize());
@@ -170,7 +184,13 @@ kmv_status prepare_layout(kmv_handle h, const kmv_points* pts, int32_t chains, c
                                 cudaMemcpyHostToDevice, st));
   }
   KMV_CUDA(h, cudaMemcpyAsync(base + o_ii, L.inst_item0.data(), b_ii, cudaMemcpyHostToDevice, st));
+  if (!wide.empty())
+    KMV_CUDA(h, cudaMemcpyAsync(base + o_wide, wide.data(), sizeof(int32_t) * wide.size(), cudaMemcpyHostToDevice, st));
   KMV_CUDA(h, cudaStreamSynchronize(st));
+  h->simt_tiles.n2 = n_wide[0];
+  h->simt_tiles.n4 = n_wide[1];
+  h->simt_tiles.item2 = reinterpret_cast<const int32_t*>(base + o_wide);
+  h->simt_tiles.item4 = h->simt_tiles.item2 + n_wide[0];
   h->dev.offsets = reinterpret_cast<const int64_t*>(base + o_off);
   h->dev.item_row0 = reinterpret_cast<const int64_t*>(base + o_row0);
   h->dev.item_inst = reinterpret_cast<const int32_t*>(base + o_inst);
@@ -248,32 +268,55 @@ kmv_status cheb_prepare(kmv_handle h, const kmv_points* pts, const double* theta
 
 // --- building blocks used by several entry points -------------------------------------
 
-// The FP32 forward, with its J range split over more CTAs when one CTA per
-// (item, chain, column chunk) would leave most SMs idle (forward_jsplit).
+// The FP32 kernels' scratch: `bytes` of partial sums and `counters` zeroed counters.
+kmv_status simt_scratch(kmv_handle h, size_t bytes, size_t counters, cudaStream_t st) {
+  if (bytes <= h->simt_part_bytes && counters <= h->simt_counters) return KMV_OK;
+  if (h->capturing)
+    return fail(h, KMV_EINVAL, "FP32 scratch not prepared: make the same call once before capturing");
+  auto grow = [&](void** p, size_t want) {
+    void* n = nullptr;
+    if (cudaMalloc(&n, want) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (*p) h->simt_retired.push_back(*p);
+    *p = n;
+    return true;
+  };
+  if (bytes > h->simt_part_bytes) {
+    size_t want = std::max(bytes, 2 * h->simt_part_bytes);
+    if (!grow(reinterpret_cast<void**>(&h->simt_part), want)) return fail(h, KMV_ENOMEM, "FP32 scratch allocation failed");
+    h->simt_part_bytes = want;
+  }
+  if (counters > h->simt_counters) {
+    const size_t want = std::max(counters, 2 * h->simt_counters);
+    if (!grow(reinterpret_cast<void**>(&h->simt_count), sizeof(uint32_t) * want))
+      return fail(h, KMV_ENOMEM, "FP32 scratch allocation failed");
+    h->simt_counters = want;
+    KMV_CUDA(h, cudaMemsetAsync(h->simt_count, 0, sizeof(uint32_t) * want, st));
+  }
+  return KMV_OK;
+}
+
+// The FP32 forward (kmv_simt_fwd.cu).
 kmv_status simt_forward(kmv_handle h, const KmvArgs& a, cudaStream_t st) {
   const Layout& L = h->layout;
   if (L.n_items == 0) return KMV_OK;
   if ((a.cg_sys || a.ms_sys) && !(a.m == 1 && a.dot_partial))
     return fail(h, KMV_EINVAL, "internal: fused CG step needs the one-column product");
-  const int js = forward_jsplit(L.n_items, L.chains, a.m, (int64_t)L.max_items_per_inst * kTile, h->num_sms);
-  if (js > 1) {
-    const size_t need = sizeof(double) * (size_t)js * L.chains * (size_t)L.n_total * a.m;
-    if (need > h->simt_part_bytes) {
-      if (h->capturing)
-        return fail(h, KMV_EINVAL, "FP32 forward scratch not prepared: make the same call once before capturing");
-      if (h->simt_part) cudaFree(h->simt_part);
-      h->simt_part = nullptr;
-      h->simt_part_bytes = 0;
-      if (cudaMalloc(&h->simt_part, need) != cudaSuccess) {
-        cudaGetLastError();
-        h->simt_part = nullptr;
-        return fail(h, KMV_ENOMEM, "FP32 forward scratch allocation failed");
-      }
-      h->simt_part_bytes = need;
-    }
-  }
-  KMV_CUDA(h, launch_forward_simt(a, L.n_items, js, h->simt_part, st));
+  SimtFwd f = simt_fwd_plan(h->simt_tiles, L.n_inst, L.n_items, L.chains, L.n_total, (int64_t)L.max_items_per_inst * kTile, a.d,
+                            a.m, h->num_sms);
+  KMV_TRY(simt_scratch(h, simt_fwd_part_bytes(f, L.chains, L.n_total, a.m), simt_fwd_counters(f, L.chains), st));
+  f.part = h->simt_part;
+  f.count = h->simt_count;
+  KMV_CUDA(h, launch_forward_simt(a, f, L.n_items, st));
   return KMV_OK;
+}
+
+SimtBwd bwd_plan(kmv_handle h, int m, bool want_gv) {
+  const Layout& L = h->layout;
+  return simt_bwd_plan(h->simt_tiles, L.n_items, L.chains, L.n_total, (int64_t)L.max_items_per_inst * kTile, L.d, m,
+                       want_gv, h->num_sms);
 }
 
 kmv_status run_forward(kmv_handle h, const KmvArgs& a, kmv_precision prec, cudaStream_t st) {
@@ -289,10 +332,9 @@ kmv_status run_forward(kmv_handle h, const KmvArgs& a, kmv_precision prec, cudaS
   return KMV_OK;
 }
 
-size_t backward_ws_bytes(const Layout& L, int m) {
-  const int mp = backward_mp(m);
-  const int nz = (m + mp - 1) / mp;
-  return sizeof(double) * (size_t)std::max(1, L.n_items) * L.chains * nz * L.n_theta;
+size_t backward_ws_bytes(kmv_handle h, int m, bool want_gv) {
+  const Layout& L = h->layout;
+  return sizeof(double) * simt_bwd_partials(bwd_plan(h, m, want_gv), L.n_items, L.chains, L.n_theta);
 }
 
 kmv_status run_backward_stationary(kmv_handle h, KmvArgs a, double* grad, double* partial,
@@ -304,15 +346,16 @@ kmv_status run_backward_stationary(kmv_handle h, KmvArgs a, double* grad, double
     const kmv_status s = tc_backward(h, a, grad, st);
     if (s != KMV_EUNSUPPORTED) return s;
   }
-  const int mp = backward_mp(a.m);
-  a.n_z = (a.m + mp - 1) / mp;
+  SimtBwd f = bwd_plan(h, a.m, a.Y != nullptr);
+  if (a.Y && L.n_items > 0) KMV_TRY(simt_scratch(h, simt_bwd_part_bytes(f, L.chains, L.n_total, a.m), 0, st));
+  f.part = h->simt_part;
+  a.n_z = f.nz;
   a.grad_partial = partial;
   if (L.n_items > 0) {
     ProfScope prof(h, KMV_KERNEL_ADJOINT, st);
-    KMV_CUDA(h, launch_backward_simt(a, L.n_items, st));
+    KMV_CUDA(h, launch_backward_simt(a, f, L.n_items, st));
   }
-  KMV_CUDA(h, launch_grad_finalize(h->dev, L.n_inst, L.chains, a.n_theta, L.ard, L.d, a.n_z,
-                                   a.theta, partial, grad, st));
+  KMV_CUDA(h, launch_grad_finalize(h->dev, f, L.n_inst, L.chains, a.n_theta, a.theta, partial, grad, st));
   return KMV_OK;
 }
 
@@ -452,6 +495,7 @@ kmv_status run_cg(kmv_handle h, const kmv_points* pts, const double* theta, cons
   // kernel at the end of the iteration.
   const bool tc_fma = prec == KMV_BF16_HILO && x_width_fma_ok(pts->d);
   const bool fused = L.n_items > 0 && (tc_fma || prec == KMV_FP32);
+  const bool p_fused = fused && !tc_fma && (int64_t)L.max_items_per_inst * kTile <= kFusedPRows;
   if (fused) {
     KMV_CUDA(h, cudaMemsetAsync(B.count, 0, sizeof(uint32_t) * 2 * n_sys, st));
     a.cg_sys = B.sys;
@@ -466,9 +510,11 @@ kmv_status run_cg(kmv_handle h, const kmv_points* pts, const double* theta, cons
     a.reuse_prep = reuse;
     KMV_TRY(run_forward(h, a, prec, s));
     if (fused) {
+      // the systems' last CTAs form p too where the largest system is small
       KMV_CUDA(h, launch_cg_update_xr_rr(h->dev, L.n_items, L.chains, L.n_total, B.sys, B.active, x, B.r, B.p,
-                                         B.q, B.partial, B.count + n_sys, tol, maxiter, B.n_active, s));
-      if (!tc_fma)
+                                         B.q, B.partial, B.count + n_sys, tol, maxiter, B.n_active,
+                                         p_fused ? kFusedPRows : 0, s));
+      if (!tc_fma && !p_fused)
         KMV_CUDA(h, launch_cg_update_p(h->dev, L.n_items, L.chains, L.n_total, B.sys, B.active, B.r, B.p, s));
       return KMV_OK;
     }
@@ -1077,6 +1123,8 @@ kmv_status kmv_destroy(kmv_handle h) {
   if (h->tables) cudaFree(h->tables);
   if (h->cheb_buf) cudaFree(h->cheb_buf);
   if (h->simt_part) cudaFree(h->simt_part);
+  if (h->simt_count) cudaFree(h->simt_count);
+  for (void* p : h->simt_retired) cudaFree(p);
   if (h->host_flag) cudaFreeHost(h->host_flag);
   if (h->side) cudaStreamDestroy(h->side);
   kmv_profile_enable(h, 0);
@@ -1135,7 +1183,7 @@ kmv_status kmv_backward(kmv_handle h, const kmv_points* pts, int32_t chains, con
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   KMV_TRY(prepare_layout(h, pts, chains, st));
   Arena ar;
-  const size_t o_part = ar.take(backward_ws_bytes(h->layout, m));
+  const size_t o_part = ar.take(backward_ws_bytes(h, m, grad_V != nullptr));
   KMV_TRY(reserve(h, ar.used));
   KMV_TRY(cheb_prepare(h, pts, theta, m, st));
   KmvArgs a = base_args(h, pts, theta);
@@ -1328,7 +1376,7 @@ kmv_status leapfrog_step(kmv_handle h, const kmv_points* pts, int32_t chains, co
   const size_t vec2 = sizeof(float) * 2 * (size_t)L.chains * std::max<int64_t>(1, L.n_total);
   const size_t o_vf = ar.take(vec2);
   const size_t o_gf = ar.take(vec2);
-  const size_t o_bp = ar.take(backward_ws_bytes(L, 2));
+  const size_t o_bp = ar.take(backward_ws_bytes(h, 2, false));
   KMV_TRY(reserve(h, ar.used));
   double* theta_h = at<double>(h, o_th);
   double* grad = at<double>(h, o_gr);
@@ -1383,7 +1431,7 @@ kmv_status kmv_implicit_step(kmv_handle h, const kmv_points* pts, int32_t chains
   const size_t o_th0 = ar.take(sizeof(double) * n_sys * n), o_pi0 = ar.take(sizeof(double) * n_sys * n);
   const size_t o_tb = ar.take(sizeof(double) * n_sys * n), o_gr = ar.take(sizeof(double) * n_sys * n);
   const size_t o_vf = ar.take(sizeof(float) * 2 * vec), o_gf = ar.take(sizeof(float) * 2 * vec);
-  const size_t o_bp = ar.take(backward_ws_bytes(L, 2));
+  const size_t o_bp = ar.take(backward_ws_bytes(h, 2, false));
   const size_t o_q = ar.take(sizeof(float) * vec), o_r = ar.take(sizeof(float) * vec), o_z = ar.take(sizeof(float) * vec);
   const size_t o_gx = ar.take(sizeof(float) * vec * k), o_fx = ar.take(sizeof(float) * vec * k);
   const size_t o_gtp = ar.take(sizeof(double) * (size_t)k * n_sys * 2 * n);

@@ -151,18 +151,23 @@ cudaError_t launch_cg_update_xr(const DevLayout& L, int n_items, int chains, int
 // x += alpha p, r -= alpha q and the r.r partials, as cg_update_xr_kernel;
 // the CTA of each system that finishes last then takes the system's r.r step
 // (as cg_reduce_rr_kernel) and keeps n_active up to date by decrements, so an
-// iteration needs no separate reduction launch.
+// iteration needs no separate reduction launch.  With p_rows > 0 that CTA also
+// forms the next direction p = r + beta p of a system of at most p_rows rows,
+// which spares the FP32 form a launch per iteration where launches count.
 __global__ void cg_update_xr_rr_kernel(DevLayout L, int chains, int64_t n_total, CgSys* sys, int32_t* active,
-                                       float* x, float* r, const float* p, const float* q, double* partial,
-                                       uint32_t* count, double tol, int maxiter, int32_t* n_active) {
+                                       float* x, float* r, float* p, const float* q, double* partial,
+                                       uint32_t* count, double tol, int maxiter, int32_t* n_active, int p_rows) {
   __shared__ double red[kTile / 32];
+  __shared__ int s_last;
+  __shared__ float s_beta;
   const int item = blockIdx.x, c = blockIdx.y;
   const int b = L.item_inst[item];
   const int s = b * chains + c;
   if (!active[s]) return;
+  const int64_t r0 = L.offsets[b], r1 = L.offsets[b + 1];
   const int64_t i = L.item_row0[item] + threadIdx.x;
   double rr = 0.0;
-  if (i < L.offsets[b + 1]) {
+  if (i < r1) {
     const int64_t v = (int64_t)c * n_total + i;
     const float al = (float)sys[s].alpha;
     x[v] = fmaf(al, p[v], x[v]);
@@ -170,23 +175,39 @@ __global__ void cg_update_xr_rr_kernel(DevLayout L, int chains, int64_t n_total,
     r[v] = ri;
     rr = (double)ri * ri;
   }
+  const bool form_p = p_rows > 0 && r1 - r0 <= p_rows;
   const double t = block_sum(rr, red);
   if (threadIdx.x == 0) {
     partial[(int64_t)item * chains + c] = t;
-    const bool last = last_block_of_system(count, s, (uint32_t)(L.inst_item0[b + 1] - L.inst_item0[b]));
-    if (last && !cg_rr_step(sys[s], sys_sum(L, b, c, chains, partial, 1, 0), tol, maxiter)) {
+    s_last = last_arrival(&count[s], 1u, (uint32_t)(L.inst_item0[b + 1] - L.inst_item0[b]));
+  }
+  __syncthreads();
+  if (!s_last) return;
+  const double rr_new = sys_sum_block(L, b, c, chains, partial, 1, 0, red);
+  if (threadIdx.x == 0) {
+    const bool go = cg_rr_step(sys[s], rr_new, tol, maxiter);
+    if (!go) {
       active[s] = 0;
       atomicSub(n_active, 1);
     }
+    s_last = go;
+    s_beta = (float)sys[s].beta;
+  }
+  if (!form_p) return;
+  __syncthreads();
+  if (!s_last) return;
+  for (int64_t j = r0 + threadIdx.x; j < r1; j += blockDim.x) {
+    const int64_t v = (int64_t)c * n_total + j;
+    p[v] = fmaf(s_beta, p[v], __ldcg(&r[v]));
   }
 }
 
 cudaError_t launch_cg_update_xr_rr(const DevLayout& L, int n_items, int chains, int64_t n_total, CgSys* sys,
-                                   int32_t* active, float* x, float* r, const float* p, const float* q,
+                                   int32_t* active, float* x, float* r, float* p, const float* q,
                                    double* partial, uint32_t* count, double tol, int maxiter, int32_t* n_active,
-                                   cudaStream_t st) {
+                                   int p_rows, cudaStream_t st) {
   cg_update_xr_rr_kernel<<<dim3(n_items, chains), kTile, 0, st>>>(L, chains, n_total, sys, active, x, r, p, q,
-                                                                  partial, count, tol, maxiter, n_active);
+                                                                  partial, count, tol, maxiter, n_active, p_rows);
   return cudaGetLastError();
 }
 

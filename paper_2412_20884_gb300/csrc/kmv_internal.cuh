@@ -124,23 +124,55 @@ struct KmvArgs {
 // point (kmv_api.cu): nullptr when they hold, else what is wrong.
 const char* points_error(const kmv_points* pts, int32_t chains);
 
-// SIMT kernels (kmv_simt.cu)
-// jsplit > 1 splits each system's J range into jsplit chunks of whole J
-// tiles, with per-chunk FP64 row sums in jpart (jsplit * chains * N_total * m
-// doubles) added in chunk order by a combine kernel.
-cudaError_t launch_forward_simt(const KmvArgs& a, int n_items, int jsplit, double* jpart, cudaStream_t st);
-// The J split for a grid of n_items * chains * column chunks CTAs: 1 from two
-// CTAs per SM up, else about two CTAs per SM with at least two J tiles (of
-// the largest instance, max_rows) per chunk, at most kMaxJSplit.
-int forward_jsplit(int n_items, int chains, int m, int64_t max_rows, int num_sms);
-cudaError_t launch_backward_simt(const KmvArgs& a, int n_items, cudaStream_t st);
+// First 128-row items of the 256- and 512-row tiles (2 and 4 items of one
+// instance) of the SIMT kernels' wide variants.
+struct SimtTiles {
+  int n2 = 0, n4 = 0;
+  const int32_t *item2 = nullptr, *item4 = nullptr;
+};
+
+// FP32 (SIMT) kernels: kmv_simt_fwd.cu, kmv_simt_bwd.cu.  A plan fixes the work
+// split of one call shape; part and count point to scratch of the sizes given
+// (count zeroed once: the kernels leave it zero).
+struct SimtFwd {
+  const int32_t* tile_item;  // first 128-row item of each R-item tile; NULL: R = 1, the items themselves
+  int n_inst, n_tiles;
+  int rows;                  // R
+  int mp, nz, z0;            // columns per CTA (the kernel's MP), column chunks, the launch's first
+  int js;                    // chunks of whole J tiles: where the FP32 sums start anew
+  int folds, upc;            // folds (512 columns) per unit, units per chunk
+  int max_units;             // js * upc; 1: every CTA writes its rows' Y itself
+  int ticket;                // the last unit of a tile adds the units and writes Y; else the combine kernel does
+  float2* part;              // (max_units, chains, m, N_total) pairs, for several units or folds
+  uint32_t* count;           // ticket: one zeroed counter per (tile, chain, column chunk)
+};
+SimtFwd simt_fwd_plan(const SimtTiles& T, int n_inst, int n_items, int chains, int64_t n_total, int64_t max_rows, int d, int m,
+                      int num_sms);
+size_t simt_fwd_part_bytes(const SimtFwd& f, int chains, int64_t n_total, int m);
+size_t simt_fwd_counters(const SimtFwd& f, int chains);
+cudaError_t launch_forward_simt(const KmvArgs& a, const SimtFwd& f, int n_items, cudaStream_t st);
+
+struct SimtBwd {
+  const int32_t* tile_item;   // first 128-row item of each tile; NULL: the items themselves
+  int n_tiles, rows, mp, nz;  // tiles, rows per thread, columns per CTA (the kernel's width), column chunks
+  int chunk;                  // columns per chunk (<= mp): W_ij is summed per chunk
+  int folds, units;           // folds (512 columns) per J unit, units
+  float2* part;               // want_gv and several units or folds: (units, chains, m, N_total) pairs
+};
 int backward_mp(int m);      // columns per backward pass
-int forward_mp(int m);
+SimtBwd simt_bwd_plan(const SimtTiles& T, int n_items, int chains, int64_t n_total, int64_t max_rows, int d, int m,
+                      bool want_gv, int num_sms);
+// The plan of one unit per 128-row item, whose partials are (n_items, chains, n_z, n_theta)
+// and which needs no part (kmv_backward_noalloc).
+SimtBwd simt_bwd_plan_plain(int n_items, int d, int m);
+// Doubles of the gradient partials: (n_items, chains, nz, units, n_theta), a tile's at its first item.
+size_t simt_bwd_partials(const SimtBwd& f, int n_items, int chains, int n_theta);
+size_t simt_bwd_part_bytes(const SimtBwd& f, int chains, int64_t n_total, int m);
+cudaError_t launch_backward_simt(const KmvArgs& a, const SimtBwd& f, int n_items, cudaStream_t st);
 
 // Gradient finalisation: sums partials per system in a fixed order and scales.
-cudaError_t launch_grad_finalize(const DevLayout& L, int n_inst, int chains, int n_theta,
-                                 int ard, int d, int n_z, const double* theta,
-                                 const double* partial, double* grad, cudaStream_t st);
+cudaError_t launch_grad_finalize(const DevLayout& L, const SimtBwd& f, int n_inst, int chains, int n_theta,
+                                 const double* theta, const double* partial, double* grad, cudaStream_t st);
 
 // CG / leapfrog / energy kernels (kmv_cg.cu)
 cudaError_t launch_cg_init(const DevLayout& L, int n_items, int chains, int64_t n_total,
@@ -152,11 +184,12 @@ cudaError_t launch_cg_reduce_init(const DevLayout& L, int n_inst, int chains, co
 cudaError_t launch_cg_reduce_pq(const DevLayout& L, int n_inst, int chains, const double* partial,
                                 CgSys* sys, int32_t* active, cudaStream_t st);
 // cg_update_xr followed, per system, by the r.r step of cg_reduce_rr in the CTA
-// that finishes last (count: one zeroed counter per system).
+// that finishes last (count: one zeroed counter per system), and for systems of at
+// most p_rows rows p = r + beta p by that CTA.
 cudaError_t launch_cg_update_xr_rr(const DevLayout& L, int n_items, int chains, int64_t n_total, CgSys* sys,
-                                   int32_t* active, float* x, float* r, const float* p, const float* q,
+                                   int32_t* active, float* x, float* r, float* p, const float* q,
                                    double* partial, uint32_t* count, double tol, int maxiter, int32_t* n_active,
-                                   cudaStream_t st);
+                                   int p_rows, cudaStream_t st);
 cudaError_t launch_cg_update_xr(const DevLayout& L, int n_items, int chains, int64_t n_total,
                                 const CgSys* sys, const int32_t* active, float* x, float* r,
                                 const float* p, const float* q, double* partial, cudaStream_t st);
@@ -388,11 +421,17 @@ struct kmv_handle_s {
   bool capturing = false;
   // stream on which the bodies of conditional (WHILE) graph nodes are captured
   cudaStream_t side = nullptr;
-  // FP32 forward's J-range split (kmv_simt_fwd.cu): per-chunk FP64 row sums,
-  // grown on first use (not under capture); the device's SM count
-  double* simt_part = nullptr;
+  // FP32 kernels: wide row tiles of the layout; the J units' partial sums and the
+  // zeroed counters, grown on first use (not under capture).  Outgrown buffers are
+  // kept until the handle goes, for graphs captured with them; they at least double,
+  // so all of them together stay below twice the last.
+  kmv::SimtTiles simt_tiles;
+  float2* simt_part = nullptr;
   size_t simt_part_bytes = 0;
-  int num_sms = 0;
+  uint32_t* simt_count = nullptr;
+  size_t simt_counters = 0;
+  std::vector<void*> simt_retired;
+  int num_sms = 0;   // of the device
   // kernel timing (kmv_profile_enable): event pairs around the main product kernels
   bool prof = false;
   std::vector<cudaEvent_t> prof_pool;

@@ -30,11 +30,16 @@
 namespace kmv {
 namespace {
 
+// Sum of a system's per-tile partials by one warp (every lane gets it).
 __device__ __forceinline__ double tile_sum(const DevLayout& L, int bi, int c, int chains, const double* partial) {
   double acc = 0.0;
-  for (int it = L.inst_item0[bi]; it < L.inst_item0[bi + 1]; ++it) acc += partial[(int64_t)it * chains + c];
+  for (int it = L.inst_item0[bi] + (int)(threadIdx.x & 31); it < L.inst_item0[bi + 1]; it += 32)
+    acc += partial[(int64_t)it * chains + c];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   return acc;
 }
+constexpr int kSysWarps = 4;   // systems (one warp each) per CTA of the per-system kernels
 
 // r = p = b, x_j = 0, p_j = b; partials of b.b
 __global__ void mscg_init_kernel(DevLayout L, int chains, int64_t n_total, int m, const float* b, float* r, float* p,
@@ -63,24 +68,15 @@ __global__ void mscg_init_kernel(DevLayout L, int chains, int64_t n_total, int m
 __global__ void mscg_setup_kernel(DevLayout L, int n_inst, int chains, int m, const double* partial,
                                   const float* shifts, double tol, MscgSys* sys, MscgShift* sh, float* base_shift,
                                   int32_t* sys_active, int32_t* n_active) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const int s = blockIdx.x * kSysWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (s >= n_inst * chains) return;
   const int bi = s / chains, c = s - bi * chains;
   const double bb = tile_sum(L, bi, c, chains, partial);
   float base = shifts[(int64_t)s * m];
   for (int j = 1; j < m; ++j) base = fminf(base, shifts[(int64_t)s * m + j]);
-  base_shift[s] = base;
   const bool finite = isfinite(bb);
   const int act = (finite && bb > 0.0 && tol < 1.0) ? 1 : 0;
-  MscgSys& y = sys[s];
-  y.rr = bb;
-  y.bb = bb;
-  y.alpha = 0.0;
-  y.beta = 0.0;
-  y.alpha_prev = 1.0;
-  y.beta_prev = 0.0;
-  y.iters = 0;
-  for (int j = 0; j < m; ++j) {
+  for (int j = lane; j < m; j += 32) {
     MscgShift& k = sh[(int64_t)s * m + j];
     k.sigma = (double)shifts[(int64_t)s * m + j] - (double)base;
     k.zeta = k.zeta_prev = k.zeta_next = 1.0;
@@ -89,6 +85,16 @@ __global__ void mscg_setup_kernel(DevLayout L, int n_inst, int chains, int m, co
     k.status = finite ? KMV_OK : KMV_ENONFINITE;
     k.active = act;
   }
+  if (lane != 0) return;
+  base_shift[s] = base;
+  MscgSys& y = sys[s];
+  y.rr = bb;
+  y.bb = bb;
+  y.alpha = 0.0;
+  y.beta = 0.0;
+  y.alpha_prev = 1.0;
+  y.beta_prev = 0.0;
+  y.iters = 0;
   sys_active[s] = act;
   if (act) atomicAdd(n_active, 1);
 }
@@ -96,10 +102,11 @@ __global__ void mscg_setup_kernel(DevLayout L, int n_inst, int chains, int m, co
 // alpha of the base CG and, per active shift, zeta_j' and alpha_j.
 __global__ void mscg_alpha_kernel(DevLayout L, int n_inst, int chains, int m, const double* partial, MscgSys* sys,
                                   MscgShift* sh, int32_t* sys_active) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const int s = blockIdx.x * kSysWarps + (threadIdx.x >> 5);
   if (s >= n_inst * chains || !sys_active[s]) return;
   const int bi = s / chains, c = s - bi * chains;
-  if (!mscg_alpha_step(sys[s], sh + (int64_t)s * m, m, tile_sum(L, bi, c, chains, partial))) sys_active[s] = 0;
+  const bool go = mscg_alpha_step(sys[s], sh + (int64_t)s * m, m, tile_sum(L, bi, c, chains, partial));
+  if (!go && (threadIdx.x & 31) == 0) sys_active[s] = 0;
 }
 
 // x_j += alpha_j p_j (active shifts), r -= alpha Bp; partials of the new r.r
@@ -138,10 +145,11 @@ __global__ void mscg_update_xr_kernel(DevLayout L, int chains, int64_t n_total, 
 __global__ void mscg_beta_kernel(DevLayout L, int n_inst, int chains, int m, const double* partial, double tol,
                                  int maxiter, MscgSys* sys, MscgShift* sh, int32_t* sys_active,
                                  int32_t* n_active) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const int s = blockIdx.x * kSysWarps + (threadIdx.x >> 5);
   if (s >= n_inst * chains || !sys_active[s]) return;
   const int bi = s / chains, c = s - bi * chains;
   const bool any = mscg_beta_step(sys[s], sh + (int64_t)s * m, m, tile_sum(L, bi, c, chains, partial), tol, maxiter);
+  if ((threadIdx.x & 31) != 0) return;
   sys_active[s] = any;
   if (any) atomicAdd(n_active, 1);
 }
@@ -156,6 +164,7 @@ __global__ void mscg_update_xr_beta_kernel(DevLayout L, int chains, int64_t n_to
   __shared__ double red[kTile / 32];
   __shared__ float as[kMaxShifts];
   __shared__ int on[kMaxShifts];
+  __shared__ int s_last;
   const int item = blockIdx.x, c = blockIdx.y;
   const int bi = L.item_inst[item];
   const int s = bi * chains + c;
@@ -179,11 +188,16 @@ __global__ void mscg_update_xr_beta_kernel(DevLayout L, int chains, int64_t n_to
   const double t = block_sum(rr, red);
   if (threadIdx.x == 0) {
     partial[(int64_t)item * chains + c] = t;
-    if (last_block_of_system(count, s, (uint32_t)(L.inst_item0[bi + 1] - L.inst_item0[bi])) &&
-        !mscg_beta_step(sys[s], sh + (int64_t)s * m, m, tile_sum(L, bi, c, chains, partial), tol, maxiter)) {
-      sys_active[s] = 0;
-      atomicSub(n_active, 1);
-    }
+    s_last = last_arrival(&count[s], 1u, (uint32_t)(L.inst_item0[bi + 1] - L.inst_item0[bi]));
+  }
+  __syncthreads();
+  if (!s_last) return;
+  double rr_new = sys_sum_block(L, bi, c, chains, partial, 1, 0, red);
+  if (threadIdx.x >= 32) return;
+  rr_new = __shfl_sync(0xffffffffu, rr_new, 0);
+  if (!mscg_beta_step(sys[s], sh + (int64_t)s * m, m, rr_new, tol, maxiter) && threadIdx.x == 0) {
+    sys_active[s] = 0;
+    atomicSub(n_active, 1);
   }
 }
 
@@ -234,7 +248,7 @@ cudaError_t launch_mscg_setup(const DevLayout& L, int n_inst, int chains, int m,
                               const float* shifts, double tol, MscgSys* sys, MscgShift* sh, float* base_shift,
                               int32_t* sys_active, int32_t* n_active, cudaStream_t st) {
   const int n = n_inst * chains;
-  mscg_setup_kernel<<<(n + 127) / 128, 128, 0, st>>>(L, n_inst, chains, m, partial, shifts, tol, sys, sh,
+  mscg_setup_kernel<<<(n + kSysWarps - 1) / kSysWarps, 32 * kSysWarps, 0, st>>>(L, n_inst, chains, m, partial, shifts, tol, sys, sh,
                                                      base_shift, sys_active, n_active);
   return cudaGetLastError();
 }
@@ -242,7 +256,7 @@ cudaError_t launch_mscg_setup(const DevLayout& L, int n_inst, int chains, int m,
 cudaError_t launch_mscg_alpha(const DevLayout& L, int n_inst, int chains, int m, const double* partial, MscgSys* sys,
                               MscgShift* sh, int32_t* sys_active, cudaStream_t st) {
   const int n = n_inst * chains;
-  mscg_alpha_kernel<<<(n + 127) / 128, 128, 0, st>>>(L, n_inst, chains, m, partial, sys, sh, sys_active);
+  mscg_alpha_kernel<<<(n + kSysWarps - 1) / kSysWarps, 32 * kSysWarps, 0, st>>>(L, n_inst, chains, m, partial, sys, sh, sys_active);
   return cudaGetLastError();
 }
 
@@ -259,7 +273,7 @@ cudaError_t launch_mscg_beta(const DevLayout& L, int n_inst, int chains, int m, 
                              int maxiter, MscgSys* sys, MscgShift* sh, int32_t* sys_active, int32_t* n_active,
                              cudaStream_t st) {
   const int n = n_inst * chains;
-  mscg_beta_kernel<<<(n + 127) / 128, 128, 0, st>>>(L, n_inst, chains, m, partial, tol, maxiter, sys, sh,
+  mscg_beta_kernel<<<(n + kSysWarps - 1) / kSysWarps, 32 * kSysWarps, 0, st>>>(L, n_inst, chains, m, partial, tol, maxiter, sys, sh,
                                                     sys_active, n_active);
   return cudaGetLastError();
 }

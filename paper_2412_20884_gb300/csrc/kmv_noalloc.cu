@@ -124,9 +124,11 @@ extern "C" kmv_status kmv_backward_noalloc(const kmv_points* pts, int32_t chains
   a.Y = grad_V;
   a.n_z = n_z;
   a.grad_partial = reinterpret_cast<double*>(base + o_part);
-  if (n_items > 0 && launch_backward_simt(a, (int)n_items, st) != cudaSuccess) return KMV_ECUDA;
-  if (launch_grad_finalize(L, pts->n_inst, chains, n_theta, pts->ard, pts->d, n_z, theta, a.grad_partial,
-                           grad_theta, st) != cudaSuccess)
+  // one unit per item: no scratch beyond the partials
+  const SimtBwd plan = simt_bwd_plan_plain((int)n_items, pts->d, m);
+  if (n_items > 0 && launch_backward_simt(a, plan, (int)n_items, st) != cudaSuccess) return KMV_ECUDA;
+  if (launch_grad_finalize(L, plan, pts->n_inst, chains, n_theta, theta, a.grad_partial, grad_theta, st) !=
+      cudaSuccess)
     return KMV_ECUDA;
   return cudaGetLastError() == cudaSuccess ? KMV_OK : KMV_ECUDA;
 }

@@ -1,244 +1,183 @@
-// Plain FP32 adjoint of L = sum G o (A V) on the FMA/MUFU pipes.
-//
-// Same tiling as the forward kernel: a CTA owns kTile rows i of one system
-// and one chunk of at most MP columns.  Per pair it recomputes K0_ij from
-// direct differences and forms
-//   W_ij = G_i . V_j             (this column chunk's share of (G V^T)_ij)
-//   Q_ij = W_ij K0_ij
-// and accumulates per row
-//   sum_j Q_ij                                   -> d/dlog alpha
-//   sum_j Q_ij (xh_ik - xh_jk)^2 (per k, or r^2) -> d/dlog l_k
-//   sum_j K0_ij G_j                              -> dL/dV = A G
-// With per-point amplitudes (Sec. 4) G and V enter as amp o G, amp o V.
-// Because every dA/dtheta_p is symmetric, summing W_ij over all ordered
-// pairs (i, j) gives the gradient without symmetrising W.  Per-CTA FP64
-// partials go to a buffer that launch_grad_finalize reduces in a fixed order.
-#include "simt_common.cuh"
+// Plain FP32 adjoint: the work split, the dispatch over dimensions and column
+// widths, and the reductions of its partial sums (the kernel is in
+// kmv_simt_bwd.cuh).
+#include <algorithm>
+
+#include "kmv_simt_bwd.cuh"
 
 namespace kmv {
 
-template <int D, int MP, bool ARD>
-__global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a) {
-  constexpr int DA = D ? D : kMaxD;
-  constexpr int DP = DA + 1;
-  constexpr int DG = ARD ? DA : 1;
-  const int dd = D ? D : a.d;
-  const int item = blockIdx.x, c = blockIdx.y, z = blockIdx.z;
-  const int b = a.L.item_inst[item];
-  const int s = b * a.chains + c;
-  if (a.sys_active && !a.sys_active[s]) return;
-
-  __shared__ float sc[DA];
-  __shared__ float sx[kJT * DP];
-  __shared__ float sv[kJT * MP];
-  __shared__ float sg[kJT * MP];
-  __shared__ double red[kTile / 32];
-
-  const int64_t j0 = a.L.offsets[b], j1 = a.L.offsets[b + 1];
-  const int64_t r0 = a.L.item_row0[item];
-  const int64_t i = r0 + threadIdx.x;
-  const bool valid = i < j1;
-  const double* th = a.theta + (int64_t)s * a.n_theta;
-  load_scale(th, dd, a.ard, sc);
-  const int c0 = z * MP;
-  const int mc = min(MP, a.m - c0);
-  const int64_t vbase = (int64_t)c * a.n_total;
-  const bool want_gv = a.Y != nullptr;
-  __syncthreads();
-
-  float xi[DA];
-  float gi[MP];
-#pragma unroll
-  for (int k = 0; k < DA; ++k) xi[k] = 0.f;
-#pragma unroll
-  for (int q = 0; q < MP; ++q) gi[q] = 0.f;
-  const float amp_i = (a.amp && valid) ? a.amp[vbase + i] : 1.f;
-  if (valid) {
-    for (int k = 0; k < dd; ++k) xi[k] = a.x[i * dd + k] * sc[k];
-#pragma unroll
-    for (int q = 0; q < MP; ++q)
-      if (q < mc) gi[q] = a.G[(vbase + i) * a.m + c0 + q] * amp_i;
-  }
-
-  float accq = 0.f, accg[DG], accv[MP];
-  double accq64 = 0.0, accg64[DG], accv64[MP];
-#pragma unroll
-  for (int k = 0; k < DG; ++k) { accg[k] = 0.f; accg64[k] = 0.0; }
-#pragma unroll
-  for (int q = 0; q < MP; ++q) { accv[q] = 0.f; accv64[q] = 0.0; }
-
-  int step = 0;
-  for (int64_t jt = j0; jt < j1; jt += kJT, ++step) {
-    const int nj = (int)min((int64_t)kJT, j1 - jt);
-    for (int e = threadIdx.x; e < kJT * dd; e += kTile) {
-      const int r = e / dd, k = e - r * dd;
-      sx[r * DP + k] = r < nj ? a.x[(jt + r) * dd + k] * sc[k] : 0.f;
-    }
-    for (int e = threadIdx.x; e < kJT * MP; e += kTile) {
-      const int r = e / MP, q = e - r * MP;
-      const bool in = r < nj && q < mc;
-      const int64_t idx = (vbase + jt + r) * a.m + c0 + q;
-      const float am = (in && a.amp) ? a.amp[vbase + jt + r] : 1.f;
-      sv[e] = in ? a.V[idx] * am : 0.f;
-      sg[e] = (in && want_gv) ? a.G[idx] * am : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 2
-    for (int jj = 0; jj < kJT; ++jj) {
-      float r2 = 0.f;
-      float df2[DG];
-      if (D) {
-#pragma unroll
-        for (int k = 0; k < DA; ++k) {
-          const float df = xi[k] - sx[jj * DP + k];
-          const float t = df * df;
-          if (ARD) df2[k] = t;
-          r2 += t;
-        }
-      } else {
-        for (int k = 0; k < dd; ++k) {
-          const float df = xi[k] - sx[jj * DP + k];
-          const float t = df * df;
-          if (ARD) df2[k] = t;
-          r2 += t;
-        }
-      }
-      const float p = ex2_approx(-r2);
-      float w = 0.f;
-#pragma unroll
-      for (int q = 0; q < MP; ++q) w = fmaf(gi[q], sv[jj * MP + q], w);
-      const float Q = w * p;
-      accq += Q;
-      if (ARD) {
-        if (D) {
-#pragma unroll
-          for (int k = 0; k < DG; ++k) accg[k] = fmaf(Q, df2[k], accg[k]);
-        } else {
-          for (int k = 0; k < dd; ++k) accg[k] = fmaf(Q, df2[k], accg[k]);
-        }
-      } else {
-        accg[0] = fmaf(Q, r2, accg[0]);
-      }
-      if (want_gv) {
-#pragma unroll
-        for (int q = 0; q < MP; ++q) accv[q] = fmaf(p, sg[jj * MP + q], accv[q]);
-      }
-    }
-    __syncthreads();
-    if ((step + 1) % (kFoldTiles * kTile / kJT) == 0) {
-      accq64 += (double)accq;
-      accq = 0.f;
-#pragma unroll
-      for (int k = 0; k < DG; ++k) { accg64[k] += (double)accg[k]; accg[k] = 0.f; }
-#pragma unroll
-      for (int q = 0; q < MP; ++q) { accv64[q] += (double)accv[q]; accv[q] = 0.f; }
-    }
-  }
-  accq64 += (double)accq;
-#pragma unroll
-  for (int k = 0; k < DG; ++k) accg64[k] += (double)accg[k];
-#pragma unroll
-  for (int q = 0; q < MP; ++q) accv64[q] += (double)accv[q];
-
-  double noise = 0.0;
-  if (valid) {
-    const double alpha = exp(th[0]);
-    const double s2 = exp(th[a.n_theta - 1]);
-#pragma unroll
-    for (int q = 0; q < MP; ++q) {
-      if (q < mc) {
-        const int64_t idx = (vbase + i) * a.m + c0 + q;
-        const double g = (double)a.G[idx];
-        noise += g * (double)a.V[idx];
-        if (want_gv) a.Y[idx] = (float)(alpha * (double)amp_i * accv64[q] + s2 * g);
-      }
-    }
-  }
-  // Per-CTA partials: [sum Q, sum Q d2 (k entries or 1), sum G.V]
-  double* out = a.grad_partial + (((int64_t)item * a.chains + c) * a.n_z + z) * a.n_theta;
-  double t = block_sum(accq64, red);
-  if (threadIdx.x == 0) out[0] = t;
-  const int kk = a.n_theta - 2;
-  for (int k = 0; k < kk; ++k) {
-    double v = 0.0;
-    if (ARD) {
-      if (D) {
-#pragma unroll
-        for (int u = 0; u < DG; ++u) v = (u == k) ? accg64[u] : v;
-      } else {
-        v = accg64[k];
-      }
-    } else {
-      v = accg64[0];
-    }
-    t = block_sum(v, red);
-    if (threadIdx.x == 0) out[1 + k] = t;
-  }
-  t = block_sum(noise, red);
-  if (threadIdx.x == 0) out[a.n_theta - 1] = t;
-}
+extern template cudaError_t bwd_launch_d<1, true>(const KmvArgs&, const SimtBwd&, dim3, cudaStream_t);
+extern template cudaError_t bwd_launch_d<1, false>(const KmvArgs&, const SimtBwd&, dim3, cudaStream_t);
+extern template cudaError_t bwd_launch_d<2, true>(const KmvArgs&, const SimtBwd&, dim3, cudaStream_t);
+extern template cudaError_t bwd_launch_d<2, false>(const KmvArgs&, const SimtBwd&, dim3, cudaStream_t);
+extern template cudaError_t bwd_launch_d<3, true>(const KmvArgs&, const SimtBwd&, dim3, cudaStream_t);
+extern template cudaError_t bwd_launch_d<3, false>(const KmvArgs&, const SimtBwd&, dim3, cudaStream_t);
+extern template cudaError_t bwd_launch_d<4, true>(const KmvArgs&, const SimtBwd&, dim3, cudaStream_t);
+extern template cudaError_t bwd_launch_d<4, false>(const KmvArgs&, const SimtBwd&, dim3, cudaStream_t);
+extern template cudaError_t bwd_launch_d<8, true>(const KmvArgs&, const SimtBwd&, dim3, cudaStream_t);
+extern template cudaError_t bwd_launch_d<8, false>(const KmvArgs&, const SimtBwd&, dim3, cudaStream_t);
+extern template cudaError_t bwd_launch_d<16, true>(const KmvArgs&, const SimtBwd&, dim3, cudaStream_t);
+extern template cudaError_t bwd_launch_d<16, false>(const KmvArgs&, const SimtBwd&, dim3, cudaStream_t);
+extern template cudaError_t bwd_launch_d<32, true>(const KmvArgs&, const SimtBwd&, dim3, cudaStream_t);
+extern template cudaError_t bwd_launch_d<32, false>(const KmvArgs&, const SimtBwd&, dim3, cudaStream_t);
+extern template cudaError_t bwd_launch_d<64, true>(const KmvArgs&, const SimtBwd&, dim3, cudaStream_t);
+extern template cudaError_t bwd_launch_d<64, false>(const KmvArgs&, const SimtBwd&, dim3, cudaStream_t);
 
 int backward_mp(int m) { return m >= kMaxMPBwd ? kMaxMPBwd : pow2ceil(m); }
 
-template <int MP, bool ARD>
-static cudaError_t bwd_by_d(const KmvArgs& a, dim3 grid, cudaStream_t st) {
-  switch (a.d) {
-    case 1: bwd_simt_kernel<1, MP, ARD><<<grid, kTile, 0, st>>>(a); break;
-    case 2: bwd_simt_kernel<2, MP, ARD><<<grid, kTile, 0, st>>>(a); break;
-    case 3: bwd_simt_kernel<3, MP, ARD><<<grid, kTile, 0, st>>>(a); break;
-    case 4: bwd_simt_kernel<4, MP, ARD><<<grid, kTile, 0, st>>>(a); break;
-    case 8: bwd_simt_kernel<8, MP, ARD><<<grid, kTile, 0, st>>>(a); break;
-    case 16: bwd_simt_kernel<16, MP, ARD><<<grid, kTile, 0, st>>>(a); break;
-    case 32: bwd_simt_kernel<32, MP, ARD><<<grid, kTile, 0, st>>>(a); break;
-    default: bwd_simt_kernel<0, MP, ARD><<<grid, kTile, 0, st>>>(a); break;
+namespace {
+
+constexpr int kDims[] = {1, 2, 3, 4, 8, 16, 32, 64};
+int dim_class(int d) {
+  for (int v : kDims)
+    if (d <= v) return v;
+  return 0;
+}
+
+// dL/dV = alpha amp sum_units part + sigma^2 G, 128 rows and kGvCols columns at a time.
+constexpr int kGvCols = 4;
+__global__ void __launch_bounds__(kTile) bwd_simt_combine_kernel(KmvArgs a, SimtBwd f) {
+  __shared__ double as2[2];
+  const int item = blockIdx.x, c = blockIdx.y;
+  const int b = a.L.item_inst[item];
+  const int s = b * a.chains + c;
+  if (a.sys_active && !a.sys_active[s]) return;
+  if (threadIdx.x < 2) as2[threadIdx.x] = exp(a.theta[(int64_t)s * a.n_theta + (threadIdx.x ? a.n_theta - 1 : 0)]);
+  const int64_t i = a.L.item_row0[item] + threadIdx.x;
+  const int64_t nb = a.L.offsets[b + 1] - a.L.offsets[b], len = (int64_t)f.folds * kFoldTiles * kTile;
+  const int units = (int)((nb + len - 1) / len);
+  __syncthreads();
+  if (i >= a.L.offsets[b + 1]) return;
+  const int64_t row = (int64_t)c * a.n_total + i;
+  const double ai = as2[0] * (double)(a.amp ? a.amp[row] : 1.f);
+  for (int c0 = blockIdx.z * kGvCols; c0 < a.m; c0 += gridDim.z * kGvCols) {
+    for (int q = c0; q < min(a.m, c0 + kGvCols); ++q) {
+      float sum = 0.f, err = 0.f;
+      for (int u = 0; u < units; ++u) {
+        const float2 p = f.part[(((size_t)u * a.chains + c) * a.m + q) * (size_t)a.n_total + i];
+        two_sum_add(sum, err, p.x);
+        err += p.y;
+      }
+      const int64_t idx = row * a.m + q;
+      a.Y[idx] = (float)(ai * ((double)sum + (double)err) + as2[1] * (double)a.G[idx]);
+    }
   }
-  return cudaGetLastError();
 }
 
-template <bool ARD>
-static cudaError_t bwd_by_mp(const KmvArgs& a, dim3 grid, int mp, cudaStream_t st) {
-  switch (mp) {
-    case 1: return bwd_by_d<1, ARD>(a, grid, st);
-    case 2: return bwd_by_d<2, ARD>(a, grid, st);
-    case 4: return bwd_by_d<4, ARD>(a, grid, st);
-    case 8: return bwd_by_d<8, ARD>(a, grid, st);
-    case 16: return bwd_by_d<16, ARD>(a, grid, st);
-    default: return bwd_by_d<32, ARD>(a, grid, st);
-  }
-}
-
-cudaError_t launch_backward_simt(const KmvArgs& a, int n_items, cudaStream_t st) {
-  const int mp = backward_mp(a.m);
-  dim3 grid(n_items, a.chains, a.n_z);
-  return a.ard ? bwd_by_mp<true>(a, grid, mp, st) : bwd_by_mp<false>(a, grid, mp, st);
-}
-
-// grad[s, p] = scale_p * sum over the instance's items and column chunks of partial[..., p]
-__global__ void grad_finalize_kernel(DevLayout L, int n_inst, int chains, int n_theta, int n_z,
-                                     const double* theta, const double* partial, double* grad) {
+// grad[s, p] = scale_p * sum over the instance's tiles, column chunks and units of
+// partial[..., p]: a warp per entry, lanes striding over the tiles, then a fixed
+// shuffle tree (one thread's serial chain over 157 items measured 75 us).
+constexpr int kGradThreads = 256;
+__global__ void __launch_bounds__(kGradThreads) grad_finalize_kernel(DevLayout L, SimtBwd f, int chains, int n_theta,
+                                                                     const double* theta, const double* partial,
+                                                                     double* grad) {
   const int s = blockIdx.x;
   const int b = s / chains, c = s - b * chains;
   const double* th = theta + (int64_t)s * n_theta;
-  for (int p = threadIdx.x; p < n_theta; p += blockDim.x) {
+  const int64_t nb = L.offsets[b + 1] - L.offsets[b], len = (int64_t)f.folds * kFoldTiles * kTile;
+  const int units = (int)((nb + len - 1) / len);
+  const int i0 = L.inst_item0[b], n_t = (L.inst_item0[b + 1] - i0 + f.rows - 1) / f.rows;
+  const int lane = threadIdx.x & 31;
+  const int n = n_t * f.nz * units;
+  for (int p = threadIdx.x >> 5; p < n_theta; p += kGradThreads / 32) {
     double acc = 0.0;
-    for (int it = L.inst_item0[b]; it < L.inst_item0[b + 1]; ++it)
-      for (int z = 0; z < n_z; ++z)
-        acc += partial[(((int64_t)it * chains + c) * n_z + z) * n_theta + p];
-    double scale;
-    if (p == 0) scale = exp(th[0]);
-    else if (p == n_theta - 1) scale = exp(th[n_theta - 1]);
-    else scale = exp(th[0]) / kHalfLog2e;
-    grad[(int64_t)s * n_theta + p] = scale * acc;
+    for (int e = lane; e < n; e += 32) {
+      const int u = e % units, tz = e / units, z = tz % f.nz, t = tz / f.nz;
+      acc += partial[((((int64_t)(i0 + t * f.rows) * chains + c) * f.nz + z) * f.units + u) * n_theta + p];
+    }
+    if (n <= 32) {
+      // few partials: in their order, whatever the batch around the system
+      double sum = 0.0;
+      for (int e = 0; e < n; ++e) sum += __shfl_sync(0xffffffffu, acc, e);
+      acc = sum;
+    } else {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    }
+    if (lane == 0) {
+      double scale;
+      if (p == 0) scale = exp(th[0]);
+      else if (p == n_theta - 1) scale = exp(th[n_theta - 1]);
+      else scale = exp(th[0]) / kHalfLog2e;
+      grad[(int64_t)s * n_theta + p] = scale * acc;
+    }
   }
 }
 
-cudaError_t launch_grad_finalize(const DevLayout& L, int n_inst, int chains, int n_theta, int ard,
-                                 int d, int n_z, const double* theta, const double* partial,
-                                 double* grad, cudaStream_t st) {
-  (void)ard;
+}  // namespace
+
+// Rows per thread and the number of J units: the wide variant once its finest split
+// (units of one fold) gives every SM two CTAs; then about 12 CTAs per SM, and with
+// dL/dV at most 512 MB of partial sums.
+SimtBwd simt_bwd_plan(const SimtTiles& T, int n_items, int chains, int64_t n_total, int64_t max_rows, int d, int m,
+                      bool want_gv, int num_sms) {
+  SimtBwd f = simt_bwd_plan_plain(n_items, d, m);
+  const int R = bwd_rows(dim_class(d), f.mp);
+  const int64_t fpc = std::max<int64_t>(1, (max_rows + kFoldTiles * kTile - 1) / (kFoldTiles * kTile));
+  const int64_t wide = (int64_t)(R == 4 ? T.n4 : R == 2 ? T.n2 : n_items) * chains * f.nz;
+  if (R > 1 && wide * fpc >= 2 * (int64_t)num_sms) {
+    f.rows = R;
+    f.tile_item = R == 4 ? T.item4 : T.item2;
+    f.n_tiles = R == 4 ? T.n4 : T.n2;
+  }
+  const int64_t ctas = (int64_t)f.n_tiles * chains * f.nz;
+  int64_t units = std::min<int64_t>(fpc, std::max<int64_t>(1, (12 * (int64_t)num_sms + ctas - 1) / std::max<int64_t>(1, ctas)));
+  units = std::min<int64_t>(units, std::max(1, 65535 / f.nz));
+  const int64_t bytes = want_gv ? (int64_t)sizeof(float2) * chains * m * std::max<int64_t>(1, n_total) : 0;
+  while (units > 1 && bytes * units > (int64_t(512) << 20)) --units;
+  f.folds = (int)((fpc + units - 1) / units);
+  f.units = (int)((fpc + f.folds - 1) / f.folds);
+  return f;
+}
+
+SimtBwd simt_bwd_plan_plain(int n_items, int d, int m) {
+  SimtBwd f{};
+  f.n_tiles = n_items;
+  f.rows = 1;
+  f.chunk = backward_mp(m);
+  f.mp = std::max(2, f.chunk);
+  f.nz = (m + f.chunk - 1) / f.chunk;
+  f.folds = 1 << 30;
+  f.units = 1;
   (void)d;
-  grad_finalize_kernel<<<n_inst * chains, 64, 0, st>>>(L, n_inst, chains, n_theta, n_z, theta,
-                                                       partial, grad);
+  return f;
+}
+
+size_t simt_bwd_partials(const SimtBwd& f, int n_items, int chains, int n_theta) {
+  return (size_t)std::max(1, n_items) * chains * f.nz * f.units * n_theta;
+}
+size_t simt_bwd_part_bytes(const SimtBwd& f, int chains, int64_t n_total, int m) {
+  return f.units > 1 || (f.folds > 1 && f.rows > 1) ? sizeof(float2) * (size_t)f.units * chains * m * (size_t)n_total : 0;
+}
+
+template <int D>
+static cudaError_t bwd_by_ard(const KmvArgs& a, const SimtBwd& f, dim3 grid, cudaStream_t st) {
+  return a.ard ? bwd_launch_d<D, true>(a, f, grid, st) : bwd_launch_d<D, false>(a, f, grid, st);
+}
+
+cudaError_t launch_backward_simt(const KmvArgs& a, const SimtBwd& f, int n_items, cudaStream_t st) {
+  const dim3 grid(f.n_tiles, a.chains, f.nz * f.units);
+  cudaError_t e = cudaErrorInvalidValue;
+  switch (dim_class(a.d)) {
+    case 1: e = bwd_by_ard<1>(a, f, grid, st); break;
+    case 2: e = bwd_by_ard<2>(a, f, grid, st); break;
+    case 3: e = bwd_by_ard<3>(a, f, grid, st); break;
+    case 4: e = bwd_by_ard<4>(a, f, grid, st); break;
+    case 8: e = bwd_by_ard<8>(a, f, grid, st); break;
+    case 16: e = bwd_by_ard<16>(a, f, grid, st); break;
+    case 32: e = bwd_by_ard<32>(a, f, grid, st); break;
+    case 64: e = bwd_by_ard<64>(a, f, grid, st); break;
+  }
+  if (e != cudaSuccess || f.units == 1 || !a.Y) return e;
+  const int gz = std::min(65535, (a.m + kGvCols - 1) / kGvCols);
+  bwd_simt_combine_kernel<<<dim3(n_items, a.chains, gz), kTile, 0, st>>>(a, f);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_grad_finalize(const DevLayout& L, const SimtBwd& f, int n_inst, int chains, int n_theta,
+                                 const double* theta, const double* partial, double* grad, cudaStream_t st) {
+  grad_finalize_kernel<<<n_inst * chains, kGradThreads, 0, st>>>(L, f, chains, n_theta, theta, partial, grad);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,326 @@
+// Plain FP32 adjoint of L = sum G o (A V) on the FMA/MUFU pipes: the kernel.
+//
+// Same tiling as the forward kernel (kmv_simt_fwd.cuh): a CTA owns R * kTile rows i
+// of one system, one chunk of at most MP columns and one range of columns j.  Per
+// pair it recomputes K0_ij from direct differences and forms
+//   W_ij = G_i . V_j             (this column chunk's share of (G V^T)_ij)
+//   Q_ij = W_ij K0_ij
+// and accumulates per row
+//   sum_j Q_ij                                   -> d/dlog alpha
+//   sum_j Q_ij (xh_ik - xh_jk)^2 (per k, or r^2) -> d/dlog l_k
+//   sum_j K0_ij G_j                              -> dL/dV = A G
+// With per-point amplitudes (Sec. 4) G and V enter as amp o G, amp o V.
+// Because every dA/dtheta_p is symmetric, summing W_ij over all ordered
+// pairs (i, j) gives the gradient without symmetrising W.  FP32 sums run over at
+// most 512 columns and are then folded into (sum, error) pairs; per-CTA FP64
+// partials go to a buffer that launch_grad_finalize reduces in a fixed order.
+//
+// What bounds it: per pair 4 D + 2 m + 3 operations of the FMA pipe (m columns with
+// dL/dV), one ex2, and the D + 2 m values of j that all lanes of a warp share (one
+// clock of shared memory each per warp, so R rows per thread divide them by R).  One
+// row per thread, one CTA per 128 rows and the whole J range took 4.38 ms at
+// N = 20,000, d = 8, m = 16 (157 CTAs: one per SM) and 84 us at N = 2048, d = 1,
+// m = 2 (16 CTAs); J units of 512 columns and R = 2 or 4 where rows are many give
+// the figures at simt_bwd_plan.
+#pragma once
+
+#include "simt_common.cuh"
+
+namespace kmv {
+
+constexpr int kXSB = kJT + 4;   // row stride of the staged x (floats)
+
+template <int D, int MP, int R, bool ARD>
+__global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
+  constexpr int DG = ARD ? D : 1;
+  const int dd = a.d;   // <= D; the dimensions past it are zero and add nothing
+  const int tile = blockIdx.x, c = blockIdx.y, u = blockIdx.z % f.units, z = blockIdx.z / f.units;
+  const int item0 = f.tile_item ? f.tile_item[tile] : tile;
+  const int b = a.L.item_inst[item0];
+  const int s = b * a.chains + c;
+  if (a.sys_active && !a.sys_active[s]) return;
+  const int64_t o0 = a.L.offsets[b], o1 = a.L.offsets[b + 1];
+  const int64_t len = (int64_t)f.folds * kFoldTiles * kTile;
+  const int64_t jb = o0 + u * len, je = min(o1, jb + len);
+  if (je <= jb) return;
+
+  // per staged row of V and G: MP columns each
+  __shared__ __align__(16) float sx[D * kXSB];
+  __shared__ __align__(16) float sv[kJT * MP];
+  __shared__ __align__(16) float sg[kJT * MP];
+  __shared__ float sc[D];
+  __shared__ double as2[2];
+  __shared__ double red[kTile / 32];
+
+  const int tid = threadIdx.x;
+  const double* th = a.theta + (int64_t)s * a.n_theta;
+  load_scale(th, dd, a.ard, sc);
+  const bool want_gv = a.Y != nullptr;
+  if (want_gv && tid >= 64 && tid < 66) as2[tid - 64] = exp(th[tid == 64 ? 0 : a.n_theta - 1]);
+  if (dd < D)
+    for (int e = tid; e < (D - dd) * kXSB; e += kTile) sx[dd * kXSB + e] = 0.f;
+  const int c0 = z * f.chunk;
+  const int mc = min(f.chunk, a.m - c0);
+  const int64_t vbase = (int64_t)c * a.n_total;
+  const int64_t r0 = a.L.item_row0[item0];
+  __syncthreads();
+
+  float xi[R][D], gi[R][MP], accq[R], accg[R][DG], accv[R][MP];
+  // running sums of the unit as pairs (several folds)
+  float sq[R], cq[R], sg2[R][DG], cg2[R][DG];
+  // those of dL/dV: in registers with one row per thread, else in f.part
+  constexpr int RV = R == 1 ? MP : 1;
+  float svp[RV], cvp[RV];
+#pragma unroll
+  for (int q = 0; q < RV; ++q) svp[q] = cvp[q] = 0.f;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int64_t i = r0 + r * kTile + tid;
+    const bool valid = i < o1;
+    const float amp_i = (a.amp && valid) ? a.amp[vbase + i] : 1.f;
+#pragma unroll
+    for (int k = 0; k < D; ++k) xi[r][k] = (k < dd && valid) ? a.x[i * dd + k] * sc[k] : 0.f;
+#pragma unroll
+    for (int q = 0; q < MP; ++q) {
+      gi[r][q] = (q < mc && valid) ? a.G[(vbase + i) * a.m + c0 + q] * amp_i : 0.f;
+      accv[r][q] = 0.f;
+    }
+    accq[r] = sq[r] = cq[r] = 0.f;
+#pragma unroll
+    for (int k = 0; k < DG; ++k) accg[r][k] = sg2[r][k] = cg2[r][k] = 0.f;
+  }
+
+  const uint32_t inv = dd > 1 ? 0xffffffffu / (uint32_t)dd + 1u : 0u;
+  const bool paired = je - jb > kFoldTiles * kTile;
+  bool first = true;
+  // dL/dV sums of this thread's rows into the pairs
+  auto fold_v = [&]() {
+    if constexpr (R == 1) {
+#pragma unroll
+      for (int q = 0; q < RV; ++q) {
+        two_sum_add(svp[q], cvp[q], accv[0][q]);
+        accv[0][q] = 0.f;
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int64_t i = r0 + r * kTile + tid;
+        if (i < o1) {
+#pragma unroll
+          for (int q = 0; q < MP; ++q)
+            if (q < mc) {
+              float2* p = &f.part[(((size_t)u * a.chains + c) * a.m + c0 + q) * (size_t)a.n_total + i];
+              float2 v = first ? make_float2(0.f, 0.f) : *p;
+              two_sum_add(v.x, v.y, accv[r][q]);
+              *p = v;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < MP; ++q) accv[r][q] = 0.f;
+      }
+      first = false;
+    }
+  };
+  auto fold_g = [&]() {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      two_sum_add(sq[r], cq[r], accq[r]);
+      accq[r] = 0.f;
+#pragma unroll
+      for (int k = 0; k < DG; ++k) {
+        two_sum_add(sg2[r][k], cg2[r][k], accg[r][k]);
+        accg[r][k] = 0.f;
+      }
+    }
+  };
+
+  int step = 0;
+  for (int64_t jt = jb; jt < je; jt += kJT, ++step) {
+    const int nj = (int)min((int64_t)kJT, je - jt);
+    for (int e = tid; e < kJT * dd; e += kTile) {
+      const int r = dd > 1 ? (int)__umulhi((uint32_t)e, inv) : e, k = e - r * dd;
+      sx[k * kXSB + r] = r < nj ? a.x[jt * dd + e] * sc[k] : 0.f;
+    }
+    for (int e = tid; e < kJT * MP; e += kTile) {
+      const int r = e / MP, q = e - r * MP;
+      const bool in = r < nj && q < mc;
+      const int64_t idx = (vbase + jt + r) * a.m + c0 + q;
+      const float am = (in && a.amp) ? a.amp[vbase + jt + r] : 1.f;
+      sv[e] = in ? a.V[idx] * am : 0.f;
+      sg[e] = (in && want_gv) ? a.G[idx] * am : 0.f;
+    }
+    __syncthreads();
+    // two points j at a time (their chains interleave), all R rows
+#pragma unroll 1
+    for (int jj = 0; jj < kJT; jj += 2) {
+      float r2[R][2], df2[R][2][DG];
+#pragma unroll
+      for (int r = 0; r < R; ++r) r2[r][0] = r2[r][1] = 0.f;
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        const float2 x2 = *reinterpret_cast<const float2*>(sx + k * kXSB + jj);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int t = 0; t < 2; ++t) {
+            const float df = __fsub_rn(xi[r][k], t ? x2.y : x2.x);
+            if (ARD) {
+              const float q2 = __fmul_rn(df, df);
+              df2[r][t][ARD ? k : 0] = q2;
+              r2[r][t] = __fadd_rn(r2[r][t], q2);
+            } else {
+              r2[r][t] = __fmaf_rn(df, df, r2[r][t]);
+            }
+          }
+      }
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        float w[R], p[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          w[r] = 0.f;
+          p[r] = ex2_approx(-r2[r][t]);
+        }
+        const float* vj = sv + (jj + t) * MP;
+        const float* gj = sg + (jj + t) * MP;
+        constexpr int QS = MP < 4 ? MP : 4;
+        float vv[QS];
+#pragma unroll
+        for (int q = 0; q < MP; q += QS) {
+          if constexpr (QS == 4) {
+            const float4 v = *reinterpret_cast<const float4*>(vj + q);
+            vv[0] = v.x;
+            vv[1 % QS] = v.y;
+            vv[2 % QS] = v.z;
+            vv[3 % QS] = v.w;
+          } else {
+            const float2 v = *reinterpret_cast<const float2*>(vj + q);
+            vv[0] = v.x;
+            vv[1 % QS] = v.y;
+          }
+#pragma unroll
+          for (int e = 0; e < QS; ++e)
+#pragma unroll
+            for (int r = 0; r < R; ++r) w[r] = __fmaf_rn(gi[r][q + e], vv[e], w[r]);
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const float Q = __fmul_rn(w[r], p[r]);
+          accq[r] = __fadd_rn(accq[r], Q);
+          if (ARD) {
+#pragma unroll
+            for (int k = 0; k < DG; ++k) accg[r][k] = __fmaf_rn(Q, df2[r][t][k], accg[r][k]);
+          } else {
+            accg[r][0] = __fmaf_rn(Q, r2[r][t], accg[r][0]);
+          }
+        }
+        if (want_gv) {
+#pragma unroll
+          for (int q = 0; q < MP; q += QS) {
+            if constexpr (QS == 4) {
+              const float4 v = *reinterpret_cast<const float4*>(gj + q);
+              vv[0] = v.x;
+              vv[1 % QS] = v.y;
+              vv[2 % QS] = v.z;
+              vv[3 % QS] = v.w;
+            } else {
+              const float2 v = *reinterpret_cast<const float2*>(gj + q);
+              vv[0] = v.x;
+              vv[1 % QS] = v.y;
+            }
+#pragma unroll
+            for (int e = 0; e < QS; ++e)
+#pragma unroll
+              for (int r = 0; r < R; ++r) accv[r][q + e] = __fmaf_rn(p[r], vv[e], accv[r][q + e]);
+          }
+        }
+      }
+    }
+    __syncthreads();
+    if (paired && jt + kJT < je && (step + 1) % (kFoldTiles * kTile / kJT) == 0) {
+      fold_g();
+      if (want_gv) fold_v();
+    }
+  }
+  fold_g();
+  const bool direct = f.units == 1;
+  if (want_gv && (R == 1 || !direct || paired)) fold_v();
+  if (R == 1 && want_gv && !direct && r0 + tid < o1) {
+#pragma unroll
+    for (int q = 0; q < RV; ++q)
+      if (q < mc)
+        f.part[(((size_t)u * a.chains + c) * a.m + c0 + q) * (size_t)a.n_total + r0 + tid] = make_float2(svp[q], cvp[q]);
+  }
+
+  // noise gradient and, in a single unit, dL/dV
+  double noise = 0.0;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int64_t i = r0 + r * kTile + tid;
+    if (i < o1 && (u == 0 || (want_gv && direct))) {
+      const double ai = want_gv ? as2[0] * (double)(a.amp ? a.amp[vbase + i] : 1.f) : 0.0;
+#pragma unroll
+      for (int q = 0; q < MP; ++q) {
+        if (q < mc) {
+          const int64_t idx = (vbase + i) * a.m + c0 + q;
+          const double g = (double)a.G[idx];
+          if (u == 0) noise += g * (double)a.V[idx];
+          if (want_gv && direct) {
+            float2 v = R == 1 ? make_float2(svp[q % RV], cvp[q % RV]) : make_float2(accv[r][q], 0.f);
+            if (R > 1 && paired) v = f.part[((size_t)c * a.m + c0 + q) * (size_t)a.n_total + i];
+            a.Y[idx] = (float)(ai * ((double)v.x + (double)v.y) + as2[1] * g);
+          }
+        }
+      }
+    }
+  }
+  // Per-CTA partials: [sum Q, sum Q d2 (k entries or 1), sum G.V]
+  double* out = a.grad_partial + ((((int64_t)item0 * a.chains + c) * f.nz + z) * f.units + u) * a.n_theta;
+  auto put = [&](int p, double v) {
+    const double t = block_sum(v, red);
+    if (tid == 0) out[p] = t;
+  };
+  double v = 0.0;
+#pragma unroll
+  for (int r = 0; r < R; ++r) v += (double)sq[r] + (double)cq[r];
+  put(0, v);
+#pragma unroll
+  for (int k = 0; k < DG; ++k) {
+    if (k < (ARD ? dd : 1)) {
+      v = 0.0;
+#pragma unroll
+      for (int r = 0; r < R; ++r) v += (double)sg2[r][k] + (double)cg2[r][k];
+      put(1 + k, v);
+    }
+  }
+  put(a.n_theta - 1, noise);
+}
+
+// Rows per thread of the wide variant: R (2 D + 2 MP + D) registers and more.
+constexpr int bwd_rows(int D, int MP) { return D <= 4 && MP <= 4 ? 4 : D + MP <= 32 ? 2 : 1; }
+
+template <int D, int MP, bool ARD>
+cudaError_t bwd_launch_mp(const KmvArgs& a, const SimtBwd& f, dim3 grid, cudaStream_t st) {
+  if (f.rows == 1) {
+    bwd_simt_kernel<D, MP, 1, ARD><<<grid, kTile, 0, st>>>(a, f);
+    return cudaGetLastError();
+  }
+  constexpr int R = bwd_rows(D, MP);
+  if (f.rows != R) return cudaErrorInvalidValue;
+  if constexpr (R > 1) bwd_simt_kernel<D, MP, R, ARD><<<grid, kTile, 0, st>>>(a, f);
+  return cudaGetLastError();
+}
+
+// The kernel for the dimension class D (kmv_simt_bwd_*.cu hold the instances).
+template <int D, bool ARD>
+cudaError_t bwd_launch_d(const KmvArgs& a, const SimtBwd& f, dim3 grid, cudaStream_t st) {
+  switch (f.mp) {
+    case 2: return bwd_launch_mp<D, 2, ARD>(a, f, grid, st);
+    case 4: return bwd_launch_mp<D, 4, ARD>(a, f, grid, st);
+    case 8: return bwd_launch_mp<D, 8, ARD>(a, f, grid, st);
+    case 16: return bwd_launch_mp<D, 16, ARD>(a, f, grid, st);
+    default: return bwd_launch_mp<D, 32, ARD>(a, f, grid, st);
+  }
+}
+
+}  // namespace kmv

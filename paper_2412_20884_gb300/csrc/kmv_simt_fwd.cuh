@@ -1,0 +1,394 @@
+// Plain FP32 forward product Y = A(theta) V on the FMA/MUFU pipes: the kernel.
+//
+// A CTA of kTile threads owns R * kTile rows i of one (instance, chain) system
+// (thread t the rows t, t + 128, ..), one chunk of at most MP columns of V and one
+// range of columns j.  It streams the points j through shared memory kJT at a time
+// and, per pair, evaluates
+//   K0_ij = 2^(-sum_k (xh_ik - xh_jk)^2),  xh = x sqrt(log2(e)/2) / l,
+// from direct differences (no |x|^2 expansion, so no cancellation), then
+// accumulates K0_ij V_j in FP32.  Every 512 columns the FP32 sums are folded into
+// (sum, error) pairs (two_sum_add).  Epilogue (Eq. kerdef): Y_i = alpha * acc_i +
+// (sigma^2 + shift) V_i.  With per-point amplitudes (the kernel family of Sec. 4)
+// V_j enters as amp_j V_j and acc_i is scaled by amp_i.
+//
+// What bounds it: per pair 2 D + m operations of the FMA pipe (128 lanes per clock
+// and SM), one ex2 (32 per clock), and a load of the D + m values of j that every
+// lane of a warp shares.  Such a broadcast still returns 128 bytes per clock and SM,
+// so with one row per thread the loads alone took D + m clocks per 32 pairs against
+// (2 D + m) / 4 for the arithmetic; R = 4 rows per thread divide them by four, and
+// the loads are 16 bytes wide (x is staged dimension by dimension).  The same
+// arithmetic in packed f32x2 form was measured at the same rate per lane
+// (60 packed against 114 scalar instructions per clock and SM), so it is not used.
+// At N = 20,000, d = 8, m = 16 one row per thread and one CTA per SM took 2.18 ms;
+// at N = 8192, d = 3, 8 chains, m = 1 0.274 ms (figures after the change stand at
+// simt_fwd_plan).
+#pragma once
+
+#include "cg_common.cuh"
+#include "simt_common.cuh"
+
+namespace kmv {
+
+constexpr int kXS = kJT + 4;   // row stride of the staged x (floats): 16-byte aligned, spreads the writes over banks
+
+// The J units of an instance of nb rows: chunks of `per` J tiles, units of `span`
+// tiles within them (32-bit arithmetic: a 64-bit division takes some 490 clocks).
+struct SimtUnits {
+  uint32_t n_jt, per, span, n_chunks;
+  __device__ __forceinline__ SimtUnits(const SimtFwd& f, int64_t nb) {
+    n_jt = (uint32_t)((nb + kJT - 1) / kJT);
+    per = f.js > 1 ? (n_jt + f.js - 1) / f.js : n_jt;
+    span = (uint32_t)f.folds * (kFoldTiles * kTile / kJT);
+    n_chunks = f.js > 1 ? (n_jt + per - 1) / per : 1;
+  }
+  // first J tile and end of unit u of chunk jc; empty when not less
+  __device__ __forceinline__ void range(uint32_t jc, uint32_t u, uint32_t& t0, uint32_t& t1) const {
+    t0 = jc * per + u * span;
+    t1 = min(min(n_jt, (jc + 1) * per), t0 + span);
+  }
+  __device__ __forceinline__ uint32_t in_chunk(uint32_t jc) const {
+    return (min(n_jt, (jc + 1) * per) - jc * per + span - 1) / span;
+  }
+  __device__ __forceinline__ uint32_t count() const { return (n_chunks - 1) * in_chunk(0) + in_chunk(n_chunks - 1); }
+};
+__device__ __forceinline__ size_t simt_part_at(const KmvArgs& a, int unit, int c, int col, int64_t i) {
+  return (((size_t)unit * a.chains + c) * a.m + col) * (size_t)a.n_total + i;
+}
+
+// Sum of the units' pairs of one element, in unit order.
+__device__ __forceinline__ double simt_part_sum(const KmvArgs& a, const SimtFwd& f, const SimtUnits& U, int c, int col,
+                                                int64_t i) {
+  float s = 0.f, e = 0.f;
+  const size_t step = (size_t)a.chains * a.m * (size_t)a.n_total;
+  for (uint32_t jc = 0; jc < U.n_chunks; ++jc) {
+    const float2* p = f.part + simt_part_at(a, jc * f.upc, c, col, i);
+    const uint32_t n = f.upc == 1 ? 1u : U.in_chunk(jc);
+#pragma unroll 4
+    for (uint32_t u = 0; u < n; ++u) {
+      const float2 v = __ldcg(p + u * step);
+      two_sum_add(s, e, v.x);
+      e += v.y;
+    }
+  }
+  return (double)s + (double)e;
+}
+
+// alpha and sigma^2 of a system: two lanes, one exp (an FP64 exp takes some 1100
+// clocks, and 2 lanes per clock and SM: once per CTA, not per thread).
+__device__ __forceinline__ void load_alpha_s2(const KmvArgs& a, int s, double* as2) {
+  if (threadIdx.x < 2) {
+    const double* th = a.theta + (int64_t)s * a.n_theta;
+    as2[threadIdx.x] = exp(th[threadIdx.x ? a.n_theta - 1 : 0]);
+  }
+}
+
+// One element of Y from its sum; returns V_i Y_i.
+__device__ __forceinline__ double simt_put_y(const KmvArgs& a, int s, int c, int64_t i, int col, double ai, double s2,
+                                             double sum) {
+  const int64_t idx = ((int64_t)c * a.n_total + i) * a.m + col;
+  const double shift = a.col_shift ? (double)a.col_shift[(int64_t)s * a.col_shift_stride + col] : 0.0;
+  const double vi = (double)a.V[idx];
+  const double y = ai * sum + (a.no_diag ? 0.0 : (s2 + shift) * vi);
+  a.Y[idx] = (float)y;
+  if (a.Y64) a.Y64[idx] = y;
+  return vi * y;
+}
+
+// The dot partials of `n` items starting at item0 (dots[r] of this thread's row in
+// item item0 + r), and inside a CG iteration the system's p.q step by the CTA that
+// completes it.
+template <int R>
+__device__ __forceinline__ void simt_put_dots(const KmvArgs& a, int b, int c, int s, int item0, int n,
+                                              const double (&dots)[R], double* red, int* s_flag) {
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    if (r < n) {
+      const double t = block_sum(dots[r], red);
+      if (threadIdx.x == 0) a.dot_partial[(int64_t)(item0 + r) * a.chains + c] = t;
+    }
+  }
+  if (!(a.cg_sys || a.ms_sys)) return;
+  if (threadIdx.x == 0)
+    *s_flag = last_arrival(&a.cg_count[s], (uint32_t)n, (uint32_t)(a.L.inst_item0[b + 1] - a.L.inst_item0[b]));
+  __syncthreads();
+  if (*s_flag) cg_finish_pq(a.L, a, b, c, s, red);
+}
+
+template <int D, int MP, int R>
+__global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
+  const int dd = a.d;   // <= D; the dimensions past it are zero and add nothing
+  const int tile = blockIdx.x, c = blockIdx.y;
+  const int u = blockIdx.z % f.upc, jc = (blockIdx.z / f.upc) % f.js, z = f.z0 + blockIdx.z / f.max_units;
+  const int item0 = f.tile_item ? f.tile_item[tile] : tile;
+  // one instance needs no look-ups (three dependent loads at the start of a small call)
+  const bool single = f.n_inst == 1;
+  const int b = single ? 0 : a.L.item_inst[item0];
+  const int s = b * a.chains + c;
+  if (a.sys_active && !a.sys_active[s]) return;
+  const int64_t o0 = single ? 0 : a.L.offsets[b], o1 = single ? a.n_total : a.L.offsets[b + 1];
+  const SimtUnits U(f, o1 - o0);
+  uint32_t t0, t1;
+  U.range(jc, u, t0, t1);
+  if (t1 <= t0) return;
+  const int64_t jb = o0 + (int64_t)t0 * kJT, je = min(o1, o0 + (int64_t)t1 * kJT);
+
+  __shared__ __align__(16) float sx[2][D * kXS];
+  __shared__ __align__(16) float sv[2][kJT * MP];
+  __shared__ float sc[D];
+  __shared__ double as2[2];
+  __shared__ double red[kTile / 32];
+  __shared__ int s_flag;
+
+  const int tid = threadIdx.x;
+  const double* th = a.theta + (int64_t)s * a.n_theta;
+  // the scales, and by two lanes of another warp alpha and sigma^2 (read at the end)
+  load_scale(th, dd, a.ard, sc);
+  if ((f.max_units == 1 || f.ticket) && tid >= 96 && tid < 98) as2[tid - 96] = exp(th[tid == 96 ? 0 : a.n_theta - 1]);
+  if (dd < D)
+    for (int e = tid; e < (D - dd) * kXS; e += kTile) sx[0][dd * kXS + e] = sx[1][dd * kXS + e] = 0.f;
+  const int c0 = z * MP;
+  const int mc = min(MP, a.m - c0);
+  const int64_t vbase = (int64_t)c * a.n_total;
+  const int64_t r0 = single ? (int64_t)item0 * kTile : a.L.item_row0[item0];
+  __syncthreads();
+
+  float xi[R][D], acc[R][MP];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int64_t i = r0 + r * kTile + tid;
+#pragma unroll
+    for (int k = 0; k < D; ++k) xi[r][k] = (k < dd && i < o1) ? a.x[i * dd + k] * sc[k] : 0.f;
+#pragma unroll
+    for (int q = 0; q < MP; ++q) acc[r][q] = 0.f;
+  }
+
+  // the next J tile's points and vectors, loaded into registers while the current
+  // one is worked on; e / dd by a multiplication (exact for e < 2^16)
+  constexpr int NX = (kJT * D + kTile - 1) / kTile, NV = (kJT * MP + kTile - 1) / kTile;
+  float fx[NX], fv[NV];
+  const uint32_t inv = dd > 1 ? 0xffffffffu / (uint32_t)dd + 1u : 0u;
+  auto split = [&](int e, int& r, int& k) {
+    r = dd > 1 ? (int)__umulhi((uint32_t)e, inv) : e;
+    k = e - r * dd;
+  };
+  auto fetch = [&](int64_t jt) {
+    const int nj = (int)min((int64_t)kJT, je - jt);
+#pragma unroll
+    for (int n = 0; n < NX; ++n) {
+      const int e = n * kTile + tid;
+      if (e < nj * dd) {
+        int r, k;
+        split(e, r, k);
+        fx[n] = a.x[jt * dd + e] * sc[k];
+      } else {
+        fx[n] = 0.f;
+      }
+    }
+#pragma unroll
+    for (int n = 0; n < NV; ++n) {
+      const int e = n * kTile + tid, r = e / MP, q = e - r * MP;
+      fv[n] = (r < nj && q < mc) ? a.V[(vbase + jt + r) * a.m + c0 + q] * (a.amp ? a.amp[vbase + jt + r] : 1.f) : 0.f;
+    }
+  };
+  auto store = [&](int buf) {
+#pragma unroll
+    for (int n = 0; n < NX; ++n) {
+      const int e = n * kTile + tid;
+      if (e < kJT * dd) {
+        int r, k;
+        split(e, r, k);
+        sx[buf][k * kXS + r] = fx[n];
+      }
+    }
+#pragma unroll
+    for (int n = 0; n < NV; ++n) {
+      const int e = n * kTile + tid;
+      if (NV * kTile == kJT * MP || e < kJT * MP) sv[buf][e] = fv[n];
+    }
+  };
+
+  const bool paired = je - jb > kFoldTiles * kTile;   // several folds: sums kept as pairs in f.part
+  const int unit = jc * f.upc + u;
+  bool first = true;
+  // adds the FP32 sums to the pairs in global memory (this thread's own elements)
+  auto fold = [&]() {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int64_t i = r0 + r * kTile + tid;
+      if (i < o1) {
+#pragma unroll
+        for (int q = 0; q < MP; ++q)
+          if (q < mc) {
+            float2* p = &f.part[simt_part_at(a, unit, c, c0 + q, i)];
+            float2 v = first ? make_float2(0.f, 0.f) : *p;
+            two_sum_add(v.x, v.y, acc[r][q]);
+            *p = v;
+          }
+      }
+#pragma unroll
+      for (int q = 0; q < MP; ++q) acc[r][q] = 0.f;
+    }
+    first = false;
+  };
+
+  fetch(jb);
+  store(0);
+  __syncthreads();
+  int step = 0;
+  for (int64_t jt = jb; jt < je; jt += kJT, ++step) {
+    const int buf = step & 1;
+    const bool more = jt + kJT < je;
+    if (more) fetch(jt + kJT);
+    const float* X = sx[buf];
+    const float* V = sv[buf];
+#pragma unroll 1
+    for (int jj = 0; jj < kJT; jj += 4) {
+      float p[R][4];
+#pragma unroll
+      for (int r = 0; r < R; ++r) p[r][0] = p[r][1] = p[r][2] = p[r][3] = 0.f;
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        const float4 x4 = *reinterpret_cast<const float4*>(X + k * kXS + jj);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const float d0 = __fsub_rn(xi[r][k], x4.x), d1 = __fsub_rn(xi[r][k], x4.y);
+          const float d2 = __fsub_rn(xi[r][k], x4.z), d3 = __fsub_rn(xi[r][k], x4.w);
+          p[r][0] = fmaf(d0, d0, p[r][0]);
+          p[r][1] = fmaf(d1, d1, p[r][1]);
+          p[r][2] = fmaf(d2, d2, p[r][2]);
+          p[r][3] = fmaf(d3, d3, p[r][3]);
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) p[r][t] = ex2_approx(-p[r][t]);
+      // the vectors of the four points: 4 MP consecutive floats
+      constexpr int NQ = MP < 4 ? MP : 4;   // float4 loads per step of 4 / (MP < 4 ? MP : 4) .. columns
+      if (MP == 1) {
+        const float4 v = *reinterpret_cast<const float4*>(V + jj);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          acc[r][0] = fmaf(p[r][0], v.x, acc[r][0]);
+          acc[r][0] = fmaf(p[r][1], v.y, acc[r][0]);
+          acc[r][0] = fmaf(p[r][2], v.z, acc[r][0]);
+          acc[r][0] = fmaf(p[r][3], v.w, acc[r][0]);
+        }
+      } else if (MP == 2) {
+        const float4 va = *reinterpret_cast<const float4*>(V + 2 * jj);
+        const float4 vb = *reinterpret_cast<const float4*>(V + 2 * jj + 4);
+        constexpr int q1 = MP > 1 ? 1 : 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          acc[r][0] = fmaf(p[r][0], va.x, acc[r][0]);
+          acc[r][q1] = fmaf(p[r][0], va.y, acc[r][q1]);
+          acc[r][0] = fmaf(p[r][1], va.z, acc[r][0]);
+          acc[r][q1] = fmaf(p[r][1], va.w, acc[r][q1]);
+          acc[r][0] = fmaf(p[r][2], vb.x, acc[r][0]);
+          acc[r][q1] = fmaf(p[r][2], vb.y, acc[r][q1]);
+          acc[r][0] = fmaf(p[r][3], vb.z, acc[r][0]);
+          acc[r][q1] = fmaf(p[r][3], vb.w, acc[r][q1]);
+        }
+      } else {
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+#pragma unroll
+          for (int q = 0; q < MP; q += NQ) {
+            const float4 v = *reinterpret_cast<const float4*>(V + (jj + t) * MP + q);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+              acc[r][(q + 0) % MP] = fmaf(p[r][t], v.x, acc[r][(q + 0) % MP]);
+              acc[r][(q + 1) % MP] = fmaf(p[r][t], v.y, acc[r][(q + 1) % MP]);
+              acc[r][(q + 2) % MP] = fmaf(p[r][t], v.z, acc[r][(q + 2) % MP]);
+              acc[r][(q + 3) % MP] = fmaf(p[r][t], v.w, acc[r][(q + 3) % MP]);
+            }
+          }
+      }
+    }
+    if (more) store(buf ^ 1);
+    __syncthreads();
+    if (paired && more && (step + 1) % (kFoldTiles * kTile / kJT) == 0) fold();
+  }
+
+  const int n_it = min(R, a.L.inst_item0[b + 1] - item0);
+  double dots[R];
+  if (f.max_units == 1) {
+    const double alpha = as2[0], s2 = as2[1];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      dots[r] = 0.0;
+      const int64_t i = r0 + r * kTile + tid;
+      if (i < o1) {
+        const double ai = a.amp ? alpha * (double)a.amp[vbase + i] : alpha;
+#pragma unroll
+        for (int q = 0; q < MP; ++q)
+          if (q < mc) {
+            float2 v = make_float2(0.f, 0.f);
+            if (paired) v = f.part[simt_part_at(a, 0, c, c0 + q, i)];
+            two_sum_add(v.x, v.y, acc[r][q]);
+            dots[r] += simt_put_y(a, s, c, i, c0 + q, ai, s2, (double)v.x + (double)v.y);
+          }
+      }
+    }
+    if (a.dot_partial) simt_put_dots<R>(a, b, c, s, item0, n_it, dots, red, &s_flag);
+    return;
+  }
+  fold();
+  if (!f.ticket) return;
+  // the tile's last unit to finish adds the units in order
+  __syncthreads();
+  if (tid == 0)
+    s_flag = last_arrival(&f.count[((size_t)tile * a.chains + c) * f.nz + z], 1u, U.count());
+  __syncthreads();
+  if (!s_flag) return;
+  const double alpha = as2[0], s2 = as2[1];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    dots[r] = 0.0;
+    const int64_t i = r0 + r * kTile + tid;
+    if (i < o1) {
+      const double ai = a.amp ? alpha * (double)a.amp[vbase + i] : alpha;
+      for (int q = 0; q < mc; ++q)
+        dots[r] += simt_put_y(a, s, c, i, c0 + q, ai, s2, simt_part_sum(a, f, U, c, c0 + q, i));
+    }
+  }
+  if (a.dot_partial) simt_put_dots<R>(a, b, c, s, item0, n_it, dots, red, &s_flag);
+}
+
+// Rows per thread of the wide variant (more rows cost registers: R (D + MP) and
+// the probabilities of four points stay below the 255 of a thread).
+constexpr int fwd_rows(int D, int MP) { return D <= 8 || (D <= 16 && MP <= 16) ? 4 : D <= 32 ? 2 : 1; }
+
+// The widest chunk built: 32 columns where the distances cost as much as they do (and
+// the staged tiles fit 48 KB); below, two 16-column chunks of four rows are cheaper
+// than one of 32 columns and two rows.
+constexpr int fwd_most_columns(int D) { return D >= 16 && D <= 32 ? 32 : 16; }
+
+template <int D, int MP>
+cudaError_t fwd_launch_mp(const KmvArgs& a, const SimtFwd& f, dim3 grid, cudaStream_t st) {
+  if (f.rows == 1) {
+    fwd_simt_kernel<D, MP, 1><<<grid, kTile, 0, st>>>(a, f);
+    return cudaGetLastError();
+  }
+  constexpr int R = fwd_rows(D, MP);
+  if (f.rows != R) return cudaErrorInvalidValue;
+  if constexpr (R > 1) fwd_simt_kernel<D, MP, R><<<grid, kTile, 0, st>>>(a, f);
+  return cudaGetLastError();
+}
+
+// The kernel for the dimension class D (kmv_simt_fwd_*.cu hold the instances).
+template <int D>
+cudaError_t fwd_launch_d(const KmvArgs& a, const SimtFwd& f, dim3 grid, cudaStream_t st) {
+  switch (f.mp) {
+    case 1: return fwd_launch_mp<D, 1>(a, f, grid, st);
+    case 2: return fwd_launch_mp<D, 2>(a, f, grid, st);
+    case 4: return fwd_launch_mp<D, 4>(a, f, grid, st);
+    case 8: return fwd_launch_mp<D, 8>(a, f, grid, st);
+    case 16: return fwd_launch_mp<D, 16>(a, f, grid, st);
+    default:
+      if constexpr (fwd_most_columns(D) == 32) return fwd_launch_mp<D, 32>(a, f, grid, st);
+      return cudaErrorInvalidValue;
+  }
+}
+
+}  // namespace kmv

@@ -943,6 +943,7 @@ __global__ void tc_fwd_epilogue_kernel(DevLayout L, TcTables T, KmvArgs a, int c
                                        const uint32_t* vmax, const int* err) {
   __shared__ double red[kTile / 32];
   __shared__ double s_alpha, s_s2;
+  __shared__ int s_last;
   const int item = blockIdx.x, c = blockIdx.y;
   const int b = L.item_inst[item];
   const int s = b * a.chains + c;
@@ -986,20 +987,16 @@ __global__ void tc_fwd_epilogue_kernel(DevLayout L, TcTables T, KmvArgs a, int c
   }
   if (a.dot_partial) {
     const double tsum = block_sum(dot, red);
+    const bool cg = a.cg_sys || a.ms_sys;
     if (threadIdx.x == 0) {
       a.dot_partial[(int64_t)item * a.chains + c] = tsum;
+      s_last = cg && last_arrival(&a.cg_count[s], 1u, (uint32_t)(L.inst_item0[b + 1] - L.inst_item0[b]));
+    }
+    if (cg) {
       // inside a (multi-shift) CG iteration: the system's last CTA takes its
       // p.q (alpha) step
-      if ((a.cg_sys || a.ms_sys) &&
-          last_block_of_system(a.cg_count, s, (uint32_t)(L.inst_item0[b + 1] - L.inst_item0[b]))) {
-        const double pq = sys_sum(L, b, c, a.chains, a.dot_partial, 1, 0);
-        const bool go = a.cg_sys ? cg_pq_step(a.cg_sys[s], pq)
-                                 : mscg_alpha_step(a.ms_sys[s], a.ms_sh + (int64_t)s * a.ms_m, a.ms_m, pq);
-        if (!go) {
-          a.cg_active[s] = 0;
-          atomicSub(a.cg_n_active, 1);
-        }
-      }
+      __syncthreads();
+      if (s_last) cg_finish_pq(L, a, b, c, s, red);
     }
   }
 }

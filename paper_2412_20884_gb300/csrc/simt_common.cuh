@@ -35,6 +35,18 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   return t;
 }
 
+// Running sum as an unevaluated pair s + c: each addition's rounding error,
+// recovered exactly by Knuth's TwoSum, is added to c, so (double)s + (double)c
+// differs from the exact sum of the terms by about u^2 times the sum of their
+// magnitudes (u = 2^-24) instead of u times it.
+__device__ __forceinline__ void two_sum_add(float& s, float& c, float x) {
+  const float t = __fadd_rn(s, x);
+  const float bp = __fsub_rn(t, s);
+  const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(x, bp));
+  c = __fadd_rn(c, err);
+  s = t;
+}
+
 inline int pow2ceil(int v) {
   int p = 1;
   while (p < v) p <<= 1;

@@ -8,6 +8,7 @@
 
 #include "exp2_poly.cuh"
 #include "kmv_internal.cuh"
+#include "simt_common.cuh"
 
 namespace kmv {
 
@@ -177,18 +178,6 @@ __device__ __forceinline__ float col_scale(uint32_t bits) {
   int e;
   frexpf(mx, &e);  // mx = f 2^e, f in [0.5, 1)
   return ldexpf(1.f, 14 - e);
-}
-
-// Running sum as an unevaluated pair s + c: each addition's rounding error,
-// recovered exactly by Knuth's TwoSum, is added to c, so (double)s + (double)c
-// differs from the exact sum of the terms by about u^2 times the sum of their
-// magnitudes (u = 2^-24) instead of u times it.
-__device__ __forceinline__ void two_sum_add(float& s, float& c, float x) {
-  const float t = __fadd_rn(s, x);
-  const float bp = __fsub_rn(t, s);
-  const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(x, bp));
-  c = __fadd_rn(c, err);
-  s = t;
 }
 
 // 1 / col_scale(bits), exactly (a power of two, formed from its exponent).
