@@ -163,6 +163,52 @@ __device__ __forceinline__ bool last_arrival(uint32_t* count, uint32_t n, uint32
   return last;
 }
 
+// p = r + beta p over [v0, v1) by one CTA, eight rows of loads in flight per thread
+// (r bypasses L1: other CTAs of this launch wrote it).
+__device__ __forceinline__ void form_direction(float* p, const float* r, float beta, int64_t v0, int64_t v1) {
+  for (int64_t v = v0 + threadIdx.x; v < v1; v += 8 * kTile) {
+    float rv[8], pv[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const bool in = v + k * kTile < v1;
+      rv[k] = in ? __ldcg(&r[v + k * kTile]) : 0.f;
+      pv[k] = in ? p[v + k * kTile] : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (v + k * kTile < v1) p[v + k * kTile] = fmaf(beta, pv[k], rv[k]);
+  }
+}
+
+// alpha = r.z / p.q of one preconditioned system; false when it stops here.
+__device__ __forceinline__ bool pcg_pq_step(PcgSys& y, double pq) {
+  if (!(pq > 0.0) || !isfinite(pq) || !(y.rz > 0.0)) {
+    y.status = isfinite(pq) && isfinite(y.rz) ? KMV_ENOTCONV : KMV_ENONFINITE;
+    y.alpha = 0.0;
+    return false;
+  }
+  y.alpha = y.rz / pq;
+  return true;
+}
+
+// beta = r.z' / r.z and the stopping test on r.r of one preconditioned system.
+__device__ __forceinline__ bool pcg_rz_step(PcgSys& y, double rr, double rz, double tol, int maxiter) {
+  y.iters += 1;
+  y.beta = rz / y.rz;
+  y.rr = rr;
+  y.rz = rz;
+  if (!isfinite(rr) || !isfinite(rz)) {
+    y.status = KMV_ENONFINITE;
+    return false;
+  }
+  if (rr <= tol * tol * y.bb) return false;
+  if (y.iters >= maxiter) {
+    y.status = KMV_ENOTCONV;
+    return false;
+  }
+  return true;
+}
+
 // The p.q (alpha) step of system s inside a (multi-shift) CG iteration, by the
 // whole CTA that completed the system's dot partials.
 __device__ __forceinline__ void cg_finish_pq(const DevLayout& L, const KmvArgs& a, int b, int c, int s, double* red) {
@@ -170,9 +216,9 @@ __device__ __forceinline__ void cg_finish_pq(const DevLayout& L, const KmvArgs& 
   if (threadIdx.x >= 32) return;
   pq = __shfl_sync(0xffffffffu, pq, 0);
   bool go;
-  if (a.cg_sys) {
+  if (a.cg_sys || a.pcg_sys) {
     if (threadIdx.x != 0) return;
-    go = cg_pq_step(a.cg_sys[s], pq);
+    go = a.cg_sys ? cg_pq_step(a.cg_sys[s], pq) : pcg_pq_step(a.pcg_sys[s], pq);
   } else {
     go = mscg_alpha_step(a.ms_sys[s], a.ms_sh + (int64_t)s * a.ms_m, a.ms_m, pq);
   }

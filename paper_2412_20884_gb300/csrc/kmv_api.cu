@@ -302,7 +302,7 @@ kmv_status simt_scratch(kmv_handle h, size_t bytes, size_t counters, cudaStream_
 kmv_status simt_forward(kmv_handle h, const KmvArgs& a, cudaStream_t st) {
   const Layout& L = h->layout;
   if (L.n_items == 0) return KMV_OK;
-  if ((a.cg_sys || a.ms_sys) && !(a.m == 1 && a.dot_partial))
+  if ((a.cg_sys || a.pcg_sys || a.ms_sys) && !(a.m == 1 && a.dot_partial))
     return fail(h, KMV_EINVAL, "internal: fused CG step needs the one-column product");
   SimtFwd f = simt_fwd_plan(h->simt_tiles, L.n_inst, L.n_items, L.chains, L.n_total, (int64_t)L.max_items_per_inst * kTile, a.d,
                             a.m, h->num_sms);
@@ -424,6 +424,29 @@ kmv_status capture_while(kmv_handle h, cudaStream_t st, const int32_t* n_active,
   return KMV_OK;
 }
 
+// The convergence test of an eager solver loop, every kCheckEvery iterations: the count
+// of active systems is copied to the host and looked at one test later, so the GPU has
+// the next iterations queued while the host waits (waiting for the copy just made left
+// it idle for about 12 us per test).  The iterations that follow convergence find every
+// system inactive and change nothing.
+constexpr int kCheckEvery = 4;
+struct Poll {
+  bool done = false, pending = false;
+  int slot = 0;
+  kmv_status step(kmv_handle h, const int32_t* n_active, cudaStream_t st) {
+    int32_t* flag = h->host_flag + 8;   // two slots, apart from the refinement's 16 bytes
+    KMV_CUDA(h, cudaMemcpyAsync(flag + slot, n_active, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    KMV_CUDA(h, cudaEventRecord(h->poll_ev[slot], st));
+    if (pending) {
+      KMV_CUDA(h, cudaEventSynchronize(h->poll_ev[slot ^ 1]));
+      done = flag[slot ^ 1] == 0;
+    }
+    pending = true;
+    slot ^= 1;
+    return KMV_OK;
+  }
+};
+
 struct CgBufs {
   float *r, *p, *q;
   double *partial, *partial2;
@@ -480,7 +503,6 @@ kmv_status run_cg(kmv_handle h, const kmv_points* pts, const double* theta, cons
                                B.p, warm, B.partial2, st));
   KMV_CUDA(h, launch_cg_reduce_init(h->dev, L.n_inst, L.chains, B.partial2, tol, B.sys, B.active,
                                     B.n_active, st));
-  const int check_every = 4;
   a.V = B.p;
   a.Y = B.q;
   a.sys_active = B.active;
@@ -503,6 +525,7 @@ kmv_status run_cg(kmv_handle h, const kmv_points* pts, const double* theta, cons
     a.cg_n_active = B.n_active;
     a.cg_count = B.count;
     a.cg_r = B.r;
+    a.chained = !h->capturing;
   }
   // one CG iteration on every active system; theta is fixed within the solve,
   // so the products after the first reuse its operand tiles
@@ -513,7 +536,7 @@ kmv_status run_cg(kmv_handle h, const kmv_points* pts, const double* theta, cons
       // the systems' last CTAs form p too where the largest system is small
       KMV_CUDA(h, launch_cg_update_xr_rr(h->dev, L.n_items, L.chains, L.n_total, B.sys, B.active, x, B.r, B.p,
                                          B.q, B.partial, B.count + n_sys, tol, maxiter, B.n_active,
-                                         p_fused ? kFusedPRows : 0, s));
+                                         p_fused ? kFusedPRows : 0, L.n_inst, a.chained, s));
       if (!tc_fma && !p_fused)
         KMV_CUDA(h, launch_cg_update_p(h->dev, L.n_items, L.chains, L.n_total, B.sys, B.active, B.r, B.p, s));
       return KMV_OK;
@@ -537,11 +560,11 @@ kmv_status run_cg(kmv_handle h, const kmv_points* pts, const double* theta, cons
       KMV_TRY(capture_while(h, st, B.n_active, [&](cudaStream_t s2) { return iteration(s2, 1); }));
     }
   } else {
+    Poll poll;
     for (int it = 0; it < maxiter; ++it) {
-      if (it % check_every == 0) {
-        KMV_CUDA(h, cudaMemcpyAsync(h->host_flag, B.n_active, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        KMV_CUDA(h, cudaStreamSynchronize(st));
-        if (*h->host_flag == 0) break;
+      if (it % kCheckEvery == 0) {
+        KMV_TRY(poll.step(h, B.n_active, st));
+        if (poll.done) break;
       }
       KMV_TRY(iteration(st, (it > 0 || warm) ? 1 : 0));
     }
@@ -554,12 +577,13 @@ kmv_status run_cg(kmv_handle h, const kmv_points* pts, const double* theta, cons
 
 struct PcgBufs {
   float *r, *p, *q, *z;
-  double *partial, *partial2, *prz, *proj, *coef;
+  double *partial, *partial2, *prz, *proj, *coef, *fac;
   PcgSys* sys;
   int32_t *active, *n_active;
+  uint32_t* count;   // 2 n_sys counters (p.q step, r.z step)
 };
 
-void pcg_layout(const Layout& L, int rank, Arena& ar, size_t off[12]) {
+void pcg_layout(const Layout& L, int rank, Arena& ar, size_t off[13]) {
   const size_t vec = sizeof(float) * (size_t)L.chains * std::max<int64_t>(1, L.n_total);
   const size_t items = (size_t)std::max(1, L.n_items) * L.chains;
   const size_t n_sys = (size_t)L.n_inst * L.chains;
@@ -571,10 +595,11 @@ void pcg_layout(const Layout& L, int rank, Arena& ar, size_t off[12]) {
   off[8] = ar.take(sizeof(double) * n_sys * rank);
   off[9] = ar.take(sizeof(PcgSys) * n_sys);
   off[10] = ar.take(sizeof(int32_t) * n_sys);
-  off[11] = ar.take(sizeof(int32_t) * 4);
+  off[11] = ar.take(sizeof(int32_t) * 4 + sizeof(uint32_t) * 2 * n_sys);
+  off[12] = ar.take(sizeof(double) * n_sys * rank);
 }
 
-PcgBufs pcg_bufs(kmv_handle h, const size_t off[12]) {
+PcgBufs pcg_bufs(kmv_handle h, const size_t off[13]) {
   PcgBufs b;
   b.r = at<float>(h, off[0]);
   b.p = at<float>(h, off[1]);
@@ -588,6 +613,8 @@ PcgBufs pcg_bufs(kmv_handle h, const size_t off[12]) {
   b.sys = at<PcgSys>(h, off[9]);
   b.active = at<int32_t>(h, off[10]);
   b.n_active = at<int32_t>(h, off[11]);
+  b.count = reinterpret_cast<uint32_t*>(b.n_active + 4);
+  b.fac = at<double>(h, off[12]);
   return b;
 }
 
@@ -608,9 +635,10 @@ kmv_status run_pcg(kmv_handle h, const kmv_points* pts, const double* theta, con
   }
   KMV_CUDA(h, launch_pcg_init(h->dev, L.n_items, L.chains, L.n_total, rhs, rhs_stride, B.q, x, B.r, warm,
                               B.partial2, st));
-  KMV_CUDA(h, launch_pcg_precond(h->dev, L.n_items, L.n_inst, L.chains, L.n_total, P, a.theta, a.n_theta, B.r, B.z,
-                                 nullptr, B.proj, B.coef, B.prz, st));
-  KMV_CUDA(h, cudaMemsetAsync(B.n_active, 0, sizeof(int32_t), st));
+  KMV_CUDA(h, launch_pcg_factors(P, n_sys, a.n_theta, a.theta, B.fac, st));
+  KMV_CUDA(h, launch_pcg_precond(h->dev, L.n_items, L.n_inst, L.chains, L.n_total, P, B.fac, B.r, B.z, nullptr, B.proj,
+                                 B.coef, B.prz, false, st));
+  KMV_CUDA(h, cudaMemsetAsync(B.n_active, 0, sizeof(int32_t) * 4 + sizeof(uint32_t) * 2 * n_sys, st));
   KMV_CUDA(h, launch_pcg_setup(h->dev, L.n_inst, L.chains, B.partial2, B.prz, tol, B.sys, B.active, B.n_active, st));
   const size_t vbytes = sizeof(float) * (size_t)L.chains * L.n_total;
   if (vbytes) KMV_CUDA(h, cudaMemcpyAsync(B.p, B.z, vbytes, cudaMemcpyDeviceToDevice, st));
@@ -618,19 +646,32 @@ kmv_status run_pcg(kmv_handle h, const kmv_points* pts, const double* theta, con
   a.Y = B.q;
   a.sys_active = B.active;
   a.dot_partial = B.partial;
-  const int check_every = 4;
+  // As in run_cg, the product's last CTA per system takes the alpha step (where the
+  // product carries the hook), the preconditioner's the beta step, and the direction
+  // is formed by the tensor-core product's preparation, a small system's last CTA or
+  // a kernel of its own.
+  const bool tc_fma = prec == KMV_BF16_HILO && x_width_fma_ok(pts->d);
+  const bool fused = L.n_items > 0 && (tc_fma || prec == KMV_FP32);
+  const bool p_fused = !tc_fma && (int64_t)L.max_items_per_inst * kTile <= kFusedPRows;
+  const bool chained = !h->capturing;
+  a.chained = chained;
+  if (fused) {
+    a.pcg_sys = B.sys;
+    a.cg_active = B.active;
+    a.cg_n_active = B.n_active;
+    a.cg_count = B.count;
+    a.cg_r = B.z;
+  }
   auto iteration = [&](cudaStream_t s, int reuse) -> kmv_status {
     a.reuse_prep = reuse;
     KMV_TRY(run_forward(h, a, prec, s));
-    KMV_CUDA(h, launch_pcg_alpha(h->dev, L.n_inst, L.chains, B.partial, B.sys, B.active, s));
-    KMV_CUDA(h, launch_pcg_update_xr(h->dev, L.n_items, L.chains, L.n_total, B.sys, B.active, x, B.r, B.p, B.q,
-                                     B.partial, s));
-    KMV_CUDA(h, launch_pcg_precond(h->dev, L.n_items, L.n_inst, L.chains, L.n_total, P, a.theta, a.n_theta, B.r,
-                                   B.z, B.active, B.proj, B.coef, B.prz, s));
-    KMV_CUDA(h, cudaMemsetAsync(B.n_active, 0, sizeof(int32_t), s));
-    KMV_CUDA(h, launch_pcg_beta(h->dev, L.n_inst, L.chains, B.partial, B.prz, tol, maxiter, B.sys, B.active,
-                                B.n_active, s));
-    KMV_CUDA(h, launch_pcg_update_p(h->dev, L.n_items, L.chains, L.n_total, B.sys, B.active, B.z, B.p, s));
+    if (!fused)
+      KMV_CUDA(h, launch_pcg_alpha(h->dev, L.n_inst, L.chains, B.partial, B.sys, B.active, B.n_active, s));
+    KMV_CUDA(h, launch_pcg_iterate(h->dev, L.n_items, L.n_inst, L.chains, L.n_total, P, B.fac, B.sys, B.active,
+                                   B.n_active, x, B.r, B.p, B.q, B.z, B.partial, B.proj, B.coef, B.prz,
+                                   B.count + n_sys, tol, maxiter, p_fused ? kFusedPRows : 0, chained, s));
+    if (!(fused && tc_fma) && !p_fused)
+      KMV_CUDA(h, launch_pcg_update_p(h->dev, L.n_items, L.chains, L.n_total, B.sys, B.active, B.z, B.p, chained, s));
     return KMV_OK;
   };
   if (h->capturing) {
@@ -640,11 +681,11 @@ kmv_status run_pcg(kmv_handle h, const kmv_points* pts, const double* theta, con
       KMV_TRY(capture_while(h, st, B.n_active, [&](cudaStream_t s2) { return iteration(s2, 1); }));
     }
   } else {
+    Poll poll;
     for (int it = 0; it < maxiter; ++it) {
-      if (it % check_every == 0) {
-        KMV_CUDA(h, cudaMemcpyAsync(h->host_flag, B.n_active, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        KMV_CUDA(h, cudaStreamSynchronize(st));
-        if (*h->host_flag == 0) break;
+      if (it % kCheckEvery == 0) {
+        KMV_TRY(poll.step(h, B.n_active, st));
+        if (poll.done) break;
       }
       KMV_TRY(iteration(st, (it > 0 || warm) ? 1 : 0));
     }
@@ -763,7 +804,7 @@ kmv_status run_cg_refined(kmv_handle h, const kmv_points* pts, const double* the
 struct SolveLayout {
   size_t cg[8];
   size_t rf[11];
-  size_t pcg[12];
+  size_t pcg[13];
   bool refined, pc;
 };
 
@@ -889,12 +930,11 @@ kmv_status run_mcg(kmv_handle h, const kmv_points* pts, const double* theta, con
   a.V = B.p;
   a.Y = B.q;
   a.sys_active = B.sys_any;
-  const int check_every = 4;
+  Poll poll;
   for (int it = 0; it < maxiter; ++it) {
-    if (it % check_every == 0) {
-      KMV_CUDA(h, cudaMemcpyAsync(h->host_flag, B.n_active, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-      KMV_CUDA(h, cudaStreamSynchronize(st));
-      if (*h->host_flag == 0) break;
+    if (it % kCheckEvery == 0) {
+      KMV_TRY(poll.step(h, B.n_active, st));
+      if (poll.done) break;
     }
     KMV_TRY(run_forward(h, a, prec, st));
     KMV_CUDA(h, launch_mcg_dot(h->dev, L.n_items, L.chains, L.n_total, m, B.p, B.q, B.sys_any, B.partial, st));
@@ -1048,12 +1088,11 @@ kmv_status run_mscg(kmv_handle h, const kmv_points* pts, const double* theta, co
     a.cg_count = B.count;
     a.cg_r = B.r;
   }
-  const int check_every = 4;
+  Poll poll;
   for (int it = 0; it < maxiter; ++it) {
-    if (it % check_every == 0) {
-      KMV_CUDA(h, cudaMemcpyAsync(h->host_flag, B.n_active, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-      KMV_CUDA(h, cudaStreamSynchronize(st));
-      if (*h->host_flag == 0) break;
+    if (it % kCheckEvery == 0) {
+      KMV_TRY(poll.step(h, B.n_active, st));
+      if (poll.done) break;
     }
     KMV_TRY(run_forward(h, a, prec, st));
     if (fused) {
@@ -1103,10 +1142,14 @@ kmv_status kmv_create(kmv_handle* out, int device) {
   if (cudaSetDevice(device) != cudaSuccess ||
       cudaMallocHost(reinterpret_cast<void**>(&h->host_flag), 64) != cudaSuccess ||
       cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&h->poll_ev[0], cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&h->poll_ev[1], cudaEventDisableTiming) != cudaSuccess ||
       cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
     cudaGetLastError();
     if (h->host_flag) cudaFreeHost(h->host_flag);
     if (h->side) cudaStreamDestroy(h->side);
+    for (cudaEvent_t e : h->poll_ev)
+      if (e) cudaEventDestroy(e);
     delete h;
     return KMV_ECUDA;
   }
@@ -1127,6 +1170,8 @@ kmv_status kmv_destroy(kmv_handle h) {
   for (void* p : h->simt_retired) cudaFree(p);
   if (h->host_flag) cudaFreeHost(h->host_flag);
   if (h->side) cudaStreamDestroy(h->side);
+  for (cudaEvent_t e : h->poll_ev)
+    if (e) cudaEventDestroy(e);
   kmv_profile_enable(h, 0);
   for (cudaEvent_t e : h->prof_pool) cudaEventDestroy(e);
   delete h;
@@ -1442,7 +1487,7 @@ kmv_status kmv_implicit_step(kmv_handle h, const kmv_points* pts, int32_t chains
   const size_t o_xp = ar.take(sizeof(double) * items * k), o_rp = ar.take(sizeof(double) * items * 2);
   const size_t o_c = ar.take(sizeof(double) * n_sys), o_pp = ar.take(sizeof(double) * items);
   const size_t o_proj = ar.take(sizeof(double) * items * rank), o_coef = ar.take(sizeof(double) * n_sys * rank);
-  const size_t o_prz = ar.take(sizeof(double) * items);
+  const size_t o_prz = ar.take(sizeof(double) * items), o_fac = ar.take(sizeof(double) * n_sys * rank);
   const size_t o_brr = ar.take(sizeof(double) * n_sys), o_bit = ar.take(sizeof(int32_t) * n_sys);
   KMV_TRY(reserve(h, ar.used));
   double* th0 = at<double>(h, o_th0);
@@ -1459,6 +1504,9 @@ kmv_status kmv_implicit_step(kmv_handle h, const kmv_points* pts, int32_t chains
   KMV_CUDA(h, cudaMemcpyAsync(th0, theta, sizeof(double) * n_sys * n, cudaMemcpyDeviceToDevice, st));
   KMV_CUDA(h, cudaMemcpyAsync(pi0, pi, sizeof(double) * n_sys * n, cudaMemcpyDeviceToDevice, st));
 
+  double* fac = at<double>(h, o_fac);
+  if (h->pc_on) KMV_CUDA(h, launch_pcg_factors(P, n_sys, n, th0, fac, st));
+
   // c ~ rho(R~ A(theta_0)) by 20 power iterations from the vector of ones, times 1.05
   KMV_TRY(cheb_prepare(h, pts, th0, 2, st));
   {
@@ -1474,8 +1522,8 @@ kmv_status kmv_implicit_step(kmv_handle h, const kmv_points* pts, int32_t chains
       KMV_TRY(run_forward(h, a, KMV_FP32, st));
       const float* w = q;
       if (h->pc_on) {
-        KMV_CUDA(h, launch_pcg_precond(h->dev, L.n_items, L.n_inst, L.chains, L.n_total, P, th0, n, q, z, nullptr,
-                                       at<double>(h, o_proj), at<double>(h, o_coef), at<double>(h, o_prz), st));
+        KMV_CUDA(h, launch_pcg_precond(h->dev, L.n_items, L.n_inst, L.chains, L.n_total, P, fac, q, z, nullptr,
+                                       at<double>(h, o_proj), at<double>(h, o_coef), at<double>(h, o_prz), false, st));
         w = z;
       }
       KMV_CUDA(h, launch_imp_scale(h->dev, L.n_items, L.chains, L.n_total, nullptr, w, z, at<double>(h, o_pp), st));
@@ -1496,12 +1544,11 @@ kmv_status kmv_implicit_step(kmv_handle h, const kmv_points* pts, int32_t chains
   // the adjoint of the force, FP32 as well, is most of an iteration's cost
   const kmv_precision lin_prec = KMV_FP32;
   (void)prec;
-  const int check_every = 4;
+  Poll poll;
   for (int it = 0; it < maxiter; ++it) {
-    if (!h->capturing && it > 0 && it % check_every == 0) {
-      KMV_CUDA(h, cudaMemcpyAsync(h->host_flag, n_active, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-      KMV_CUDA(h, cudaStreamSynchronize(st));
-      if (*h->host_flag == 0) break;
+    if (!h->capturing && it > 0 && it % kCheckEvery == 0) {
+      KMV_TRY(poll.step(h, n_active, st));
+      if (poll.done) break;
     }
     const int slot = it % k, cnt = std::min(it + 1, k);
     KMV_CUDA(h, launch_imp_mid(n_sys * n, th0, theta, tb, st));
@@ -1515,8 +1562,8 @@ kmv_status kmv_implicit_step(kmv_handle h, const kmv_points* pts, int32_t chains
     KMV_CUDA(h, launch_imp_resid(h->dev, L.n_items, L.chains, L.n_total, y, q, active, r, at<double>(h, o_rp), st));
     const float* zz = r;
     if (h->pc_on) {
-      KMV_CUDA(h, launch_pcg_precond(h->dev, L.n_items, L.n_inst, L.chains, L.n_total, P, th0, n, r, z, active,
-                                     at<double>(h, o_proj), at<double>(h, o_coef), at<double>(h, o_prz), st));
+      KMV_CUDA(h, launch_pcg_precond(h->dev, L.n_items, L.n_inst, L.chains, L.n_total, P, fac, r, z, active,
+                                     at<double>(h, o_proj), at<double>(h, o_coef), at<double>(h, o_prz), false, st));
       zz = z;
     }
     KMV_CUDA(h, launch_imp_x(h->dev, L.n_items, L.chains, L.n_total, k, slot, cnt, x_work, zz, cscale, active,

@@ -156,16 +156,21 @@ cudaError_t launch_cg_update_xr(const DevLayout& L, int n_items, int chains, int
 // which spares the FP32 form a launch per iteration where launches count.
 __global__ void cg_update_xr_rr_kernel(DevLayout L, int chains, int64_t n_total, CgSys* sys, int32_t* active,
                                        float* x, float* r, float* p, const float* q, double* partial,
-                                       uint32_t* count, double tol, int maxiter, int32_t* n_active, int p_rows) {
+                                       uint32_t* count, double tol, int maxiter, int32_t* n_active, int p_rows,
+                                       int n_inst) {
   __shared__ double red[kTile / 32];
   __shared__ int s_last;
   __shared__ float s_beta;
+  chain_trigger();
   const int item = blockIdx.x, c = blockIdx.y;
-  const int b = L.item_inst[item];
+  const bool single = n_inst == 1;   // no look-ups needed
+  const int b = single ? 0 : L.item_inst[item];
   const int s = b * chains + c;
+  const int64_t r0 = single ? 0 : L.offsets[b], r1 = single ? n_total : L.offsets[b + 1];
+  const int64_t i = (single ? (int64_t)item * kTile : L.item_row0[item]) + threadIdx.x;
+  const uint32_t n_of_system = single ? gridDim.x : (uint32_t)(L.inst_item0[b + 1] - L.inst_item0[b]);
+  chain_wait();
   if (!active[s]) return;
-  const int64_t r0 = L.offsets[b], r1 = L.offsets[b + 1];
-  const int64_t i = L.item_row0[item] + threadIdx.x;
   double rr = 0.0;
   if (i < r1) {
     const int64_t v = (int64_t)c * n_total + i;
@@ -179,7 +184,7 @@ __global__ void cg_update_xr_rr_kernel(DevLayout L, int chains, int64_t n_total,
   const double t = block_sum(rr, red);
   if (threadIdx.x == 0) {
     partial[(int64_t)item * chains + c] = t;
-    s_last = last_arrival(&count[s], 1u, (uint32_t)(L.inst_item0[b + 1] - L.inst_item0[b]));
+    s_last = last_arrival(&count[s], 1u, n_of_system);
   }
   __syncthreads();
   if (!s_last) return;
@@ -196,19 +201,15 @@ __global__ void cg_update_xr_rr_kernel(DevLayout L, int chains, int64_t n_total,
   if (!form_p) return;
   __syncthreads();
   if (!s_last) return;
-  for (int64_t j = r0 + threadIdx.x; j < r1; j += blockDim.x) {
-    const int64_t v = (int64_t)c * n_total + j;
-    p[v] = fmaf(s_beta, p[v], __ldcg(&r[v]));
-  }
+  form_direction(p, r, s_beta, (int64_t)c * n_total + r0, (int64_t)c * n_total + r1);
 }
 
 cudaError_t launch_cg_update_xr_rr(const DevLayout& L, int n_items, int chains, int64_t n_total, CgSys* sys,
                                    int32_t* active, float* x, float* r, float* p, const float* q,
                                    double* partial, uint32_t* count, double tol, int maxiter, int32_t* n_active,
-                                   int p_rows, cudaStream_t st) {
-  cg_update_xr_rr_kernel<<<dim3(n_items, chains), kTile, 0, st>>>(L, chains, n_total, sys, active, x, r, p, q,
-                                                                  partial, count, tol, maxiter, n_active, p_rows);
-  return cudaGetLastError();
+                                   int p_rows, int n_inst, bool chained, cudaStream_t st) {
+  return launch_chained(chained, cg_update_xr_rr_kernel, dim3(n_items, chains), kTile, 0, st, L, chains, n_total, sys,
+                        active, x, r, p, q, partial, count, tol, maxiter, n_active, p_rows, n_inst);
 }
 
 __global__ void cg_reduce_rr_kernel(DevLayout L, int n_inst, int chains, const double* partial,

@@ -66,11 +66,47 @@ struct MscgShift {
   int32_t active, iters, status, pad;
 };
 
+// Per-system state of the preconditioned CG.
+struct PcgSys {
+  double rr, bb, rz, alpha, beta;
+  int32_t iters, status;
+};
 // Per-system CG state, kept in the handle workspace.
 struct CgSys {
   double rr, bb, pq, alpha, beta;
   int32_t iters, status;
 };
+
+// ---------------------------------------------------------------------------
+// Programmatic dependent launch: a kernel launched with launch_chained starts while
+// the kernel before it on the stream still runs, and must call chain_wait before it
+// touches anything that kernel (or one before it) writes or reads; chain_wait returns
+// when that kernel has completed.  What stands before it may read only what was
+// complete when the chain began (the points, theta, the layout tables).  Every kernel
+// of a chain calls chain_trigger first thing, so that the next one's CTAs are resident
+// and set up when it ends: a dependent launch of the small solver kernels otherwise
+// costs about 2 us of launch latency and the set-up each.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void chain_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// chained == false: an ordinary launch (stream captures, whose graphs may place it in
+// the body of a conditional node).
+template <class... Params, class... Args>
+cudaError_t launch_chained(bool chained, void (*kernel)(Params...), dim3 grid, int block, size_t smem, cudaStream_t st,
+                           Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
 
 // ---------------------------------------------------------------------------
 // Kernel argument blocks
@@ -109,6 +145,8 @@ struct KmvArgs {
   int32_t* cg_n_active;
   uint32_t* cg_count;
   const float* cg_r;
+  // the same inside a preconditioned CG iteration (pcg_sys set; cg_r is z)
+  PcgSys* pcg_sys;
   // the same inside a multi-shift CG iteration (ms_sys set; cg_active,
   // cg_n_active, cg_count and cg_r as above): the last CTA takes the system's
   // alpha step for its ms_m shifts, and the tensor-core FMA-pipe product first
@@ -118,6 +156,7 @@ struct KmvArgs {
   MscgShift* ms_sh;
   int ms_m;
   float* ms_ps;
+  int chained;   // inside a solver's chain of dependent launches (launch_chained)
 };
 
 // The argument rules of a point set and chain count shared by every entry
@@ -189,7 +228,7 @@ cudaError_t launch_cg_reduce_pq(const DevLayout& L, int n_inst, int chains, cons
 cudaError_t launch_cg_update_xr_rr(const DevLayout& L, int n_items, int chains, int64_t n_total, CgSys* sys,
                                    int32_t* active, float* x, float* r, float* p, const float* q,
                                    double* partial, uint32_t* count, double tol, int maxiter, int32_t* n_active,
-                                   int p_rows, cudaStream_t st);
+                                   int p_rows, int n_inst, bool chained, cudaStream_t st);
 cudaError_t launch_cg_update_xr(const DevLayout& L, int n_items, int chains, int64_t n_total,
                                 const CgSys* sys, const int32_t* active, float* x, float* r,
                                 const float* p, const float* q, double* partial, cudaStream_t st);
@@ -228,10 +267,6 @@ cudaError_t launch_phi_status(int n_sys, int n_poles, const int32_t* col_status,
 
 // Randomized Nystrom preconditioner (kmv_nystrom.cu) and preconditioned CG (kmv_pcg.cu)
 constexpr int kMaxRank = 128;
-struct PcgSys {
-  double rr, bb, rz, alpha, beta;
-  int32_t iters, status;
-};
 struct PcgPrecond {
   int rank;
   const float* U;     // (chains, rank, N_total)
@@ -243,21 +278,28 @@ cudaError_t launch_nystrom_finish(const DevLayout& L, int n_items, int n_inst, i
 cudaError_t launch_pcg_init(const DevLayout& L, int n_items, int chains, int64_t n_total, const float* rhs,
                             int64_t rhs_stride, const float* q, float* x, float* r, int warm, double* partial2,
                             cudaStream_t st);
+// d[s, k] = (lambda_r + mu_s) / (lambda_k + mu_s) - 1 with mu_s = sigma_s^2 of theta,
+// the Woodbury factors of launch_pcg_precond: once per solve.
+cudaError_t launch_pcg_factors(const PcgPrecond& P, int n_sys, int n_theta, const double* theta, double* d,
+                               cudaStream_t st);
+// z = r + U (d o (U^T r)); partials of r.z in prz.
 cudaError_t launch_pcg_precond(const DevLayout& L, int n_items, int n_inst, int chains, int64_t n_total,
-                               const PcgPrecond& P, const double* theta, int n_theta, const float* r, float* z,
-                               const int32_t* active, double* proj, double* coef, double* prz, cudaStream_t st);
+                               const PcgPrecond& P, const double* d, const float* r, float* z, const int32_t* active,
+                               double* proj, double* coef, double* prz, bool chained, cudaStream_t st);
 cudaError_t launch_pcg_setup(const DevLayout& L, int n_inst, int chains, const double* partial2, const double* prz,
                              double tol, PcgSys* sys, int32_t* active, int32_t* n_active, cudaStream_t st);
 cudaError_t launch_pcg_alpha(const DevLayout& L, int n_inst, int chains, const double* partial, PcgSys* sys,
-                             int32_t* active, cudaStream_t st);
-cudaError_t launch_pcg_update_xr(const DevLayout& L, int n_items, int chains, int64_t n_total, const PcgSys* sys,
-                                 const int32_t* active, float* x, float* r, const float* p, const float* q,
-                                 double* partial, cudaStream_t st);
-cudaError_t launch_pcg_beta(const DevLayout& L, int n_inst, int chains, const double* prr, const double* prz,
-                            double tol, int maxiter, PcgSys* sys, int32_t* active, int32_t* n_active,
-                            cudaStream_t st);
+                             int32_t* active, int32_t* n_active, cudaStream_t st);
+// After the product and alpha: x, r, U^T r; the coefficients; z, and by each system's
+// last CTA (count: one zeroed counter per system) its beta and stopping test, and for
+// systems of at most p_rows rows p = z + beta p.
+cudaError_t launch_pcg_iterate(const DevLayout& L, int n_items, int n_inst, int chains, int64_t n_total,
+                               const PcgPrecond& P, const double* d, PcgSys* sys, int32_t* active, int32_t* n_active,
+                               float* x, float* r, float* p, const float* q, float* z, double* partial, double* proj,
+                               double* coef, double* prz, uint32_t* count, double tol, int maxiter, int p_rows,
+                               bool chained, cudaStream_t st);
 cudaError_t launch_pcg_update_p(const DevLayout& L, int n_items, int chains, int64_t n_total, const PcgSys* sys,
-                                const int32_t* active, const float* z, float* p, cudaStream_t st);
+                                const int32_t* active, const float* z, float* p, bool chained, cudaStream_t st);
 cudaError_t launch_pcg_finish(int n_sys, const PcgSys* sys, const int32_t* active, int32_t* status, int32_t* iters,
                               cudaStream_t st);
 
@@ -403,6 +445,7 @@ struct kmv_handle_s {
   void* ws = nullptr;
   size_t ws_bytes = 0;
   int32_t* host_flag = nullptr;   // pinned, for convergence checks
+  cudaEvent_t poll_ev[2] = {nullptr, nullptr};
   void* tc = nullptr;             // tensor-core path state (kmv_tc.cu)
   // Chebyshev-amplitude family: internal parameters, amplitudes and the
   // backward's scratch for the current theta (kmv_api.cu, cheb_prepare)

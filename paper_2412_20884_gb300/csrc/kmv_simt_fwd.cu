@@ -38,7 +38,8 @@ __global__ void __launch_bounds__(kTile) fwd_simt_combine_kernel(KmvArgs a, Simt
     const int mc = min(kCombineCols, a.m - c0);
     if (valid)
       for (int q = 0; q < mc; ++q)
-        simt_put_y(a, s, c, i, c0 + q, ai, as2[1], simt_part_sum(a, f, U, c, c0 + q, i));
+        simt_put_y(a, s, c, i, c0 + q, ai, as2[1], simt_part_sum(a, f, U, c, c0 + q, i),
+                   a.V[((int64_t)c * a.n_total + i) * a.m + c0 + q]);
   }
 }
 

@@ -55,20 +55,31 @@ __device__ __forceinline__ size_t simt_part_at(const KmvArgs& a, int unit, int c
   return (((size_t)unit * a.chains + c) * a.m + col) * (size_t)a.n_total + i;
 }
 
+// Adds n pairs a fixed step apart to (s, e), eight loads in flight at a time (one
+// after the other, 16 of them took 5 us of a small product's last CTA).
+__device__ __forceinline__ void simt_add_pairs(const float2* p, size_t step, uint32_t n, float& s, float& e) {
+  for (uint32_t u0 = 0; u0 < n; u0 += 8) {
+    float2 v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = u0 + k < n ? __ldcg(p + (u0 + k) * step) : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      two_sum_add(s, e, v[k].x);
+      e += v[k].y;
+    }
+  }
+}
+
 // Sum of the units' pairs of one element, in unit order.
 __device__ __forceinline__ double simt_part_sum(const KmvArgs& a, const SimtFwd& f, const SimtUnits& U, int c, int col,
                                                 int64_t i) {
   float s = 0.f, e = 0.f;
   const size_t step = (size_t)a.chains * a.m * (size_t)a.n_total;
-  for (uint32_t jc = 0; jc < U.n_chunks; ++jc) {
-    const float2* p = f.part + simt_part_at(a, jc * f.upc, c, col, i);
-    const uint32_t n = f.upc == 1 ? 1u : U.in_chunk(jc);
-#pragma unroll 4
-    for (uint32_t u = 0; u < n; ++u) {
-      const float2 v = __ldcg(p + u * step);
-      two_sum_add(s, e, v.x);
-      e += v.y;
-    }
+  const float2* p = f.part + simt_part_at(a, 0, c, col, i);
+  if (f.upc == 1) {
+    simt_add_pairs(p, step, U.n_chunks, s, e);
+  } else {
+    for (uint32_t jc = 0; jc < U.n_chunks; ++jc) simt_add_pairs(p + jc * f.upc * step, step, U.in_chunk(jc), s, e);
   }
   return (double)s + (double)e;
 }
@@ -82,12 +93,12 @@ __device__ __forceinline__ void load_alpha_s2(const KmvArgs& a, int s, double* a
   }
 }
 
-// One element of Y from its sum; returns V_i Y_i.
+// One element of Y from its sum and V_i; returns V_i Y_i.
 __device__ __forceinline__ double simt_put_y(const KmvArgs& a, int s, int c, int64_t i, int col, double ai, double s2,
-                                             double sum) {
+                                             double sum, float v) {
   const int64_t idx = ((int64_t)c * a.n_total + i) * a.m + col;
   const double shift = a.col_shift ? (double)a.col_shift[(int64_t)s * a.col_shift_stride + col] : 0.0;
-  const double vi = (double)a.V[idx];
+  const double vi = (double)v;
   const double y = ai * sum + (a.no_diag ? 0.0 : (s2 + shift) * vi);
   a.Y[idx] = (float)y;
   if (a.Y64) a.Y64[idx] = y;
@@ -107,7 +118,7 @@ __device__ __forceinline__ void simt_put_dots(const KmvArgs& a, int b, int c, in
       if (threadIdx.x == 0) a.dot_partial[(int64_t)(item0 + r) * a.chains + c] = t;
     }
   }
-  if (!(a.cg_sys || a.ms_sys)) return;
+  if (!(a.cg_sys || a.ms_sys || a.pcg_sys)) return;
   if (threadIdx.x == 0)
     *s_flag = last_arrival(&a.cg_count[s], (uint32_t)n, (uint32_t)(a.L.inst_item0[b + 1] - a.L.inst_item0[b]));
   __syncthreads();
@@ -116,6 +127,7 @@ __device__ __forceinline__ void simt_put_dots(const KmvArgs& a, int b, int c, in
 
 template <int D, int MP, int R>
 __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
+  chain_trigger();
   const int dd = a.d;   // <= D; the dimensions past it are zero and add nothing
   const int tile = blockIdx.x, c = blockIdx.y;
   const int u = blockIdx.z % f.upc, jc = (blockIdx.z / f.upc) % f.js, z = f.z0 + blockIdx.z / f.max_units;
@@ -124,12 +136,11 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
   const bool single = f.n_inst == 1;
   const int b = single ? 0 : a.L.item_inst[item0];
   const int s = b * a.chains + c;
-  if (a.sys_active && !a.sys_active[s]) return;
   const int64_t o0 = single ? 0 : a.L.offsets[b], o1 = single ? a.n_total : a.L.offsets[b + 1];
   const SimtUnits U(f, o1 - o0);
   uint32_t t0, t1;
   U.range(jc, u, t0, t1);
-  if (t1 <= t0) return;
+  if (t1 <= t0) return;   // an empty unit: the last ones of a short instance
   const int64_t jb = o0 + (int64_t)t0 * kJT, je = min(o1, o0 + (int64_t)t1 * kJT);
 
   __shared__ __align__(16) float sx[2][D * kXS];
@@ -141,23 +152,20 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
 
   const int tid = threadIdx.x;
   const double* th = a.theta + (int64_t)s * a.n_theta;
-  // the scales, and by two lanes of another warp alpha and sigma^2 (read at the end)
-  load_scale(th, dd, a.ard, sc);
-  if ((f.max_units == 1 || f.ticket) && tid >= 96 && tid < 98) as2[tid - 96] = exp(th[tid == 96 ? 0 : a.n_theta - 1]);
-  if (dd < D)
-    for (int e = tid; e < (D - dd) * kXS; e += kTile) sx[0][dd * kXS + e] = sx[1][dd * kXS + e] = 0.f;
   const int c0 = z * MP;
   const int mc = min(MP, a.m - c0);
   const int64_t vbase = (int64_t)c * a.n_total;
   const int64_t r0 = single ? (int64_t)item0 * kTile : a.L.item_row0[item0];
-  __syncthreads();
 
   float xi[R][D], acc[R][MP];
+  // few columns: V_i for the epilogue too, loaded here so that the last CTA has it
+  constexpr int PV = MP <= 2 ? MP : 1;
+  float vi[R][PV];
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int64_t i = r0 + r * kTile + tid;
 #pragma unroll
-    for (int k = 0; k < D; ++k) xi[r][k] = (k < dd && i < o1) ? a.x[i * dd + k] * sc[k] : 0.f;
+    for (int k = 0; k < D; ++k) xi[r][k] = (k < dd && i < o1) ? a.x[i * dd + k] : 0.f;
 #pragma unroll
     for (int q = 0; q < MP; ++q) acc[r][q] = 0.f;
   }
@@ -171,19 +179,16 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
     r = dd > 1 ? (int)__umulhi((uint32_t)e, inv) : e;
     k = e - r * dd;
   };
-  auto fetch = [&](int64_t jt) {
+  auto fetch_x = [&](int64_t jt) {
     const int nj = (int)min((int64_t)kJT, je - jt);
 #pragma unroll
     for (int n = 0; n < NX; ++n) {
       const int e = n * kTile + tid;
-      if (e < nj * dd) {
-        int r, k;
-        split(e, r, k);
-        fx[n] = a.x[jt * dd + e] * sc[k];
-      } else {
-        fx[n] = 0.f;
-      }
+      fx[n] = e < nj * dd ? a.x[jt * dd + e] : 0.f;
     }
+  };
+  auto fetch_v = [&](int64_t jt) {
+    const int nj = (int)min((int64_t)kJT, je - jt);
 #pragma unroll
     for (int n = 0; n < NV; ++n) {
       const int e = n * kTile + tid, r = e / MP, q = e - r * MP;
@@ -197,7 +202,7 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
       if (e < kJT * dd) {
         int r, k;
         split(e, r, k);
-        sx[buf][k * kXS + r] = fx[n];
+        sx[buf][k * kXS + r] = fx[n] * sc[k];
       }
     }
 #pragma unroll
@@ -206,6 +211,30 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
       if (NV * kTile == kJT * MP || e < kJT * MP) sv[buf][e] = fv[n];
     }
   };
+  fetch_x(jb);
+  // the scales, and by two lanes of another warp alpha and sigma^2 (read at the end),
+  // while the loads above are in flight
+  load_scale(th, dd, a.ard, sc);
+  if ((f.max_units == 1 || f.ticket) && tid >= 96 && tid < 98) as2[tid - 96] = exp(th[tid == 96 ? 0 : a.n_theta - 1]);
+  if (dd < D)
+    for (int e = tid; e < (D - dd) * kXS; e += kTile) sx[0][dd * kXS + e] = sx[1][dd * kXS + e] = 0.f;
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int k = 0; k < D; ++k)
+      if (k < dd) xi[r][k] *= sc[k];
+  // from here on, what the solver's kernels before this one write: V and the masks
+  chain_wait();
+  if (a.sys_active && !a.sys_active[s]) return;
+  fetch_v(jb);
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int q = 0; q < PV; ++q) {
+      const int64_t i = r0 + r * kTile + tid;
+      vi[r][q] = (MP <= 2 && q < mc && i < o1) ? a.V[(vbase + i) * a.m + c0 + q] : 0.f;
+    }
 
   const bool paired = je - jb > kFoldTiles * kTile;   // several folds: sums kept as pairs in f.part
   const int unit = jc * f.upc + u;
@@ -231,17 +260,20 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
     first = false;
   };
 
-  fetch(jb);
   store(0);
   __syncthreads();
   int step = 0;
   for (int64_t jt = jb; jt < je; jt += kJT, ++step) {
     const int buf = step & 1;
     const bool more = jt + kJT < je;
-    if (more) fetch(jt + kJT);
+    if (more) {
+      fetch_x(jt + kJT);
+      fetch_v(jt + kJT);
+    }
     const float* X = sx[buf];
     const float* V = sv[buf];
-#pragma unroll 1
+    // one row per thread leaves a chain of dependent steps: two steps in flight there
+#pragma unroll (R == 1 && D * MP <= 64 ? 2 : 1)
     for (int jj = 0; jj < kJT; jj += 4) {
       float p[R][4];
 #pragma unroll
@@ -326,7 +358,8 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
             float2 v = make_float2(0.f, 0.f);
             if (paired) v = f.part[simt_part_at(a, 0, c, c0 + q, i)];
             two_sum_add(v.x, v.y, acc[r][q]);
-            dots[r] += simt_put_y(a, s, c, i, c0 + q, ai, s2, (double)v.x + (double)v.y);
+            dots[r] += simt_put_y(a, s, c, i, c0 + q, ai, s2, (double)v.x + (double)v.y,
+                                  MP <= 2 ? vi[r][q % PV] : a.V[(vbase + i) * a.m + c0 + q]);
           }
       }
     }
@@ -348,8 +381,9 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
     const int64_t i = r0 + r * kTile + tid;
     if (i < o1) {
       const double ai = a.amp ? alpha * (double)a.amp[vbase + i] : alpha;
-      for (int q = 0; q < mc; ++q)
-        dots[r] += simt_put_y(a, s, c, i, c0 + q, ai, s2, simt_part_sum(a, f, U, c, c0 + q, i));
+#pragma unroll
+      for (int q = 0; q < PV; ++q)   // (ticket: at most two columns)
+        if (q < mc) dots[r] += simt_put_y(a, s, c, i, c0 + q, ai, s2, simt_part_sum(a, f, U, c, c0 + q, i), vi[r][q]);
     }
   }
   if (a.dot_partial) simt_put_dots<R>(a, b, c, s, item0, n_it, dots, red, &s_flag);
@@ -367,13 +401,12 @@ constexpr int fwd_most_columns(int D) { return D >= 16 && D <= 32 ? 32 : 16; }
 template <int D, int MP>
 cudaError_t fwd_launch_mp(const KmvArgs& a, const SimtFwd& f, dim3 grid, cudaStream_t st) {
   if (f.rows == 1) {
-    fwd_simt_kernel<D, MP, 1><<<grid, kTile, 0, st>>>(a, f);
-    return cudaGetLastError();
+    return launch_chained(a.chained, fwd_simt_kernel<D, MP, 1>, grid, kTile, 0, st, a, f);
   }
   constexpr int R = fwd_rows(D, MP);
-  if (f.rows != R) return cudaErrorInvalidValue;
-  if constexpr (R > 1) fwd_simt_kernel<D, MP, R><<<grid, kTile, 0, st>>>(a, f);
-  return cudaGetLastError();
+  if constexpr (R > 1)
+    if (f.rows == R) return launch_chained(a.chained, fwd_simt_kernel<D, MP, R>, grid, kTile, 0, st, a, f);
+  return cudaErrorInvalidValue;
 }
 
 // The kernel for the dimension class D (kmv_simt_fwd_*.cu hold the instances).

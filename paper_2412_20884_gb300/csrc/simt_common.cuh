@@ -47,6 +47,22 @@ __device__ __forceinline__ void two_sum_add(float& s, float& c, float x) {
   s = t;
 }
 
+// Adds u v to the pair (s, e): the product's rounding error is recovered by an FMA.
+__device__ __forceinline__ void pair_add_product(float& s, float& e, float u, float v) {
+  const float p = __fmul_rn(u, v);
+  two_sum_add(s, e, p);
+  e = __fadd_rn(e, __fmaf_rn(u, v, -p));
+}
+// Sum of the warp's pairs, in every lane.
+__device__ __forceinline__ void pair_warp_sum(float& s, float& e) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float so = __shfl_xor_sync(0xffffffffu, s, o), eo = __shfl_xor_sync(0xffffffffu, e, o);
+    two_sum_add(s, e, so);
+    e = __fadd_rn(e, eo);
+  }
+}
+
 inline int pow2ceil(int v) {
   int p = 1;
   while (p < v) p <<= 1;
