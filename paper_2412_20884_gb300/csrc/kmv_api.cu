@@ -355,7 +355,7 @@ kmv_status run_backward_stationary(kmv_handle h, KmvArgs a, double* grad, double
     ProfScope prof(h, KMV_KERNEL_ADJOINT, st);
     KMV_CUDA(h, launch_backward_simt(a, f, L.n_items, st));
   }
-  KMV_CUDA(h, launch_grad_finalize(h->dev, f, L.n_inst, L.chains, a.n_theta, a.theta, partial, grad, st));
+  KMV_CUDA(h, launch_grad_finalize(h->dev, f, L.n_inst, L.chains, a.n_theta, a.theta, partial, grad, a.chained, st));
   return KMV_OK;
 }
 
@@ -842,6 +842,7 @@ struct McgBufs {
   double *partial, *partial2;
   McgCol* cols;
   int32_t *sys_any, *n_active;
+  uint32_t* count;   // 2 n_sys counters (alpha steps, beta steps)
 };
 
 void mcg_layout(const Layout& L, int m, Arena& ar, size_t off[8]) {
@@ -855,7 +856,8 @@ void mcg_layout(const Layout& L, int m, Arena& ar, size_t off[8]) {
   off[4] = ar.take(sizeof(double) * items * 2);
   off[5] = ar.take(sizeof(McgCol) * n_sys * m);
   off[6] = ar.take(sizeof(int32_t) * n_sys);
-  off[7] = ar.take(sizeof(double) * 2);   // n_active (int32) + worst rr/bb (double at +8)
+  // n_active (int32), worst rr/bb (double at +8), and the fused steps' counters
+  off[7] = ar.take(sizeof(double) * 2 + sizeof(uint32_t) * 2 * n_sys);
 }
 
 McgBufs mcg_bufs(kmv_handle h, const size_t off[8]) {
@@ -868,6 +870,7 @@ McgBufs mcg_bufs(kmv_handle h, const size_t off[8]) {
   b.cols = at<McgCol>(h, off[5]);
   b.sys_any = at<int32_t>(h, off[6]);
   b.n_active = at<int32_t>(h, off[7]);
+  b.count = reinterpret_cast<uint32_t*>(b.n_active + 4);
   return b;
 }
 
@@ -876,25 +879,27 @@ McgBufs mcg_bufs(kmv_handle h, const size_t off[8]) {
 struct McgPre {
   PcgPrecond P;
   float* z;
-  double *proj, *coef, *prz;
+  double *proj, *coef, *prz, *fac;
 };
 
-void mcg_pre_layout(const Layout& L, int m, int rank, Arena& ar, size_t off[4]) {
+void mcg_pre_layout(const Layout& L, int m, int rank, Arena& ar, size_t off[5]) {
   const size_t vec = sizeof(float) * (size_t)L.chains * std::max<int64_t>(1, L.n_total) * m;
   const size_t items = (size_t)std::max(1, L.n_items) * L.chains * m;
   off[0] = ar.take(vec);
   off[1] = ar.take(sizeof(double) * items * rank);
   off[2] = ar.take(sizeof(double) * (size_t)L.n_inst * L.chains * m * rank);
   off[3] = ar.take(sizeof(double) * items);
+  off[4] = ar.take(sizeof(double) * (size_t)L.n_inst * L.chains * m * rank);
 }
 
-McgPre mcg_pre(kmv_handle h, const size_t off[4]) {
+McgPre mcg_pre(kmv_handle h, const size_t off[5]) {
   McgPre p;
   p.P = PcgPrecond{h->pc.rank, h->pc.U, h->pc.lam};
   p.z = at<float>(h, off[0]);
   p.proj = at<double>(h, off[1]);
   p.coef = at<double>(h, off[2]);
   p.prz = at<double>(h, off[3]);
+  p.fac = at<double>(h, off[4]);
   return p;
 }
 
@@ -921,15 +926,22 @@ kmv_status run_mcg(kmv_handle h, const kmv_points* pts, const double* theta, con
   KMV_CUDA(h, launch_mcg_reduce_init(h->dev, L.n_inst, L.chains, m, B.partial2, tol, B.cols, B.sys_any,
                                      B.n_active, st));
   const size_t vbytes = sizeof(float) * (size_t)L.chains * L.n_total * m;
+  const int n_sys = L.n_inst * L.chains;
+  const McgBetaHook none{};
   if (pre) {
-    KMV_CUDA(h, launch_mcg_precond(h->dev, L.n_items, L.n_inst, L.chains, L.n_total, m, pre->P, a.theta, a.n_theta,
-                                   shifts, B.r, pre->z, B.sys_any, pre->proj, pre->coef, pre->prz, st));
+    KMV_CUDA(h, launch_mcg_factors(pre->P, n_sys, m, a.n_theta, a.theta, shifts, pre->fac, st));
+    KMV_CUDA(h, launch_mcg_precond(h->dev, L.n_items, L.n_inst, L.chains, L.n_total, m, pre->P, pre->fac, B.r, pre->z,
+                                   B.sys_any, pre->proj, pre->coef, pre->prz, none, false, st));
     KMV_CUDA(h, launch_mcg_set_rz(h->dev, L.n_inst, L.chains, m, pre->prz, B.cols, st));
     if (vbytes) KMV_CUDA(h, cudaMemcpyAsync(B.p, pre->z, vbytes, cudaMemcpyDeviceToDevice, st));
   }
   a.V = B.p;
   a.Y = B.q;
   a.sys_active = B.sys_any;
+  KMV_CUDA(h, cudaMemsetAsync(B.count, 0, sizeof(uint32_t) * 2 * n_sys, st));
+  const bool chained = !h->capturing;
+  a.chained = chained;
+  const McgBetaHook hook{B.count + n_sys, B.cols, B.partial, tol, maxiter, B.n_active};
   Poll poll;
   for (int it = 0; it < maxiter; ++it) {
     if (it % kCheckEvery == 0) {
@@ -937,18 +949,15 @@ kmv_status run_mcg(kmv_handle h, const kmv_points* pts, const double* theta, con
       if (poll.done) break;
     }
     KMV_TRY(run_forward(h, a, prec, st));
-    KMV_CUDA(h, launch_mcg_dot(h->dev, L.n_items, L.chains, L.n_total, m, B.p, B.q, B.sys_any, B.partial, st));
-    KMV_CUDA(h, launch_mcg_alpha(h->dev, L.n_inst, L.chains, m, B.partial, B.cols, B.sys_any, pre ? 1 : 0, st));
-    KMV_CUDA(h, launch_mcg_update_xr(h->dev, L.n_items, L.chains, L.n_total, m, B.cols, B.sys_any, x, B.r, B.p,
-                                     B.q, B.partial, st));
+    KMV_CUDA(h, launch_mcg_dot(h->dev, L.n_items, L.chains, L.n_total, m, B.p, B.q, B.sys_any, B.partial, B.count,
+                               B.cols, pre ? 1 : 0, B.n_active, chained, st));
+    KMV_CUDA(h, launch_mcg_update_xr(h->dev, L.n_items, L.chains, L.n_total, m, B.cols, B.sys_any, x, B.r, B.p, B.q,
+                                     B.partial, pre ? nullptr : B.count + n_sys, tol, maxiter, B.n_active, chained, st));
     if (pre)
-      KMV_CUDA(h, launch_mcg_precond(h->dev, L.n_items, L.n_inst, L.chains, L.n_total, m, pre->P, a.theta,
-                                     a.n_theta, shifts, B.r, pre->z, B.sys_any, pre->proj, pre->coef, pre->prz, st));
-    KMV_CUDA(h, cudaMemsetAsync(B.n_active, 0, sizeof(int32_t), st));
-    KMV_CUDA(h, launch_mcg_beta(h->dev, L.n_inst, L.chains, m, B.partial, pre ? pre->prz : nullptr, tol, maxiter,
-                                B.cols, B.sys_any, B.n_active, st));
-    KMV_CUDA(h, launch_mcg_update_p(h->dev, L.n_items, L.chains, L.n_total, m, B.cols, B.sys_any,
-                                    pre ? pre->z : B.r, B.p, st));
+      KMV_CUDA(h, launch_mcg_precond(h->dev, L.n_items, L.n_inst, L.chains, L.n_total, m, pre->P, pre->fac, B.r, pre->z,
+                                     B.sys_any, pre->proj, pre->coef, pre->prz, hook, chained, st));
+    KMV_CUDA(h, launch_mcg_update_p(h->dev, L.n_items, L.chains, L.n_total, m, B.cols, B.sys_any, pre ? pre->z : B.r,
+                                    B.p, chained, st));
   }
   return KMV_OK;
 }
@@ -1083,6 +1092,7 @@ kmv_status run_mscg(kmv_handle h, const kmv_points* pts, const double* theta, co
     a.ms_sh = B.sh;
     a.ms_m = m;
     a.ms_ps = B.ps;
+    a.chained = !h->capturing;
     a.cg_active = B.sys_active;
     a.cg_n_active = B.n_active;
     a.cg_count = B.count;
@@ -1098,10 +1108,10 @@ kmv_status run_mscg(kmv_handle h, const kmv_points* pts, const double* theta, co
     if (fused) {
       KMV_CUDA(h, launch_mscg_update_xr_beta(h->dev, L.n_items, L.chains, L.n_total, m, B.sys, B.sh, B.sys_active,
                                              B.r, B.q, x, B.ps, B.partial, B.count + n_sys, tol, maxiter, B.n_active,
-                                             st));
+                                             a.chained, st));
       if (!tc_fma)
         KMV_CUDA(h, launch_mscg_update_p(h->dev, L.n_items, L.chains, L.n_total, m, B.sys, B.sh, B.sys_active, B.r,
-                                         B.p, B.ps, st));
+                                         B.p, B.ps, a.chained, st));
       continue;
     }
     KMV_CUDA(h, launch_mscg_alpha(h->dev, L.n_inst, L.chains, m, B.partial, B.sys, B.sh, B.sys_active, st));
@@ -1111,7 +1121,7 @@ kmv_status run_mscg(kmv_handle h, const kmv_points* pts, const double* theta, co
     KMV_CUDA(h, launch_mscg_beta(h->dev, L.n_inst, L.chains, m, B.partial, tol, maxiter, B.sys, B.sh, B.sys_active,
                                  B.n_active, st));
     KMV_CUDA(h, launch_mscg_update_p(h->dev, L.n_items, L.chains, L.n_total, m, B.sys, B.sh, B.sys_active, B.r, B.p,
-                                     B.ps, st));
+                                     B.ps, false, st));
   }
   KMV_CUDA(h, launch_mscg_finish(n_cols, B.sh, col_status, col_iters, st));
   return KMV_OK;
@@ -1285,7 +1295,7 @@ kmv_status kmv_phi_refresh(kmv_handle h, const kmv_points* pts, int32_t chains, 
   if (h->pc_on && !use_pc)
     return fail(h, KMV_EINVAL, "the preconditioner was built for another layout (n_inst, chains, N_total)");
   Arena ar;
-  size_t ob[8], orf[8], oms[10], opre[4];
+  size_t ob[8], orf[8], oms[10], opre[5];
   if (!use_pc) mscg_layout(L, n_poles, ar, oms);
   if (refined || use_pc) mcg_layout(L, n_poles, ar, ob);
   if (refined && !use_pc) mcg_layout(L, n_poles, ar, orf);
@@ -1379,7 +1389,7 @@ kmv_status kmv_nystrom_build(kmv_handle h, const kmv_points* pts, int32_t chains
   KMV_TRY(run_forward(h, a, prec, st));
   KMV_CUDA(h, launch_nystrom_finish(h->dev, L.n_items, L.n_inst, L.chains, L.n_total, rank, omega, at<float>(h, o_y),
                                     at<double>(h, o_g), at<double>(h, o_s), at<double>(h, o_t), at<double>(h, o_nu), U,
-                                    lam, chain_status, st));
+                                    lam, chain_status, h->num_sms, st));
   return KMV_OK;
 }
 
@@ -1545,47 +1555,52 @@ kmv_status kmv_implicit_step(kmv_handle h, const kmv_points* pts, int32_t chains
   const kmv_precision lin_prec = KMV_FP32;
   (void)prec;
   Poll poll;
+  const bool chained = !h->capturing;
+  KMV_CUDA(h, launch_fill_i32(n_active, 1, n_sys, st));
+  // the midpoint and the force's columns of the first iterate; each iteration forms the next ones
+  KMV_CUDA(h, launch_imp_mid(n_sys * n, th0, theta, tb, st));
+  KMV_CUDA(h, launch_pack_force(L.chains, L.n_total, x_work, phi, at<float>(h, o_vf), at<float>(h, o_gf), st));
   for (int it = 0; it < maxiter; ++it) {
     if (!h->capturing && it > 0 && it % kCheckEvery == 0) {
       KMV_TRY(poll.step(h, n_active, st));
       if (poll.done) break;
     }
     const int slot = it % k, cnt = std::min(it + 1, k);
-    KMV_CUDA(h, launch_imp_mid(n_sys * n, th0, theta, tb, st));
     KMV_TRY(cheb_prepare(h, pts, tb, 2, st));
     KmvArgs a = base_args(h, pts, tb);
     a.m = 1;
     a.V = x_work;
     a.Y = q;
     a.sys_active = active;
+    a.chained = chained ? 2 : 0;
     KMV_TRY(run_forward(h, a, lin_prec, st));
-    KMV_CUDA(h, launch_imp_resid(h->dev, L.n_items, L.chains, L.n_total, y, q, active, r, at<double>(h, o_rp), st));
+    KMV_CUDA(h, launch_imp_resid(h->dev, L.n_items, L.chains, L.n_total, y, q, active, r, at<double>(h, o_rp), chained,
+                                 st));
     const float* zz = r;
     if (h->pc_on) {
       KMV_CUDA(h, launch_pcg_precond(h->dev, L.n_items, L.n_inst, L.chains, L.n_total, P, fac, r, z, active,
-                                     at<double>(h, o_proj), at<double>(h, o_coef), at<double>(h, o_prz), false, st));
+                                     at<double>(h, o_proj), at<double>(h, o_coef), at<double>(h, o_prz), chained, st));
       zz = z;
     }
     KMV_CUDA(h, launch_imp_x(h->dev, L.n_items, L.chains, L.n_total, k, slot, cnt, x_work, zz, cscale, active,
-                             at<float>(h, o_gx), at<float>(h, o_fx), at<double>(h, o_xp), st));
+                             at<float>(h, o_gx), at<float>(h, o_fx), at<double>(h, o_xp), chained, st));
     // the frozen-x force at theta_bar (FP32 adjoint, as in the leapfrog step)
-    KMV_CUDA(h, launch_pack_force(L.chains, L.n_total, x_work, phi, at<float>(h, o_vf), at<float>(h, o_gf), st));
     KmvArgs fa = base_args(h, pts, tb);
     fa.V = at<float>(h, o_vf);
     fa.G = at<float>(h, o_gf);
     fa.m = 2;
     fa.Y = nullptr;
     fa.sys_active = active;
+    fa.chained = a.chained;
     KMV_TRY(run_backward(h, fa, grad, at<double>(h, o_bp), KMV_FP32, st));
-    KMV_CUDA(h, cudaMemsetAsync(n_active, 0, sizeof(int32_t), st));
     KMV_CUDA(h, launch_imp_aa(h->dev, L.n_inst, L.chains, n, k, slot, cnt, th0, pi0, theta, pi, grad, prior_mu,
                               prior_prec, free_mask, dt, at<double>(h, o_xp), at<double>(h, o_rp), tol, it, maxiter,
                               at<double>(h, o_gtp), at<double>(h, o_ftp), at<double>(h, o_h), at<double>(h, o_al),
                               active, at<int32_t>(h, o_dn), chain_status, iters, n_active, at<double>(h, o_brr),
-                              at<int32_t>(h, o_bit), st));
-    KMV_CUDA(h, launch_imp_mix(h->dev, L.n_items, L.n_inst, L.chains, L.n_total, n, k, slot, cnt,
-                               at<double>(h, o_gtp), at<float>(h, o_gx), at<double>(h, o_al), active,
-                               at<int32_t>(h, o_dn), theta, pi, x_work, st));
+                              at<int32_t>(h, o_bit), tb, chained, st));
+    KMV_CUDA(h, launch_imp_mix(h->dev, L.n_items, L.chains, L.n_total, k, slot, cnt, at<float>(h, o_gx),
+                               at<double>(h, o_al), active, at<int32_t>(h, o_dn), x_work, at<float>(h, o_vf),
+                               at<float>(h, o_gf), chained, st));
   }
   return KMV_OK;
 }

@@ -156,7 +156,7 @@ struct KmvArgs {
   MscgShift* ms_sh;
   int ms_m;
   float* ms_ps;
-  int chained;   // inside a solver's chain of dependent launches (launch_chained)
+  int chained;   // inside a solver's chain of dependent launches (launch_chained); 2: theta changes within it
 };
 
 // The argument rules of a point set and chain count shared by every entry
@@ -211,7 +211,8 @@ cudaError_t launch_backward_simt(const KmvArgs& a, const SimtBwd& f, int n_items
 
 // Gradient finalisation: sums partials per system in a fixed order and scales.
 cudaError_t launch_grad_finalize(const DevLayout& L, const SimtBwd& f, int n_inst, int chains, int n_theta,
-                                 const double* theta, const double* partial, double* grad, cudaStream_t st);
+                                 const double* theta, const double* partial, double* grad, bool chained,
+                                 cudaStream_t st);
 
 // CG / leapfrog / energy kernels (kmv_cg.cu)
 cudaError_t launch_cg_init(const DevLayout& L, int n_items, int chains, int64_t n_total,
@@ -274,7 +275,7 @@ struct PcgPrecond {
 };
 cudaError_t launch_nystrom_finish(const DevLayout& L, int n_items, int n_inst, int chains, int64_t n_total, int r,
                                   const float* Om, const float* Y, double* grams, double* scratch, double* T,
-                                  double* nu, float* U, double* lam, int32_t* status, cudaStream_t st);
+                                  double* nu, float* U, double* lam, int32_t* status, int num_sms, cudaStream_t st);
 cudaError_t launch_pcg_init(const DevLayout& L, int n_items, int chains, int64_t n_total, const float* rhs,
                             int64_t rhs_stride, const float* q, float* x, float* r, int warm, double* partial2,
                             cudaStream_t st);
@@ -314,20 +315,21 @@ constexpr int kMaxAA = 16;
 cudaError_t launch_fill_i32(int32_t* v, int n, int32_t val, cudaStream_t st);
 cudaError_t launch_imp_mid(int n, const double* th0, const double* th, double* tb, cudaStream_t st);
 cudaError_t launch_imp_resid(const DevLayout& L, int n_items, int chains, int64_t n_total, const float* y,
-                             const float* q, const int32_t* active, float* r, double* partial2, cudaStream_t st);
+                             const float* q, const int32_t* active, float* r, double* partial2, bool chained,
+                             cudaStream_t st);
 cudaError_t launch_imp_x(const DevLayout& L, int n_items, int chains, int64_t n_total, int k, int slot, int cnt,
                          const float* x, const float* z, const double* cscale, const int32_t* active, float* Gx,
-                         float* Fx, double* partial, cudaStream_t st);
+                         float* Fx, double* partial, bool chained, cudaStream_t st);
 cudaError_t launch_imp_aa(const DevLayout& L, int n_inst, int chains, int n, int k, int slot, int cnt,
-                          const double* th0, const double* pi0, const double* th, const double* pi,
-                          const double* grad, const double* mu, const double* prec, const uint8_t* mask, double dt,
-                          const double* xpart, const double* rpart, double tol, int iter, int maxiter, double* Gtp,
-                          double* Ftp, double* H, double* alpha, int32_t* active, int32_t* done_now, int32_t* status,
-                          int32_t* iters, int32_t* n_active, double* best_rr, int32_t* best_it, cudaStream_t st);
-cudaError_t launch_imp_mix(const DevLayout& L, int n_items, int n_inst, int chains, int64_t n_total, int n, int k,
-                           int slot, int cnt, const double* Gtp, const float* Gx, const double* alpha,
-                           const int32_t* active, const int32_t* done_now, double* th, double* pi, float* x,
-                           cudaStream_t st);
+                          const double* th0, const double* pi0, double* th, double* pi, const double* grad,
+                          const double* mu, const double* prec, const uint8_t* mask, double dt, const double* xpart,
+                          const double* rpart, double tol, int iter, int maxiter, double* Gtp, double* Ftp, double* H,
+                          double* alpha, int32_t* active, int32_t* done_now, int32_t* status, int32_t* iters,
+                          int32_t* n_active, double* best_rr, int32_t* best_it, double* tb_next, bool chained,
+                          cudaStream_t st);
+cudaError_t launch_imp_mix(const DevLayout& L, int n_items, int chains, int64_t n_total, int k, int slot, int cnt,
+                           const float* Gx, const double* alpha, const int32_t* active, const int32_t* done_now,
+                           float* x, float* Vf, float* Gf, bool chained, cudaStream_t st);
 cudaError_t launch_imp_scale(const DevLayout& L, int n_items, int chains, int64_t n_total, const double* norm,
                              const float* w, float* v, double* partial, cudaStream_t st);
 cudaError_t launch_imp_norm(const DevLayout& L, int n_inst, int chains, const double* partial, double* cscale,
@@ -367,10 +369,10 @@ cudaError_t launch_mscg_beta(const DevLayout& L, int n_inst, int chains, int m, 
 cudaError_t launch_mscg_update_xr_beta(const DevLayout& L, int n_items, int chains, int64_t n_total, int m,
                                        MscgSys* sys, MscgShift* sh, int32_t* sys_active, float* r, const float* q,
                                        float* xs, const float* ps, double* partial, uint32_t* count, double tol,
-                                       int maxiter, int32_t* n_active, cudaStream_t st);
+                                       int maxiter, int32_t* n_active, bool chained, cudaStream_t st);
 cudaError_t launch_mscg_update_p(const DevLayout& L, int n_items, int chains, int64_t n_total, int m,
                                  const MscgSys* sys, const MscgShift* sh, const int32_t* sys_active, const float* r,
-                                 float* p, float* ps, cudaStream_t st);
+                                 float* p, float* ps, bool chained, cudaStream_t st);
 cudaError_t launch_mscg_finish(int64_t n_cols, const MscgShift* sh, int32_t* col_status, int32_t* col_iters,
                                cudaStream_t st);
 
@@ -380,16 +382,16 @@ cudaError_t launch_mcg_init(const DevLayout& L, int n_items, int chains, int64_t
                             cudaStream_t st);
 cudaError_t launch_mcg_reduce_init(const DevLayout& L, int n_inst, int chains, int m, const double* partial2,
                                    double tol, McgCol* st, int32_t* sys_any, int32_t* n_active, cudaStream_t s);
+// p.q per column, and the columns' alpha steps by each system's last CTA (count: one
+// zeroed counter per system).
 cudaError_t launch_mcg_dot(const DevLayout& L, int n_items, int chains, int64_t n_total, int m, const float* p,
-                           const float* q, const int32_t* sys_any, double* partial, cudaStream_t st);
-cudaError_t launch_mcg_alpha(const DevLayout& L, int n_inst, int chains, int m, const double* partial, McgCol* st,
-                             const int32_t* sys_any, int pre, cudaStream_t s);
-cudaError_t launch_mcg_update_xr(const DevLayout& L, int n_items, int chains, int64_t n_total, int m,
-                                 const McgCol* stt, const int32_t* sys_any, float* x, float* r, const float* p,
-                                 const float* q, double* partial, cudaStream_t st);
-cudaError_t launch_mcg_beta(const DevLayout& L, int n_inst, int chains, int m, const double* partial,
-                            const double* prz, double tol, int maxiter, McgCol* st, int32_t* sys_any,
-                            int32_t* n_active, cudaStream_t s);
+                           const float* q, int32_t* sys_any, double* partial, uint32_t* count, McgCol* cols, int pre,
+                           int32_t* n_active, bool chained, cudaStream_t st);
+// x, r and r.r; with count (no preconditioner) the beta steps likewise.
+cudaError_t launch_mcg_update_xr(const DevLayout& L, int n_items, int chains, int64_t n_total, int m, McgCol* cols,
+                                 int32_t* sys_any, float* x, float* r, const float* p, const float* q, double* partial,
+                                 uint32_t* count, double tol, int maxiter, int32_t* n_active, bool chained,
+                                 cudaStream_t st);
 cudaError_t launch_mcg_finish(int64_t n_cols, const McgCol* cols, int accumulate, int32_t* col_status,
                               int32_t* col_iters, cudaStream_t st);
 cudaError_t launch_mcg_mask(const DevLayout& L, int n_items, int chains, int64_t n_total, int m, const McgCol* cols,
@@ -400,14 +402,25 @@ cudaError_t launch_mcg_undo(const DevLayout& L, int n_items, int chains, int64_t
                             const float* dx, float* x, cudaStream_t st);
 cudaError_t launch_mcg_refine_finish(int64_t n_cols, const McgCol* cols, int32_t* col_status, cudaStream_t st);
 // preconditioned multi-column CG: z_q = r_q + U (d_q o (U^T r_q)), d from mu_q = sigma^2 + shift_q
+// (once per solve); with the hook's count the columns' beta steps by each system's last CTA
+struct McgBetaHook {
+  uint32_t* count;
+  McgCol* cols;
+  const double* prr;
+  double tol;
+  int maxiter;
+  int32_t* n_active;
+};
+cudaError_t launch_mcg_factors(const PcgPrecond& P, int n_sys, int m, int n_theta, const double* theta,
+                               const float* shifts, double* d, cudaStream_t st);
 cudaError_t launch_mcg_precond(const DevLayout& L, int n_items, int n_inst, int chains, int64_t n_total, int m,
-                               const PcgPrecond& P, const double* theta, int n_theta, const float* shifts,
-                               const float* r, float* z, const int32_t* sys_any, double* proj, double* coef,
-                               double* prz, cudaStream_t st);
+                               const PcgPrecond& P, const double* d, const float* r, float* z, int32_t* sys_any,
+                               double* proj, double* coef, double* prz, const McgBetaHook& h, bool chained,
+                               cudaStream_t st);
 cudaError_t launch_mcg_set_rz(const DevLayout& L, int n_inst, int chains, int m, const double* prz, McgCol* cols,
                               cudaStream_t st);
 cudaError_t launch_mcg_update_p(const DevLayout& L, int n_items, int chains, int64_t n_total, int m,
-                                const McgCol* stt, const int32_t* sys_any, const float* r, float* p,
+                                const McgCol* stt, const int32_t* sys_any, const float* r, float* p, bool chained,
                                 cudaStream_t st);
 
 

@@ -165,9 +165,11 @@ __global__ void mscg_update_xr_beta_kernel(DevLayout L, int chains, int64_t n_to
   __shared__ float as[kMaxShifts];
   __shared__ int on[kMaxShifts];
   __shared__ int s_last;
+  chain_trigger();
   const int item = blockIdx.x, c = blockIdx.y;
   const int bi = L.item_inst[item];
   const int s = bi * chains + c;
+  chain_wait();
   if (!sys_active[s]) return;
   if (threadIdx.x < m) {
     const MscgShift& k = sh[(int64_t)s * m + threadIdx.x];
@@ -207,9 +209,11 @@ __global__ void mscg_update_p_kernel(DevLayout L, int chains, int64_t n_total, i
                                      float* ps) {
   __shared__ float zs[kMaxShifts], bs[kMaxShifts];
   __shared__ int on[kMaxShifts];
+  chain_trigger();
   const int item = blockIdx.x, c = blockIdx.y;
   const int bi = L.item_inst[item];
   const int s = bi * chains + c;
+  chain_wait();
   if (!sys_active[s]) return;
   if (threadIdx.x < m) {
     const MscgShift& k = sh[(int64_t)s * m + threadIdx.x];
@@ -281,21 +285,18 @@ cudaError_t launch_mscg_beta(const DevLayout& L, int n_inst, int chains, int m, 
 cudaError_t launch_mscg_update_xr_beta(const DevLayout& L, int n_items, int chains, int64_t n_total, int m,
                                        MscgSys* sys, MscgShift* sh, int32_t* sys_active, float* r, const float* q,
                                        float* xs, const float* ps, double* partial, uint32_t* count, double tol,
-                                       int maxiter, int32_t* n_active, cudaStream_t st) {
+                                       int maxiter, int32_t* n_active, bool chained, cudaStream_t st) {
   if (n_items == 0) return cudaSuccess;
-  mscg_update_xr_beta_kernel<<<dim3(n_items, chains), kTile, 0, st>>>(L, chains, n_total, m, sys, sh, sys_active, r,
-                                                                      q, xs, ps, partial, count, tol, maxiter,
-                                                                      n_active);
-  return cudaGetLastError();
+  return launch_chained(chained, mscg_update_xr_beta_kernel, dim3(n_items, chains), kTile, 0, st, L, chains, n_total, m,
+                        sys, sh, sys_active, r, q, xs, ps, partial, count, tol, maxiter, n_active);
 }
 
 cudaError_t launch_mscg_update_p(const DevLayout& L, int n_items, int chains, int64_t n_total, int m,
                                  const MscgSys* sys, const MscgShift* sh, const int32_t* sys_active, const float* r,
-                                 float* p, float* ps, cudaStream_t st) {
+                                 float* p, float* ps, bool chained, cudaStream_t st) {
   if (n_items == 0) return cudaSuccess;
-  mscg_update_p_kernel<<<dim3(n_items, chains), kTile, 0, st>>>(L, chains, n_total, m, sys, sh, sys_active, r, p,
-                                                                ps);
-  return cudaGetLastError();
+  return launch_chained(chained, mscg_update_p_kernel, dim3(n_items, chains), kTile, 0, st, L, chains, n_total, m, sys,
+                        sh, sys_active, r, p, ps);
 }
 
 cudaError_t launch_mscg_finish(int64_t n_cols, const MscgShift* sh, int32_t* col_status, int32_t* col_iters,

@@ -23,50 +23,74 @@ namespace {
 constexpr int kGB = 32;   // Gram / U block edge
 
 // grams[s] = [O^T Y, O^T O, Y^T Y] (r x r each, FP64 products and sums), one
-// 32 x 32 block per CTA, rows staged 32 at a time.  FP64 throughout: the columns
-// of U = Y_nu T come out orthonormal only as far as these sums are exact, and
+// 32 x 32 block of one matrix per CTA, rows staged 32 at a time.  FP64 throughout: the
+// columns of U = Y_nu T come out orthonormal only as far as these sums are exact, and
 // the preconditioner stays positive definite only while that error is below
-// (lambda_r + mu) / (lambda_1 + mu).
+// (lambda_r + mu) / (lambda_1 + mu).  Every entry is one chain over the rows in order.
+// Bound by the FP64 pipe (2 lanes per clock and SM, conversions included): the staged
+// values are converted once, and the symmetric matrices' lower blocks are mirrored
+// (u v and v u round alike): 36 blocks in place of 48 at r = 128, 24.8 ms before at
+// N = 16,384 with 8 chains.
 __global__ void __launch_bounds__(256) ny_gram_kernel(DevLayout L, int chains, int64_t n_total, int r, int nb,
                                                       const float* Om, const float* Y, double* grams) {
-  __shared__ float ok[kGB][kGB + 1], ol[kGB][kGB + 1], yk[kGB][kGB + 1], yl[kGB][kGB + 1];
+  __shared__ double ak[kGB][kGB + 1], bl[kGB][kGB + 1];
   const int s = blockIdx.x;
   const int b = s / chains, c = s - b * chains;
-  const int kb = blockIdx.y / nb, lb = blockIdx.y - (blockIdx.y / nb) * nb;
+  // block index -> matrix g and block (kb, lb): all of O^T Y, the upper blocks of the others
+  int e = blockIdx.y, g = 0, kb, lb;
+  if (e < nb * nb) {
+    kb = e / nb;
+    lb = e - kb * nb;
+  } else {
+    e -= nb * nb;
+    const int half = nb * (nb + 1) / 2;
+    g = 1 + e / half;
+    e -= (g - 1) * half;
+    kb = 0;
+    while (e >= nb - kb) e -= nb - kb++;
+    lb = kb + e;
+  }
+  const float* A = g == 2 ? Y : Om;
+  const float* B = g == 1 ? Om : Y;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
   const int64_t j0 = L.offsets[b], j1 = L.offsets[b + 1];
-  double a64[3][4] = {};
-  for (int64_t i0 = j0; i0 < j1; i0 += kGB) {
-    for (int e = threadIdx.x; e < kGB * kGB; e += 256) {
-      const int rr = e / kGB, cc = e - rr * kGB;
-      const int64_t i = i0 + rr;
-      const bool in = i < j1;
-      const int k = kb * kGB + cc, l = lb * kGB + cc;
+  double acc[4] = {};
+  float fa[4], fb[4];   // the next rows, loaded while the current ones are summed
+  auto fetch = [&](int64_t i0) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int64_t i = i0 + ty + 8 * q;
+      const int k = kb * kGB + tx, l = lb * kGB + tx;
       const int64_t base = ((int64_t)c * n_total + i) * r;
-      ok[rr][cc] = (in && k < r) ? Om[base + k] : 0.f;
-      yk[rr][cc] = (in && k < r) ? Y[base + k] : 0.f;
-      ol[rr][cc] = (in && l < r) ? Om[base + l] : 0.f;
-      yl[rr][cc] = (in && l < r) ? Y[base + l] : 0.f;
+      fa[q] = i < j1 && k < r ? A[base + k] : 0.f;
+      fb[q] = i < j1 && l < r ? B[base + l] : 0.f;
+    }
+  };
+  fetch(j0);
+  for (int64_t i0 = j0; i0 < j1; i0 += kGB) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      ak[ty + 8 * q][tx] = fa[q];
+      bl[ty + 8 * q][tx] = fb[q];
     }
     __syncthreads();
+    if (i0 + kGB < j1) fetch(i0 + kGB);
+#pragma unroll 4
     for (int rr = 0; rr < kGB; ++rr) {
-      const double oL = ol[rr][tx], yL = yl[rr][tx];
+      const double v = bl[rr][tx];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int kk = ty + 8 * q;
-        const double oK = ok[rr][kk], yK = yk[rr][kk];
-        a64[0][q] = fma(oK, yL, a64[0][q]);
-        a64[1][q] = fma(oK, oL, a64[1][q]);
-        a64[2][q] = fma(yK, yL, a64[2][q]);
-      }
+      for (int q = 0; q < 4; ++q) acc[q] = fma(ak[rr][ty + 8 * q], v, acc[q]);
     }
     __syncthreads();
   }
   const int l = lb * kGB + tx;
+  double* out = grams + ((int64_t)s * 3 + g) * r * r;
   for (int q = 0; q < 4; ++q) {
     const int k = kb * kGB + ty + 8 * q;
-    if (k < r && l < r)
-      for (int g = 0; g < 3; ++g) grams[(((int64_t)s * 3 + g) * r + k) * r + l] = a64[g][q];
+    if (k < r && l < r) {
+      out[k * r + l] = acc[q];
+      if (g > 0 && kb != lb) out[l * r + k] = acc[q];
+    }
   }
 }
 
@@ -108,18 +132,17 @@ __device__ bool block_cholesky(double* W, int r, int* fail) {
   return ok;
 }
 
-// The r x r part per system (one CTA, FP64, matrices in the system's scratch):
-// nu, W = sym(O^T Y) + nu O^T O = L L^T, M = L^{-1} G_nu L^{-T}, Jacobi M = V S2 V^T,
-// sorted descending; lam = max(S2 - nu, 0); T = L^{-T} V S2^{-1/2} (FP32 out).
+// The r x r part per system (FP64, matrices in the system's scratch), in three
+// kernels: here (one CTA) nu, W = sym(O^T Y) + nu O^T O = L L^T and
+// M = L^{-1} G_nu L^{-T}; then the Jacobi eigendecomposition M = V S2 V^T; then,
+// sorted descending, lam = max(S2 - nu, 0) and T = L^{-T} V S2^{-1/2}.
 // A system whose Cholesky fails at every shift (or with fewer rows than r) gets
 // lam = 0 and T = 0: its preconditioner is the identity.
-__global__ void __launch_bounds__(256) ny_small_kernel(DevLayout L, int chains, int r, const double* grams,
-                                                       double* scratch, double* T, double* lam, double* nu_out,
-                                                       int32_t* status) {
+__global__ void __launch_bounds__(256) ny_factor_kernel(DevLayout L, int chains, int r, const double* grams,
+                                                        double* scratch, double* T, double* lam, double* nu_out,
+                                                        int32_t* status) {
   __shared__ double red[8];
-  __shared__ double cs[kMaxRank / 2 + 1][2];
-  __shared__ int pq[kMaxRank / 2 + 1][2];
-  __shared__ int perm[kMaxRank];
+  __shared__ double cs[8][2];
   __shared__ int fail;
   const int s = blockIdx.x;
   const int b = s / chains;
@@ -130,7 +153,6 @@ __global__ void __launch_bounds__(256) ny_small_kernel(DevLayout L, int chains, 
   double* W = scratch + (int64_t)s * 4 * r * r;   // W, then L in its lower triangle
   double* G = W + r * r;                          // G_nu, then X = L^{-1} G_nu
   double* M = G + r * r;
-  double* V = M + r * r;
   const int tid = threadIdx.x, nt = blockDim.x;
   const int rr = r * r;
 
@@ -211,76 +233,156 @@ __global__ void __launch_bounds__(256) ny_small_kernel(DevLayout L, int chains, 
   __syncthreads();
   for (int e = tid; e < rr; e += nt) {
     const int k = e / r, l = e - k * r;
-    V[e] = k == l ? 1.0 : 0.0;
     if (k < l) {
       const double v = 0.5 * (M[e] + M[l * r + k]);
       M[e] = v;
       M[l * r + k] = v;
     }
   }
-  __syncthreads();
-  // cyclic Jacobi, round-robin pairs (r rounded up to even; index r is a bye)
+  if (tid == 0) {
+    nu_out[s] = nu;
+    status[s] = KMV_OK;
+  }
+}
+
+// Cyclic Jacobi on a system's M (r x r), round-robin pairs (r rounded up to even; index
+// r is a bye), V the product of the rotations.  A round's rotations are disjoint, so the
+// 2 x 2 block of M at the rows of pair I and the columns of pair J is rotated on both
+// sides by one thread from values of before the round, and every element sees the same
+// operations in the same order however the blocks are spread.  Some 100 K FP64
+// operations per round against 2 lanes per clock and SM: one CTA per system took
+// 106 ms for 8 systems of rank 128, so a cluster of `cl` CTAs shares the blocks (M in
+// L2, V by rows in shared memory) with one cluster barrier per round.
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+constexpr int kJacThreads = 256;
+__global__ void __launch_bounds__(kJacThreads) ny_jacobi_kernel(int r, int cl, double* scratch, const int32_t* status) {
+  extern __shared__ double vrow[];   // this CTA's rows of V
+  __shared__ double red[kJacThreads / 32];
+  __shared__ double cs[kMaxRank / 2 + 1][2];
+  const int s = blockIdx.x / cl, rank = blockIdx.x % cl;
+  if (status[s] != KMV_OK) return;   // (the whole cluster)
+  double* M = scratch + (int64_t)s * 4 * r * r + 2 * (int64_t)r * r;
+  double* V = M + (int64_t)r * r;
+  const int tid = threadIdx.x, rr = r * r;
+  const int v0 = r * rank / cl, v1 = r * (rank + 1) / cl, nv = v1 - v0;
+  for (int e = tid; e < nv * r; e += kJacThreads) vrow[e] = e / r + v0 == e % r ? 1.0 : 0.0;
   const int n2 = r + (r & 1), np = n2 / 2;
+  const int per = (np * np + cl - 1) / cl, e0 = rank * per, e1 = min(np * np, e0 + per);
+  auto pair_of = [&](int t, int k, int& p, int& q) {
+    if (k == 0) {
+      p = t;
+      q = n2 - 1;
+    } else {
+      p = t + k;
+      if (p >= n2 - 1) p -= n2 - 1;
+      q = t - k;
+      if (q < 0) q += n2 - 1;
+    }
+    if (p > q) {
+      const int u = p;
+      p = q;
+      q = u;
+    }
+  };
+  __syncthreads();
   for (int sweep = 0; sweep < 20; ++sweep) {
     for (int t = 0; t < n2 - 1; ++t) {
-      for (int k = tid; k < np; k += nt) {
+      // rotations of the round (every CTA of the cluster computes them all)
+      for (int k = tid; k < np; k += kJacThreads) {
         int p, q;
-        if (k == 0) {
-          p = t;
-          q = n2 - 1;
-        } else {
-          p = (t + k) % (n2 - 1);
-          q = (t - k + n2 - 1) % (n2 - 1);
-        }
-        if (p > q) {
-          const int u = p;
-          p = q;
-          q = u;
-        }
+        pair_of(t, k, p, q);
         double c = 1.0, sn = 0.0;
         if (q < r) {
-          const double apq = M[p * r + q];
+          const double apq = __ldcg(&M[p * r + q]);
           if (apq != 0.0) {
-            const double th = (M[q * r + q] - M[p * r + p]) / (2.0 * apq);
+            const double th = (__ldcg(&M[q * r + q]) - __ldcg(&M[p * r + p])) / (2.0 * apq);
             const double tt = copysign(1.0, th) / (fabs(th) + sqrt(th * th + 1.0));
             c = 1.0 / sqrt(tt * tt + 1.0);
             sn = tt * c;
           }
         }
-        pq[k][0] = p;
-        pq[k][1] = q;
         cs[k][0] = c;
         cs[k][1] = sn;
       }
+      // two blocks at a time; the first two loaded before the rotations are known
+      double m00[2], m01[2], m10[2], m11[2];
+      int at[2][4];
+      auto load = [&](int e, int u) {
+        at[u][0] = -1;
+        if (e >= e1) return;
+        int pi, qi, pj, qj;
+        const int I = e / np, J = e - I * np;
+        pair_of(t, I, pi, qi);
+        pair_of(t, J, pj, qj);
+        at[u][0] = pi * r + pj;
+        at[u][1] = qj < r ? pi * r + qj : -1;
+        at[u][2] = qi < r ? qi * r + pj : -1;
+        at[u][3] = qi < r && qj < r ? qi * r + qj : -1;
+        m00[u] = __ldcg(&M[at[u][0]]);
+        m01[u] = at[u][1] >= 0 ? __ldcg(&M[at[u][1]]) : 0.0;
+        m10[u] = at[u][2] >= 0 ? __ldcg(&M[at[u][2]]) : 0.0;
+        m11[u] = at[u][3] >= 0 ? __ldcg(&M[at[u][3]]) : 0.0;
+      };
+      load(e0 + tid, 0);
+      load(e0 + tid + kJacThreads, 1);
       __syncthreads();
-      for (int e = tid; e < np * r; e += nt) {   // rows p, q of J^T M
-        const int k = e / r, col = e - k * r;
-        const int p = pq[k][0], q = pq[k][1];
+      // every read of the old M by this cluster precedes every write of the new one:
+      // the rotations read entries that other CTAs write
+      cluster_barrier();
+      for (int e = e0 + tid; e < e1; e += 2 * kJacThreads) {
+        if (e != e0 + tid) {
+          load(e, 0);
+          load(e + kJacThreads, 1);
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          if (at[u][0] < 0) continue;
+          const int eu = e + u * kJacThreads, I = eu / np, J = eu - I * np;
+          if (at[u][2] >= 0) {
+            const double c = cs[I][0], sn = cs[I][1];
+            const double mp = m00[u], mq = m10[u];
+            m00[u] = c * mp - sn * mq;
+            m10[u] = sn * mp + c * mq;
+            const double np_ = m01[u], nq = m11[u];
+            m01[u] = c * np_ - sn * nq;
+            m11[u] = sn * np_ + c * nq;
+          }
+          if (at[u][1] >= 0) {
+            const double c = cs[J][0], sn = cs[J][1];
+            const double mp = m00[u], mq = m01[u];
+            m00[u] = c * mp - sn * mq;
+            m01[u] = sn * mp + c * mq;
+            const double np_ = m10[u], nq = m11[u];
+            m10[u] = c * np_ - sn * nq;
+            m11[u] = sn * np_ + c * nq;
+            __stcg(&M[at[u][1]], m01[u]);
+            if (at[u][3] >= 0) __stcg(&M[at[u][3]], m11[u]);
+          }
+          __stcg(&M[at[u][0]], m00[u]);
+          if (at[u][2] >= 0) __stcg(&M[at[u][2]], m10[u]);
+        }
+      }
+      for (int e = tid; e < np * nv; e += kJacThreads) {   // columns p, q of V J
+        const int k = e % np, row = e / np;
+        int p, q;
+        pair_of(t, k, p, q);
         if (q >= r) continue;
         const double c = cs[k][0], sn = cs[k][1];
-        const double mp = M[p * r + col], mq = M[q * r + col];
-        M[p * r + col] = c * mp - sn * mq;
-        M[q * r + col] = sn * mp + c * mq;
+        const double vp = vrow[row * r + p], vq = vrow[row * r + q];
+        vrow[row * r + p] = c * vp - sn * vq;
+        vrow[row * r + q] = sn * vp + c * vq;
       }
-      __syncthreads();
-      for (int e = tid; e < np * r; e += nt) {   // columns p, q of (J^T M) J and of V J
-        const int k = e / r, row = e - k * r;
-        const int p = pq[k][0], q = pq[k][1];
-        if (q >= r) continue;
-        const double c = cs[k][0], sn = cs[k][1];
-        const double mp = M[row * r + p], mq = M[row * r + q];
-        M[row * r + p] = c * mp - sn * mq;
-        M[row * r + q] = sn * mp + c * mq;
-        const double vp = V[row * r + p], vq = V[row * r + q];
-        V[row * r + p] = c * vp - sn * vq;
-        V[row * r + q] = sn * vp + c * vq;
-      }
-      __syncthreads();
+      __syncthreads();   // cs is rewritten by the next round
+      cluster_barrier();
     }
-    // stop when the off-diagonal part is at rounding level
+    // stop when the off-diagonal part is at rounding level (every CTA sums all of M, in
+    // the same order, so that all of a cluster's stop together)
     double off = 0.0, all = 0.0;
-    for (int e = tid; e < rr; e += nt) {
-      const double v = M[e] * M[e];
+    for (int e = tid; e < rr; e += kJacThreads) {
+      const double m = __ldcg(&M[e]);
+      const double v = m * m;
       all += v;
       if (e / r != e % r) off += v;
     }
@@ -289,27 +391,44 @@ __global__ void __launch_bounds__(256) ny_small_kernel(DevLayout L, int chains, 
       all += __shfl_down_sync(0xffffffffu, all, o);
     }
     __syncthreads();
-    if ((tid & 31) == 0) {
-      red[tid >> 5] = off;
-    }
+    if ((tid & 31) == 0) red[tid >> 5] = off;
     __syncthreads();
     double off_t = 0.0;
-    for (int w = 0; w < nt / 32; ++w) off_t += red[w];
+    for (int w = 0; w < kJacThreads / 32; ++w) off_t += red[w];
     __syncthreads();
     if ((tid & 31) == 0) red[tid >> 5] = all;
     __syncthreads();
     double all_t = 0.0;
-    for (int w = 0; w < nt / 32; ++w) all_t += red[w];
+    for (int w = 0; w < kJacThreads / 32; ++w) all_t += red[w];
     __syncthreads();
+    cluster_barrier();   // M is read to the end before the next sweep writes it
     if (off_t <= 1e-30 * all_t) break;
   }
+  for (int e = tid; e < nv * r; e += kJacThreads) V[(int64_t)v0 * r + e] = vrow[e];
+}
+
+__global__ void __launch_bounds__(256) ny_finish_kernel(int r, double* scratch, double* T, double* lam,
+                                                        const double* nu_in, const int32_t* status) {
+  __shared__ int perm[kMaxRank];
+  __shared__ double diag[kMaxRank];
+  const int s = blockIdx.x;
+  if (status[s] != KMV_OK) return;
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const int rr = r * r;
+  const double* W = scratch + (int64_t)s * 4 * rr;
+  double* G = scratch + (int64_t)s * 4 * rr + rr;
+  const double* M = G + rr;
+  const double* V = M + rr;
+  const double nu = nu_in[s];
+  for (int k = tid; k < r; k += nt) diag[k] = M[k * r + k];
+  __syncthreads();
   // eigenvalues in descending order
   if (tid == 0) {
     for (int k = 0; k < r; ++k) perm[k] = k;
     for (int a = 0; a < r; ++a) {
       int best = a;
       for (int k = a + 1; k < r; ++k)
-        if (M[perm[k] * r + perm[k]] > M[perm[best] * r + perm[best]]) best = k;
+        if (diag[perm[k]] > diag[perm[best]]) best = k;
       const int u = perm[a];
       perm[a] = perm[best];
       perm[best] = u;
@@ -319,7 +438,7 @@ __global__ void __launch_bounds__(256) ny_small_kernel(DevLayout L, int chains, 
   // T[:, j] = L^{-T} V[:, perm_j] / sqrt(s2_j) (back substitution per column)
   for (int j = tid; j < r; j += nt) {
     const int pj = perm[j];
-    const double s2 = M[pj * r + pj];
+    const double s2 = diag[pj];
     lam[(int64_t)s * r + j] = fmax(s2 - nu, 0.0);
     double* t = G + j;   // column j of G as scratch (X is no longer needed), stride r
     for (int i = r - 1; i >= 0; --i) {
@@ -329,10 +448,6 @@ __global__ void __launch_bounds__(256) ny_small_kernel(DevLayout L, int chains, 
     }
     const double inv = s2 > 0.0 ? 1.0 / sqrt(s2) : 0.0;
     for (int i = 0; i < r; ++i) T[(int64_t)s * rr + i * r + j] = t[i * r] * inv;
-  }
-  if (tid == 0) {
-    nu_out[s] = nu;
-    status[s] = KMV_OK;
   }
 }
 
@@ -374,12 +489,31 @@ __global__ void __launch_bounds__(kTile) ny_u_kernel(DevLayout L, int chains, in
 
 cudaError_t launch_nystrom_finish(const DevLayout& L, int n_items, int n_inst, int chains, int64_t n_total, int r,
                                   const float* Om, const float* Y, double* grams, double* scratch, double* T,
-                                  double* nu, float* U, double* lam, int32_t* status, cudaStream_t st) {
+                                  double* nu, float* U, double* lam, int32_t* status, int num_sms, cudaStream_t st) {
   const int n_sys = n_inst * chains;
   if (n_sys == 0) return cudaSuccess;
   const int nb = (r + kGB - 1) / kGB, nu_b = (r + kUB - 1) / kUB;
-  ny_gram_kernel<<<dim3(n_sys, nb * nb), 256, 0, st>>>(L, chains, n_total, r, nb, Om, Y, grams);
-  ny_small_kernel<<<n_sys, 256, 0, st>>>(L, chains, r, grams, scratch, T, lam, nu, status);
+  ny_gram_kernel<<<dim3(n_sys, nb * nb + nb * (nb + 1)), 256, 0, st>>>(L, chains, n_total, r, nb, Om, Y, grams);
+  ny_factor_kernel<<<n_sys, 256, 0, st>>>(L, chains, r, grams, scratch, T, lam, nu, status);
+  // CTAs per system: as many as leave one per SM over all systems, at most 8
+  int cl = 8;
+  while (cl > 1 && (int64_t)n_sys * cl > num_sms) cl /= 2;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)n_sys * cl);
+  cfg.blockDim = dim3(kJacThreads);
+  cfg.dynamicSmemBytes = sizeof(double) * (size_t)((r + cl - 1) / cl) * r;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = cl;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaError_t e = cudaFuncSetAttribute(ny_jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)(sizeof(double) * kMaxRank * kMaxRank));
+  if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, ny_jacobi_kernel, r, cl, scratch, (const int32_t*)status);
+  if (e != cudaSuccess) return e;
+  ny_finish_kernel<<<n_sys, 256, 0, st>>>(r, scratch, T, lam, nu, status);
   if (n_items > 0)
     ny_u_kernel<<<dim3(n_items, chains, nu_b), kTile, sizeof(double) * r * kUB, st>>>(L, chains, n_total, r, Om, Y,
                                                                                       T, nu, U);

@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(32 * kCoefShares) pcg_coef_kernel(DevLayout L,
                                                                     double* coef) {
   __shared__ double red[kCoefShares][32];
   chain_trigger();
-  const int s = blockIdx.y, lane = threadIdx.x & 31, y = threadIdx.x >> 5, k = blockIdx.x * 32 + lane;
+  const int s = blockIdx.x, lane = threadIdx.x & 31, y = threadIdx.x >> 5, k = blockIdx.y * 32 + lane;
   const int b = s / chains, c = s - b * chains;
   const int i0 = L.inst_item0[b], i1 = L.inst_item0[b + 1];
   chain_wait();
@@ -288,7 +288,7 @@ cudaError_t launch_pcg_precond(const DevLayout& L, int n_items, int n_inst, int 
   cudaError_t e = launch_chained(chained, pcg_proj_kernel<false>, grid, kTile, 0, st, L, chains, n_total, P.rank, P.U,
                                  nullptr, active, nullptr, const_cast<float*>(r), nullptr, nullptr, nullptr, proj);
   if (e == cudaSuccess)
-    e = launch_chained(chained, pcg_coef_kernel, dim3((P.rank + 31) / 32, n_inst * chains), 32 * kCoefShares, 0, st, L,
+    e = launch_chained(chained, pcg_coef_kernel, dim3(n_inst * chains, (P.rank + 31) / 32), 32 * kCoefShares, 0, st, L,
                        chains, P.rank, d, proj, active, coef);
   if (e == cudaSuccess)
     e = launch_chained(chained, pcg_apply_kernel, grid, kTile, 0, st, L, chains, n_total, P.rank, P.U, coef, r, z,
@@ -306,7 +306,7 @@ cudaError_t launch_pcg_iterate(const DevLayout& L, int n_items, int n_inst, int 
   cudaError_t e = launch_chained(chained, pcg_proj_kernel<true>, grid, kTile, 0, st, L, chains, n_total, P.rank, P.U,
                                  sys, active, x, r, p, q, partial, proj);
   if (e == cudaSuccess)
-    e = launch_chained(chained, pcg_coef_kernel, dim3((P.rank + 31) / 32, n_inst * chains), 32 * kCoefShares, 0, st, L,
+    e = launch_chained(chained, pcg_coef_kernel, dim3(n_inst * chains, (P.rank + 31) / 32), 32 * kCoefShares, 0, st, L,
                        chains, P.rank, d, proj, active, coef);
   if (e == cudaSuccess)
     e = launch_chained(chained, pcg_apply_kernel, grid, kTile, 0, st, L, chains, n_total, P.rank, P.U, coef, r, z,

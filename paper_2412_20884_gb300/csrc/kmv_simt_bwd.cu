@@ -72,6 +72,8 @@ constexpr int kGradThreads = 256;
 __global__ void __launch_bounds__(kGradThreads) grad_finalize_kernel(DevLayout L, SimtBwd f, int chains, int n_theta,
                                                                      const double* theta, const double* partial,
                                                                      double* grad) {
+  chain_trigger();
+  chain_wait();
   const int s = blockIdx.x;
   const int b = s / chains, c = s - b * chains;
   const double* th = theta + (int64_t)s * n_theta;
@@ -81,6 +83,9 @@ __global__ void __launch_bounds__(kGradThreads) grad_finalize_kernel(DevLayout L
   const int lane = threadIdx.x & 31;
   const int n = n_t * f.nz * units;
   for (int p = threadIdx.x >> 5; p < n_theta; p += kGradThreads / 32) {
+    // (the exp first: its thousand clocks run while the partials come in)
+    double scale = exp(p == n_theta - 1 ? th[n_theta - 1] : th[0]);
+    if (p != 0 && p != n_theta - 1) scale = scale / kHalfLog2e;
     double acc = 0.0;
     for (int e = lane; e < n; e += 32) {
       const int u = e % units, tz = e / units, z = tz % f.nz, t = tz / f.nz;
@@ -95,13 +100,7 @@ __global__ void __launch_bounds__(kGradThreads) grad_finalize_kernel(DevLayout L
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
     }
-    if (lane == 0) {
-      double scale;
-      if (p == 0) scale = exp(th[0]);
-      else if (p == n_theta - 1) scale = exp(th[n_theta - 1]);
-      else scale = exp(th[0]) / kHalfLog2e;
-      grad[(int64_t)s * n_theta + p] = scale * acc;
-    }
+    if (lane == 0) grad[(int64_t)s * n_theta + p] = scale * acc;
   }
 }
 
@@ -176,9 +175,10 @@ cudaError_t launch_backward_simt(const KmvArgs& a, const SimtBwd& f, int n_items
 }
 
 cudaError_t launch_grad_finalize(const DevLayout& L, const SimtBwd& f, int n_inst, int chains, int n_theta,
-                                 const double* theta, const double* partial, double* grad, cudaStream_t st) {
-  grad_finalize_kernel<<<n_inst * chains, kGradThreads, 0, st>>>(L, f, chains, n_theta, theta, partial, grad);
-  return cudaGetLastError();
+                                 const double* theta, const double* partial, double* grad, bool chained,
+                                 cudaStream_t st) {
+  return launch_chained(chained, grad_finalize_kernel, dim3(n_inst * chains), kGradThreads, 0, st, L, f, chains, n_theta,
+                        theta, partial, grad);
 }
 
 }  // namespace kmv

@@ -33,6 +33,8 @@ constexpr int kXSB = kJT + 4;   // row stride of the staged x (floats)
 template <int D, int MP, int R, bool ARD>
 __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
   constexpr int DG = ARD ? D : 1;
+  chain_trigger();
+  chain_wait();
   const int dd = a.d;   // <= D; the dimensions past it are zero and add nothing
   const int tile = blockIdx.x, c = blockIdx.y, u = blockIdx.z % f.units, z = blockIdx.z / f.units;
   const int item0 = f.tile_item ? f.tile_item[tile] : tile;
@@ -50,7 +52,7 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
   __shared__ __align__(16) float sg[kJT * MP];
   __shared__ float sc[D];
   __shared__ double as2[2];
-  __shared__ double red[kTile / 32];
+  __shared__ double red[kTile / 32 * (2 + DG)];
 
   const int tid = threadIdx.x;
   const double* th = a.theta + (int64_t)s * a.n_theta;
@@ -150,8 +152,9 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
       sg[e] = (in && want_gv) ? a.G[idx] * am : 0.f;
     }
     __syncthreads();
-    // two points j at a time (their chains interleave), all R rows
-#pragma unroll 1
+    // two points j at a time (their chains interleave), all R rows; one row per thread
+    // has eight in flight where registers allow
+#pragma unroll (R == 1 && D * MP <= 32 ? 4 : 1)
     for (int jj = 0; jj < kJT; jj += 2) {
       float r2[R][2], df2[R][2][DG];
 #pragma unroll
@@ -276,24 +279,23 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
   }
   // Per-CTA partials: [sum Q, sum Q d2 (k entries or 1), sum G.V]
   double* out = a.grad_partial + ((((int64_t)item0 * a.chains + c) * f.nz + z) * f.units + u) * a.n_theta;
-  auto put = [&](int p, double v) {
-    const double t = block_sum(v, red);
-    if (tid == 0) out[p] = t;
-  };
-  double v = 0.0;
+  constexpr int NE = 2 + DG;
+  double ev[NE];   // [q, g_0 .. , noise]
+  ev[0] = 0.0;
 #pragma unroll
-  for (int r = 0; r < R; ++r) v += (double)sq[r] + (double)cq[r];
-  put(0, v);
+  for (int r = 0; r < R; ++r) ev[0] += (double)sq[r] + (double)cq[r];
 #pragma unroll
   for (int k = 0; k < DG; ++k) {
-    if (k < (ARD ? dd : 1)) {
-      v = 0.0;
+    ev[1 + k] = 0.0;
 #pragma unroll
-      for (int r = 0; r < R; ++r) v += (double)sg2[r][k] + (double)cg2[r][k];
-      put(1 + k, v);
-    }
+    for (int r = 0; r < R; ++r) ev[1 + k] += (double)sg2[r][k] + (double)cg2[r][k];
   }
-  put(a.n_theta - 1, noise);
+  ev[NE - 1] = noise;
+  block_sum_many<NE>(ev, NE, red, [&](int e, double t) {
+    // the dimensions past d are not written
+    if (e == NE - 1) out[a.n_theta - 1] = t;
+    else if (e < a.n_theta - 1) out[e] = t;
+  });
 }
 
 // Rows per thread of the wide variant: R (2 D + 2 MP + D) registers and more.
@@ -302,13 +304,12 @@ constexpr int bwd_rows(int D, int MP) { return D <= 4 && MP <= 4 ? 4 : D + MP <=
 template <int D, int MP, bool ARD>
 cudaError_t bwd_launch_mp(const KmvArgs& a, const SimtBwd& f, dim3 grid, cudaStream_t st) {
   if (f.rows == 1) {
-    bwd_simt_kernel<D, MP, 1, ARD><<<grid, kTile, 0, st>>>(a, f);
-    return cudaGetLastError();
+    return launch_chained(a.chained, bwd_simt_kernel<D, MP, 1, ARD>, grid, kTile, 0, st, a, f);
   }
   constexpr int R = bwd_rows(D, MP);
-  if (f.rows != R) return cudaErrorInvalidValue;
-  if constexpr (R > 1) bwd_simt_kernel<D, MP, R, ARD><<<grid, kTile, 0, st>>>(a, f);
-  return cudaGetLastError();
+  if constexpr (R > 1)
+    if (f.rows == R) return launch_chained(a.chained, bwd_simt_kernel<D, MP, R, ARD>, grid, kTile, 0, st, a, f);
+  return cudaErrorInvalidValue;
 }
 
 // The kernel for the dimension class D (kmv_simt_bwd_*.cu hold the instances).

@@ -128,6 +128,7 @@ __device__ __forceinline__ void simt_put_dots(const KmvArgs& a, int b, int c, in
 template <int D, int MP, int R>
 __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
   chain_trigger();
+  if (a.chained == 2) chain_wait();
   const int dd = a.d;   // <= D; the dimensions past it are zero and add nothing
   const int tile = blockIdx.x, c = blockIdx.y;
   const int u = blockIdx.z % f.upc, jc = (blockIdx.z / f.upc) % f.js, z = f.z0 + blockIdx.z / f.max_units;

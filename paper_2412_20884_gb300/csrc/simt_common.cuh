@@ -63,6 +63,70 @@ __device__ __forceinline__ void pair_warp_sum(float& s, float& e) {
   }
 }
 
+// block_sum of N values at once, each in block_sum's order: the shuffles of the values
+// interleave, where N calls would wait for N chains of dependent FP64 adds (some 900
+// clocks each).  red: blockDim / 32 rows of N; out(v, sum) is called by thread v < n.
+template <int N, class Out>
+__device__ __forceinline__ void block_sum_many(double (&v)[N], int n, double* red, Out&& out) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  __syncthreads();
+  if (l == 0) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) red[w * N + k] = v[k];
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    double t = 0.0;
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[i * N + k];
+    out(k, t);
+  }
+}
+
+// Sums NC (16 or 32) pairs per lane over the warp: the lanes halve the vector between
+// them step by step; lane l returns with column l % NC in (s[0], e[0]).
+template <int NC>
+__device__ __forceinline__ void pair_reduce_scatter(float (&s)[NC], float (&e)[NC]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int h = NC / 2; h >= 1; h /= 2) {
+    const bool up = lane & h;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const float so = __shfl_xor_sync(0xffffffffu, up ? s[i] : s[i + h], h);
+      const float eo = __shfl_xor_sync(0xffffffffu, up ? e[i] : e[i + h], h);
+      float sk = up ? s[i + h] : s[i], ek = up ? e[i + h] : e[i];
+      two_sum_add(sk, ek, so);
+      s[i] = sk;
+      e[i] = __fadd_rn(ek, eo);
+    }
+  }
+  if (NC == 16) {
+    const float so = __shfl_xor_sync(0xffffffffu, s[0], 16), eo = __shfl_xor_sync(0xffffffffu, e[0], 16);
+    two_sum_add(s[0], e[0], so);
+    e[0] = __fadd_rn(e[0], eo);
+  }
+}
+// Block sums of NC pairs per thread (kTile threads): out(col, sum) by thread col < n.
+// red: kTile / 32 rows of NC.
+template <int NC, class Out>
+__device__ __forceinline__ void pair_block_sums(float (&s)[NC], float (&e)[NC], int n, double* red, Out&& out) {
+  pair_reduce_scatter<NC>(s, e);
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  __syncthreads();
+  if (l < NC) red[w * NC + l] = (double)s[0] + (double)e[0];
+  __syncthreads();
+  if ((int)threadIdx.x < n) {
+    double t = 0.0;
+#pragma unroll
+    for (int i = 0; i < kTile / 32; ++i) t += red[i * NC + threadIdx.x];
+    out((int)threadIdx.x, t);
+  }
+}
+
 inline int pow2ceil(int v) {
   int p = 1;
   while (p < v) p <<= 1;
