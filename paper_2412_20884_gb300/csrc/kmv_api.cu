@@ -1104,6 +1104,7 @@ kmv_status run_mscg(kmv_handle h, const kmv_points* pts, const double* theta, co
       KMV_TRY(poll.step(h, B.n_active, st));
       if (poll.done) break;
     }
+    a.reuse_prep = it > 0;   // theta is fixed within the solve
     KMV_TRY(run_forward(h, a, prec, st));
     if (fused) {
       KMV_CUDA(h, launch_mscg_update_xr_beta(h->dev, L.n_items, L.chains, L.n_total, m, B.sys, B.sh, B.sys_active,

@@ -36,7 +36,7 @@ int dim_class(int d) {
 }
 
 // dL/dV = alpha amp sum_units part + sigma^2 G, 128 rows and kGvCols columns at a time.
-constexpr int kGvCols = 4;
+constexpr int kGvCols = 2;
 __global__ void __launch_bounds__(kTile) bwd_simt_combine_kernel(KmvArgs a, SimtBwd f) {
   __shared__ double as2[2];
   const int item = blockIdx.x, c = blockIdx.y;
@@ -66,48 +66,48 @@ __global__ void __launch_bounds__(kTile) bwd_simt_combine_kernel(KmvArgs a, Simt
 }
 
 // grad[s, p] = scale_p * sum over the instance's tiles, column chunks and units of
-// partial[..., p]: a warp per entry, lanes striding over the tiles, then a fixed
-// shuffle tree (one thread's serial chain over 157 items measured 75 us).
-constexpr int kGradThreads = 256;
+// partial[..., p]: a CTA per (system, entry), threads striding over the partials, then
+// the fixed order of block_sum; a few partials in their own order, whatever the batch
+// around the system (one thread's serial chain over 157 items measured 75 us).
+constexpr int kGradThreads = 128;
 __global__ void __launch_bounds__(kGradThreads) grad_finalize_kernel(DevLayout L, SimtBwd f, int chains, int n_theta,
                                                                      const double* theta, const double* partial,
                                                                      double* grad) {
+  __shared__ double red[kGradThreads / 32];
   chain_trigger();
   chain_wait();
-  const int s = blockIdx.x;
+  const int s = blockIdx.x / n_theta, p = blockIdx.x - s * n_theta;
   const int b = s / chains, c = s - b * chains;
   const double* th = theta + (int64_t)s * n_theta;
   const int64_t nb = L.offsets[b + 1] - L.offsets[b], len = (int64_t)f.folds * kFoldTiles * kTile;
   const int units = (int)((nb + len - 1) / len);
   const int i0 = L.inst_item0[b], n_t = (L.inst_item0[b + 1] - i0 + f.rows - 1) / f.rows;
-  const int lane = threadIdx.x & 31;
-  const int n = n_t * f.nz * units;
-  for (int p = threadIdx.x >> 5; p < n_theta; p += kGradThreads / 32) {
-    // (the exp first: its thousand clocks run while the partials come in)
-    double scale = exp(p == n_theta - 1 ? th[n_theta - 1] : th[0]);
-    if (p != 0 && p != n_theta - 1) scale = scale / kHalfLog2e;
-    double acc = 0.0;
-    for (int e = lane; e < n; e += 32) {
-      const int u = e % units, tz = e / units, z = tz % f.nz, t = tz / f.nz;
-      acc += partial[((((int64_t)(i0 + t * f.rows) * chains + c) * f.nz + z) * f.units + u) * n_theta + p];
+  const int n = n_t * f.nz * units, per_tile = f.nz * units;
+  auto at = [&](int e) {
+    const int t = e / per_tile, zu = e - t * per_tile, z = zu / units, u = zu - z * units;
+    return partial[((((int64_t)(i0 + t * f.rows) * chains + c) * f.nz + z) * f.units + u) * n_theta + p];
+  };
+  double acc = 0.0;
+  if (n <= 32) {
+    if (threadIdx.x < 32) {
+      const double v = (int)threadIdx.x < n ? at(threadIdx.x) : 0.0;
+      for (int e = 0; e < n; ++e) acc += __shfl_sync(0xffffffffu, v, e);
     }
-    if (n <= 32) {
-      // few partials: in their order, whatever the batch around the system
-      double sum = 0.0;
-      for (int e = 0; e < n; ++e) sum += __shfl_sync(0xffffffffu, acc, e);
-      acc = sum;
-    } else {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    }
-    if (lane == 0) grad[(int64_t)s * n_theta + p] = scale * acc;
+  } else {
+#pragma unroll 4
+    for (int e = threadIdx.x; e < n; e += kGradThreads) acc += at(e);
+    acc = block_sum(acc, red);
   }
+  if (threadIdx.x != 0) return;
+  double scale = exp(p == n_theta - 1 ? th[n_theta - 1] : th[0]);
+  if (p != 0 && p != n_theta - 1) scale = scale / kHalfLog2e;
+  grad[(int64_t)s * n_theta + p] = scale * acc;
 }
 
 }  // namespace
 
 // Rows per thread and the number of J units: the wide variant once its finest split
-// (units of one fold) gives every SM two CTAs; then about 12 CTAs per SM, and with
+// (units of one fold) gives every SM two CTAs; then about 8 CTAs per SM, and with
 // dL/dV at most 512 MB of partial sums.
 SimtBwd simt_bwd_plan(const SimtTiles& T, int n_items, int chains, int64_t n_total, int64_t max_rows, int d, int m,
                       bool want_gv, int num_sms) {
@@ -121,7 +121,7 @@ SimtBwd simt_bwd_plan(const SimtTiles& T, int n_items, int chains, int64_t n_tot
     f.n_tiles = R == 4 ? T.n4 : T.n2;
   }
   const int64_t ctas = (int64_t)f.n_tiles * chains * f.nz;
-  int64_t units = std::min<int64_t>(fpc, std::max<int64_t>(1, (12 * (int64_t)num_sms + ctas - 1) / std::max<int64_t>(1, ctas)));
+  int64_t units = std::min<int64_t>(fpc, std::max<int64_t>(1, (8 * (int64_t)num_sms + ctas - 1) / std::max<int64_t>(1, ctas)));
   units = std::min<int64_t>(units, std::max(1, 65535 / f.nz));
   const int64_t bytes = want_gv ? (int64_t)sizeof(float2) * chains * m * std::max<int64_t>(1, n_total) : 0;
   while (units > 1 && bytes * units > (int64_t(512) << 20)) --units;
@@ -177,7 +177,7 @@ cudaError_t launch_backward_simt(const KmvArgs& a, const SimtBwd& f, int n_items
 cudaError_t launch_grad_finalize(const DevLayout& L, const SimtBwd& f, int n_inst, int chains, int n_theta,
                                  const double* theta, const double* partial, double* grad, bool chained,
                                  cudaStream_t st) {
-  return launch_chained(chained, grad_finalize_kernel, dim3(n_inst * chains), kGradThreads, 0, st, L, f, chains, n_theta,
+  return launch_chained(chained, grad_finalize_kernel, dim3((unsigned)n_inst * chains * n_theta), kGradThreads, 0, st, L, f, chains, n_theta,
                         theta, partial, grad);
 }
 

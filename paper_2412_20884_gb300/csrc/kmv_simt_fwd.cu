@@ -20,7 +20,7 @@ extern template cudaError_t fwd_launch_d<32>(const KmvArgs&, const SimtFwd&, dim
 extern template cudaError_t fwd_launch_d<64>(const KmvArgs&, const SimtFwd&, dim3, cudaStream_t);
 
 // Adds the units' sums and writes Y, 128 rows and kCombineCols columns at a time.
-constexpr int kCombineCols = 4;
+constexpr int kCombineCols = 2;
 __global__ void __launch_bounds__(kTile) fwd_simt_combine_kernel(KmvArgs a, SimtFwd f) {
   __shared__ double as2[2];
   const int item = blockIdx.x, c = blockIdx.y;
@@ -105,9 +105,9 @@ SimtFwd simt_fwd_plan(const SimtTiles& T, int n_inst, int n_items, int chains, i
   f.tile_item = !big ? nullptr : R == 4 ? T.item4 : T.item2;
   f.n_tiles = !big ? n_items : R == 4 ? T.n4 : T.n2;
   const int64_t ctas = (int64_t)f.n_tiles * chains * f.nz * f.js;
-  // about 12 CTAs per SM (three or four resident, so that the last wave is short),
-  // with at most 512 MB of partial sums
-  int64_t upc = std::min<int64_t>(fpc, std::max<int64_t>(1, (12 * (int64_t)num_sms + ctas - 1) / std::max<int64_t>(1, ctas)));
+  // about 8 CTAs per SM (two to four resident, so that the last wave is short), with at
+  // most 512 MB of partial sums
+  int64_t upc = std::min<int64_t>(fpc, std::max<int64_t>(1, (8 * (int64_t)num_sms + ctas - 1) / std::max<int64_t>(1, ctas)));
   const int64_t bytes = (int64_t)sizeof(float2) * f.js * chains * m * std::max<int64_t>(1, n_total);
   while (upc > 1 && bytes * upc > (int64_t(512) << 20)) --upc;
   f.folds = (int)((fpc + upc - 1) / upc);

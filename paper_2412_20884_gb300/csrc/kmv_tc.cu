@@ -99,8 +99,11 @@ struct TcFwdArgs {
   int* err;
 };
 
-// RM > 0: the FP64 fold accumulators of up to RM columns live in registers;
-// RM == 0: they live in the per-item partial (global read-modify-write).
+// RM > 0: the fold sums of up to RM columns (FP32 pairs) live in registers; RM == 0:
+// they live as pairs in the place of the per-item FP64 partials (global
+// read-modify-write by the row's own thread), converted after the item's last fold.
+// As FP64 sums they cost 64 conversions and adds per row and fold at m = 64, on a pipe
+// of 2 lanes per clock: 14% of the kernel.
 template <int RM, int POLY>
 __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
   using namespace ptx;
@@ -337,9 +340,16 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
           uint32_t a0[32], a1[32], b0[32], b1[32], pk[32];
           tmem_ld32(tl + s_col, a0);
           tmem_ld32(tl + s_col + 32, a1);
-          tmem_ld_wait_regs(a0, a1);
+          if (RM > 0) tmem_ld_wait_regs(a0, a1);
           tmem_ld32(tl + s_col + 64, b0);
           tmem_ld32(tl + s_col + 96, b1);
+          if (RM == 0) {
+            // many columns or dimensions: the next S takes the tensor core long enough
+            // to be worth starting before the exps
+            tmem_ld_wait_regs(a0, a1, b0, b1);
+            tc_fence_before();
+            mbar_arrive(&s_free[g]);
+          }
 #pragma unroll
           for (int q = 0; q < 16; ++q)
             pk[q] = pack_f16x2(exp2_mix<POLY, 3>(__uint_as_float(a0[2 * q]), 2 * q),
@@ -348,10 +358,12 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
           for (int q = 0; q < 16; ++q)
             pk[16 + q] = pack_f16x2(exp2_mix<POLY, 3>(__uint_as_float(a1[2 * q]), 2 * q),
                                exp2_mix<POLY, 3>(__uint_as_float(a1[2 * q + 1]), 2 * q + 1));
-          tmem_ld_wait_regs(b0, b1);
-          // S(k) is fully in registers: the tensor core may overwrite it
-          tc_fence_before();
-          mbar_arrive(&s_free[g]);
+          if (RM > 0) {
+            tmem_ld_wait_regs(b0, b1);
+            // S(k) is fully in registers: the tensor core may overwrite it
+            tc_fence_before();
+            mbar_arrive(&s_free[g]);
+          }
           if (k > 0) {
             // P(k-1) must have been consumed before P(k) overwrites it
             ok = mbar_wait(&p_free[g], pf_ph, abort, a.err, 10);
@@ -403,9 +415,13 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
               for (int q = 0; q < 16; ++q) {
                 const int col = c0 + q;
                 if (col < a.mz) {
-                  const double v = (double)__uint_as_float(o[q]);
-                  double& pv = a.part[part_idx(t, a.mz, col, rowp)];
-                  pv = first ? v : pv + v;
+                  float2* pv = reinterpret_cast<float2*>(&a.part[part_idx(t, a.mz, col, rowp)]);
+                  float2 v = first ? make_float2(0.f, 0.f) : *pv;
+                  two_sum_add(v.x, v.y, __uint_as_float(o[q]));
+                  if (j == item.w - 1)
+                    a.part[part_idx(t, a.mz, col, rowp)] = (double)v.x + (double)v.y;
+                  else
+                    *pv = v;
                 }
               }
             }
@@ -441,6 +457,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
 template <int MZ, int POLY>
 __global__ void __launch_bounds__(kFmaThreads, 1) tc_fwd_fma_kernel(TcFwdArgs a) {
   using namespace ptx;
+  chain_trigger();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
   const uint32_t A_TILE = a.KX * 256u, V_TILE = MZ * 512u;
@@ -489,6 +506,7 @@ __global__ void __launch_bounds__(kFmaThreads, 1) tc_fwd_fma_kernel(TcFwdArgs a)
   __syncthreads();
   tc_fence_after();
   const uint32_t tbase = *tslot;
+  chain_wait();   // the tensor memory and barriers are set up; VF and the masks come from the kernels before
 
   if (warp == kFmaLoadWarp) {
     const bool leader = elect_one();
@@ -605,64 +623,80 @@ __global__ void __launch_bounds__(kFmaThreads, 1) tc_fwd_fma_kernel(TcFwdArgs a)
         acc64[q] = 0.0;
         acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.f;
       }
-      for (int j = 0; j < item.w; ++j, ++k) {
-        const int buf = (int)(k & 1);
-        const uint32_t s_col = 256 * buf + g * 128 + 64 * hf;
-        bool ok = mbar_wait(&s_full[2 * g + buf], (sph >> buf) & 1u, abort, a.err, 16);
-        // the VF tile of this stage is visible once its copy has completed
-        ok = ok && mbar_wait(&full[stage], fph, abort, a.err, 17);
-        if (!__all_sync(0xffffffffu, ok)) goto fma_exp_out;
-        sph ^= 1u << buf;
-        tc_fence_after();
-        // this half's 64 columns of v: float4 16 hf .. 16 hf + 15 of each column's 32
-        const float4* vs = reinterpret_cast<const float4*>(sV + stage * V_TILE) + 16 * hf;
-        {
-          // 32 columns at a time (registers are 96 a thread at 608 threads; the
-          // other warps of the scheduler cover the second load)
-          uint32_t a0[32];
-          tmem_ld32(tl + s_col, a0);
-          tmem_ld_wait_regs(a0);
+      // The half's 64 columns in four chunks of 16, each chunk's TMEM load in flight
+      // while the one before it is worked on, the next tile's first chunk included if
+      // that tile's S is there by then (it usually is: the issuers run a tile ahead).
+      // Two 32-column chunks in flight would spill at the 96 registers of 608 threads.
+      uint32_t a0[16], a1[16];
+      auto fma16 = [&](const uint32_t (&a)[16], const float4* vs, int u0) {
 #pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const float p0 = exp2_mix<POLY, 5>(__uint_as_float(a0[4 * u]), 4 * u);
-            const float p1 = exp2_mix<POLY, 5>(__uint_as_float(a0[4 * u + 1]), 4 * u + 1);
-            const float p2 = exp2_mix<POLY, 5>(__uint_as_float(a0[4 * u + 2]), 4 * u + 2);
-            const float p3 = exp2_mix<POLY, 5>(__uint_as_float(a0[4 * u + 3]), 4 * u + 3);
+        for (int u = 0; u < 4; ++u) {
+          const float p0 = exp2_mix<POLY, 5>(__uint_as_float(a[4 * u]), 4 * u);
+          const float p1 = exp2_mix<POLY, 5>(__uint_as_float(a[4 * u + 1]), 4 * u + 1);
+          const float p2 = exp2_mix<POLY, 5>(__uint_as_float(a[4 * u + 2]), 4 * u + 2);
+          const float p3 = exp2_mix<POLY, 5>(__uint_as_float(a[4 * u + 3]), 4 * u + 3);
 #pragma unroll
-            for (int q = 0; q < MZ; ++q) {
-              const float4 v = vs[q * 32 + u];
-              acc[q][0] = fmaf(p0, v.x, acc[q][0]);
-              acc[q][1] = fmaf(p1, v.y, acc[q][1]);
-              acc[q][2] = fmaf(p2, v.z, acc[q][2]);
-              acc[q][3] = fmaf(p3, v.w, acc[q][3]);
-            }
-          }
-          uint32_t a1[32];
-          tmem_ld32(tl + s_col + 32, a1);
-          tmem_ld_wait_regs(a1);
-          // this half of S(k) is in registers: once both halves are, the tensor core may overwrite it
-          tc_fence_before();
-          mbar_arrive(&s_free[2 * g + buf]);
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const float p0 = exp2_mix<POLY, 5>(__uint_as_float(a1[4 * u]), 4 * u);
-            const float p1 = exp2_mix<POLY, 5>(__uint_as_float(a1[4 * u + 1]), 4 * u + 1);
-            const float p2 = exp2_mix<POLY, 5>(__uint_as_float(a1[4 * u + 2]), 4 * u + 2);
-            const float p3 = exp2_mix<POLY, 5>(__uint_as_float(a1[4 * u + 3]), 4 * u + 3);
-#pragma unroll
-            for (int q = 0; q < MZ; ++q) {
-              const float4 v = vs[q * 32 + 8 + u];
-              acc[q][0] = fmaf(p0, v.x, acc[q][0]);
-              acc[q][1] = fmaf(p1, v.y, acc[q][1]);
-              acc[q][2] = fmaf(p2, v.z, acc[q][2]);
-              acc[q][3] = fmaf(p3, v.w, acc[q][3]);
-            }
+          for (int q = 0; q < MZ; ++q) {
+            const float4 v = vs[q * 32 + u0 + u];
+            acc[q][0] = fmaf(p0, v.x, acc[q][0]);
+            acc[q][1] = fmaf(p1, v.y, acc[q][1]);
+            acc[q][2] = fmaf(p2, v.z, acc[q][2]);
+            acc[q][3] = fmaf(p3, v.w, acc[q][3]);
           }
         }
+      };
+      bool loaded = false;   // this tile's first chunk is already on its way
+      for (int j0 = 0; j0 < item.w; j0 += kFold) {
+        const int j1 = min(item.w, j0 + kFold);
+#pragma unroll 1
+        for (int j = j0; j < j1; ++j, ++k) {
+        const int buf = (int)(k & 1);
+        const uint32_t s_col = 256 * buf + g * 128 + 64 * hf;
+        if (!loaded) {
+          const bool ok = mbar_wait(&s_full[2 * g + buf], (sph >> buf) & 1u, abort, a.err, 16);
+          if (!__all_sync(0xffffffffu, ok)) goto fma_exp_out;
+          sph ^= 1u << buf;
+          tc_fence_after();
+          tmem_ld16(tl + s_col, a0);
+        }
+        {
+          // the VF tile of this stage is visible once its copy has completed
+          const bool ok = mbar_wait(&full[stage], fph, abort, a.err, 17);
+          if (!__all_sync(0xffffffffu, ok)) goto fma_exp_out;
+        }
+        // this half's 64 columns of v: float4 16 hf .. 16 hf + 15 of each column's 32
+        const float4* vs = reinterpret_cast<const float4*>(sV + stage * V_TILE) + 16 * hf;
+        tmem_ld_wait_regs(a0);
+        tmem_ld16(tl + s_col + 16, a1);
+        fma16(a0, vs, 0);
+        tmem_ld_wait_regs(a1);
+        tmem_ld16(tl + s_col + 32, a0);
+        fma16(a1, vs, 4);
+        tmem_ld_wait_regs(a0);
+        tmem_ld16(tl + s_col + 48, a1);
+        fma16(a0, vs, 8);
+        tmem_ld_wait_regs(a1);
+        // this half of S(k) is in registers: once both halves are, the tensor core may overwrite it
+        tc_fence_before();
+        mbar_arrive(&s_free[2 * g + buf]);
+        loaded = false;
+        if (j + 1 < item.w) {
+          const int nb = buf ^ 1;
+          if (__all_sync(0xffffffffu, mbar_try_wait(smem_u32(&s_full[2 * g + nb]), (sph >> nb) & 1u))) {
+            loaded = true;
+            sph ^= 1u << nb;
+            tc_fence_after();
+            tmem_ld16(tl + 256 * nb + g * 128 + 64 * hf, a0);
+          }
+        }
+        fma16(a1, vs, 12);
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[stage]);
         if (++stage == (uint32_t)S) { stage = 0; fph ^= 1; }
-        if ((j % kFold) == kFold - 1) {
+        }
+        // (after the chunk of kFold tiles, not inside its loop: there the compiler
+        // predicated the FP64 conversions and adds, and every tile issued them)
+        if (j1 - j0 == kFold) {
 #pragma unroll
           for (int q = 0; q < MZ; ++q) {
             acc64[q] += (double)((acc[q][0] + acc[q][1]) + (acc[q][2] + acc[q][3]));
@@ -711,12 +745,14 @@ __global__ void tc_prep_vf_kernel(DevLayout L, TcTables T, int chains, int64_t n
                                   int mz, int T_total, const int32_t* sys_active, const float* amp, float* VF,
                                   const CgSys* cg_sys, const PcgSys* pcg_sys, const MscgSys* ms_sys, const MscgShift* ms_sh, int ms_m,
                                   float* ms_ps, const float* cg_r, float* cg_p) {
+  chain_trigger();
   const int t = blockIdx.x, c = blockIdx.y, r = threadIdx.x;
   const int b = T.tile_inst[t];
   const int s = b * chains + c;
-  if (sys_active && !sys_active[s]) return;
   const int64_t nb = L.offsets[b + 1] - L.offsets[b];
   const int64_t rl = (int64_t)(t - T.inst_tile0[b]) * 128 + r;
+  chain_wait();
+  if (sys_active && !sys_active[s]) return;
   const bool valid = rl < nb;
   const int64_t i = L.offsets[b] + rl;
   float* dst = VF + ((size_t)c * T_total + t) * (size_t)mz * 128;
@@ -944,17 +980,16 @@ __global__ void tc_fwd_epilogue_kernel(DevLayout L, TcTables T, KmvArgs a, int c
   __shared__ double red[kTile / 32];
   __shared__ double s_alpha, s_s2;
   __shared__ int s_last;
+  chain_trigger();
   const int item = blockIdx.x, c = blockIdx.y;
   const int b = L.item_inst[item];
   const int s = b * a.chains + c;
-  if (a.sys_active && !a.sys_active[s]) return;
-  if (threadIdx.x == 0) {
-    // alpha and sigma^2 of the system (FP64 exp once per block)
+  if (threadIdx.x < 2) {
+    // alpha and sigma^2 of the system (one FP64 exp per block)
     const double* th = a.theta + (int64_t)s * a.n_theta;
-    s_alpha = exp(th[0]);
-    s_s2 = exp(th[a.n_theta - 1]);
+    const double e = exp(th[threadIdx.x ? a.n_theta - 1 : 0]);
+    (threadIdx.x ? s_s2 : s_alpha) = e;
   }
-  __syncthreads();
   const int64_t i = L.item_row0[item] + threadIdx.x;
   const bool valid = i < L.offsets[b + 1];
   const int tile_in_inst = (int)((L.item_row0[item] - L.offsets[b]) / 128);
@@ -962,7 +997,10 @@ __global__ void tc_fwd_epilogue_kernel(DevLayout L, TcTables T, KmvArgs a, int c
   const int nk = T.inst_nk[b];
   const int64_t it0 = T.sys_item0[s] + (int64_t)p * nk;
   const int rowp = half * 128 + threadIdx.x;
+  __syncthreads();
   const double alpha = s_alpha, s2 = s_s2;
+  chain_wait();
+  if (a.sys_active && !a.sys_active[s]) return;
   const bool bad = *err != 0;
   double dot = 0.0;
   if (valid) {
@@ -1210,8 +1248,8 @@ void tc_launch_prep_x(kmv_handle h, TcState* S, const KmvArgs& a, int KX, int ns
 
 void tc_launch_epilogue(kmv_handle h, TcState* S, const KmvArgs& a, int c0, int mz, const double* part,
                         const uint32_t* colmax, const int* err, cudaStream_t st) {
-  tc_fwd_epilogue_kernel<<<dim3(h->layout.n_items, h->layout.chains), kTile, 0, st>>>(h->dev, S->dev, a, c0, mz,
-                                                                                      part, colmax, err);
+  launch_chained(a.chained, tc_fwd_epilogue_kernel, dim3(h->layout.n_items, h->layout.chains), kTile, 0, st, h->dev,
+                 S->dev, a, c0, mz, part, colmax, err);
 }
 
 using FwdKernel = void (*)(TcFwdArgs);
@@ -1291,12 +1329,13 @@ kmv_status tc_forward(kmv_handle h, const KmvArgs& a, cudaStream_t st) {
     if (fwd_kernels_set_smem() != cudaSuccess) return tc_fail(h, KMV_ECUDA, "cudaFuncSetAttribute failed");
     S->attr_set = true;
   }
-  if (cudaMemsetAsync(err, 0, sizeof(int), st) != cudaSuccess) return tc_fail(h, KMV_ECUDA, "memset failed");
   // the operand tiles depend on theta and x only: a solve's later products
-  // reuse those of its first one
+  // reuse those of its first one (and keep its error word: a product that gave up
+  // ends the solve)
   const bool reuse = a.reuse_prep && S->prep_valid && S->prep_theta == a.theta && S->prep_x == a.x &&
                      S->prep_nsplit == nsplit && S->prep_d == a.d;
   if (!reuse) {
+    if (cudaMemsetAsync(err, 0, sizeof(int), st) != cudaSuccess) return tc_fail(h, KMV_ECUDA, "memset failed");
     tc_launch_center(h, a, ckeys, st);
     tc_launch_prep_x(h, S, a, KX, nsplit, ckeys, XA, XB, nullptr, st);
     S->prep_valid = true;
@@ -1315,10 +1354,9 @@ kmv_status tc_forward(kmv_handle h, const KmvArgs& a, cudaStream_t st) {
     const int stages =
         (int)std::max<size_t>(2, std::min<size_t>(max_stages, (kMaxSmem - fixed - tail) / (A_TILE + V_TILE + 16)));
     const size_t smem = std::max(kMinSmem, fixed + stages * (A_TILE + V_TILE + 16) + tail);
-    tc_prep_vf_kernel<<<dim3(S->T_total, L.chains), 128, 0, st>>>(
-        h->dev, S->dev, L.chains, L.n_total, a.V, a.m, mz, S->T_total, a.sys_active, a.amp,
-        reinterpret_cast<float*>(VT), a.cg_sys, a.pcg_sys, a.ms_sys, a.ms_sh, a.ms_m, a.ms_ps, a.cg_r,
-        const_cast<float*>(a.V));
+    launch_chained(a.chained, tc_prep_vf_kernel, dim3(S->T_total, L.chains), 128, 0, st, h->dev, S->dev, L.chains,
+                   L.n_total, a.V, a.m, mz, S->T_total, a.sys_active, a.amp, reinterpret_cast<float*>(VT), a.cg_sys,
+                   a.pcg_sys, a.ms_sys, a.ms_sh, a.ms_m, a.ms_ps, a.cg_r, const_cast<float*>(a.V));
     TcFwdArgs fa;
     fa.items = S->d_items;
     fa.n_items = S->n_items;
@@ -1337,7 +1375,7 @@ kmv_status tc_forward(kmv_handle h, const KmvArgs& a, cudaStream_t st) {
     const int grid = std::min(S->n_items, S->num_sms);
     {
       ProfScope prof(h, KMV_KERNEL_FORWARD, st);
-      fwd_kernel(true, mz, tl.exp_split)<<<grid, kFmaThreads, smem, st>>>(fa);
+      launch_chained(a.chained, fwd_kernel(true, mz, tl.exp_split), dim3(grid), kFmaThreads, smem, st, fa);
     }
     // no column maxima: the epilogue's column scale is 1
     tc_launch_epilogue(h, S, a, 0, mz, part, nullptr, err, st);

@@ -7,17 +7,18 @@
 // tiles (J >= I) is evaluated, off-diagonal tiles weighted twice.
 //
 // A work item is one I tile of one system against a range of J tiles; each J
-// tile is split into two 64-column halves, half b for warpgroup b.  The two
-// warpgroups run as independent pipelines, each with its own MMA issuer warp,
-// TMEM buffers and accumulator, sharing only the operand stages.  For its half
-// of a J tile, issuer b writes into TMEM
+// tile is split into two 64-column halves, half b for warpgroup b.  Issuer warp 0
+// writes into TMEM, per J tile (its 128 columns in one MMA per K step: with the A
+// operand in shared memory an MMA of 64 columns takes 48 clocks, one of 128 takes 64,
+// and an issuing warp manages one per 50 to 120 clocks)
 //   S = XA_I XB_J^T           the base-2 exponent from F16 hi/lo operands of the
 //                             centred points (|dS| ~ 2^-24 |xh|^2); XA from TMEM
 //   W = GI_I VJ_J^T           = G_i . V_j + V_i . G_j with GI rows
 //                             [gh gh gl vh vh vl] (shared memory, once per item)
 //                             and VJ rows [vh vl vh gh gl gh] (F16 hi/lo, G and V
 //                             each scaled by a power of two)
-// warpgroup b forms Q = W 2^S in FP32 (halved on the diagonal tile, and zero for
+// Both warpgroups read their half of S and W into registers at once, so that the next
+// tile's products run during this tile's exps.  Warpgroup b forms Q = W 2^S in FP32 (halved on the diagonal tile, and zero for
 // i = j, whose (xt_i - xt_i)^2 is 0), splits it exactly into Q = Qh + Ql with Qh
 // holding 11 significant bits (Veltkamp's splitting), stores both as F16, and
 // issuer b accumulates, per row i,
@@ -122,9 +123,9 @@ __device__ __forceinline__ void split_q(float q, float& hi, float& lo) {
   lo = __fsub_rn(q, hi);
 }
 
-// Warps: 0-7 the two warpgroups, 8 the issuer of warpgroup 0 (and TMEM owner),
-// 9 the producer, 10 the issuer of warpgroup 1.  TMEM (512 columns):
-//   S_b [128 b, +64), W_b [128 b + 64, +64), Qh_b [256 + 64 b, +32), Ql_b [+32, +32),
+// Warps: 0-7 the two warpgroups, 8 the issuer of S and W (and TMEM owner), 9 the
+// producer, 10 the issuer of the feature sums.  TMEM (512 columns):
+//   S [0, 128), W [128, 256), Qh_b [256 + 64 b, +32), Ql_b [+32, +32),
 //   XA [384, 384 + KX/2) unless XS, ACC_b [512 - 2 NACC + b NACC, +NACC).
 // Shared memory: the item's GI tile, the item's XA tile when XS (large d), and
 // the stages [XB | VJ | BG] of the J tiles.
@@ -169,15 +170,15 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
   uint64_t* empty = full + S;        // both issuers done with the stage (2 commits)
   uint64_t* a_ready = empty + S;     // XA of the item stored in TMEM (128 arrivals of warpgroup 0)
   uint64_t* seg = a_ready + 1;       // both warpgroups finished the previous item (256)
-  uint64_t* sw_full = seg + 1;       // [b] S_b, W_b written
-  uint64_t* s_free = sw_full + 2;    // [b] S_b, W_b loaded into registers
-  uint64_t* q_ready = s_free + 2;    // [b] Q_b written
+  uint64_t* sw_full = seg + 1;       // S, W of the tile written
+  uint64_t* s_free = sw_full + 1;    // S, W loaded into registers (256: both warpgroups)
+  uint64_t* q_ready = s_free + 1;    // [b] Q_b written
   uint64_t* q_free = q_ready + 2;    // [b] the feature sums of Q_b done
-  uint64_t* done = q_free + 2;       // [issuer b]
+  uint64_t* done = q_free + 2;       // [issuer]
   uint64_t* xa_full = done + 2;      // XS: XA tile landed
-  uint64_t* xa_empty = xa_full + 1;  // XS: both issuers done with it (2 commits)
+  uint64_t* xa_empty = xa_full + 1;  // XS: the S products are done with it
   uint64_t* gi_full = xa_empty + 1;  // GI tile landed
-  uint64_t* gi_empty = gi_full + 1;  // both issuers done with it (2 commits)
+  uint64_t* gi_empty = gi_full + 1;  // the W products are done with it
   uint32_t* tslot = reinterpret_cast<uint32_t*>(gi_empty + 1);
   volatile int* abort = reinterpret_cast<volatile int*>(tslot + 1);
 
@@ -189,17 +190,17 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
     }
     mbar_init(a_ready, 128);
     mbar_init(seg, 256);
+    mbar_init(sw_full, 1);
+    mbar_init(s_free, 256);
     for (int b = 0; b < 2; ++b) {
-      mbar_init(&sw_full[b], 1);
-      mbar_init(&s_free[b], 128);
       mbar_init(&q_ready[b], 128);
       mbar_init(&q_free[b], 1);
       mbar_init(&done[b], 1);
     }
     mbar_init(xa_full, 1);
-    mbar_init(xa_empty, 2);
+    mbar_init(xa_empty, 1);
     mbar_init(gi_full, 1);
-    mbar_init(gi_empty, 2);
+    mbar_init(gi_empty, 1);
     *abort = 0;
     fence_barrier_init();
   }
@@ -265,44 +266,21 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
         mbar_drain(gi_full, (uint32_t)(n_items_done - 1) & 1u, 500000000ull);
       }
     }
-  } else if (warp == kMmaWarp || warp == kBwdIssue1Warp) {
-    // ------------------------------------------------------------ issuer of warpgroup b
-    // Per own half k of the item: S(k), W(k) once the warpgroup has read
-    // S(k-1), W(k-1); then the feature sums of Q(k-1) once it is written.
+  } else if (warp == kMmaWarp) {
+    // ------------------------------------------------------------ issuer of S and W
+    // Per J tile: S and W of its 128 columns (both halves at once) when both warpgroups
+    // have read the previous tile's.
     const bool leader = elect_one();
-    const int b = warp == kMmaWarp ? 0 : 1;
-    const uint32_t idSW = idesc_f16(128, 64, 0, 0);
-    const uint32_t idA = idesc_f16(128, a.NACC, 0, 0);
+    const uint32_t idSW = idesc_f16(128, 128, 0, 0);
     const int nkx = a.KX / 16, nkg = a.KG / 16;
     const uint64_t dXA = sdesc(smem_u32(sXA), 128, a.KX * 16u);
     const uint64_t dGI = sdesc(smem_u32(sGI), 128, a.KG * 16u);
-    const uint64_t dXB = sdesc(smem_u32(sS + b * a.KX * 128u), 128, a.KX * 16u);
-    const uint64_t dVJ = sdesc(smem_u32(sS + XT + b * a.KG * 128u), 128, a.KG * 16u);
-    const uint64_t dBG = sdesc(smem_u32(sS + XT + GT + b * 1024u), 128, 2048);
-    const uint32_t lo_bytes = (uint32_t)a.NACC * 256u;   // ksplit: the lo block of BG
-    const uint32_t tS = tbase + 128 * b, tW = tS + 64, tA = tbase + kColXA;
-    const uint32_t tQh = tbase + 256 + 64 * b, tQl = tQh + 32;
-    const uint32_t tACC = tbase + 512 - 2 * a.NACC + b * a.NACC;
+    const uint64_t dXB = sdesc(smem_u32(sS), 128, a.KX * 16u);
+    const uint64_t dVJ = sdesc(smem_u32(sS + XT), 128, a.KG * 16u);
+    const uint32_t tS = tbase, tW = tbase + 128, tA = tbase + kColXA;
     int it = 0;
-    long long uses = 0, qr = 0;
+    long long uses = 0;
     uint32_t stage = 0, sph = 0;
-    // the feature sums of own half jj (stored in Q_b), from stage st_
-    auto issue_acc = [&](uint32_t st_, int jj) -> bool {
-      if (!warp_wait(&q_ready[b], (uint32_t)(qr & 1), abort, a.err, 26)) return false;
-      ++qr;
-      tc_fence_after();
-      const uint32_t acc = (jj % kFoldOwn) != 0;
-      const uint64_t dbg = sdesc_add(dBG, st_ * STG);
-      if (leader) {
-        issue_ts4(tACC, tQh, dbg, idA, acc);
-        if (a.ksplit) issue_ts4(tACC, tQh, sdesc_add(dbg, lo_bytes), idA, 1);
-        issue_ts4(tACC, tQl, dbg, idA, 1);
-        tc_commit(&q_free[b]);
-        tc_commit(&empty[st_]);
-      }
-      __syncwarp();
-      return true;
-    };
     for (int t = blockIdx.x; t < a.n_items; t += gridDim.x) {
       const int4 item = a.items[t];
       if (a.sys_active && !a.sys_active[item.x]) continue;
@@ -310,9 +288,8 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
       if (!warp_wait(XS ? xa_full : a_ready, ip, abort, a.err, XS ? 34 : 31)) goto sw_out;
       if (!warp_wait(gi_full, ip, abort, a.err, 36)) goto sw_out;
       ++it;
-      uint32_t prev_stage = 0;
       for (int j = 0; j < item.w; ++j) {
-        if (uses > 0 && !warp_wait(&s_free[b], (uint32_t)((uses - 1) & 1), abort, a.err, 23)) goto sw_out;
+        if (uses > 0 && !warp_wait(s_free, (uint32_t)((uses - 1) & 1), abort, a.err, 23)) goto sw_out;
         if (!warp_wait(&full[stage], sph, abort, a.err, 25)) goto sw_out;
         tc_fence_after();
         // operands computed by the whole warp (warp-uniform), issued by the leader
@@ -330,7 +307,8 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
           }
 #pragma unroll 4
           for (int q = 0; q < nkg; ++q) mma_ss(tW, dGI + 16 * q, dv + 16 * q, idSW, q > 0);
-          tc_commit(&sw_full[b]);
+          tc_commit(sw_full);
+          tc_commit(&empty[stage]);
           // the item's XA and GI tiles are released after its last S, W products
           if (j == item.w - 1) {
             tc_commit(gi_empty);
@@ -339,22 +317,57 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
         }
         __syncwarp();
         ++uses;
-        if (j > 0 && !issue_acc(prev_stage, j - 1)) goto sw_out;
-        prev_stage = stage;
         if (++stage == (uint32_t)S) { stage = 0; sph ^= 1; }
       }
-      if (item.w > 0 && !issue_acc(prev_stage, item.w - 1)) goto sw_out;
     }
   sw_out:
-    if (leader) tc_commit(&done[b]);
+    if (leader) tc_commit(&done[0]);
     __syncwarp();
-    mbar_drain(&done[b], 0, 500000000ull);
+    mbar_drain(&done[0], 0, 500000000ull);
+  } else if (warp == kBwdIssue1Warp) {
+    // ------------------------------------------------------------ issuer of the feature sums
+    // Per J tile the sums of Q_0, then of Q_1, once each is written.
+    const bool leader = elect_one();
+    const uint32_t idA = idesc_f16(128, a.NACC, 0, 0);
+    const uint64_t dBG = sdesc(smem_u32(sS + XT + GT), 128, 2048);
+    const uint32_t lo_bytes = (uint32_t)a.NACC * 256u;   // ksplit: the lo block of BG
+    long long qr = 0;
+    uint32_t stage = 0, sph = 0;
+    for (int t = blockIdx.x; t < a.n_items; t += gridDim.x) {
+      const int4 item = a.items[t];
+      if (a.sys_active && !a.sys_active[item.x]) continue;
+      for (int j = 0; j < item.w; ++j, ++qr) {
+        if (!warp_wait(&full[stage], sph, abort, a.err, 25)) goto acc_out;
+        const uint32_t acc = (j % kFoldOwn) != 0;
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          if (!warp_wait(&q_ready[b], (uint32_t)(qr & 1), abort, a.err, 26)) goto acc_out;
+          tc_fence_after();
+          const uint32_t tQh = tbase + 256 + 64 * b, tQl = tQh + 32;
+          const uint32_t tACC = tbase + 512 - 2 * a.NACC + b * a.NACC;
+          const uint64_t dbg = sdesc_add(dBG, stage * STG + b * 1024u);
+          if (leader) {
+            issue_ts4(tACC, tQh, dbg, idA, acc);
+            if (a.ksplit) issue_ts4(tACC, tQh, sdesc_add(dbg, lo_bytes), idA, 1);
+            issue_ts4(tACC, tQl, dbg, idA, 1);
+            tc_commit(&q_free[b]);
+            if (b == 1) tc_commit(&empty[stage]);
+          }
+          __syncwarp();
+        }
+        if (++stage == (uint32_t)S) { stage = 0; sph ^= 1; }
+      }
+    }
+  acc_out:
+    if (leader) tc_commit(&done[1]);
+    __syncwarp();
+    mbar_drain(&done[1], 0, 500000000ull);
   } else {
     // ------------------------------------------------------------ warpgroups
     const int b = warp >> 2, w = warp & 3;
     const int row = 32 * w + lane;
     const uint32_t lofs = static_cast<uint32_t>(32 * w) << 16;
-    const uint32_t tS = tbase + lofs + 128 * b, tQh = tbase + lofs + 256 + 64 * b;
+    const uint32_t tS = tbase + lofs + 64 * b, tW = tS + 128, tQh = tbase + lofs + 256 + 64 * b;
     const uint32_t tQl = tQh + 32;
     const uint32_t tACC = tbase + lofs + 512 - 2 * a.NACC + b * a.NACC;
     const int d = a.d, dk = a.dk, k0 = a.k0;
@@ -483,7 +496,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
         }
       };
       for (int j = 0; j < item.w; ++j, ++uses) {
-        bool ok = mbar_wait(&sw_full[b], (uint32_t)(uses & 1), abort, a.err, 28);
+        bool ok = mbar_wait(sw_full, (uint32_t)(uses & 1), abort, a.err, 28);
         if (!__all_sync(0xffffffffu, ok)) goto exp_out;
         tc_fence_after();
         {
@@ -492,11 +505,11 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
           uint32_t s0[32], s1[32], w0[32], w1[32], qq[32];
           tmem_ld32(tS, s0);
           tmem_ld32(tS + 32, s1);
-          tmem_ld32(tS + 64, w0);
-          tmem_ld32(tS + 96, w1);
+          tmem_ld32(tW, w0);
+          tmem_ld32(tW + 32, w1);
           tmem_ld_wait_regs(s0, s1, w0, w1);
           tc_fence_before();
-          mbar_arrive(&s_free[b]);
+          mbar_arrive(s_free);
           if (item.z + j == item.y) {
             // diagonal tile of the upper triangle: counted once, off-diagonal
             // tiles twice; the pair i = j is left out (its distance is 0, and its

@@ -86,6 +86,20 @@ __device__ __forceinline__ void block_sum_many(double (&v)[N], int n, double* re
   }
 }
 
+// Block sum of one pair per thread; result valid in thread 0.  (An FP64 block_sum keeps
+// the FP64 pipe, 2 lanes per clock and SM, busy for six operations per warp.)
+__device__ __forceinline__ double pair_block_sum(float s, float e, double* red) {
+  pair_warp_sum(s, e);
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  __syncthreads();
+  if (l == 0) red[w] = (double)s + (double)e;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x == 0)
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[i];
+  return t;
+}
+
 // Sums NC (16 or 32) pairs per lane over the warp: the lanes halve the vector between
 // them step by step; lane l returns with column l % NC in (s[0], e[0]).
 template <int NC>
