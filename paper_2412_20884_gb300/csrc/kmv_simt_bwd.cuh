@@ -24,6 +24,7 @@
 // the figures at simt_bwd_plan.
 #pragma once
 
+#include "f32x2.cuh"
 #include "simt_common.cuh"
 
 namespace kmv {
@@ -46,9 +47,9 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
   const int64_t jb = o0 + u * len, je = min(o1, jb + len);
   if (je <= jb) return;
 
-  // per staged row of V and G: MP columns each
+  // V by column (pairs of points for W), G by point (pairs of columns for dL/dV)
   __shared__ __align__(16) float sx[D * kXSB];
-  __shared__ __align__(16) float sv[kJT * MP];
+  __shared__ __align__(16) float sv[MP * kXSB];
   __shared__ __align__(16) float sg[kJT * MP];
   __shared__ float sc[D];
   __shared__ double as2[2];
@@ -67,7 +68,9 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
   const int64_t r0 = a.L.item_row0[item0];
   __syncthreads();
 
-  float xi[R][D], gi[R][MP], accq[R], accg[R][DG], accv[R][MP];
+  float xi[R][D], gi[R][MP], accq[R], accg[R][DG];
+  uint64_t accv[R][MP / 2];   // columns 2q, 2q + 1 in a packed pair
+  auto accv_at = [&](int r, int q) { return (q & 1) ? hi_f32x2(accv[r][q / 2]) : lo_f32x2(accv[r][q / 2]); };
   // running sums of the unit as pairs (several folds)
   float sq[R], cq[R], sg2[R][DG], cg2[R][DG];
   // those of dL/dV: in registers with one row per thread, else in f.part
@@ -85,7 +88,7 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
 #pragma unroll
     for (int q = 0; q < MP; ++q) {
       gi[r][q] = (q < mc && valid) ? a.G[(vbase + i) * a.m + c0 + q] * amp_i : 0.f;
-      accv[r][q] = 0.f;
+      accv[r][q / 2] = 0;
     }
     accq[r] = sq[r] = cq[r] = 0.f;
 #pragma unroll
@@ -100,9 +103,10 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
     if constexpr (R == 1) {
 #pragma unroll
       for (int q = 0; q < RV; ++q) {
-        two_sum_add(svp[q], cvp[q], accv[0][q]);
-        accv[0][q] = 0.f;
+        two_sum_add(svp[q], cvp[q], accv_at(0, q));
       }
+#pragma unroll
+      for (int q = 0; q < MP / 2; ++q) accv[0][q] = 0;
     } else {
 #pragma unroll
       for (int r = 0; r < R; ++r) {
@@ -113,12 +117,12 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
             if (q < mc) {
               float2* p = &f.part[(((size_t)u * a.chains + c) * a.m + c0 + q) * (size_t)a.n_total + i];
               float2 v = first ? make_float2(0.f, 0.f) : *p;
-              two_sum_add(v.x, v.y, accv[r][q]);
+              two_sum_add(v.x, v.y, accv_at(r, q));
               *p = v;
             }
         }
 #pragma unroll
-        for (int q = 0; q < MP; ++q) accv[r][q] = 0.f;
+        for (int q = 0; q < MP / 2; ++q) accv[r][q] = 0;
       }
       first = false;
     }
@@ -148,7 +152,7 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
       const bool in = r < nj && q < mc;
       const int64_t idx = (vbase + jt + r) * a.m + c0 + q;
       const float am = (in && a.amp) ? a.amp[vbase + jt + r] : 1.f;
-      sv[e] = in ? a.V[idx] * am : 0.f;
+      sv[q * kXSB + r] = in ? a.V[idx] * am : 0.f;
       sg[e] = (in && want_gv) ? a.G[idx] * am : 0.f;
     }
     __syncthreads();
@@ -156,85 +160,73 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
     // has eight in flight where registers allow
 #pragma unroll (R == 1 && D * MP <= 32 ? 4 : 1)
     for (int jj = 0; jj < kJT; jj += 2) {
-      float r2[R][2], df2[R][2][DG];
+      uint64_t r2[R], df2[R][DG];
 #pragma unroll
-      for (int r = 0; r < R; ++r) r2[r][0] = r2[r][1] = 0.f;
+      for (int r = 0; r < R; ++r) r2[r] = 0;
 #pragma unroll
       for (int k = 0; k < D; ++k) {
-        const float2 x2 = *reinterpret_cast<const float2*>(sx + k * kXSB + jj);
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-#pragma unroll
-          for (int t = 0; t < 2; ++t) {
-            const float df = __fsub_rn(xi[r][k], t ? x2.y : x2.x);
-            if (ARD) {
-              const float q2 = __fmul_rn(df, df);
-              df2[r][t][ARD ? k : 0] = q2;
-              r2[r][t] = __fadd_rn(r2[r][t], q2);
-            } else {
-              r2[r][t] = __fmaf_rn(df, df, r2[r][t]);
-            }
-          }
-      }
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        float w[R], p[R];
+        const uint64_t x2 = *reinterpret_cast<const uint64_t*>(sx + k * kXSB + jj);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          w[r] = 0.f;
-          p[r] = ex2_approx(-r2[r][t]);
-        }
-        const float* vj = sv + (jj + t) * MP;
-        const float* gj = sg + (jj + t) * MP;
-        constexpr int QS = MP < 4 ? MP : 4;
-        float vv[QS];
-#pragma unroll
-        for (int q = 0; q < MP; q += QS) {
-          if constexpr (QS == 4) {
-            const float4 v = *reinterpret_cast<const float4*>(vj + q);
-            vv[0] = v.x;
-            vv[1 % QS] = v.y;
-            vv[2 % QS] = v.z;
-            vv[3 % QS] = v.w;
-          } else {
-            const float2 v = *reinterpret_cast<const float2*>(vj + q);
-            vv[0] = v.x;
-            vv[1 % QS] = v.y;
-          }
-#pragma unroll
-          for (int e = 0; e < QS; ++e)
-#pragma unroll
-            for (int r = 0; r < R; ++r) w[r] = __fmaf_rn(gi[r][q + e], vv[e], w[r]);
-        }
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          const float Q = __fmul_rn(w[r], p[r]);
-          accq[r] = __fadd_rn(accq[r], Q);
+          const uint64_t df = sub_f32x2(pack_f32x2(xi[r][k], xi[r][k]), x2);
           if (ARD) {
-#pragma unroll
-            for (int k = 0; k < DG; ++k) accg[r][k] = __fmaf_rn(Q, df2[r][t][k], accg[r][k]);
+            const uint64_t q2 = mul_f32x2(df, df);
+            df2[r][ARD ? k : 0] = q2;
+            r2[r] = add_f32x2(r2[r], q2);
           } else {
-            accg[r][0] = __fmaf_rn(Q, r2[r][t], accg[r][0]);
+            r2[r] = fma_f32x2(df, df, r2[r]);
           }
         }
-        if (want_gv) {
+      }
+      uint64_t w[R];
 #pragma unroll
-          for (int q = 0; q < MP; q += QS) {
-            if constexpr (QS == 4) {
-              const float4 v = *reinterpret_cast<const float4*>(gj + q);
-              vv[0] = v.x;
-              vv[1 % QS] = v.y;
-              vv[2 % QS] = v.z;
-              vv[3 % QS] = v.w;
-            } else {
-              const float2 v = *reinterpret_cast<const float2*>(gj + q);
-              vv[0] = v.x;
-              vv[1 % QS] = v.y;
+      for (int r = 0; r < R; ++r) w[r] = 0;
+#pragma unroll
+      for (int q = 0; q < MP; ++q) {
+        const uint64_t v2 = *reinterpret_cast<const uint64_t*>(sv + q * kXSB + jj);
+#pragma unroll
+        for (int r = 0; r < R; ++r) w[r] = fma_f32x2(pack_f32x2(gi[r][q], gi[r][q]), v2, w[r]);
+      }
+      float p[R][2];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        p[r][0] = ex2_approx(-lo_f32x2(r2[r]));
+        p[r][1] = ex2_approx(-hi_f32x2(r2[r]));
+        const uint64_t Q2 = mul_f32x2(w[r], pack_f32x2(p[r][0], p[r][1]));
+        const float Q0 = lo_f32x2(Q2), Q1 = hi_f32x2(Q2);
+        accq[r] = __fadd_rn(__fadd_rn(accq[r], Q0), Q1);
+        if (ARD) {
+#pragma unroll
+          for (int k = 0; k < DG; ++k) {
+            accg[r][k] = __fmaf_rn(Q0, lo_f32x2(df2[r][k]), accg[r][k]);
+            accg[r][k] = __fmaf_rn(Q1, hi_f32x2(df2[r][k]), accg[r][k]);
+          }
+        } else {
+          accg[r][0] = __fmaf_rn(Q0, lo_f32x2(r2[r]), accg[r][0]);
+          accg[r][0] = __fmaf_rn(Q1, hi_f32x2(r2[r]), accg[r][0]);
+        }
+      }
+      if (want_gv) {
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          const float* gj = sg + (jj + t) * MP;
+          uint64_t pp[R];
+#pragma unroll
+          for (int r = 0; r < R; ++r) pp[r] = pack_f32x2(p[r][t], p[r][t]);
+          if constexpr (MP == 2) {
+            const uint64_t v2 = *reinterpret_cast<const uint64_t*>(gj);
+#pragma unroll
+            for (int r = 0; r < R; ++r) accv[r][0] = fma_f32x2(pp[r], v2, accv[r][0]);
+          } else {
+#pragma unroll
+            for (int q = 0; q < MP / 2; q += 2) {
+              const ulonglong2 v2 = *reinterpret_cast<const ulonglong2*>(gj + 2 * q);
+#pragma unroll
+              for (int r = 0; r < R; ++r) {
+                accv[r][q] = fma_f32x2(pp[r], v2.x, accv[r][q]);
+                accv[r][(q + 1) % (MP / 2)] = fma_f32x2(pp[r], v2.y, accv[r][(q + 1) % (MP / 2)]);
+              }
             }
-#pragma unroll
-            for (int e = 0; e < QS; ++e)
-#pragma unroll
-              for (int r = 0; r < R; ++r) accv[r][q + e] = __fmaf_rn(p[r], vv[e], accv[r][q + e]);
           }
         }
       }
@@ -269,7 +261,7 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
           const double g = (double)a.G[idx];
           if (u == 0) noise += g * (double)a.V[idx];
           if (want_gv && direct) {
-            float2 v = R == 1 ? make_float2(svp[q % RV], cvp[q % RV]) : make_float2(accv[r][q], 0.f);
+            float2 v = R == 1 ? make_float2(svp[q % RV], cvp[q % RV]) : make_float2(accv_at(r, q), 0.f);
             if (R > 1 && paired) v = f.part[((size_t)c * a.m + c0 + q) * (size_t)a.n_total + i];
             a.Y[idx] = (float)(ai * ((double)v.x + (double)v.y) + as2[1] * g);
           }

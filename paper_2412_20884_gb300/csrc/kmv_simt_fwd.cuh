@@ -16,15 +16,17 @@
 // lane of a warp shares.  Such a broadcast still returns 128 bytes per clock and SM,
 // so with one row per thread the loads alone took D + m clocks per 32 pairs against
 // (2 D + m) / 4 for the arithmetic; R = 4 rows per thread divide them by four, and
-// the loads are 16 bytes wide (x is staged dimension by dimension).  The same
-// arithmetic in packed f32x2 form was measured at the same rate per lane
-// (60 packed against 114 scalar instructions per clock and SM), so it is not used.
+// the loads are 16 bytes wide (x is staged dimension by dimension).  Distances of two
+// points and sums of two columns share packed f32x2 instructions: the FMA pipe runs them
+// at the same rate per value (60 packed against 114 scalar instructions per clock and
+// SM), but the scalar form needed an issue slot per clock and scheduler for it alone.
 // At N = 20,000, d = 8, m = 16 one row per thread and one CTA per SM took 2.18 ms;
 // at N = 8192, d = 3, 8 chains, m = 1 0.274 ms (figures after the change stand at
 // simt_fwd_plan).
 #pragma once
 
 #include "cg_common.cuh"
+#include "f32x2.cuh"
 #include "simt_common.cuh"
 
 namespace kmv {
@@ -158,7 +160,11 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
   const int64_t vbase = (int64_t)c * a.n_total;
   const int64_t r0 = single ? (int64_t)item0 * kTile : a.L.item_row0[item0];
 
-  float xi[R][D], acc[R][MP];
+  float xi[R][D];
+  // sums: columns 2q, 2q + 1 of a row in a packed pair (one column: plain)
+  constexpr int NP = MP > 1 ? MP / 2 : 1;
+  uint64_t acc[R][NP];
+  auto acc_at = [&](int r, int q) { return (q & 1) ? hi_f32x2(acc[r][q / 2]) : lo_f32x2(acc[r][q / 2]); };
   // few columns: V_i for the epilogue too, loaded here so that the last CTA has it
   constexpr int PV = MP <= 2 ? MP : 1;
   float vi[R][PV];
@@ -168,7 +174,7 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
 #pragma unroll
     for (int k = 0; k < D; ++k) xi[r][k] = (k < dd && i < o1) ? a.x[i * dd + k] : 0.f;
 #pragma unroll
-    for (int q = 0; q < MP; ++q) acc[r][q] = 0.f;
+    for (int q = 0; q < NP; ++q) acc[r][q] = 0;
   }
 
   // the next J tile's points and vectors, loaded into registers while the current
@@ -251,12 +257,12 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
           if (q < mc) {
             float2* p = &f.part[simt_part_at(a, unit, c, c0 + q, i)];
             float2 v = first ? make_float2(0.f, 0.f) : *p;
-            two_sum_add(v.x, v.y, acc[r][q]);
+            two_sum_add(v.x, v.y, acc_at(r, q));
             *p = v;
           }
       }
 #pragma unroll
-      for (int q = 0; q < MP; ++q) acc[r][q] = 0.f;
+      for (int q = 0; q < NP; ++q) acc[r][q] = 0;
     }
     first = false;
   };
@@ -276,66 +282,66 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
     // one row per thread leaves a chain of dependent steps: two steps in flight there
 #pragma unroll (R == 1 && D * MP <= 64 ? 2 : 1)
     for (int jj = 0; jj < kJT; jj += 4) {
-      float p[R][4];
+      uint64_t d01[R], d23[R];   // squared distances of the four points
 #pragma unroll
-      for (int r = 0; r < R; ++r) p[r][0] = p[r][1] = p[r][2] = p[r][3] = 0.f;
+      for (int r = 0; r < R; ++r) d01[r] = d23[r] = 0;
 #pragma unroll
       for (int k = 0; k < D; ++k) {
-        const float4 x4 = *reinterpret_cast<const float4*>(X + k * kXS + jj);
+        const ulonglong2 x4 = *reinterpret_cast<const ulonglong2*>(X + k * kXS + jj);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          const float d0 = __fsub_rn(xi[r][k], x4.x), d1 = __fsub_rn(xi[r][k], x4.y);
-          const float d2 = __fsub_rn(xi[r][k], x4.z), d3 = __fsub_rn(xi[r][k], x4.w);
-          p[r][0] = fmaf(d0, d0, p[r][0]);
-          p[r][1] = fmaf(d1, d1, p[r][1]);
-          p[r][2] = fmaf(d2, d2, p[r][2]);
-          p[r][3] = fmaf(d3, d3, p[r][3]);
+          const uint64_t xx = pack_f32x2(xi[r][k], xi[r][k]);
+          const uint64_t da = sub_f32x2(xx, x4.x), db = sub_f32x2(xx, x4.y);
+          d01[r] = fma_f32x2(da, da, d01[r]);
+          d23[r] = fma_f32x2(db, db, d23[r]);
         }
       }
+      float p[R][4];
 #pragma unroll
-      for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int t = 0; t < 4; ++t) p[r][t] = ex2_approx(-p[r][t]);
+      for (int r = 0; r < R; ++r) {
+        p[r][0] = ex2_approx(-lo_f32x2(d01[r]));
+        p[r][1] = ex2_approx(-hi_f32x2(d01[r]));
+        p[r][2] = ex2_approx(-lo_f32x2(d23[r]));
+        p[r][3] = ex2_approx(-hi_f32x2(d23[r]));
+      }
       // the vectors of the four points: 4 MP consecutive floats
-      constexpr int NQ = MP < 4 ? MP : 4;   // float4 loads per step of 4 / (MP < 4 ? MP : 4) .. columns
       if (MP == 1) {
         const float4 v = *reinterpret_cast<const float4*>(V + jj);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          acc[r][0] = fmaf(p[r][0], v.x, acc[r][0]);
-          acc[r][0] = fmaf(p[r][1], v.y, acc[r][0]);
-          acc[r][0] = fmaf(p[r][2], v.z, acc[r][0]);
-          acc[r][0] = fmaf(p[r][3], v.w, acc[r][0]);
+          float s1 = lo_f32x2(acc[r][0]);
+          s1 = fmaf(p[r][0], v.x, s1);
+          s1 = fmaf(p[r][1], v.y, s1);
+          s1 = fmaf(p[r][2], v.z, s1);
+          s1 = fmaf(p[r][3], v.w, s1);
+          acc[r][0] = pack_f32x2(s1, 0.f);
         }
       } else if (MP == 2) {
-        const float4 va = *reinterpret_cast<const float4*>(V + 2 * jj);
-        const float4 vb = *reinterpret_cast<const float4*>(V + 2 * jj + 4);
-        constexpr int q1 = MP > 1 ? 1 : 0;
+        const ulonglong2 va = *reinterpret_cast<const ulonglong2*>(V + 2 * jj);
+        const ulonglong2 vb = *reinterpret_cast<const ulonglong2*>(V + 2 * jj + 4);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          acc[r][0] = fmaf(p[r][0], va.x, acc[r][0]);
-          acc[r][q1] = fmaf(p[r][0], va.y, acc[r][q1]);
-          acc[r][0] = fmaf(p[r][1], va.z, acc[r][0]);
-          acc[r][q1] = fmaf(p[r][1], va.w, acc[r][q1]);
-          acc[r][0] = fmaf(p[r][2], vb.x, acc[r][0]);
-          acc[r][q1] = fmaf(p[r][2], vb.y, acc[r][q1]);
-          acc[r][0] = fmaf(p[r][3], vb.z, acc[r][0]);
-          acc[r][q1] = fmaf(p[r][3], vb.w, acc[r][q1]);
+          acc[r][0] = fma_f32x2(pack_f32x2(p[r][0], p[r][0]), va.x, acc[r][0]);
+          acc[r][0] = fma_f32x2(pack_f32x2(p[r][1], p[r][1]), va.y, acc[r][0]);
+          acc[r][0] = fma_f32x2(pack_f32x2(p[r][2], p[r][2]), vb.x, acc[r][0]);
+          acc[r][0] = fma_f32x2(pack_f32x2(p[r][3], p[r][3]), vb.y, acc[r][0]);
         }
       } else {
 #pragma unroll
-        for (int t = 0; t < 4; ++t)
+        for (int t = 0; t < 4; ++t) {
+          uint64_t pp[R];
 #pragma unroll
-          for (int q = 0; q < MP; q += NQ) {
-            const float4 v = *reinterpret_cast<const float4*>(V + (jj + t) * MP + q);
+          for (int r = 0; r < R; ++r) pp[r] = pack_f32x2(p[r][t], p[r][t]);
+#pragma unroll
+          for (int q = 0; q < MP; q += 4) {
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(V + (jj + t) * MP + q);
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-              acc[r][(q + 0) % MP] = fmaf(p[r][t], v.x, acc[r][(q + 0) % MP]);
-              acc[r][(q + 1) % MP] = fmaf(p[r][t], v.y, acc[r][(q + 1) % MP]);
-              acc[r][(q + 2) % MP] = fmaf(p[r][t], v.z, acc[r][(q + 2) % MP]);
-              acc[r][(q + 3) % MP] = fmaf(p[r][t], v.w, acc[r][(q + 3) % MP]);
+              acc[r][(q / 2) % NP] = fma_f32x2(pp[r], v.x, acc[r][(q / 2) % NP]);
+              acc[r][(q / 2 + 1) % NP] = fma_f32x2(pp[r], v.y, acc[r][(q / 2 + 1) % NP]);
             }
           }
+        }
       }
     }
     if (more) store(buf ^ 1);
@@ -358,7 +364,7 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
           if (q < mc) {
             float2 v = make_float2(0.f, 0.f);
             if (paired) v = f.part[simt_part_at(a, 0, c, c0 + q, i)];
-            two_sum_add(v.x, v.y, acc[r][q]);
+            two_sum_add(v.x, v.y, acc_at(r, q));
             dots[r] += simt_put_y(a, s, c, i, c0 + q, ai, s2, (double)v.x + (double)v.y,
                                   MP <= 2 ? vi[r][q % PV] : a.V[(vbase + i) * a.m + c0 + q]);
           }

@@ -615,13 +615,20 @@ __global__ void __launch_bounds__(kFmaThreads, 1) tc_fwd_fma_kernel(TcFwdArgs a)
       const int4 item = a.items[t];
       if (a.sys_active && !a.sys_active[item.x]) continue;
       const int rowp = g * 128 + row;
-      // four independent FP32 chains per column (short FMA dependency chains)
+      // four independent FP32 chains per column (short FMA dependency chains), two to a
+      // packed register pair
       double acc64[MZ];
-      float acc[MZ][4];
+      uint64_t acc[MZ][2];
+      auto acc_sum = [&](int q) {
+        float c0, c1, c2, c3;
+        unpack_f32x2(acc[q][0], c0, c1);
+        unpack_f32x2(acc[q][1], c2, c3);
+        return (double)((c0 + c1) + (c2 + c3));
+      };
 #pragma unroll
       for (int q = 0; q < MZ; ++q) {
         acc64[q] = 0.0;
-        acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.f;
+        acc[q][0] = acc[q][1] = 0;
       }
       // The half's 64 columns in four chunks of 16, each chunk's TMEM load in flight
       // while the one before it is worked on, the next tile's first chunk included if
@@ -638,10 +645,8 @@ __global__ void __launch_bounds__(kFmaThreads, 1) tc_fwd_fma_kernel(TcFwdArgs a)
 #pragma unroll
           for (int q = 0; q < MZ; ++q) {
             const float4 v = vs[q * 32 + u0 + u];
-            acc[q][0] = fmaf(p0, v.x, acc[q][0]);
-            acc[q][1] = fmaf(p1, v.y, acc[q][1]);
-            acc[q][2] = fmaf(p2, v.z, acc[q][2]);
-            acc[q][3] = fmaf(p3, v.w, acc[q][3]);
+            acc[q][0] = fma_f32x2(pack_f32x2(p0, p1), pack_f32x2(v.x, v.y), acc[q][0]);
+            acc[q][1] = fma_f32x2(pack_f32x2(p2, p3), pack_f32x2(v.z, v.w), acc[q][1]);
           }
         }
       };
@@ -699,8 +704,8 @@ __global__ void __launch_bounds__(kFmaThreads, 1) tc_fwd_fma_kernel(TcFwdArgs a)
         if (j1 - j0 == kFold) {
 #pragma unroll
           for (int q = 0; q < MZ; ++q) {
-            acc64[q] += (double)((acc[q][0] + acc[q][1]) + (acc[q][2] + acc[q][3]));
-            acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.f;
+            acc64[q] += acc_sum(q);
+            acc[q][0] = acc[q][1] = 0;
           }
         }
       }
@@ -717,7 +722,7 @@ __global__ void __launch_bounds__(kFmaThreads, 1) tc_fwd_fma_kernel(TcFwdArgs a)
         }
 #pragma unroll
         for (int q = 0; q < MZ; ++q)
-          cb[q * 128 + row] = acc64[q] + (double)((acc[q][0] + acc[q][1]) + (acc[q][2] + acc[q][3]));
+          cb[q * 128 + row] = acc64[q] + acc_sum(q);
         mbar_arrive(&comb_full[2 * g + par]);
       } else {
         const bool okc = mbar_wait(&comb_full[2 * g + par], (cph >> par) & 1u, abort, a.err, 18);
@@ -726,7 +731,7 @@ __global__ void __launch_bounds__(kFmaThreads, 1) tc_fwd_fma_kernel(TcFwdArgs a)
 #pragma unroll
         for (int q = 0; q < MZ; ++q)
           a.part[part_idx(t, a.mz, q, rowp)] =
-              (acc64[q] + (double)((acc[q][0] + acc[q][1]) + (acc[q][2] + acc[q][3]))) + cb[q * 128 + row];
+              (acc64[q] + acc_sum(q)) + cb[q * 128 + row];
         mbar_arrive(&comb_free[2 * g + par]);
       }
       ++it;

@@ -7,21 +7,25 @@
 // tiles (J >= I) is evaluated, off-diagonal tiles weighted twice.
 //
 // A work item is one I tile of one system against a range of J tiles; each J
-// tile is split into two 64-column halves, half b for warpgroup b.  Issuer warp 0
-// writes into TMEM, per J tile (its 128 columns in one MMA per K step: with the A
-// operand in shared memory an MMA of 64 columns takes 48 clocks, one of 128 takes 64,
-// and an issuing warp manages one per 50 to 120 clocks)
+// tile is split into two 64-column halves, half b for warpgroup b, with two MMA issuer
+// warps.  XA in tensor memory (small d): the warpgroups run as independent pipelines,
+// an issuer each, so that one computes while the other waits (1.17 ms at N = 65,536,
+// d = 8, m = 16; with the products of a tile issued for both at once they wait
+// together, 1.27 ms).  XA in shared memory (large d, where S is 7 K steps and more):
+// one issuer writes S and W of a J tile's 128 columns in one MMA per K step (an MMA of
+// 64 columns with A in shared memory takes 48 clocks, one of 128 takes 64), the other
+// the feature sums.  Per J tile
 //   S = XA_I XB_J^T           the base-2 exponent from F16 hi/lo operands of the
 //                             centred points (|dS| ~ 2^-24 |xh|^2); XA from TMEM
 //   W = GI_I VJ_J^T           = G_i . V_j + V_i . G_j with GI rows
 //                             [gh gh gl vh vh vl] (shared memory, once per item)
 //                             and VJ rows [vh vl vh gh gl gh] (F16 hi/lo, G and V
 //                             each scaled by a power of two)
-// Both warpgroups read their half of S and W into registers at once, so that the next
-// tile's products run during this tile's exps.  Warpgroup b forms Q = W 2^S in FP32 (halved on the diagonal tile, and zero for
-// i = j, whose (xt_i - xt_i)^2 is 0), splits it exactly into Q = Qh + Ql with Qh
-// holding 11 significant bits (Veltkamp's splitting), stores both as F16, and
-// issuer b accumulates, per row i,
+// Each warpgroup reads its half of S and W into registers at once, so that the next
+// products run during the exps.  Warpgroup b forms Q = W 2^S in FP32 (halved on the
+// diagonal tile, and zero for i = j, whose (xt_i - xt_i)^2 is 0), splits it exactly into
+// Q = Qh + Ql with Qh holding 11 significant bits (Veltkamp's splitting), stores both as
+// F16, and an issuer accumulates, per row i,
 //   ACC_b += Qh BG + Ql BG    BG: F16 hi/lo of xt_jk and xt_jk^2 and a ones column
 //                             (the hi and lo parts in separate accumulator
 //                             columns, or, for large d, in the same columns by
@@ -114,18 +118,29 @@ __device__ __forceinline__ double row_scale(uint32_t bits) {
 
 // Exact split q = hi + lo with hi holding 11 significant bits (Veltkamp's
 // splitting with the factor 2^13 + 1), so that hi is an F16 value and lo
-// carries the next 11 bits when stored as F16.  The rounded intrinsics keep
-// the compiler from contracting the steps into FMAs, which would break the
-// split.
-__device__ __forceinline__ void split_q(float q, float& hi, float& lo) {
-  const float t = __fmul_rn(q, 8193.f);
-  hi = __fsub_rn(t, __fsub_rn(t, q));
-  lo = __fsub_rn(q, hi);
+// carries the next 11 bits when stored as F16; q = w 2^s of two neighbouring columns at
+// a time in packed FP32 instructions (the same roundings, half the issue slots: the
+// kernel's exp warps issue on 55% of the cycles).  The packed intrinsics keep the
+// compiler from contracting the steps into FMAs, which would break the split.
+__device__ __forceinline__ void split_q2(uint32_t s0, uint32_t s1, uint32_t w0, uint32_t w1, uint32_t& hi, uint32_t& lo) {
+  using namespace ptx;
+  const uint64_t q = mul_f32x2(pack_f32x2(ex2(__uint_as_float(s0)), ex2(__uint_as_float(s1))),
+                               pack_f32x2(__uint_as_float(w0), __uint_as_float(w1)));
+  const uint64_t t = mul_f32x2(q, pack_f32x2(8193.f, 8193.f));
+  const uint64_t h = sub_f32x2(t, sub_f32x2(t, q));
+  const uint64_t l = sub_f32x2(q, h);
+  float a, b;
+  unpack_f32x2(h, a, b);
+  hi = pack_f16x2(a, b);
+  unpack_f32x2(l, a, b);
+  lo = pack_f16x2(a, b);
 }
 
-// Warps: 0-7 the two warpgroups, 8 the issuer of S and W (and TMEM owner), 9 the
-// producer, 10 the issuer of the feature sums.  TMEM (512 columns):
-//   S [0, 128), W [128, 256), Qh_b [256 + 64 b, +32), Ql_b [+32, +32),
+// Warps: 0-7 the two warpgroups, 8 and 10 the issuers (8 also owns the TMEM), 9 the
+// producer.  XS: warp 8 issues S and W of whole J tiles, warp 10 the feature sums;
+// else warp 8 all products of warpgroup 0 and warp 10 those of warpgroup 1.  TMEM (512
+// columns):
+//   S [0, 128), W [128, 256) (half b at + 64 b), Qh_b [256 + 64 b, +32), Ql_b [+32, +32),
 //   XA [384, 384 + KX/2) unless XS, ACC_b [512 - 2 NACC + b NACC, +NACC).
 // Shared memory: the item's GI tile, the item's XA tile when XS (large d), and
 // the stages [XB | VJ | BG] of the J tiles.
@@ -170,15 +185,15 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
   uint64_t* empty = full + S;        // both issuers done with the stage (2 commits)
   uint64_t* a_ready = empty + S;     // XA of the item stored in TMEM (128 arrivals of warpgroup 0)
   uint64_t* seg = a_ready + 1;       // both warpgroups finished the previous item (256)
-  uint64_t* sw_full = seg + 1;       // S, W of the tile written
-  uint64_t* s_free = sw_full + 1;    // S, W loaded into registers (256: both warpgroups)
-  uint64_t* q_ready = s_free + 1;    // [b] Q_b written
+  uint64_t* sw_full = seg + 1;       // [b] S_b, W_b written (XS: [0], both)
+  uint64_t* s_free = sw_full + 2;    // [b] S_b, W_b loaded into registers (XS: [0], by both warpgroups)
+  uint64_t* q_ready = s_free + 2;    // [b] Q_b written
   uint64_t* q_free = q_ready + 2;    // [b] the feature sums of Q_b done
   uint64_t* done = q_free + 2;       // [issuer]
   uint64_t* xa_full = done + 2;      // XS: XA tile landed
   uint64_t* xa_empty = xa_full + 1;  // XS: the S products are done with it
   uint64_t* gi_full = xa_empty + 1;  // GI tile landed
-  uint64_t* gi_empty = gi_full + 1;  // the W products are done with it
+  uint64_t* gi_empty = gi_full + 1;  // the W products are done with it (a commit per issuer of W)
   uint32_t* tslot = reinterpret_cast<uint32_t*>(gi_empty + 1);
   volatile int* abort = reinterpret_cast<volatile int*>(tslot + 1);
 
@@ -190,9 +205,9 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
     }
     mbar_init(a_ready, 128);
     mbar_init(seg, 256);
-    mbar_init(sw_full, 1);
-    mbar_init(s_free, 256);
     for (int b = 0; b < 2; ++b) {
+      mbar_init(&sw_full[b], 1);
+      mbar_init(&s_free[b], XS ? 256 : 128);
       mbar_init(&q_ready[b], 128);
       mbar_init(&q_free[b], 1);
       mbar_init(&done[b], 1);
@@ -200,7 +215,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
     mbar_init(xa_full, 1);
     mbar_init(xa_empty, 1);
     mbar_init(gi_full, 1);
-    mbar_init(gi_empty, 1);
+    mbar_init(gi_empty, XS ? 1 : 2);
     *abort = 0;
     fence_barrier_init();
   }
@@ -266,7 +281,84 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
         mbar_drain(gi_full, (uint32_t)(n_items_done - 1) & 1u, 500000000ull);
       }
     }
-  } else if (warp == kMmaWarp) {
+  } else if (!XS && (warp == kMmaWarp || warp == kBwdIssue1Warp)) {
+    // ------------------------------------------------------------ issuer of warpgroup b
+    // Per own half k of the item: S(k), W(k) once the warpgroup has read
+    // S(k-1), W(k-1); then the feature sums of Q(k-1) once it is written.
+    const bool leader = elect_one();
+    const int b = warp == kMmaWarp ? 0 : 1;
+    const uint32_t idSW = idesc_f16(128, 64, 0, 0);
+    const uint32_t idA = idesc_f16(128, a.NACC, 0, 0);
+    const int nkx = a.KX / 16, nkg = a.KG / 16;
+    const uint64_t dGI = sdesc(smem_u32(sGI), 128, a.KG * 16u);
+    const uint64_t dXB = sdesc(smem_u32(sS + b * a.KX * 128u), 128, a.KX * 16u);
+    const uint64_t dVJ = sdesc(smem_u32(sS + XT + b * a.KG * 128u), 128, a.KG * 16u);
+    const uint64_t dBG = sdesc(smem_u32(sS + XT + GT + b * 1024u), 128, 2048);
+    const uint32_t lo_bytes = (uint32_t)a.NACC * 256u;   // ksplit: the lo block of BG
+    const uint32_t tS = tbase + 64 * b, tW = tS + 128, tA = tbase + kColXA;
+    const uint32_t tQh = tbase + 256 + 64 * b, tQl = tQh + 32;
+    const uint32_t tACC = tbase + 512 - 2 * a.NACC + b * a.NACC;
+    int it = 0;
+    long long uses = 0, qr = 0;
+    uint32_t stage = 0, sph = 0;
+    // the feature sums of own half jj (stored in Q_b), from stage st_
+    auto issue_acc = [&](uint32_t st_, int jj) -> bool {
+      if (!warp_wait(&q_ready[b], (uint32_t)(qr & 1), abort, a.err, 26)) return false;
+      ++qr;
+      tc_fence_after();
+      const uint32_t acc = (jj % kFoldOwn) != 0;
+      const uint64_t dbg = sdesc_add(dBG, st_ * STG);
+      if (leader) {
+        issue_ts4(tACC, tQh, dbg, idA, acc);
+        if (a.ksplit) issue_ts4(tACC, tQh, sdesc_add(dbg, lo_bytes), idA, 1);
+        issue_ts4(tACC, tQl, dbg, idA, 1);
+        tc_commit(&q_free[b]);
+        tc_commit(&empty[st_]);
+      }
+      __syncwarp();
+      return true;
+    };
+    for (int t = blockIdx.x; t < a.n_items; t += gridDim.x) {
+      const int4 item = a.items[t];
+      if (a.sys_active && !a.sys_active[item.x]) continue;
+      const uint32_t ip = (uint32_t)(it & 1);
+      if (!warp_wait(a_ready, ip, abort, a.err, 31)) goto own_out;
+      if (!warp_wait(gi_full, ip, abort, a.err, 36)) goto own_out;
+      ++it;
+      uint32_t prev_stage = 0;
+      for (int j = 0; j < item.w; ++j) {
+        if (uses > 0 && !warp_wait(&s_free[b], (uint32_t)((uses - 1) & 1), abort, a.err, 23)) goto own_out;
+        if (!warp_wait(&full[stage], sph, abort, a.err, 25)) goto own_out;
+        tc_fence_after();
+        // operands computed by the whole warp (warp-uniform), issued by the leader
+        const uint64_t db = sdesc_add(dXB, stage * STG);
+        const uint64_t dv = sdesc_add(dVJ, stage * STG);
+        if (leader) {
+#pragma unroll
+          for (int q = 0; q < kMaxKX / 16; ++q) {
+            if (q < nkx) {
+              mma_ts(tS, tA + 8 * q, db + 16 * q, idSW, q > 0);
+            }
+          }
+#pragma unroll 4
+          for (int q = 0; q < nkg; ++q) mma_ss(tW, dGI + 16 * q, dv + 16 * q, idSW, q > 0);
+          tc_commit(&sw_full[b]);
+          // the item's GI tile is released after its last W products
+          if (j == item.w - 1) tc_commit(gi_empty);
+        }
+        __syncwarp();
+        ++uses;
+        if (j > 0 && !issue_acc(prev_stage, j - 1)) goto own_out;
+        prev_stage = stage;
+        if (++stage == (uint32_t)S) { stage = 0; sph ^= 1; }
+      }
+      if (item.w > 0 && !issue_acc(prev_stage, item.w - 1)) goto own_out;
+    }
+  own_out:
+    if (leader) tc_commit(&done[b]);
+    __syncwarp();
+    mbar_drain(&done[b], 0, 500000000ull);
+  } else if (XS && warp == kMmaWarp) {
     // ------------------------------------------------------------ issuer of S and W
     // Per J tile: S and W of its 128 columns (both halves at once) when both warpgroups
     // have read the previous tile's.
@@ -277,7 +369,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
     const uint64_t dGI = sdesc(smem_u32(sGI), 128, a.KG * 16u);
     const uint64_t dXB = sdesc(smem_u32(sS), 128, a.KX * 16u);
     const uint64_t dVJ = sdesc(smem_u32(sS + XT), 128, a.KG * 16u);
-    const uint32_t tS = tbase, tW = tbase + 128, tA = tbase + kColXA;
+    const uint32_t tS = tbase, tW = tbase + 128;
     int it = 0;
     long long uses = 0;
     uint32_t stage = 0, sph = 0;
@@ -285,7 +377,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
       const int4 item = a.items[t];
       if (a.sys_active && !a.sys_active[item.x]) continue;
       const uint32_t ip = (uint32_t)(it & 1);
-      if (!warp_wait(XS ? xa_full : a_ready, ip, abort, a.err, XS ? 34 : 31)) goto sw_out;
+      if (!warp_wait(xa_full, ip, abort, a.err, 34)) goto sw_out;
       if (!warp_wait(gi_full, ip, abort, a.err, 36)) goto sw_out;
       ++it;
       for (int j = 0; j < item.w; ++j) {
@@ -299,10 +391,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
 #pragma unroll
           for (int q = 0; q < kMaxKX / 16; ++q) {
             if (q < nkx) {
-              if (XS)
-                mma_ss(tS, dXA + 16 * q, db + 16 * q, idSW, q > 0);
-              else
-                mma_ts(tS, tA + 8 * q, db + 16 * q, idSW, q > 0);
+              mma_ss(tS, dXA + 16 * q, db + 16 * q, idSW, q > 0);
             }
           }
 #pragma unroll 4
@@ -312,7 +401,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
           // the item's XA and GI tiles are released after its last S, W products
           if (j == item.w - 1) {
             tc_commit(gi_empty);
-            if (XS) tc_commit(xa_empty);
+            tc_commit(xa_empty);
           }
         }
         __syncwarp();
@@ -324,7 +413,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
     if (leader) tc_commit(&done[0]);
     __syncwarp();
     mbar_drain(&done[0], 0, 500000000ull);
-  } else if (warp == kBwdIssue1Warp) {
+  } else if (XS && warp == kBwdIssue1Warp) {
     // ------------------------------------------------------------ issuer of the feature sums
     // Per J tile the sums of Q_0, then of Q_1, once each is written.
     const bool leader = elect_one();
@@ -496,7 +585,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
         }
       };
       for (int j = 0; j < item.w; ++j, ++uses) {
-        bool ok = mbar_wait(sw_full, (uint32_t)(uses & 1), abort, a.err, 28);
+        bool ok = mbar_wait(&sw_full[XS ? 0 : b], (uint32_t)(uses & 1), abort, a.err, 28);
         if (!__all_sync(0xffffffffu, ok)) goto exp_out;
         tc_fence_after();
         {
@@ -509,7 +598,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
           tmem_ld32(tW + 32, w1);
           tmem_ld_wait_regs(s0, s1, w0, w1);
           tc_fence_before();
-          mbar_arrive(s_free);
+          mbar_arrive(&s_free[XS ? 0 : b]);
           if (item.z + j == item.y) {
             // diagonal tile of the upper triangle: counted once, off-diagonal
             // tiles twice; the pair i = j is left out (its distance is 0, and its
@@ -525,19 +614,8 @@ __global__ void __launch_bounds__(kTsThreads, 1) tc_bwd_ts_kernel(TcBwdArgs a) {
           uint32_t qh[32];
 #pragma unroll
           for (int q = 0; q < 16; ++q) {
-            float h0, l0, h1, l1;
-            split_q(ex2(__uint_as_float(s0[2 * q])) * __uint_as_float(w0[2 * q]), h0, l0);
-            split_q(ex2(__uint_as_float(s0[2 * q + 1])) * __uint_as_float(w0[2 * q + 1]), h1, l1);
-            qh[q] = pack_f16x2(h0, h1);
-            qq[q] = pack_f16x2(l0, l1);
-          }
-#pragma unroll
-          for (int q = 0; q < 16; ++q) {
-            float h0, l0, h1, l1;
-            split_q(ex2(__uint_as_float(s1[2 * q])) * __uint_as_float(w1[2 * q]), h0, l0);
-            split_q(ex2(__uint_as_float(s1[2 * q + 1])) * __uint_as_float(w1[2 * q + 1]), h1, l1);
-            qh[16 + q] = pack_f16x2(h0, h1);
-            qq[16 + q] = pack_f16x2(l0, l1);
+            split_q2(s0[2 * q], s0[2 * q + 1], w0[2 * q], w0[2 * q + 1], qh[q], qq[q]);
+            split_q2(s1[2 * q], s1[2 * q + 1], w1[2 * q], w1[2 * q + 1], qh[16 + q], qq[16 + q]);
           }
           if (j > 0) {
             // the feature sums of Q(j-1) are done: Q_b may be overwritten, and
