@@ -14,16 +14,13 @@
 //
 // Main kernel (one CTA per SM, persistent over work items): an item is one
 // pair of 128-row I tiles of one system against a contiguous range of J tiles.
-//   warp 9       : bulk-copy producer (A tiles per item, XB/VT tiles per J step)
-//   warps 8, 10  : one MMA issuer per I tile g: S_g = A_g XB^T into TMEM (a
-//                  128x128 FP32 accumulator), then O_g += P_g VT^T with P_g
-//                  read from TMEM.  Two issuers let the two tiles' thin P.V
-//                  MMAs overlap in the tensor pipe and keep the warpgroups
-//                  independent of each other.
-//   warps 0-7    : two exp warpgroups, one per I tile: TMEM S -> ex2 -> F16 P
-//                  written to its own TMEM columns (the second half tile's
-//                  TMEM loads overlap the first half's exps), and every kFold
-//                  J tiles the FP32 O accumulator is folded into per-column
+//   warp 17      : bulk-copy producer (A tiles per item, XB/VT tiles per J step)
+//   warps 16, 18, 19 : MMA issuers: S_g = A_g XB^T of both I tiles g into TMEM
+//                  (128x128 FP32 accumulators), and per I tile O_g += P_g VT^T
+//                  with P_g read from TMEM.
+//   warps 0-15   : four exp warpgroups, two per I tile on the halves of S: TMEM
+//                  S -> ex2 -> F16 P written to its own TMEM columns, and every
+//                  kFold J tiles the FP32 O accumulator is folded into per-column
 //                  FP32 pair sums (TwoSum), written in FP64 once per item.
 // An epilogue kernel sums the per-item partials in a fixed order and applies
 // Y = alpha O + (sigma^2 + shift) V.
@@ -47,13 +44,15 @@ namespace {
 // J tiles accumulated in FP32 in TMEM before each fold (4096 columns) into
 // the per-column TwoSum pairs.
 constexpr int kFold = 32;
-// Forward warp roles: warps 0-7 two exp warpgroups, warp 8 MMA issuer for I
-// tile 0 (and TMEM owner), warp 9 producer, warp 10 MMA issuer for I tile 1.
-constexpr int kFwdThreads = 352;
-constexpr int kIssue1Warp = 10;
-// FMA-pipe forward warp roles: warps 0-15 four exp warpgroups (I tile
-// (w >> 2) & 1, S columns 64 (w >> 3) .. + 63), warp 16 MMA issuer for I
-// tile 0 (and TMEM owner), warp 17 producer, warp 18 MMA issuer for I tile 1.
+// Warp roles of both forward kernels: warps 0-15 four exp warpgroups (I tile
+// (w >> 2) & 1, S columns 64 (w >> 3) .. + 63), warp 17 producer.
+// Forward: warp 16 issuer of S (and TMEM owner), warps 18, 19 issuers of P.V of I
+// tiles 0, 1.  One issuer per I tile for both was busy 72% of the time at d = 8, m = 16
+// (10 MMAs per tile, 50 to 140 clocks to issue one) and set the kernel's pace.
+constexpr int kFwdThreads = 640;
+constexpr int kFwdSWarp = 16, kFwdLoadWarp = 17, kFwdPvWarp = 18;
+// FMA-pipe forward: warp 16 MMA issuer for I tile 0 (and TMEM owner), warp 18 for I
+// tile 1.
 constexpr int kFmaThreads = 608;
 constexpr int kFmaMmaWarp = 16, kFmaLoadWarp = 17, kFmaIssue1Warp = 18;
 
@@ -99,12 +98,17 @@ struct TcFwdArgs {
   int* err;
 };
 
-// RM > 0: the fold sums of up to RM columns (FP32 pairs) live in registers; RM == 0:
-// they live as pairs in the place of the per-item FP64 partials (global
-// read-modify-write by the row's own thread), converted after the item's last fold.
-// As FP64 sums they cost 64 conversions and adds per row and fold at m = 64, on a pipe
-// of 2 lanes per clock: 14% of the kernel.
-template <int RM, int POLY>
+// The fold sums of O (FP32 pairs, TwoSum): SP (up to 16 columns) in shared memory,
+// else in the place of the per-item FP64 partials (global read-modify-write by the
+// row's own thread), converted after the item's last fold.
+//
+// Bound by the exp warps: one ex2 per pair at 32 per clock and SM, with a pack, the
+// TMEM load and the TMEM store around it.  With two warps per scheduler the latencies
+// between them left XU at 58% (0.82 ms at N = 65,536, d = 8, m = 16, ROOF 0.43 ms); four
+// warps per scheduler, two per I tile on the column halves of S, each take their 64
+// columns in one load (S is free for the next tile before the exps), pack in place and
+// store P once, late enough that the previous P.V is done with the buffer.
+template <bool SP, int POLY>
 __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
   using namespace ptx;
   extern __shared__ uint8_t smem_raw[];
@@ -124,31 +128,33 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
   uint64_t* p_free = p_ready + 2;    // [g] P_g consumed by the P.V MMAs
   uint64_t* o_ready = p_free + 2;
   uint64_t* o_free = o_ready + 2;
-  uint64_t* done = o_free + 2;       // [g]
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 2);
+  uint64_t* done = o_free + 2;       // [issuer]
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 3);
   volatile int* abort = reinterpret_cast<volatile int*>(tslot + 1);
+  float2* s_pair = reinterpret_cast<float2*>(tslot + 2);   // SP: [column of the half][exp thread]
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int i = 0; i < S; ++i) {
       mbar_init(&full[i], 1);
-      mbar_init(&empty[i], 2);
+      mbar_init(&empty[i], 3);   // S, and P.V of each I tile, done with the stage
     }
     for (int g = 0; g < 2; ++g) {
       mbar_init(&a_full[g], 1);
-      mbar_init(&a_empty[g], 2);
+      mbar_init(&a_empty[g], 1);
       mbar_init(&s_full[g], 1);
-      mbar_init(&s_free[g], 128);
-      mbar_init(&p_ready[g], 128);
+      mbar_init(&s_free[g], 256);
+      mbar_init(&p_ready[g], 256);
       mbar_init(&p_free[g], 1);
       mbar_init(&o_ready[g], 1);
-      mbar_init(&o_free[g], 128);
+      mbar_init(&o_free[g], 256);
       mbar_init(&done[g], 1);
     }
+    mbar_init(&done[2], 1);
     *abort = 0;
     fence_barrier_init();
   }
-  if (warp == kMmaWarp) {
+  if (warp == kFwdSWarp) {
     tmem_alloc(tslot, 512);
     tmem_relinquish();
   }
@@ -162,7 +168,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
   // addresses and descriptors stay warp-uniform, and one elected lane issues
   // the copies, MMAs and commits: issuing from a lone lane was measured at
   // 2-3x the cost per tcgen05.mma.
-  if (warp == kLoadWarp) {
+  if (warp == kFwdLoadWarp) {
     const bool leader = elect_one();
     {
       // ------------------------------------------------------------ producer
@@ -209,127 +215,108 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
         }
       }
     }
-  } else if (warp == kMmaWarp || warp == kIssue1Warp) {
+  } else if (warp == kFwdSWarp) {
+    // ------------------------------------------------------------ issuer of S
+    // Tile stream k = 0, 1, ... over this CTA's items: S_g(k) of each I tile once its
+    // warpgroups have read S_g(k-1).
     const bool leader = elect_one();
-    {
-      // ------------------------------------------------------------ MMA issuer of I tile g
-      // Tile stream k = 0, 1, ... over this CTA's items.  For tile k it issues
-      // S(k) once warpgroup g has read S(k-1), then P.V of tile k-1 once P(k-1)
-      // is written, so the tensor core computes the next S while the
-      // warpgroup computes exps, and P.V runs during the next tile's exps.
-      const int g = warp == kMmaWarp ? 0 : 1;
-      const uint32_t idS = idesc_f16(128, 128, 1, 1);
-      const uint32_t idP = idesc_f16(128, a.MP, 0, 0);
-      const uint32_t sboX = a.KX * 16u;
-      const int nkx = a.KX / 16;
-      const uint64_t dA = sdesc(smem_u32(sA + g * A_TILE), 128, sboX);
-      const uint64_t dB = sdesc(smem_u32(sB), 128, sboX);
-      const uint64_t dV = sdesc(smem_u32(sV), 128, 2048);
-      const uint32_t s_tmem = tbase + g * 128, p_tmem = tbase + 256 + g * 64, o_tmem = tbase + 384 + g * 64;
-      int it = 0;
-      uint32_t stage = 0, sph = 0;
-      uint32_t sf_ph = 0, pr_ph = 0, of_ph = 0;
-      bool opend = false;
-      long long k = 0;
-      // the previous tile, whose P.V is still to be issued
-      bool have_prev = false;
-      uint32_t prev_stage = 0;
-      int prev_j = 0, prev_nJ = 0, prev_ab = 0;
-      for (int t = blockIdx.x; t < a.n_items; t += gridDim.x) {
-        const int4 item = a.items[t];
-        if (a.sys_active && !a.sys_active[item.x]) continue;
-        const int ab = it & 1;
-        const uint64_t dAg = sdesc_add(dA, 2 * ab * A_TILE);
-        for (int j = 0; j < item.w; ++j, ++k) {
-          // ---- S(k)
-          if (k > 0) {
-            if (!warp_wait(&s_free[g], sf_ph, abort, a.err, 3)) goto mma_out;
-            sf_ph ^= 1;
-          }
-          if (j == 0 && !warp_wait(&a_full[ab], (it >> 1) & 1, abort, a.err, 4)) goto mma_out;
-          if (!warp_wait(&full[stage], sph, abort, a.err, 5)) goto mma_out;
+    const uint32_t idS = idesc_f16(128, 128, 1, 1);
+    const uint32_t sboX = a.KX * 16u;
+    const int nkx = a.KX / 16;
+    const uint64_t dA = sdesc(smem_u32(sA), 128, sboX);
+    const uint64_t dB = sdesc(smem_u32(sB), 128, sboX);
+    int it = 0;
+    uint32_t stage = 0, sph = 0, sf_ph = 0;
+    bool begun = false;
+    for (int t = blockIdx.x; t < a.n_items; t += gridDim.x) {
+      const int4 item = a.items[t];
+      if (a.sys_active && !a.sys_active[item.x]) continue;
+      const int ab = it & 1;
+      const uint64_t dAt = sdesc_add(dA, 2 * ab * A_TILE);
+      if (!warp_wait(&a_full[ab], (it >> 1) & 1, abort, a.err, 4)) goto s_out;
+      for (int j = 0; j < item.w; ++j) {
+        if (!warp_wait(&full[stage], sph, abort, a.err, 5)) goto s_out;
+        // operands computed by the whole warp (warp-uniform), issued by the leader
+        const uint64_t db = sdesc_add(dB, stage * A_TILE);
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          if (begun && !warp_wait(&s_free[g], sf_ph, abort, a.err, 3)) goto s_out;
           tc_fence_after();
-          // operands computed by the whole warp (warp-uniform), issued by the leader
-          const uint64_t db = sdesc_add(dB, stage * A_TILE);
+          const uint64_t da = sdesc_add(dAt, g * A_TILE);
           if (leader) {
-            issue_s(s_tmem, dAg, db, nkx, idS);
+            issue_s(tbase + g * 128, da, db, nkx, idS);
             tc_commit(&s_full[g]);
+            if (g == 1) {
+              tc_commit(&empty[stage]);
+              if (j == item.w - 1) tc_commit(&a_empty[ab]);
+            }
           }
           __syncwarp();
-          // ---- P.V of tile k-1
-          if (have_prev) {
-            if (!warp_wait(&p_ready[g], pr_ph, abort, a.err, 6)) goto mma_out;
-            pr_ph ^= 1;
-            tc_fence_after();
-            const uint32_t acc = (prev_j % kFold) != 0;
-            if (!acc && opend) {
-              if (!warp_wait(&o_free[g], of_ph, abort, a.err, 7)) goto mma_out;
-              of_ph ^= 1;
-              opend = false;
-              tc_fence_after();
-            }
-            const bool fold_end = (prev_j % kFold) == kFold - 1 || prev_j == prev_nJ - 1;
-            const uint64_t dv = sdesc_add(dV, prev_stage * V_TILE);
-            if (leader) {
-              issue_pv(o_tmem, p_tmem, dv, idP, acc);
-              tc_commit(&p_free[g]);
-              if (fold_end) tc_commit(&o_ready[g]);
-              tc_commit(&empty[prev_stage]);
-              if (prev_j == prev_nJ - 1) tc_commit(&a_empty[prev_ab]);
-            }
-            __syncwarp();
-            if (fold_end) opend = true;
-          }
-          have_prev = true;
-          prev_stage = stage;
-          prev_j = j;
-          prev_nJ = item.w;
-          prev_ab = ab;
-          if (++stage == (uint32_t)S) { stage = 0; sph ^= 1; }
         }
-        ++it;
+        if (begun) sf_ph ^= 1;
+        begun = true;
+        if (++stage == (uint32_t)S) { stage = 0; sph ^= 1; }
       }
-      if (have_prev) {
-        if (!warp_wait(&p_ready[g], pr_ph, abort, a.err, 6)) goto mma_out;
-        tc_fence_after();
-        const uint32_t acc = (prev_j % kFold) != 0;
+      ++it;
+    }
+  s_out:
+    if (leader) tc_commit(&done[2]);
+    __syncwarp();
+    mbar_drain(&done[2], 0, 500000000ull);
+  } else if (warp >= kFwdPvWarp) {
+    // ------------------------------------------------------------ issuer of P.V of I tile g
+    const bool leader = elect_one();
+    const int g = warp - kFwdPvWarp;
+    const uint32_t idP = idesc_f16(128, a.MP, 0, 0);
+    const uint64_t dV = sdesc(smem_u32(sV), 128, 2048);
+    const uint32_t p_tmem = tbase + 256 + g * 64, o_tmem = tbase + 384 + g * 64;
+    uint32_t stage = 0, sph = 0, pr_ph = 0, of_ph = 0;
+    bool opend = false;   // O was handed to the warpgroups and not yet taken back
+    for (int t = blockIdx.x; t < a.n_items; t += gridDim.x) {
+      const int4 item = a.items[t];
+      if (a.sys_active && !a.sys_active[item.x]) continue;
+      for (int j = 0; j < item.w; ++j) {
+        if (!warp_wait(&full[stage], sph, abort, a.err, 5)) goto pv_out;
+        if (!warp_wait(&p_ready[g], pr_ph, abort, a.err, 6)) goto pv_out;
+        pr_ph ^= 1;
+        const uint32_t acc = (j % kFold) != 0;
         if (!acc && opend) {
-          if (!warp_wait(&o_free[g], of_ph, abort, a.err, 7)) goto mma_out;
-          tc_fence_after();
+          if (!warp_wait(&o_free[g], of_ph, abort, a.err, 7)) goto pv_out;
+          of_ph ^= 1;
+          opend = false;
         }
-        const uint64_t dv = sdesc_add(dV, prev_stage * V_TILE);
+        tc_fence_after();
+        const bool fold_end = (j % kFold) == kFold - 1 || j == item.w - 1;
+        const uint64_t dv = sdesc_add(dV, stage * V_TILE);
         if (leader) {
           issue_pv(o_tmem, p_tmem, dv, idP, acc);
           tc_commit(&p_free[g]);
-          tc_commit(&o_ready[g]);
-          tc_commit(&empty[prev_stage]);
-          tc_commit(&a_empty[prev_ab]);
+          if (fold_end) tc_commit(&o_ready[g]);
+          tc_commit(&empty[stage]);
         }
         __syncwarp();
+        if (fold_end) opend = true;
+        if (++stage == (uint32_t)S) { stage = 0; sph ^= 1; }
       }
-    mma_out:
-      if (leader) tc_commit(&done[g]);
-      __syncwarp();
-      mbar_drain(&done[g], 0, 500000000ull);
     }
+  pv_out:
+    if (leader) tc_commit(&done[g]);
     __syncwarp();
+    mbar_drain(&done[g], 0, 500000000ull);
   } else {
     // ------------------------------------------------------------ exp warpgroups
-    const int g = warp >> 2, w = warp & 3;
+    const int g = (warp >> 2) & 1, w = warp & 3, hf = warp >> 3;
     const int row = 32 * w + lane;
     const uint32_t tl = tbase + (static_cast<uint32_t>(32 * w) << 16);
-    const uint32_t s_col = g * 128, p_col = 256 + g * 64, o_col = 384 + g * 64;
+    const uint32_t s_col = g * 128 + 64 * hf, p_col = 256 + g * 64 + 32 * hf, o_col = 384 + g * 64;
+    // this half's columns of O: [oc0, oc1)
+    const int oc0 = hf * (a.MP / 2), oc1 = oc0 + a.MP / 2;
+    const int rowp = g * 128 + row;
     uint32_t sph = 0, pf_ph = 0, oph = 0;
     long long k = 0;
     for (int t = blockIdx.x; t < a.n_items; t += gridDim.x) {
       const int4 item = a.items[t];
       if (a.sys_active && !a.sys_active[item.x]) continue;
-      const int rowp = g * 128 + row;
-      // the item's O sums per column as FP32 pairs (TwoSum; the FP64 pipe is a
-      // small fraction of the FP32 rate on this GPU), written in FP64
-      float rs[RM > 0 ? RM : 1], rc[RM > 0 ? RM : 1];
-#pragma unroll
-      for (int q = 0; q < (RM > 0 ? RM : 1); ++q) rs[q] = rc[q] = 0.f;
       bool first = true;
       for (int j = 0; j < item.w; ++j, ++k) {
         bool ok = mbar_wait(&s_full[g], sph, abort, a.err, 8);
@@ -337,32 +324,22 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
         sph ^= 1;
         tc_fence_after();
         {
-          uint32_t a0[32], a1[32], b0[32], b1[32], pk[32];
+          uint32_t a0[32], a1[32], pk[32];
           tmem_ld32(tl + s_col, a0);
           tmem_ld32(tl + s_col + 32, a1);
-          if (RM > 0) tmem_ld_wait_regs(a0, a1);
-          tmem_ld32(tl + s_col + 64, b0);
-          tmem_ld32(tl + s_col + 96, b1);
-          if (RM == 0) {
-            // many columns or dimensions: the next S takes the tensor core long enough
-            // to be worth starting before the exps
-            tmem_ld_wait_regs(a0, a1, b0, b1);
-            tc_fence_before();
-            mbar_arrive(&s_free[g]);
-          }
+          tmem_ld_wait_regs(a0, a1);
+          // this half of S(k) is in registers: once both are, the tensor core may overwrite it
+          tc_fence_before();
+          mbar_arrive(&s_free[g]);
 #pragma unroll
-          for (int q = 0; q < 16; ++q)
+          for (int q = 0; q < 16; ++q) {
             pk[q] = pack_f16x2(exp2_mix<POLY, 3>(__uint_as_float(a0[2 * q]), 2 * q),
                                exp2_mix<POLY, 3>(__uint_as_float(a0[2 * q + 1]), 2 * q + 1));
+          }
 #pragma unroll
-          for (int q = 0; q < 16; ++q)
+          for (int q = 0; q < 16; ++q) {
             pk[16 + q] = pack_f16x2(exp2_mix<POLY, 3>(__uint_as_float(a1[2 * q]), 2 * q),
-                               exp2_mix<POLY, 3>(__uint_as_float(a1[2 * q + 1]), 2 * q + 1));
-          if (RM > 0) {
-            tmem_ld_wait_regs(b0, b1);
-            // S(k) is fully in registers: the tensor core may overwrite it
-            tc_fence_before();
-            mbar_arrive(&s_free[g]);
+                                    exp2_mix<POLY, 3>(__uint_as_float(a1[2 * q + 1]), 2 * q + 1));
           }
           if (k > 0) {
             // P(k-1) must have been consumed before P(k) overwrites it
@@ -372,57 +349,33 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
             tc_fence_after();
           }
           tmem_st32(tl + p_col, pk);
-          // the second half's exps in place; pk, the source of the store just
-          // issued, is rewritten only after tcgen05.wait::st
-#pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            b0[e] = __float_as_uint(exp2_mix<POLY, 3>(__uint_as_float(b0[e]), e));
-            b1[e] = __float_as_uint(exp2_mix<POLY, 3>(__uint_as_float(b1[e]), e));
-          }
+          // the store has read its registers before the next tile's load fills them
           tmem_st_wait();
-#pragma unroll
-          for (int q = 0; q < 16; ++q) {
-            pk[q] = pack_f16x2(__uint_as_float(b0[2 * q]), __uint_as_float(b0[2 * q + 1]));
-            pk[16 + q] = pack_f16x2(__uint_as_float(b1[2 * q]), __uint_as_float(b1[2 * q + 1]));
-          }
-          tmem_st32(tl + p_col + 32, pk);
         }
-        tmem_st_wait();
         tc_fence_before();
         mbar_arrive(&p_ready[g]);
         if ((j % kFold) == kFold - 1 || j == item.w - 1) {
+          const bool last = j == item.w - 1;
           ok = mbar_wait(&o_ready[g], oph, abort, a.err, 9);
           if (!__all_sync(0xffffffffu, ok)) goto exp_out;
           oph ^= 1;
           tc_fence_after();
-          if (RM > 0) {
+          for (int c0 = oc0; c0 < oc1; c0 += 8) {
+            uint32_t o[8];
+            tmem_ld8(tl + o_col + c0, o);
+            tmem_ld_wait_regs(o);
 #pragma unroll
-            for (int c0 = 0; c0 < (RM > 0 ? RM : 16); c0 += 16) {
-              if (c0 < a.MP) {
-                uint32_t o[16];
-                tmem_ld16(tl + o_col + c0, o);
-                tmem_ld_wait_regs(o);
-#pragma unroll
-                for (int q = 0; q < 16; ++q) two_sum_add(rs[c0 + q], rc[c0 + q], __uint_as_float(o[q]));
-              }
-            }
-          } else {
-            for (int c0 = 0; c0 < a.MP; c0 += 16) {
-              uint32_t o[16];
-              tmem_ld16(tl + o_col + c0, o);
-              tmem_ld_wait_regs(o);
-#pragma unroll
-              for (int q = 0; q < 16; ++q) {
-                const int col = c0 + q;
-                if (col < a.mz) {
-                  float2* pv = reinterpret_cast<float2*>(&a.part[part_idx(t, a.mz, col, rowp)]);
-                  float2 v = first ? make_float2(0.f, 0.f) : *pv;
-                  two_sum_add(v.x, v.y, __uint_as_float(o[q]));
-                  if (j == item.w - 1)
-                    a.part[part_idx(t, a.mz, col, rowp)] = (double)v.x + (double)v.y;
-                  else
-                    *pv = v;
-                }
+            for (int q = 0; q < 8; ++q) {
+              const int col = c0 + q;
+              if (col < a.mz) {
+                float2* pv = SP ? &s_pair[q * 512 + (int)threadIdx.x]
+                                : reinterpret_cast<float2*>(&a.part[part_idx(t, a.mz, col, rowp)]);
+                float2 v = first ? make_float2(0.f, 0.f) : *pv;
+                two_sum_add(v.x, v.y, __uint_as_float(o[q]));
+                if (last)
+                  a.part[part_idx(t, a.mz, col, rowp)] = (double)v.x + (double)v.y;
+                else
+                  *pv = v;
               }
             }
           }
@@ -431,11 +384,6 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
           mbar_arrive(&o_free[g]);
         }
       }
-      if (RM > 0) {
-#pragma unroll
-        for (int q = 0; q < (RM > 0 ? RM : 1); ++q)
-          if (q < a.mz) a.part[part_idx(t, a.mz, q, rowp)] = (double)rs[q] + (double)rc[q];
-      }
     }
   exp_out:;
   }
@@ -443,7 +391,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == kMmaWarp) tmem_dealloc(tbase, 512);
+  if (warp == kFwdSWarp) tmem_dealloc(tbase, 512);
 }
 
 // Forward for one or two columns (the CG product): S = XA XB^T on the tensor
@@ -1259,7 +1207,7 @@ void tc_launch_epilogue(kmv_handle h, TcState* S, const KmvArgs& a, int c0, int 
 
 using FwdKernel = void (*)(TcFwdArgs);
 
-// The instantiation for RM (16: register fold accumulators, 0: global) or MZ
+// The instantiation for the fold sums' place (16: shared memory, 0: global) or MZ
 // (FMA path) and the exp split; exp splits other than 0, 4 and 8 take the
 // nearest built one.
 FwdKernel fwd_kernel(bool fma, int cols, int split) {
@@ -1268,8 +1216,9 @@ FwdKernel fwd_kernel(bool fma, int cols, int split) {
     if (cols == 1) return sp == 0 ? tc_fwd_fma_kernel<1, 0> : sp == 4 ? tc_fwd_fma_kernel<1, 4> : tc_fwd_fma_kernel<1, 8>;
     return sp == 0 ? tc_fwd_fma_kernel<2, 0> : sp == 4 ? tc_fwd_fma_kernel<2, 4> : tc_fwd_fma_kernel<2, 8>;
   }
-  if (cols == 16) return sp == 0 ? tc_fwd_kernel<16, 0> : sp == 4 ? tc_fwd_kernel<16, 4> : tc_fwd_kernel<16, 8>;
-  return sp == 0 ? tc_fwd_kernel<0, 0> : sp == 4 ? tc_fwd_kernel<0, 4> : tc_fwd_kernel<0, 8>;
+  if (cols == 16)
+    return sp == 0 ? tc_fwd_kernel<true, 0> : sp == 4 ? tc_fwd_kernel<true, 4> : tc_fwd_kernel<true, 8>;
+  return sp == 0 ? tc_fwd_kernel<false, 0> : sp == 4 ? tc_fwd_kernel<false, 4> : tc_fwd_kernel<false, 8>;
 }
 
 cudaError_t fwd_kernels_set_smem() {
@@ -1307,9 +1256,11 @@ kmv_status tc_forward(kmv_handle h, const KmvArgs& a, cudaStream_t st) {
   // column chunk: as wide as shared memory allows (at least two pipeline stages)
   const size_t fixed = 1024 + 4 * A_TILE + 256;
   int mz_max = std::min(a.m, kMaxMP);
+  // up to 16 columns: the fold sums' pairs, 8 columns for each of the 512 exp threads
+  auto pair_bytes = [&](int mz) { return mz <= 16 ? (size_t)8 * 512 * sizeof(float2) : (size_t)0; };
   auto stages_for = [&](int mz) {
     const size_t vt = (size_t)std::max(16, (mz + 15) / 16 * 16) * 256;
-    return (int)std::min<size_t>(max_stages, (kMaxSmem - fixed - 20 * 8) / (A_TILE + vt + 16));
+    return (int)std::min<size_t>(max_stages, (kMaxSmem - fixed - pair_bytes(mz) - 20 * 8) / (A_TILE + vt + 16));
   };
   while (stages_for(mz_max) < 2 && mz_max > 16) mz_max = std::max(16, mz_max / 2);
   if (stages_for(mz_max) < 2) return tc_fail(h, KMV_EUNSUPPORTED, "tensor-core tiles do not fit in shared memory");
@@ -1393,7 +1344,8 @@ kmv_status tc_forward(kmv_handle h, const KmvArgs& a, cudaStream_t st) {
     const int MP = std::max(16, (mz + 15) / 16 * 16);
     const size_t V_TILE = (size_t)MP * 256;
     const int stages = stages_for(mz);
-    const size_t smem = std::max(kMinSmem, fixed + stages * (A_TILE + V_TILE) + (2 * stages + 20) * 8);
+    const size_t smem =
+        std::max(kMinSmem, fixed + stages * (A_TILE + V_TILE) + (2 * stages + 20) * 8 + pair_bytes(mz));
     if (cudaMemsetAsync(vmax, 0, sizeof(uint32_t) * (size_t)n_sys * mz, st) != cudaSuccess)
       return tc_fail(h, KMV_ECUDA, "memset failed");
     tc_vmax_kernel<<<dim3(L.n_items, L.chains), kTile, 0, st>>>(h->dev, L.chains, L.n_total, a.V, a.m, c0, mz,
