@@ -46,9 +46,8 @@ namespace {
 constexpr int kFold = 32;
 // Warp roles of both forward kernels: warps 0-15 four exp warpgroups (I tile
 // (w >> 2) & 1, S columns 64 (w >> 3) .. + 63), warp 17 producer.
-// Forward: warp 16 issuer of S (and TMEM owner), warps 18, 19 issuers of P.V of I
-// tiles 0, 1.  One issuer per I tile for both was busy 72% of the time at d = 8, m = 16
-// (10 MMAs per tile, 50 to 140 clocks to issue one) and set the kernel's pace.
+// Forward: warp 16 issuer of S (and TMEM owner), warps 18, 19 issuers of P.V of I tiles
+// 0, 1.
 constexpr int kFwdThreads = 640;
 constexpr int kFwdSWarp = 16, kFwdLoadWarp = 17, kFwdPvWarp = 18;
 // FMA-pipe forward: warp 16 MMA issuer for I tile 0 (and TMEM owner), warp 18 for I
@@ -102,12 +101,17 @@ struct TcFwdArgs {
 // else in the place of the per-item FP64 partials (global read-modify-write by the
 // row's own thread), converted after the item's last fold.
 //
-// Bound by the exp warps: one ex2 per pair at 32 per clock and SM, with a pack, the
-// TMEM load and the TMEM store around it.  With two warps per scheduler the latencies
-// between them left XU at 58% (0.82 ms at N = 65,536, d = 8, m = 16, ROOF 0.43 ms); four
-// warps per scheduler, two per I tile on the column halves of S, each take their 64
-// columns in one load (S is free for the next tile before the exps), pack in place and
-// store P once, late enough that the previous P.V is done with the buffer.
+// Bound by the exp warps' chain: one ex2 per pair at 32 per clock and SM (ROOF 0.43 ms at
+// N = 65,536, d = 8, m = 16), with TMEM loads and stores, packs and barrier waits that go
+// through the same issue queue.  With two warps per scheduler (two exp warpgroups of 128
+// columns a row) it took 0.82 ms there.  Four warpgroups, two per I tile on the column
+// halves of S, an issuer for S and one per I tile for P.V: 0.80 ms.  Of a step of 1630
+// clocks (both I tiles) each warpgroup then spent 180 on its load, 755 on its exps, 325 on
+// the P buffer and the store, 370 waiting for S.  Loading the half's 64 columns in two
+// chunks, the second under the first's exps, and storing P in two, the first under the
+// second's exps: 0.75 ms and no spills.  Measured slower: one arrival per warp in place of
+// one per thread (+14%), an issuer of S per I tile (+7%), a suspend time hint at the
+// barrier waits (+3%), the second I tile started half a step late (+2% at d = 2).
 template <bool SP, int POLY>
 __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
   using namespace ptx;
@@ -324,23 +328,19 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
         sph ^= 1;
         tc_fence_after();
         {
-          uint32_t a0[32], a1[32], pk[32];
+          uint32_t a0[32], a1[32], pk[16], pk2[16];
           tmem_ld32(tl + s_col, a0);
+          tmem_ld_wait_regs(a0);
           tmem_ld32(tl + s_col + 32, a1);
-          tmem_ld_wait_regs(a0, a1);
-          // this half of S(k) is in registers: once both are, the tensor core may overwrite it
-          tc_fence_before();
-          mbar_arrive(&s_free[g]);
 #pragma unroll
           for (int q = 0; q < 16; ++q) {
             pk[q] = pack_f16x2(exp2_mix<POLY, 3>(__uint_as_float(a0[2 * q]), 2 * q),
                                exp2_mix<POLY, 3>(__uint_as_float(a0[2 * q + 1]), 2 * q + 1));
           }
-#pragma unroll
-          for (int q = 0; q < 16; ++q) {
-            pk[16 + q] = pack_f16x2(exp2_mix<POLY, 3>(__uint_as_float(a1[2 * q]), 2 * q),
-                                    exp2_mix<POLY, 3>(__uint_as_float(a1[2 * q + 1]), 2 * q + 1));
-          }
+          tmem_ld_wait_regs(a1);
+          // this half of S(k) is in registers: once both are, the tensor core may overwrite it
+          tc_fence_before();
+          mbar_arrive(&s_free[g]);
           if (k > 0) {
             // P(k-1) must have been consumed before P(k) overwrites it
             ok = mbar_wait(&p_free[g], pf_ph, abort, a.err, 10);
@@ -348,9 +348,17 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
             pf_ph ^= 1;
             tc_fence_after();
           }
-          tmem_st32(tl + p_col, pk);
-          // the store has read its registers before the next tile's load fills them
+          tmem_st16(tl + p_col, pk);
+#pragma unroll
+          for (int q = 0; q < 16; ++q) {
+            pk2[q] = pack_f16x2(exp2_mix<POLY, 3>(__uint_as_float(a1[2 * q]), 2 * q),
+                                exp2_mix<POLY, 3>(__uint_as_float(a1[2 * q + 1]), 2 * q + 1));
+          }
+          tmem_st16(tl + p_col + 16, pk2);
           tmem_st_wait();
+          // the stores' source registers are theirs until the wait has passed
+#pragma unroll
+          for (int q = 0; q < 16; ++q) asm volatile("" ::"r"(pk[q]), "r"(pk2[q]));
         }
         tc_fence_before();
         mbar_arrive(&p_ready[g]);
@@ -372,7 +380,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
                                 : reinterpret_cast<float2*>(&a.part[part_idx(t, a.mz, col, rowp)]);
                 float2 v = first ? make_float2(0.f, 0.f) : *pv;
                 two_sum_add(v.x, v.y, __uint_as_float(o[q]));
-                if (last)
+                if (SP && last)
                   a.part[part_idx(t, a.mz, col, rowp)] = (double)v.x + (double)v.y;
                 else
                   *pv = v;
@@ -382,6 +390,16 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
           first = false;
           tc_fence_before();
           mbar_arrive(&o_free[g]);
+        }
+      }
+      if (!SP) {
+        // the pairs to FP64, once per item: as a branch of the fold the conversions were
+        // predicated and issued at every fold (25% of the kernel's cycles on the FP64 pipe
+        // at m = 64; with 16 columns the branch is the faster form)
+        for (int q = oc0; q < min(oc1, a.mz); ++q) {
+          double* pd = &a.part[part_idx(t, a.mz, q, rowp)];
+          const float2 v = *reinterpret_cast<const float2*>(pd);
+          *pd = (double)v.x + (double)v.y;
         }
       }
     }
