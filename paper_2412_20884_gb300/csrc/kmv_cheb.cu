@@ -27,11 +27,10 @@ __device__ __forceinline__ void cheb_values(double x, int n, double* t) {
 
 // Basis value T_t(x_i) of flat multi-index t (row-major over d digits base n).
 __device__ __forceinline__ double basis_at(const double* tv, int d, int n, int t) {
-  double v = 1.0;
-  for (int k = d - 1; k >= 0; --k) {
-    const int dig = t % n;
+  double v = tv[(d - 1) * kMaxChebOrder + t % n];
+  for (int k = d - 2; k >= 0; --k) {
     t /= n;
-    v *= tv[k * kMaxChebOrder + dig];
+    v *= tv[k * kMaxChebOrder + t % n];
   }
   return v;
 }
@@ -70,6 +69,9 @@ __global__ void cheb_theta_kernel(int n_sys, int n_coef, int n_theta, int n_thet
 }
 
 // Per (tile, chain): partial[t] = sum_i T_t(x_i) h_i over the tile's rows.
+// Bound by the FP64 pipe (1.9 lanes per clock and SM): the warp sums eight terms at a time
+// by a reduce-scatter, 9 adds a lane where a tree per term takes 40, pairing the lanes in
+// the same order: 100 -> 57 us at N = 65,536, d = 2, N_cheb = 8, m = 16.
 __global__ void cheb_grad_kernel(DevLayout L, int chains, int64_t n_total, int d, int n_cheb, int n_coef, int m,
                                  const float* x, const float* V, const float* G, const float* KV, const float* KG,
                                  const int32_t* sys_active, double* partial) {
@@ -91,10 +93,24 @@ __global__ void cheb_grad_kernel(DevLayout L, int chains, int64_t n_total, int d
       for (int k = 0; k < d; ++k) cheb_values((double)x[i * d + k], n_cheb, tv + k * kMaxChebOrder);
   }
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  for (int t = 0; t < n_coef; ++t) {
-    double v = valid ? (n_cheb > 1 ? h * basis_at(tv, d, n_cheb, t) : h) : 0.0;
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (l == 0) red[w * n_coef + t] = v;
+  for (int t0 = 0; t0 < n_coef; t0 += 8) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      v[u] = valid && t0 + u < n_coef ? (n_cheb > 1 ? h * basis_at(tv, d, n_cheb, t0 + u) : h) : 0.0;
+#pragma unroll
+    for (int o = 16, n = 4; o >= 4; o >>= 1, n >>= 1) {
+      const bool up = l & o;
+#pragma unroll
+      for (int u = 0; u < n; ++u) {
+        const double mine = up ? v[u + n] : v[u], other = up ? v[u] : v[u + n];
+        v[u] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+      }
+    }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    const int t = t0 + (l >> 2);
+    if ((l & 3) == 0 && t < n_coef) red[w * n_coef + t] = v[0];
   }
   __syncthreads();
   double* out = partial + ((int64_t)item * chains + c) * n_coef;
@@ -106,7 +122,12 @@ __global__ void cheb_grad_kernel(DevLayout L, int chains, int64_t n_total, int d
 }
 
 // grad[s] = [sum over the instance's tiles of the Theta partials, the internal
-// lengthscale and noise gradients]; tiles summed in a fixed order.
+// lengthscale and noise gradients]; tiles summed in a fixed order: one after the other
+// up to 32 tiles, else in 32 strided sums and a tree.  A warp per (system, term): a
+// thread per term was a chain of as many dependent loads and FP64 adds as tiles
+// (125 -> 10 us at 512 tiles, 64 terms).
+constexpr int kFinWarps = 4;
+
 __global__ void cheb_grad_finalize_kernel(DevLayout L, int n_inst, int chains, int n_coef, int n_theta,
                                           int n_theta_int, const double* partial, const double* grad_int,
                                           const int32_t* sys_active, double* grad) {
@@ -115,14 +136,24 @@ __global__ void cheb_grad_finalize_kernel(DevLayout L, int n_inst, int chains, i
   if (sys_active && !sys_active[s]) return;
   const int b = s / chains, c = s - b * chains;
   double* g = grad + (int64_t)s * n_theta;
-  for (int t = threadIdx.x; t < n_coef; t += blockDim.x) {
+  const int t = blockIdx.y * kFinWarps + (threadIdx.x >> 5), l = threadIdx.x & 31;
+  if (t < n_coef) {
+    const int it0 = L.inst_item0[b], n = L.inst_item0[b + 1] - it0;
+    double v = 0.0;
+    for (int u = l; u < n; u += 32) v += partial[((int64_t)(it0 + u) * chains + c) * n_coef + t];
     double acc = 0.0;
-    for (int it = L.inst_item0[b]; it < L.inst_item0[b + 1]; ++it)
-      acc += partial[((int64_t)it * chains + c) * n_coef + t];
-    g[t] = acc;
+    if (n <= 32) {
+      for (int u = 0; u < n; ++u) acc += __shfl_sync(0xffffffffu, v, u);
+    } else {
+      acc = v;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    }
+    if (l == 0) g[t] = acc;
   }
-  for (int k = 1 + threadIdx.x; k < n_theta_int; k += blockDim.x)
-    g[n_coef + k - 1] = grad_int[(int64_t)s * n_theta_int + k];
+  if (blockIdx.y == 0)
+    for (int k = 1 + threadIdx.x; k < n_theta_int; k += blockDim.x)
+      g[n_coef + k - 1] = grad_int[(int64_t)s * n_theta_int + k];
 }
 
 }  // namespace
@@ -159,8 +190,8 @@ cudaError_t launch_cheb_grad(const DevLayout& L, int n_items, int n_inst, int ch
   }
   const int n_sys = n_inst * chains;
   if (n_sys > 0)
-    cheb_grad_finalize_kernel<<<n_sys, 128, 0, st>>>(L, n_inst, chains, n_coef, n_theta, n_theta_int, partial,
-                                                     grad_int, sys_active, grad);
+    cheb_grad_finalize_kernel<<<dim3(n_sys, (n_coef + kFinWarps - 1) / kFinWarps), 32 * kFinWarps, 0, st>>>(
+        L, n_inst, chains, n_coef, n_theta, n_theta_int, partial, grad_int, sys_active, grad);
   return cudaGetLastError();
 }
 
