@@ -48,6 +48,10 @@ constexpr int kFold = 32;
 // (w >> 2) & 1, S columns 64 (w >> 3) .. + 63), warp 17 producer.
 // Forward: warp 16 issuer of S (and TMEM owner), warps 18, 19 issuers of P.V of I tiles
 // 0, 1.
+// The two-warpgroup forward: warps 0-7 the exp warpgroups, warp 8 issuer of I tile 0 (and
+// TMEM owner), warp 9 producer, warp 10 issuer of I tile 1.
+constexpr int kFwd2Threads = 352, kFwd2Issue1Warp = 10;
+constexpr int kFwd2KX = 96;
 constexpr int kFwdThreads = 640;
 constexpr int kFwdSWarp = 16, kFwdLoadWarp = 17, kFwdPvWarp = 18;
 // FMA-pipe forward: warp 16 MMA issuer for I tile 0 (and TMEM owner), warp 18 for I
@@ -322,6 +326,46 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
       const int4 item = a.items[t];
       if (a.sys_active && !a.sys_active[item.x]) continue;
       bool first = true;
+      // The wide form's fold.  The item's last one forms the FP64 partials and stands
+      // outside the tile loop: as a branch of the loop's fold the conversions were
+      // predicated and issued at every fold (25% of the kernel's cycles on the FP64 pipe
+      // at m = 64, N = 100,000; with 16 columns the branch is the faster form).  The
+      // pairs of 8 columns are loaded together, and an item of one fold loads none and
+      // converts once per sum (three FP64 operations each took 50 us at N = 9001, d = 3,
+      // m = 40: 294 against 237 us a call).
+      auto fold_wide = [&](bool fresh, bool last) -> bool {
+        if (!__all_sync(0xffffffffu, mbar_wait(&o_ready[g], oph, abort, a.err, 9))) return false;
+        oph ^= 1;
+        tc_fence_after();
+        for (int c0 = oc0; c0 < oc1; c0 += 8) {
+          uint32_t o[8];
+          tmem_ld8(tl + o_col + c0, o);
+          float2 v[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            v[q] = make_float2(0.f, 0.f);
+            if (!fresh && c0 + q < a.mz)
+              v[q] = *reinterpret_cast<const float2*>(&a.part[part_idx(t, a.mz, c0 + q, rowp)]);
+          }
+          tmem_ld_wait_regs(o);
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            two_sum_add(v[q].x, v[q].y, __uint_as_float(o[q]));
+            if (c0 + q < a.mz) {
+              double* pd = &a.part[part_idx(t, a.mz, c0 + q, rowp)];
+              if (last && fresh)
+                *pd = (double)v[q].x;   // one value: no error term
+              else if (last)
+                *pd = (double)v[q].x + (double)v[q].y;
+              else
+                *reinterpret_cast<float2*>(pd) = v[q];
+            }
+          }
+        }
+        tc_fence_before();
+        mbar_arrive(&o_free[g]);
+        return true;
+      };
       for (int j = 0; j < item.w; ++j, ++k) {
         bool ok = mbar_wait(&s_full[g], sph, abort, a.err, 8);
         if (!__all_sync(0xffffffffu, ok)) goto exp_out;
@@ -362,7 +406,12 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
         }
         tc_fence_before();
         mbar_arrive(&p_ready[g]);
-        if ((j % kFold) == kFold - 1 || j == item.w - 1) {
+        if (!SP) {
+          if ((j % kFold) == kFold - 1 && j != item.w - 1) {
+            if (!fold_wide(first, false)) goto exp_out;
+            first = false;
+          }
+        } else if ((j % kFold) == kFold - 1 || j == item.w - 1) {
           const bool last = j == item.w - 1;
           ok = mbar_wait(&o_ready[g], oph, abort, a.err, 9);
           if (!__all_sync(0xffffffffu, ok)) goto exp_out;
@@ -376,11 +425,10 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
             for (int q = 0; q < 8; ++q) {
               const int col = c0 + q;
               if (col < a.mz) {
-                float2* pv = SP ? &s_pair[q * 512 + (int)threadIdx.x]
-                                : reinterpret_cast<float2*>(&a.part[part_idx(t, a.mz, col, rowp)]);
+                float2* pv = &s_pair[q * 512 + (int)threadIdx.x];
                 float2 v = first ? make_float2(0.f, 0.f) : *pv;
                 two_sum_add(v.x, v.y, __uint_as_float(o[q]));
-                if (SP && last)
+                if (last)
                   a.part[part_idx(t, a.mz, col, rowp)] = (double)v.x + (double)v.y;
                 else
                   *pv = v;
@@ -392,14 +440,11 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
           mbar_arrive(&o_free[g]);
         }
       }
-      if (!SP) {
-        // the pairs to FP64, once per item: as a branch of the fold the conversions were
-        // predicated and issued at every fold (25% of the kernel's cycles on the FP64 pipe
-        // at m = 64; with 16 columns the branch is the faster form)
-        for (int q = oc0; q < min(oc1, a.mz); ++q) {
-          double* pd = &a.part[part_idx(t, a.mz, q, rowp)];
-          const float2 v = *reinterpret_cast<const float2*>(pd);
-          *pd = (double)v.x + (double)v.y;
+      if (!SP && item.w > 0) {
+        if (first) {
+          if (!fold_wide(true, true)) goto exp_out;
+        } else {
+          if (!fold_wide(false, true)) goto exp_out;
         }
       }
     }
@@ -410,6 +455,315 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
   __syncthreads();
   tc_fence_after();
   if (warp == kFwdSWarp) tmem_dealloc(tbase, 512);
+}
+
+// The forward for up to 16 columns of many-dimensional points (KX >= kFwd2KX): two exp
+// warpgroups, one per I tile, with an issuer each for both products, fold sums in
+// registers.  S is 6 or 7 K steps there, and its MMAs set the pace: a single issuer of S
+// took 1.40 ms at N = 70,000, d = 32, m = 16 (1.33 at m = 3) where this form takes 1.23
+// (1.20), and two issuers of S beside one of P.V 1.72.  At d = 20 (KX = 80) this form is
+// the slower one, 1.09 against 1.04 ms.
+template <int POLY>
+__global__ void __launch_bounds__(kFwd2Threads, 1) tc_fwd2_kernel(TcFwdArgs a) {
+  using namespace ptx;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = align1024(smem_raw);
+  const uint32_t A_TILE = a.KX * 256u, V_TILE = a.MP * 256u;
+  const int S = a.S;
+  uint8_t* sA = smem;                       // [buffer 2][tile 2]
+  uint8_t* sB = sA + 4 * A_TILE;            // [stage]
+  uint8_t* sV = sB + S * A_TILE;            // [stage]
+  uint64_t* full = reinterpret_cast<uint64_t*>(sV + S * V_TILE);
+  uint64_t* empty = full + S;
+  uint64_t* a_full = empty + S;
+  uint64_t* a_empty = a_full + 2;
+  uint64_t* s_full = a_empty + 2;    // [g] S_g written by the tensor core
+  uint64_t* s_free = s_full + 2;     // [g] S_g read into registers by warpgroup g
+  uint64_t* p_ready = s_free + 2;    // [g] P_g written by warpgroup g
+  uint64_t* p_free = p_ready + 2;    // [g] P_g consumed by the P.V MMAs
+  uint64_t* o_ready = p_free + 2;
+  uint64_t* o_free = o_ready + 2;
+  uint64_t* done = o_free + 2;       // [g]
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 2);
+  volatile int* abort = reinterpret_cast<volatile int*>(tslot + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < S; ++i) {
+      mbar_init(&full[i], 1);
+      mbar_init(&empty[i], 2);
+    }
+    for (int g = 0; g < 2; ++g) {
+      mbar_init(&a_full[g], 1);
+      mbar_init(&a_empty[g], 2);
+      mbar_init(&s_full[g], 1);
+      mbar_init(&s_free[g], 128);
+      mbar_init(&p_ready[g], 128);
+      mbar_init(&p_free[g], 1);
+      mbar_init(&o_ready[g], 1);
+      mbar_init(&o_free[g], 128);
+      mbar_init(&done[g], 1);
+    }
+    *abort = 0;
+    fence_barrier_init();
+  }
+  if (warp == kMmaWarp) {
+    tmem_alloc(tslot, 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tbase = *tslot;
+  // TMEM columns: S_g [128 g, 128 g + 128), P_g [256 + 64 g, +64), O_g [384 + 64 g, +MP)
+
+  // The producer and issuer warps run their loops with all 32 lanes, so that
+  // addresses and descriptors stay warp-uniform, and one elected lane issues
+  // the copies, MMAs and commits: issuing from a lone lane was measured at
+  // 2-3x the cost per tcgen05.mma.
+  if (warp == kLoadWarp) {
+    const bool leader = elect_one();
+    {
+      // ------------------------------------------------------------ producer
+      int it = 0;
+      uint32_t stage = 0, sph = 0;
+      int n_issued = 0, n_a_issued = 0;
+      bool aborted = false;
+      for (int t = blockIdx.x; t < a.n_items && !aborted; t += gridDim.x) {
+        const int4 item = a.items[t];
+        if (a.sys_active && !a.sys_active[item.x]) continue;
+        const int c = item.x % a.chains;
+        const int ab = it & 1;
+        if (!warp_wait(&a_empty[ab], ((it >> 1) & 1) ^ 1, abort, a.err, 1)) { aborted = true; break; }
+        if (leader) {
+          mbar_arrive_expect_tx(&a_full[ab], 2 * A_TILE);
+          bulk_g2s(sA + (2 * ab) * A_TILE, a.XA + ((size_t)c * a.T_total + item.y) * A_TILE, 2 * A_TILE,
+                   &a_full[ab]);
+        }
+        __syncwarp();
+        ++n_a_issued;
+        for (int j = 0; j < item.w; ++j) {
+          if (!warp_wait(&empty[stage], sph ^ 1, abort, a.err, 2)) { aborted = true; break; }
+          if (leader) {
+            mbar_arrive_expect_tx(&full[stage], A_TILE + V_TILE);
+            const size_t tj = (size_t)c * a.T_total + item.z + j;
+            bulk_g2s(sB + stage * A_TILE, a.XB + tj * A_TILE, A_TILE, &full[stage]);
+            bulk_g2s(sV + stage * V_TILE, a.VT + tj * V_TILE, V_TILE, &full[stage]);
+          }
+          __syncwarp();
+          ++n_issued;
+          if (++stage == (uint32_t)S) { stage = 0; sph ^= 1; }
+        }
+        ++it;
+      }
+      if (aborted) {
+        // drain: the copies already issued must land before the CTA exits
+        for (int k = 1; k <= min(n_issued, S); ++k) {
+          const int idx = n_issued - k;
+          mbar_drain(&full[idx % S], (idx / S) & 1, 500000000ull);
+        }
+        for (int k = 1; k <= min(n_a_issued, 2); ++k) {
+          const int idx = n_a_issued - k;
+          mbar_drain(&a_full[idx & 1], (idx >> 1) & 1, 500000000ull);
+        }
+      }
+    }
+  } else if (warp == kMmaWarp || warp == kFwd2Issue1Warp) {
+    const bool leader = elect_one();
+    {
+      // ------------------------------------------------------------ MMA issuer of I tile g
+      // Tile stream k = 0, 1, ... over this CTA's items.  For tile k it issues
+      // S(k) once warpgroup g has read S(k-1), then P.V of tile k-1 once P(k-1)
+      // is written, so the tensor core computes the next S while the
+      // warpgroup computes exps, and P.V runs during the next tile's exps.
+      const int g = warp == kMmaWarp ? 0 : 1;
+      const uint32_t idS = idesc_f16(128, 128, 1, 1);
+      const uint32_t idP = idesc_f16(128, a.MP, 0, 0);
+      const uint32_t sboX = a.KX * 16u;
+      const int nkx = a.KX / 16;
+      const uint64_t dA = sdesc(smem_u32(sA + g * A_TILE), 128, sboX);
+      const uint64_t dB = sdesc(smem_u32(sB), 128, sboX);
+      const uint64_t dV = sdesc(smem_u32(sV), 128, 2048);
+      const uint32_t s_tmem = tbase + g * 128, p_tmem = tbase + 256 + g * 64, o_tmem = tbase + 384 + g * 64;
+      int it = 0;
+      uint32_t stage = 0, sph = 0;
+      uint32_t sf_ph = 0, pr_ph = 0, of_ph = 0;
+      bool opend = false;
+      long long k = 0;
+      // the previous tile, whose P.V is still to be issued
+      bool have_prev = false;
+      uint32_t prev_stage = 0;
+      int prev_j = 0, prev_nJ = 0, prev_ab = 0;
+      for (int t = blockIdx.x; t < a.n_items; t += gridDim.x) {
+        const int4 item = a.items[t];
+        if (a.sys_active && !a.sys_active[item.x]) continue;
+        const int ab = it & 1;
+        const uint64_t dAg = sdesc_add(dA, 2 * ab * A_TILE);
+        for (int j = 0; j < item.w; ++j, ++k) {
+          // ---- S(k)
+          if (k > 0) {
+            if (!warp_wait(&s_free[g], sf_ph, abort, a.err, 3)) goto mma_out;
+            sf_ph ^= 1;
+          }
+          if (j == 0 && !warp_wait(&a_full[ab], (it >> 1) & 1, abort, a.err, 4)) goto mma_out;
+          if (!warp_wait(&full[stage], sph, abort, a.err, 5)) goto mma_out;
+          tc_fence_after();
+          // operands computed by the whole warp (warp-uniform), issued by the leader
+          const uint64_t db = sdesc_add(dB, stage * A_TILE);
+          if (leader) {
+            issue_s(s_tmem, dAg, db, nkx, idS);
+            tc_commit(&s_full[g]);
+          }
+          __syncwarp();
+          // ---- P.V of tile k-1
+          if (have_prev) {
+            if (!warp_wait(&p_ready[g], pr_ph, abort, a.err, 6)) goto mma_out;
+            pr_ph ^= 1;
+            tc_fence_after();
+            const uint32_t acc = (prev_j % kFold) != 0;
+            if (!acc && opend) {
+              if (!warp_wait(&o_free[g], of_ph, abort, a.err, 7)) goto mma_out;
+              of_ph ^= 1;
+              opend = false;
+              tc_fence_after();
+            }
+            const bool fold_end = (prev_j % kFold) == kFold - 1 || prev_j == prev_nJ - 1;
+            const uint64_t dv = sdesc_add(dV, prev_stage * V_TILE);
+            if (leader) {
+              issue_pv(o_tmem, p_tmem, dv, idP, acc);
+              tc_commit(&p_free[g]);
+              if (fold_end) tc_commit(&o_ready[g]);
+              tc_commit(&empty[prev_stage]);
+              if (prev_j == prev_nJ - 1) tc_commit(&a_empty[prev_ab]);
+            }
+            __syncwarp();
+            if (fold_end) opend = true;
+          }
+          have_prev = true;
+          prev_stage = stage;
+          prev_j = j;
+          prev_nJ = item.w;
+          prev_ab = ab;
+          if (++stage == (uint32_t)S) { stage = 0; sph ^= 1; }
+        }
+        ++it;
+      }
+      if (have_prev) {
+        if (!warp_wait(&p_ready[g], pr_ph, abort, a.err, 6)) goto mma_out;
+        tc_fence_after();
+        const uint32_t acc = (prev_j % kFold) != 0;
+        if (!acc && opend) {
+          if (!warp_wait(&o_free[g], of_ph, abort, a.err, 7)) goto mma_out;
+          tc_fence_after();
+        }
+        const uint64_t dv = sdesc_add(dV, prev_stage * V_TILE);
+        if (leader) {
+          issue_pv(o_tmem, p_tmem, dv, idP, acc);
+          tc_commit(&p_free[g]);
+          tc_commit(&o_ready[g]);
+          tc_commit(&empty[prev_stage]);
+          tc_commit(&a_empty[prev_ab]);
+        }
+        __syncwarp();
+      }
+    mma_out:
+      if (leader) tc_commit(&done[g]);
+      __syncwarp();
+      mbar_drain(&done[g], 0, 500000000ull);
+    }
+    __syncwarp();
+  } else {
+    // ------------------------------------------------------------ exp warpgroups
+    const int g = warp >> 2, w = warp & 3;
+    const int row = 32 * w + lane;
+    const uint32_t tl = tbase + (static_cast<uint32_t>(32 * w) << 16);
+    const uint32_t s_col = g * 128, p_col = 256 + g * 64, o_col = 384 + g * 64;
+    uint32_t sph = 0, pf_ph = 0, oph = 0;
+    long long k = 0;
+    for (int t = blockIdx.x; t < a.n_items; t += gridDim.x) {
+      const int4 item = a.items[t];
+      if (a.sys_active && !a.sys_active[item.x]) continue;
+      const int rowp = g * 128 + row;
+      // the item's O sums per column as FP32 pairs (TwoSum; the FP64 pipe is a
+      // small fraction of the FP32 rate on this GPU), written in FP64
+      float rs[16], rc[16];
+#pragma unroll
+      for (int q = 0; q < 16; ++q) rs[q] = rc[q] = 0.f;
+      for (int j = 0; j < item.w; ++j, ++k) {
+        bool ok = mbar_wait(&s_full[g], sph, abort, a.err, 8);
+        if (!__all_sync(0xffffffffu, ok)) goto exp_out;
+        sph ^= 1;
+        tc_fence_after();
+        {
+          uint32_t a0[32], a1[32], b0[32], b1[32], pk[32];
+          tmem_ld32(tl + s_col, a0);
+          tmem_ld32(tl + s_col + 32, a1);
+          tmem_ld_wait_regs(a0, a1);
+          tmem_ld32(tl + s_col + 64, b0);
+          tmem_ld32(tl + s_col + 96, b1);
+#pragma unroll
+          for (int q = 0; q < 16; ++q)
+            pk[q] = pack_f16x2(exp2_mix<POLY, 3>(__uint_as_float(a0[2 * q]), 2 * q),
+                               exp2_mix<POLY, 3>(__uint_as_float(a0[2 * q + 1]), 2 * q + 1));
+#pragma unroll
+          for (int q = 0; q < 16; ++q)
+            pk[16 + q] = pack_f16x2(exp2_mix<POLY, 3>(__uint_as_float(a1[2 * q]), 2 * q),
+                               exp2_mix<POLY, 3>(__uint_as_float(a1[2 * q + 1]), 2 * q + 1));
+          tmem_ld_wait_regs(b0, b1);
+          // S(k) is fully in registers: the tensor core may overwrite it
+          tc_fence_before();
+          mbar_arrive(&s_free[g]);
+          if (k > 0) {
+            // P(k-1) must have been consumed before P(k) overwrites it
+            ok = mbar_wait(&p_free[g], pf_ph, abort, a.err, 10);
+            if (!__all_sync(0xffffffffu, ok)) goto exp_out;
+            pf_ph ^= 1;
+            tc_fence_after();
+          }
+          tmem_st32(tl + p_col, pk);
+          // the second half's exps in place; pk, the source of the store just
+          // issued, is rewritten only after tcgen05.wait::st
+#pragma unroll
+          for (int e = 0; e < 32; ++e) {
+            b0[e] = __float_as_uint(exp2_mix<POLY, 3>(__uint_as_float(b0[e]), e));
+            b1[e] = __float_as_uint(exp2_mix<POLY, 3>(__uint_as_float(b1[e]), e));
+          }
+          tmem_st_wait();
+#pragma unroll
+          for (int q = 0; q < 16; ++q) {
+            pk[q] = pack_f16x2(__uint_as_float(b0[2 * q]), __uint_as_float(b0[2 * q + 1]));
+            pk[16 + q] = pack_f16x2(__uint_as_float(b1[2 * q]), __uint_as_float(b1[2 * q + 1]));
+          }
+          tmem_st32(tl + p_col + 32, pk);
+        }
+        tmem_st_wait();
+        tc_fence_before();
+        mbar_arrive(&p_ready[g]);
+        if ((j % kFold) == kFold - 1 || j == item.w - 1) {
+          ok = mbar_wait(&o_ready[g], oph, abort, a.err, 9);
+          if (!__all_sync(0xffffffffu, ok)) goto exp_out;
+          oph ^= 1;
+          tc_fence_after();
+          uint32_t o[16];
+          tmem_ld16(tl + o_col, o);
+          tmem_ld_wait_regs(o);
+#pragma unroll
+          for (int q = 0; q < 16; ++q) two_sum_add(rs[q], rc[q], __uint_as_float(o[q]));
+          tc_fence_before();
+          mbar_arrive(&o_free[g]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 16; ++q)
+        if (q < a.mz) a.part[part_idx(t, a.mz, q, rowp)] = (double)rs[q] + (double)rc[q];
+    }
+  exp_out:;
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == kMmaWarp) tmem_dealloc(tbase, 512);
 }
 
 // Forward for one or two columns (the CG product): S = XA XB^T on the tensor
@@ -1234,6 +1588,7 @@ FwdKernel fwd_kernel(bool fma, int cols, int split) {
     if (cols == 1) return sp == 0 ? tc_fwd_fma_kernel<1, 0> : sp == 4 ? tc_fwd_fma_kernel<1, 4> : tc_fwd_fma_kernel<1, 8>;
     return sp == 0 ? tc_fwd_fma_kernel<2, 0> : sp == 4 ? tc_fwd_fma_kernel<2, 4> : tc_fwd_fma_kernel<2, 8>;
   }
+  if (cols == 17) return sp == 0 ? tc_fwd2_kernel<0> : sp == 4 ? tc_fwd2_kernel<4> : tc_fwd2_kernel<8>;
   if (cols == 16)
     return sp == 0 ? tc_fwd_kernel<true, 0> : sp == 4 ? tc_fwd_kernel<true, 4> : tc_fwd_kernel<true, 8>;
   return sp == 0 ? tc_fwd_kernel<false, 0> : sp == 4 ? tc_fwd_kernel<false, 4> : tc_fwd_kernel<false, 8>;
@@ -1241,7 +1596,7 @@ FwdKernel fwd_kernel(bool fma, int cols, int split) {
 
 cudaError_t fwd_kernels_set_smem() {
   for (bool fma : {false, true})
-    for (int cols : {0, 1, 2, 16})
+    for (int cols : {0, 1, 2, 16, 17})
       for (int sp : {0, 4, 8}) {
         if (fma != (cols == 1 || cols == 2)) continue;
         const cudaError_t e =
@@ -1275,7 +1630,7 @@ kmv_status tc_forward(kmv_handle h, const KmvArgs& a, cudaStream_t st) {
   const size_t fixed = 1024 + 4 * A_TILE + 256;
   int mz_max = std::min(a.m, kMaxMP);
   // up to 16 columns: the fold sums' pairs, 8 columns for each of the 512 exp threads
-  auto pair_bytes = [&](int mz) { return mz <= 16 ? (size_t)8 * 512 * sizeof(float2) : (size_t)0; };
+  auto pair_bytes = [&](int mz) { return mz <= 16 && KX < kFwd2KX ? (size_t)8 * 512 * sizeof(float2) : (size_t)0; };
   auto stages_for = [&](int mz) {
     const size_t vt = (size_t)std::max(16, (mz + 15) / 16 * 16) * 256;
     return (int)std::min<size_t>(max_stages, (kMaxSmem - fixed - pair_bytes(mz) - 20 * 8) / (A_TILE + vt + 16));
@@ -1388,7 +1743,8 @@ kmv_status tc_forward(kmv_handle h, const KmvArgs& a, cudaStream_t st) {
     const int grid = std::min(S->n_items, S->num_sms);
     {
       ProfScope prof(h, KMV_KERNEL_FORWARD, st);
-      fwd_kernel(false, MP <= 16 ? 16 : 0, tl.exp_split)<<<grid, kFwdThreads, smem, st>>>(fa);
+      const bool two = MP <= 16 && KX >= kFwd2KX;
+      fwd_kernel(false, two ? 17 : MP <= 16 ? 16 : 0, tl.exp_split)<<<grid, two ? kFwd2Threads : kFwdThreads, smem, st>>>(fa);
     }
     tc_launch_epilogue(h, S, a, c0, mz, part, vmax, err, st);
     const cudaError_t e = cudaGetLastError();
