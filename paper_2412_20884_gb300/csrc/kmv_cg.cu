@@ -171,17 +171,17 @@ __global__ void cg_update_xr_rr_kernel(DevLayout L, int chains, int64_t n_total,
   const uint32_t n_of_system = single ? gridDim.x : (uint32_t)(L.inst_item0[b + 1] - L.inst_item0[b]);
   chain_wait();
   if (!active[s]) return;
-  float rs = 0.f, re = 0.f;
+  double rr = 0.0;
   if (i < r1) {
     const int64_t v = (int64_t)c * n_total + i;
     const float al = (float)sys[s].alpha;
     x[v] = fmaf(al, p[v], x[v]);
     const float ri = fmaf(-al, q[v], r[v]);
     r[v] = ri;
-    pair_add_product(rs, re, ri, ri);
+    rr = (double)ri * ri;
   }
   const bool form_p = p_rows > 0 && r1 - r0 <= p_rows;
-  const double t = pair_block_sum(rs, re, red);
+  const double t = block_sum(rr, red);
   if (threadIdx.x == 0) {
     partial[(int64_t)item * chains + c] = t;
     s_last = last_arrival(&count[s], 1u, n_of_system);

@@ -6,12 +6,12 @@
 // product.  FP64 scalars, per-(tile, chain, column) partial sums reduced in a
 // fixed order, so the iterates are bitwise reproducible.
 //
-// The columns' dot products are exact FP32 products summed as (sum, error) pairs
-// (2^-48), all columns of a row tile in one reduce-scatter; the per-column scalar
-// steps run in the CTA that finishes a system last, a warp per column.  (FP64 products
-// and one thread per system took 63 + 91 us per iteration for 8 systems of 64 tiles
-// and 15 columns, the projections 467 us: the FP64 pipe of this GPU gives 2 lanes per
-// clock and SM.)
+// The columns' dot products are FP64 throughout (a solve is to give the same iterates
+// for any scale of its right-hand side, and FP32 squares of a residual below 1e-19 are
+// subnormal), all columns of a row tile in one reduce-scatter; the per-column scalar
+// steps run in the CTA that finishes a system last, a warp per column.  (A block sum per
+// column and one thread per system took 63 + 91 us per iteration for 8 systems of 64
+// tiles and 15 columns.)
 #include <algorithm>
 
 #include "cg_common.cuh"
@@ -150,16 +150,16 @@ __global__ void __launch_bounds__(kTile) mcg_dot_kernel(DevLayout L, int chains,
   const bool valid = i < L.offsets[bi + 1];
   chain_wait();
   if (!sys_any[s]) return;
-  float sm[NC], er[NC];
+  double v[NC];
 #pragma unroll
   for (int col = 0; col < NC; ++col) {
-    sm[col] = er[col] = 0.f;
+    v[col] = 0.0;
     if (valid && col < m) {
       const int64_t o = ((int64_t)c * n_total + i) * m + col;
-      pair_add_product(sm[col], er[col], p[o], q[o]);
+      v[col] = (double)p[o] * q[o];
     }
   }
-  pair_block_sums<NC>(sm, er, m, red, [&](int col, double t) { partial[((int64_t)item * chains + c) * m + col] = t; });
+  block_sums<NC>(v, m, red, [&](int col, double t) { partial[((int64_t)item * chains + c) * m + col] = t; });
   __syncthreads();
   if (threadIdx.x == 0) s_last = last_arrival(&count[s], 1u, (uint32_t)(L.inst_item0[bi + 1] - L.inst_item0[bi]));
   __syncthreads();
@@ -201,10 +201,10 @@ __global__ void __launch_bounds__(kTile) mcg_update_xr_kernel(DevLayout L, int c
     on[threadIdx.x] = k.active;
   }
   __syncthreads();
-  float sm[NC], er[NC];
+  double v[NC];
 #pragma unroll
   for (int col = 0; col < NC; ++col) {
-    sm[col] = er[col] = 0.f;
+    v[col] = 0.0;
     if (valid && col < m) {
       const int64_t o = ((int64_t)c * n_total + i) * m + col;
       float rv = r[o];
@@ -213,10 +213,10 @@ __global__ void __launch_bounds__(kTile) mcg_update_xr_kernel(DevLayout L, int c
         rv = fmaf(-al[col], q[o], rv);
         r[o] = rv;
       }
-      pair_add_product(sm[col], er[col], rv, rv);
+      v[col] = (double)rv * rv;
     }
   }
-  pair_block_sums<NC>(sm, er, m, red, [&](int col, double t) { partial[((int64_t)item * chains + c) * m + col] = t; });
+  block_sums<NC>(v, m, red, [&](int col, double t) { partial[((int64_t)item * chains + c) * m + col] = t; });
   if (!count) return;
   __syncthreads();
   if (threadIdx.x == 0) s_last = last_arrival(&count[s], 1u, (uint32_t)(L.inst_item0[bi + 1] - L.inst_item0[bi]));
@@ -470,19 +470,19 @@ __global__ void __launch_bounds__(kTile) mcg_apply_kernel(DevLayout L, int chain
       }
     }
   }
-  float sm[NC], er[NC];
+  double v[NC];
 #pragma unroll
   for (int q = 0; q < NC; ++q) {
-    sm[q] = er[q] = 0.f;
+    v[q] = 0.0;
     if (valid && q < m) {
       const int64_t o = ((int64_t)c * n_total + i) * m + q;
       const float rv = r[o];
       const float zv = rv + acc[q];
       z[o] = zv;
-      pair_add_product(sm[q], er[q], rv, zv);
+      v[q] = (double)rv * zv;
     }
   }
-  pair_block_sums<NC>(sm, er, m, red, [&](int q, double t) { prz[((int64_t)item * chains + c) * m + q] = t; });
+  block_sums<NC>(v, m, red, [&](int q, double t) { prz[((int64_t)item * chains + c) * m + q] = t; });
   if (!count) return;
   __syncthreads();
   if (threadIdx.x == 0) s_last = last_arrival(&count[s], 1u, (uint32_t)(L.inst_item0[b + 1] - L.inst_item0[b]));

@@ -178,16 +178,16 @@ __global__ void mscg_update_xr_beta_kernel(DevLayout L, int chains, int64_t n_to
   }
   __syncthreads();
   const int64_t i = L.item_row0[item] + threadIdx.x;
-  float rs = 0.f, re = 0.f;
+  double rr = 0.0;
   if (i < L.offsets[bi + 1]) {
     const int64_t v = (int64_t)c * n_total + i;
     for (int j = 0; j < m; ++j)
       if (on[j]) xs[v * m + j] = fmaf(as[j], ps[v * m + j], xs[v * m + j]);
     const float rv = fmaf(-(float)sys[s].alpha, q[v], r[v]);
     r[v] = rv;
-    pair_add_product(rs, re, rv, rv);
+    rr = (double)rv * rv;
   }
-  const double t = pair_block_sum(rs, re, red);
+  const double t = block_sum(rr, red);
   if (threadIdx.x == 0) {
     partial[(int64_t)item * chains + c] = t;
     s_last = last_arrival(&count[s], 1u, (uint32_t)(L.inst_item0[bi + 1] - L.inst_item0[bi]));

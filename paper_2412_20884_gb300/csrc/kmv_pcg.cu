@@ -112,9 +112,7 @@ __global__ void pcg_proj_kernel(DevLayout L, int chains, int64_t n_total, int ra
   }
   rs[threadIdx.x] = rv;
   if (UPDATE) {
-    float sm = 0.f, er = 0.f;
-    if (i < r1) pair_add_product(sm, er, rv, rv);
-    const double t = pair_block_sum(sm, er, red);
+    const double t = block_sum((double)rv * rv, red);
     if (threadIdx.x == 0) partial[(int64_t)item * chains + c] = t;
   } else {
     __syncthreads();
@@ -170,7 +168,7 @@ __global__ void pcg_apply_kernel(DevLayout L, int chains, int64_t n_total, int r
   if (active && !active[s]) return;
   for (int k = threadIdx.x; k < rank; k += blockDim.x) cf[k] = (float)coef[(int64_t)s * rank + k];
   __syncthreads();
-  float sm = 0.f, er = 0.f;
+  double rz = 0.0;
   if (i < r1) {
     const int64_t v = (int64_t)c * n_total + i;
     const float rv = r[v];
@@ -180,9 +178,9 @@ __global__ void pcg_apply_kernel(DevLayout L, int chains, int64_t n_total, int r
     for (int k = 0; k < rank; ++k) acc = fmaf(Ui[(int64_t)k * n_total], cf[k], acc);
     const float zv = rv + acc;
     z[v] = zv;
-    pair_add_product(sm, er, rv, zv);
+    rz = (double)rv * zv;
   }
-  const double t = pair_block_sum(sm, er, red);
+  const double t = block_sum(rz, red);
   if (threadIdx.x == 0) {
     prz[(int64_t)item * chains + c] = t;
     s_last = sys && last_arrival(&count[s], 1u, (uint32_t)n_of_system);

@@ -47,7 +47,11 @@ __device__ __forceinline__ void two_sum_add(float& s, float& c, float x) {
   s = t;
 }
 
-// Adds u v to the pair (s, e): the product's rounding error is recovered by an FMA.
+// Adds u v to the pair (s, e): the product's rounding error is recovered by an FMA.  FP32's
+// range holds for the product, and for its error (2^-24 of it): for sums of which only
+// FP32 accuracy near the size of u and v is needed (the preconditioner's projections),
+// not for the r.r, r.z and p.q of a solver, whose squares leave FP32's range where the
+// vectors are still well inside it.
 __device__ __forceinline__ void pair_add_product(float& s, float& e, float u, float v) {
   const float p = __fmul_rn(u, v);
   two_sum_add(s, e, p);
@@ -86,20 +90,6 @@ __device__ __forceinline__ void block_sum_many(double (&v)[N], int n, double* re
   }
 }
 
-// Block sum of one pair per thread; result valid in thread 0.  (An FP64 block_sum keeps
-// the FP64 pipe, 2 lanes per clock and SM, busy for six operations per warp.)
-__device__ __forceinline__ double pair_block_sum(float s, float e, double* red) {
-  pair_warp_sum(s, e);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) red[w] = (double)s + (double)e;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[i];
-  return t;
-}
-
 // Sums NC (16 or 32) pairs per lane over the warp: the lanes halve the vector between
 // them step by step; lane l returns with column l % NC in (s[0], e[0]).
 template <int NC>
@@ -124,14 +114,25 @@ __device__ __forceinline__ void pair_reduce_scatter(float (&s)[NC], float (&e)[N
     e[0] = __fadd_rn(e[0], eo);
   }
 }
-// Block sums of NC pairs per thread (kTile threads): out(col, sum) by thread col < n.
+// Block sums of NC (16 or 32) values per thread (kTile threads): out(col, sum) by thread
+// col < n.  The lanes halve the vector between them step by step, NC - 1 adds a lane
+// where a tree per value takes 5 NC (the FP64 pipe gives 2 lanes per clock and SM).
 // red: kTile / 32 rows of NC.
 template <int NC, class Out>
-__device__ __forceinline__ void pair_block_sums(float (&s)[NC], float (&e)[NC], int n, double* red, Out&& out) {
-  pair_reduce_scatter<NC>(s, e);
+__device__ __forceinline__ void block_sums(double (&v)[NC], int n, double* red, Out&& out) {
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+#pragma unroll
+  for (int h = NC / 2; h >= 1; h /= 2) {
+    const bool up = l & h;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const double other = __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + h], h);
+      v[i] = (up ? v[i + h] : v[i]) + other;
+    }
+  }
+  if (NC == 16) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 16);
   __syncthreads();
-  if (l < NC) red[w * NC + l] = (double)s[0] + (double)e[0];
+  if (l < NC) red[w * NC + l] = v[0];
   __syncthreads();
   if ((int)threadIdx.x < n) {
     double t = 0.0;
