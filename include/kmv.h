@@ -72,7 +72,7 @@ typedef enum {
 
 typedef enum {
   /* Plain FP32 on the FMA/MUFU pipes: direct differences, FP32 exp2, FP32
-   * products folded exactly (TwoSum pairs) every 512 columns.  Relative
+   * products folded into FP64 accumulators every 512 columns.  Relative
    * error against FP64 <= 1e-5 on outputs, <= 1e-4 on gradients. */
   KMV_FP32 = 0,
   /* Tensor-core form (tcgen05).  Points are centred per instance (midrange,

@@ -182,7 +182,7 @@ struct SimtFwd {
   int folds, upc;            // folds (512 columns) per unit, units per chunk
   int max_units;             // js * upc; 1: every CTA writes its rows' Y itself
   int ticket;                // the last unit of a tile adds the units and writes Y; else the combine kernel does
-  float2* part;              // (max_units, chains, m, N_total) pairs, for several units or folds
+  double* part;              // (max_units, chains, m, N_total) sums, for several units or folds
   uint32_t* count;           // ticket: one zeroed counter per (tile, chain, column chunk)
 };
 SimtFwd simt_fwd_plan(const SimtTiles& T, int n_inst, int n_items, int chains, int64_t n_total, int64_t max_rows, int d, int m,
@@ -196,7 +196,7 @@ struct SimtBwd {
   int n_tiles, rows, mp, nz;  // tiles, rows per thread, columns per CTA (the kernel's width), column chunks
   int chunk;                  // columns per chunk (<= mp): W_ij is summed per chunk
   int folds, units;           // folds (512 columns) per J unit, units
-  float2* part;               // want_gv and several units or folds: (units, chains, m, N_total) pairs
+  double* part;               // want_gv and several units or folds: (units, chains, m, N_total) sums
 };
 int backward_mp(int m);      // columns per backward pass
 SimtBwd simt_bwd_plan(const SimtTiles& T, int n_items, int chains, int64_t n_total, int64_t max_rows, int d, int m,
@@ -482,7 +482,7 @@ struct kmv_handle_s {
   // kept until the handle goes, for graphs captured with them; they at least double,
   // so all of them together stay below twice the last.
   kmv::SimtTiles simt_tiles;
-  float2* simt_part = nullptr;
+  double* simt_part = nullptr;
   size_t simt_part_bytes = 0;
   uint32_t* simt_count = nullptr;
   size_t simt_counters = 0;

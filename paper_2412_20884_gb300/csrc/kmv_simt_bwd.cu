@@ -53,14 +53,10 @@ __global__ void __launch_bounds__(kTile) bwd_simt_combine_kernel(KmvArgs a, Simt
   const double ai = as2[0] * (double)(a.amp ? a.amp[row] : 1.f);
   for (int c0 = blockIdx.z * kGvCols; c0 < a.m; c0 += gridDim.z * kGvCols) {
     for (int q = c0; q < min(a.m, c0 + kGvCols); ++q) {
-      float sum = 0.f, err = 0.f;
-      for (int u = 0; u < units; ++u) {
-        const float2 p = f.part[(((size_t)u * a.chains + c) * a.m + q) * (size_t)a.n_total + i];
-        two_sum_add(sum, err, p.x);
-        err += p.y;
-      }
+      double sum = 0.0;
+      for (int u = 0; u < units; ++u) sum += f.part[(((size_t)u * a.chains + c) * a.m + q) * (size_t)a.n_total + i];
       const int64_t idx = row * a.m + q;
-      a.Y[idx] = (float)(ai * ((double)sum + (double)err) + as2[1] * (double)a.G[idx]);
+      a.Y[idx] = (float)(ai * sum + as2[1] * (double)a.G[idx]);
     }
   }
 }
@@ -124,7 +120,7 @@ SimtBwd simt_bwd_plan(const SimtTiles& T, int n_items, int chains, int64_t n_tot
   const int64_t ctas = (int64_t)f.n_tiles * chains * f.nz;
   int64_t units = std::min<int64_t>(fpc, std::max<int64_t>(1, (8 * (int64_t)num_sms + ctas - 1) / std::max<int64_t>(1, ctas)));
   units = std::min<int64_t>(units, std::max(1, 65535 / f.nz));
-  const int64_t bytes = want_gv ? (int64_t)sizeof(float2) * chains * m * std::max<int64_t>(1, n_total) : 0;
+  const int64_t bytes = want_gv ? (int64_t)sizeof(double) * chains * m * std::max<int64_t>(1, n_total) : 0;
   while (units > 1 && bytes * units > (int64_t(512) << 20)) --units;
   f.folds = (int)((fpc + units - 1) / units);
   f.units = (int)((fpc + f.folds - 1) / f.folds);
@@ -148,7 +144,7 @@ size_t simt_bwd_partials(const SimtBwd& f, int n_items, int chains, int n_theta)
   return (size_t)std::max(1, n_items) * chains * f.nz * f.units * n_theta;
 }
 size_t simt_bwd_part_bytes(const SimtBwd& f, int chains, int64_t n_total, int m) {
-  return f.units > 1 || (f.folds > 1 && f.rows > 1) ? sizeof(float2) * (size_t)f.units * chains * m * (size_t)n_total : 0;
+  return f.units > 1 || (f.folds > 1 && f.rows > 1) ? sizeof(double) * (size_t)f.units * chains * m * (size_t)n_total : 0;
 }
 
 template <int D>

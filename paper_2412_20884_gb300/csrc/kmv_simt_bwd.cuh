@@ -12,7 +12,7 @@
 // With per-point amplitudes (Sec. 4) G and V enter as amp o G, amp o V.
 // Because every dA/dtheta_p is symmetric, summing W_ij over all ordered
 // pairs (i, j) gives the gradient without symmetrising W.  FP32 sums run over at
-// most 512 columns and are then folded into (sum, error) pairs; per-CTA FP64
+// most 512 columns and are then folded into FP64 sums; per-CTA FP64
 // partials go to a buffer that launch_grad_finalize reduces in a fixed order.
 //
 // What bounds it: per pair 4 D + 2 m + 3 operations of the FMA pipe (m columns with
@@ -71,13 +71,19 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
   float xi[R][D], gi[R][MP], accq[R], accg[R][DG];
   uint64_t accv[R][MP / 2];   // columns 2q, 2q + 1 in a packed pair
   auto accv_at = [&](int r, int q) { return (q & 1) ? hi_f32x2(accv[r][q / 2]) : lo_f32x2(accv[r][q / 2]); };
-  // running sums of the unit as pairs (several folds)
-  float sq[R], cq[R], sg2[R][DG], cg2[R][DG];
+  // running sums of the unit; those of many dimensions in local memory (64 FP64 sums are
+  // 128 registers, used once in 512 columns), by a pointer hidden from the compiler, which
+  // would put the array into registers and spill the loop's values
+  constexpr bool kLocalG = R * DG >= 32;
+  double sq[R], sg2[kLocalG ? 1 : R][kLocalG ? 1 : DG], sg_store[kLocalG ? R * DG : 1];
+  double* sgl = sg_store;
+  if constexpr (kLocalG) asm volatile("" : "+l"(sgl));
+  bool first_g = true;
   // those of dL/dV: in registers with one row per thread, else in f.part
   constexpr int RV = R == 1 ? MP : 1;
-  float svp[RV], cvp[RV];
+  double svp[RV];
 #pragma unroll
-  for (int q = 0; q < RV; ++q) svp[q] = cvp[q] = 0.f;
+  for (int q = 0; q < RV; ++q) svp[q] = 0.0;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int64_t i = r0 + r * kTile + tid;
@@ -90,21 +96,23 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
       gi[r][q] = (q < mc && valid) ? a.G[(vbase + i) * a.m + c0 + q] * amp_i : 0.f;
       accv[r][q / 2] = 0;
     }
-    accq[r] = sq[r] = cq[r] = 0.f;
+    accq[r] = 0.f;
+    sq[r] = 0.0;
 #pragma unroll
-    for (int k = 0; k < DG; ++k) accg[r][k] = sg2[r][k] = cg2[r][k] = 0.f;
+    for (int k = 0; k < DG; ++k) {
+      accg[r][k] = 0.f;
+      if constexpr (!kLocalG) sg2[r][k] = 0.0;
+    }
   }
 
   const uint32_t inv = dd > 1 ? 0xffffffffu / (uint32_t)dd + 1u : 0u;
   const bool paired = je - jb > kFoldTiles * kTile;
   bool first = true;
-  // dL/dV sums of this thread's rows into the pairs
+  // adds the FP32 sums of dL/dV of this thread's rows to the FP64 ones
   auto fold_v = [&]() {
     if constexpr (R == 1) {
 #pragma unroll
-      for (int q = 0; q < RV; ++q) {
-        two_sum_add(svp[q], cvp[q], accv_at(0, q));
-      }
+      for (int q = 0; q < RV; ++q) svp[q] += (double)accv_at(0, q);
 #pragma unroll
       for (int q = 0; q < MP / 2; ++q) accv[0][q] = 0;
     } else {
@@ -115,10 +123,9 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
 #pragma unroll
           for (int q = 0; q < MP; ++q)
             if (q < mc) {
-              float2* p = &f.part[(((size_t)u * a.chains + c) * a.m + c0 + q) * (size_t)a.n_total + i];
-              float2 v = first ? make_float2(0.f, 0.f) : *p;
-              two_sum_add(v.x, v.y, accv_at(r, q));
-              *p = v;
+              double* p = &f.part[(((size_t)u * a.chains + c) * a.m + c0 + q) * (size_t)a.n_total + i];
+              const double v = (double)accv_at(r, q);
+              *p = first ? v : *p + v;
             }
         }
 #pragma unroll
@@ -130,14 +137,22 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
   auto fold_g = [&]() {
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      two_sum_add(sq[r], cq[r], accq[r]);
+      sq[r] += (double)accq[r];
       accq[r] = 0.f;
 #pragma unroll
       for (int k = 0; k < DG; ++k) {
-        two_sum_add(sg2[r][k], cg2[r][k], accg[r][k]);
+        if constexpr (kLocalG) {
+          if (k < dd) {   // (the FP64 pipe is slow)
+            const double v = (double)accg[r][k];
+            sgl[r * DG + k] = first_g ? v : sgl[r * DG + k] + v;
+          }
+        } else {
+          if (k < dd) sg2[r][k] += (double)accg[r][k];
+        }
         accg[r][k] = 0.f;
       }
     }
+    first_g = false;
   };
 
   int step = 0;
@@ -244,7 +259,7 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
 #pragma unroll
     for (int q = 0; q < RV; ++q)
       if (q < mc)
-        f.part[(((size_t)u * a.chains + c) * a.m + c0 + q) * (size_t)a.n_total + r0 + tid] = make_float2(svp[q], cvp[q]);
+        f.part[(((size_t)u * a.chains + c) * a.m + c0 + q) * (size_t)a.n_total + r0 + tid] = svp[q];
   }
 
   // noise gradient and, in a single unit, dL/dV
@@ -261,9 +276,9 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
           const double g = (double)a.G[idx];
           if (u == 0) noise += g * (double)a.V[idx];
           if (want_gv && direct) {
-            float2 v = R == 1 ? make_float2(svp[q % RV], cvp[q % RV]) : make_float2(accv_at(r, q), 0.f);
+            double v = R == 1 ? svp[q % RV] : (double)accv_at(r, q);
             if (R > 1 && paired) v = f.part[((size_t)c * a.m + c0 + q) * (size_t)a.n_total + i];
-            a.Y[idx] = (float)(ai * ((double)v.x + (double)v.y) + as2[1] * g);
+            a.Y[idx] = (float)(ai * v + as2[1] * g);
           }
         }
       }
@@ -275,12 +290,15 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
   double ev[NE];   // [q, g_0 .. , noise]
   ev[0] = 0.0;
 #pragma unroll
-  for (int r = 0; r < R; ++r) ev[0] += (double)sq[r] + (double)cq[r];
+  for (int r = 0; r < R; ++r) ev[0] += sq[r];
 #pragma unroll
   for (int k = 0; k < DG; ++k) {
     ev[1 + k] = 0.0;
 #pragma unroll
-    for (int r = 0; r < R; ++r) ev[1 + k] += (double)sg2[r][k] + (double)cg2[r][k];
+    for (int r = 0; r < R; ++r) {
+      if constexpr (kLocalG) ev[1 + k] += k < dd ? sgl[r * DG + k] : 0.0;
+      else ev[1 + k] += sg2[r][k];
+    }
   }
   ev[NE - 1] = noise;
   block_sum_many<NE>(ev, NE, red, [&](int e, double t) {

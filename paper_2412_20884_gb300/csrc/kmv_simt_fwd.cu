@@ -86,7 +86,7 @@ int forward_jsplit(int n_items, int chains, int m, int64_t max_rows, int num_sms
 
 // Rows per thread and the number of J units.  Units end at multiples of 512 columns
 // of a chunk, where the FP32 sums are folded anyway, so the split changes the result
-// only in the pairs' last bits (2^-48).
+// only in the FP64 sums' last bits.
 // One CTA of one-row threads per 128 rows took 2.18 ms at N = 20,000, d = 8, m = 16 (one
 // to two CTAs per SM); four rows and units of 512 columns and up take 0.46 ms, with
 // 0.03 ms for their sum.  The wide variant starts where its finest split fills every SM
@@ -115,7 +115,7 @@ SimtFwd simt_fwd_plan(const SimtTiles& T, int n_inst, int n_items, int chains, i
   // about 8 CTAs per SM (two to four resident, so that the last wave is short), with at
   // most 512 MB of partial sums
   int64_t upc = std::min<int64_t>(fpc, std::max<int64_t>(1, (8 * (int64_t)num_sms + ctas - 1) / std::max<int64_t>(1, ctas)));
-  const int64_t bytes = (int64_t)sizeof(float2) * f.js * chains * m * std::max<int64_t>(1, n_total);
+  const int64_t bytes = (int64_t)sizeof(double) * f.js * chains * m * std::max<int64_t>(1, n_total);
   while (upc > 1 && bytes * upc > (int64_t(512) << 20)) --upc;
   f.folds = (int)((fpc + upc - 1) / upc);
   f.upc = (int)((fpc + f.folds - 1) / f.folds);
@@ -125,7 +125,7 @@ SimtFwd simt_fwd_plan(const SimtTiles& T, int n_inst, int n_items, int chains, i
 }
 
 size_t simt_fwd_part_bytes(const SimtFwd& f, int chains, int64_t n_total, int m) {
-  return f.max_units > 1 || f.folds > 1 ? sizeof(float2) * (size_t)f.max_units * chains * m * (size_t)n_total : 0;
+  return f.max_units > 1 || f.folds > 1 ? sizeof(double) * (size_t)f.max_units * chains * m * (size_t)n_total : 0;
 }
 size_t simt_fwd_counters(const SimtFwd& f, int chains) { return f.ticket ? (size_t)f.n_tiles * chains * f.nz : 0; }
 

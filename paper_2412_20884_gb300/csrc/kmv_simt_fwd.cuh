@@ -7,7 +7,7 @@
 //   K0_ij = 2^(-sum_k (xh_ik - xh_jk)^2),  xh = x sqrt(log2(e)/2) / l,
 // from direct differences (no |x|^2 expansion, so no cancellation), then
 // accumulates K0_ij V_j in FP32.  Every 512 columns the FP32 sums are folded into
-// (sum, error) pairs (two_sum_add).  Epilogue (Eq. kerdef): Y_i = alpha * acc_i +
+// FP64 sums.  Epilogue (Eq. kerdef): Y_i = alpha * acc_i +
 // (sigma^2 + shift) V_i.  With per-point amplitudes (the kernel family of Sec. 4)
 // V_j enters as amp_j V_j and acc_i is scaled by amp_i.
 //
@@ -57,33 +57,37 @@ __device__ __forceinline__ size_t simt_part_at(const KmvArgs& a, int unit, int c
   return (((size_t)unit * a.chains + c) * a.m + col) * (size_t)a.n_total + i;
 }
 
-// Adds n pairs a fixed step apart to (s, e), eight loads in flight at a time (one
-// after the other, 16 of them took 5 us of a small product's last CTA).
-__device__ __forceinline__ void simt_add_pairs(const float2* p, size_t step, uint32_t n, float& s, float& e) {
+// Adds n sums a fixed step apart to s, eight loads in flight at a time (one after the
+// other, 16 of them took 5 us of a small product's last CTA).
+__device__ __forceinline__ void simt_add_parts(const double* p, size_t step, uint32_t n, double& s) {
   for (uint32_t u0 = 0; u0 < n; u0 += 8) {
-    float2 v[8];
+    double v[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = u0 + k < n ? __ldcg(p + (u0 + k) * step) : make_float2(0.f, 0.f);
+    for (int k = 0; k < 8; ++k) v[k] = u0 + k < n ? __ldcg(p + (u0 + k) * step) : 0.0;
+    if (u0 + 8 <= n) {
+      // (a tree: 16 dependent FP64 adds of 65 clocks were 0.4 us of a small product)
+      s += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+    } else {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      two_sum_add(s, e, v[k].x);
-      e += v[k].y;
+      for (int k = 0; k < 8; ++k)
+        if (u0 + k < n) s += v[k];
     }
   }
 }
 
-// Sum of the units' pairs of one element, in unit order.
+// Sum of the units' sums of one element, in a fixed order.
 __device__ __forceinline__ double simt_part_sum(const KmvArgs& a, const SimtFwd& f, const SimtUnits& U, int c, int col,
                                                 int64_t i) {
-  float s = 0.f, e = 0.f;
+  double s = 0.0;
   const size_t step = (size_t)a.chains * a.m * (size_t)a.n_total;
-  const float2* p = f.part + simt_part_at(a, 0, c, col, i);
-  if (f.upc == 1) {
-    simt_add_pairs(p, step, U.n_chunks, s, e);
-  } else {
-    for (uint32_t jc = 0; jc < U.n_chunks; ++jc) simt_add_pairs(p + jc * f.upc * step, step, U.in_chunk(jc), s, e);
-  }
-  return (double)s + (double)e;
+  const double* p = f.part + simt_part_at(a, 0, c, col, i);
+  // one run of units, or a run per chunk where this instance's chunks have fewer than upc
+  // (upc == 1 without the divisions)
+  const bool one_run = f.upc == 1 || U.in_chunk(0) == (uint32_t)f.upc;
+  const uint32_t runs = one_run ? 1 : U.n_chunks;
+  for (uint32_t jc = 0; jc < runs; ++jc)
+    simt_add_parts(p + jc * f.upc * step, step, f.upc == 1 ? U.n_chunks : one_run ? U.count() : U.in_chunk(jc), s);
+  return s;
 }
 
 // alpha and sigma^2 of a system: two lanes, one exp (an FP64 exp takes some 1100
@@ -243,10 +247,10 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
       vi[r][q] = (MP <= 2 && q < mc && i < o1) ? a.V[(vbase + i) * a.m + c0 + q] : 0.f;
     }
 
-  const bool paired = je - jb > kFoldTiles * kTile;   // several folds: sums kept as pairs in f.part
+  const bool paired = je - jb > kFoldTiles * kTile;   // several folds: sums kept in f.part
   const int unit = jc * f.upc + u;
   bool first = true;
-  // adds the FP32 sums to the pairs in global memory (this thread's own elements)
+  // adds the FP32 sums to the FP64 ones in global memory (this thread's own elements)
   auto fold = [&]() {
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -255,10 +259,9 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
 #pragma unroll
         for (int q = 0; q < MP; ++q)
           if (q < mc) {
-            float2* p = &f.part[simt_part_at(a, unit, c, c0 + q, i)];
-            float2 v = first ? make_float2(0.f, 0.f) : *p;
-            two_sum_add(v.x, v.y, acc_at(r, q));
-            *p = v;
+            double* p = &f.part[simt_part_at(a, unit, c, c0 + q, i)];
+            const double v = (double)acc_at(r, q);
+            *p = first ? v : *p + v;
           }
       }
 #pragma unroll
@@ -362,10 +365,9 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
 #pragma unroll
         for (int q = 0; q < MP; ++q)
           if (q < mc) {
-            float2 v = make_float2(0.f, 0.f);
-            if (paired) v = f.part[simt_part_at(a, 0, c, c0 + q, i)];
-            two_sum_add(v.x, v.y, acc_at(r, q));
-            dots[r] += simt_put_y(a, s, c, i, c0 + q, ai, s2, (double)v.x + (double)v.y,
+            double v = (double)acc_at(r, q);
+            if (paired) v = f.part[simt_part_at(a, 0, c, c0 + q, i)] + v;
+            dots[r] += simt_put_y(a, s, c, i, c0 + q, ai, s2, v,
                                   MP <= 2 ? vi[r][q % PV] : a.V[(vbase + i) * a.m + c0 + q]);
           }
       }
