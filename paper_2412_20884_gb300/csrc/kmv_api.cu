@@ -269,33 +269,55 @@ kmv_status cheb_prepare(kmv_handle h, const kmv_points* pts, const double* theta
 // --- building blocks used by several entry points -------------------------------------
 
 // The FP32 kernels' scratch: `bytes` of partial sums and `counters` zeroed counters.
+// KMV_ENOMEM (no message recorded) when they are not there and cannot be had, under
+// capture above all: the caller then takes the plan of one unit.
 kmv_status simt_scratch(kmv_handle h, size_t bytes, size_t counters, cudaStream_t st) {
-  if (bytes <= h->simt_part_bytes && counters <= h->simt_counters) return KMV_OK;
-  if (h->capturing)
-    return fail(h, KMV_EINVAL, "FP32 scratch not prepared: make the same call once before capturing");
-  auto grow = [&](void** p, size_t want) {
-    void* n = nullptr;
-    if (cudaMalloc(&n, want) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
+  if (bytes > h->simt_part_bytes || counters > h->simt_counters) {
+    if (h->capturing) return KMV_ENOMEM;
+    // replaces *p (of `have` bytes) by `want` bytes, or `least` if those are not to be had
+    auto grow = [&](void** p, size_t& have, size_t want, size_t least) -> kmv_status {
+      if (*p && h->simt_captured) {
+        try {
+          h->simt_retired.push_back(*p);
+        } catch (const std::bad_alloc&) {
+          return KMV_ENOMEM;
+        }
+        h->simt_retired_bytes += have;
+      } else if (*p) {
+        KMV_CUDA(h, cudaFree(*p));
+      }
+      *p = nullptr;
+      have = 0;
+      for (size_t size : {want, least}) {
+        if (cudaMalloc(p, size) == cudaSuccess) {
+          have = size;
+          return KMV_OK;
+        }
+        cudaGetLastError();
+        *p = nullptr;
+      }
+      return KMV_ENOMEM;
+    };
+    if (bytes > h->simt_part_bytes) {
+      const size_t twice = std::min<size_t>(2 * h->simt_part_bytes, (size_t)kSimtPartMax);
+      KMV_TRY(grow(reinterpret_cast<void**>(&h->simt_part), h->simt_part_bytes, std::max(bytes, twice), bytes));
     }
-    if (*p) h->simt_retired.push_back(*p);
-    *p = n;
-    return true;
-  };
-  if (bytes > h->simt_part_bytes) {
-    size_t want = std::max(bytes, 2 * h->simt_part_bytes);
-    if (!grow(reinterpret_cast<void**>(&h->simt_part), want)) return fail(h, KMV_ENOMEM, "FP32 scratch allocation failed");
-    h->simt_part_bytes = want;
+    if (counters > h->simt_counters) {
+      size_t have = sizeof(uint32_t) * h->simt_counters;
+      const kmv_status s = grow(reinterpret_cast<void**>(&h->simt_count), have,
+                                sizeof(uint32_t) * std::max(counters, 2 * h->simt_counters), sizeof(uint32_t) * counters);
+      h->simt_counters = have / sizeof(uint32_t);
+      KMV_TRY(s);
+      KMV_CUDA(h, cudaMemsetAsync(h->simt_count, 0, have, st));
+    }
   }
-  if (counters > h->simt_counters) {
-    const size_t want = std::max(counters, 2 * h->simt_counters);
-    if (!grow(reinterpret_cast<void**>(&h->simt_count), sizeof(uint32_t) * want))
-      return fail(h, KMV_ENOMEM, "FP32 scratch allocation failed");
-    h->simt_counters = want;
-    KMV_CUDA(h, cudaMemsetAsync(h->simt_count, 0, sizeof(uint32_t) * want, st));
-  }
+  if (h->capturing && (bytes > 0 || counters > 0)) h->simt_captured = true;
   return KMV_OK;
+}
+
+kmv_status no_simt_scratch(kmv_handle h) {
+  return h->capturing ? fail(h, KMV_EINVAL, "FP32 scratch not prepared: make the same call once before capturing")
+                      : fail(h, KMV_ENOMEM, "FP32 scratch allocation failed");
 }
 
 // The FP32 forward (kmv_simt_fwd.cu).
@@ -304,19 +326,26 @@ kmv_status simt_forward(kmv_handle h, const KmvArgs& a, cudaStream_t st) {
   if (L.n_items == 0) return KMV_OK;
   if ((a.cg_sys || a.pcg_sys || a.ms_sys) && !(a.m == 1 && a.dot_partial))
     return fail(h, KMV_EINVAL, "internal: fused CG step needs the one-column product");
-  SimtFwd f = simt_fwd_plan(h->simt_tiles, L.n_inst, L.n_items, L.chains, L.n_total, (int64_t)L.max_items_per_inst * kTile, a.d,
-                            a.m, h->num_sms);
-  KMV_TRY(simt_scratch(h, simt_fwd_part_bytes(f, L.chains, L.n_total, a.m), simt_fwd_counters(f, L.chains), st));
+  SimtFwd f;
+  auto take = [&](bool one_unit) {
+    f = simt_fwd_plan(h->simt_tiles, L.n_inst, L.n_items, L.chains, L.n_total, (int64_t)L.max_items_per_inst * kTile, a.d,
+                      a.m, h->num_sms, one_unit);
+    return simt_scratch(h, simt_fwd_part_bytes(f, L.chains, L.n_total, a.m), simt_fwd_counters(f, L.chains), st);
+  };
+  kmv_status got = take(false);
+  if (got == KMV_ENOMEM && f.upc > 1) got = take(true);
+  if (got == KMV_ENOMEM) return no_simt_scratch(h);
+  KMV_TRY(got);
   f.part = h->simt_part;
   f.count = h->simt_count;
   KMV_CUDA(h, launch_forward_simt(a, f, L.n_items, st));
   return KMV_OK;
 }
 
-SimtBwd bwd_plan(kmv_handle h, int m, bool want_gv) {
+SimtBwd bwd_plan(kmv_handle h, int m, bool want_gv, bool one_unit) {
   const Layout& L = h->layout;
   return simt_bwd_plan(h->simt_tiles, L.n_items, L.chains, L.n_total, (int64_t)L.max_items_per_inst * kTile, L.d, m,
-                       want_gv, h->num_sms);
+                       want_gv, h->num_sms, one_unit);
 }
 
 kmv_status run_forward(kmv_handle h, const KmvArgs& a, kmv_precision prec, cudaStream_t st) {
@@ -332,9 +361,15 @@ kmv_status run_forward(kmv_handle h, const KmvArgs& a, kmv_precision prec, cudaS
   return KMV_OK;
 }
 
-size_t backward_ws_bytes(kmv_handle h, int m, bool want_gv) {
+// The adjoint's partial sums, the last region of a call's workspace.  Under capture, where
+// the workspace cannot grow, the plan of one unit (fewer partials) if theirs do not fit.
+size_t take_backward(kmv_handle h, Arena& ar, int m, bool want_gv) {
   const Layout& L = h->layout;
-  return sizeof(double) * simt_bwd_partials(bwd_plan(h, m, want_gv), L.n_items, L.chains, L.n_theta);
+  auto bytes = [&](bool one_unit) {
+    return sizeof(double) * simt_bwd_partials(bwd_plan(h, m, want_gv, one_unit), L.n_items, L.chains, L.n_theta);
+  };
+  h->bwd_one_unit = h->capturing && ar.used + bytes(false) > h->ws_bytes;
+  return ar.take(bytes(h->bwd_one_unit));
 }
 
 kmv_status run_backward_stationary(kmv_handle h, KmvArgs a, double* grad, double* partial,
@@ -346,8 +381,12 @@ kmv_status run_backward_stationary(kmv_handle h, KmvArgs a, double* grad, double
     const kmv_status s = tc_backward(h, a, grad, st);
     if (s != KMV_EUNSUPPORTED) return s;
   }
-  SimtBwd f = bwd_plan(h, a.m, a.Y != nullptr);
-  if (a.Y && L.n_items > 0) KMV_TRY(simt_scratch(h, simt_bwd_part_bytes(f, L.chains, L.n_total, a.m), 0, st));
+  SimtBwd f = bwd_plan(h, a.m, a.Y != nullptr, h->bwd_one_unit);
+  if (a.Y && L.n_items > 0) {
+    const kmv_status got = simt_scratch(h, simt_bwd_part_bytes(f, L.chains, L.n_total, a.m), 0, st);
+    if (got == KMV_ENOMEM) f = bwd_plan(h, a.m, true, true);   // needs no scratch
+    else KMV_TRY(got);
+  }
   f.part = h->simt_part;
   a.n_z = f.nz;
   a.grad_partial = partial;
@@ -1206,7 +1245,9 @@ const char* kmv_status_string(kmv_status s) {
 const char* kmv_last_error(kmv_handle h) { return h ? h->last_error.c_str() : ""; }
 
 int64_t kmv_workspace_bytes(kmv_handle h) {
-  return h ? (int64_t)(h->ws_bytes + h->tables_bytes + h->cheb_bytes + tc_workspace_bytes(h)) : 0;
+  return h ? (int64_t)(h->ws_bytes + h->tables_bytes + h->cheb_bytes + tc_workspace_bytes(h) + h->simt_part_bytes +
+                       sizeof(uint32_t) * h->simt_counters + h->simt_retired_bytes)
+           : 0;
 }
 
 kmv_status kmv_forward(kmv_handle h, const kmv_points* pts, int32_t chains, const double* theta,
@@ -1239,7 +1280,7 @@ kmv_status kmv_backward(kmv_handle h, const kmv_points* pts, int32_t chains, con
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   KMV_TRY(prepare_layout(h, pts, chains, st));
   Arena ar;
-  const size_t o_part = ar.take(backward_ws_bytes(h, m, grad_V != nullptr));
+  const size_t o_part = take_backward(h, ar, m, grad_V != nullptr);
   KMV_TRY(reserve(h, ar.used));
   KMV_TRY(cheb_prepare(h, pts, theta, m, st));
   KmvArgs a = base_args(h, pts, theta);
@@ -1432,7 +1473,7 @@ kmv_status leapfrog_step(kmv_handle h, const kmv_points* pts, int32_t chains, co
   const size_t vec2 = sizeof(float) * 2 * (size_t)L.chains * std::max<int64_t>(1, L.n_total);
   const size_t o_vf = ar.take(vec2);
   const size_t o_gf = ar.take(vec2);
-  const size_t o_bp = ar.take(backward_ws_bytes(h, 2, false));
+  const size_t o_bp = take_backward(h, ar, 2, false);
   KMV_TRY(reserve(h, ar.used));
   double* theta_h = at<double>(h, o_th);
   double* grad = at<double>(h, o_gr);
@@ -1487,7 +1528,6 @@ kmv_status kmv_implicit_step(kmv_handle h, const kmv_points* pts, int32_t chains
   const size_t o_th0 = ar.take(sizeof(double) * n_sys * n), o_pi0 = ar.take(sizeof(double) * n_sys * n);
   const size_t o_tb = ar.take(sizeof(double) * n_sys * n), o_gr = ar.take(sizeof(double) * n_sys * n);
   const size_t o_vf = ar.take(sizeof(float) * 2 * vec), o_gf = ar.take(sizeof(float) * 2 * vec);
-  const size_t o_bp = ar.take(backward_ws_bytes(h, 2, false));
   const size_t o_q = ar.take(sizeof(float) * vec), o_r = ar.take(sizeof(float) * vec), o_z = ar.take(sizeof(float) * vec);
   const size_t o_gx = ar.take(sizeof(float) * vec * k), o_fx = ar.take(sizeof(float) * vec * k);
   const size_t o_gtp = ar.take(sizeof(double) * (size_t)k * n_sys * 2 * n);
@@ -1500,6 +1540,7 @@ kmv_status kmv_implicit_step(kmv_handle h, const kmv_points* pts, int32_t chains
   const size_t o_proj = ar.take(sizeof(double) * items * rank), o_coef = ar.take(sizeof(double) * n_sys * rank);
   const size_t o_prz = ar.take(sizeof(double) * items), o_fac = ar.take(sizeof(double) * n_sys * rank);
   const size_t o_brr = ar.take(sizeof(double) * n_sys), o_bit = ar.take(sizeof(int32_t) * n_sys);
+  const size_t o_bp = take_backward(h, ar, 2, false);
   KMV_TRY(reserve(h, ar.used));
   double* th0 = at<double>(h, o_th0);
   double* pi0 = at<double>(h, o_pi0);

@@ -182,11 +182,14 @@ struct SimtFwd {
   int folds, upc;            // folds (512 columns) per unit, units per chunk
   int max_units;             // js * upc; 1: every CTA writes its rows' Y itself
   int ticket;                // the last unit of a tile adds the units and writes Y; else the combine kernel does
-  double* part;              // (max_units, chains, m, N_total) sums, for several units or folds
+  double* part;              // (max_units, chains, m, N_total) sums, for several units
   uint32_t* count;           // ticket: one zeroed counter per (tile, chain, column chunk)
 };
+// Most bytes of one call's J-unit sums (js > 1 only at sizes that stay below 20 MB).
+constexpr int64_t kSimtPartMax = int64_t(512) << 20;
+// one_unit: the plan that needs no scratch (for js == 1), where there is none to be had.
 SimtFwd simt_fwd_plan(const SimtTiles& T, int n_inst, int n_items, int chains, int64_t n_total, int64_t max_rows, int d, int m,
-                      int num_sms);
+                      int num_sms, bool one_unit);
 size_t simt_fwd_part_bytes(const SimtFwd& f, int chains, int64_t n_total, int m);
 size_t simt_fwd_counters(const SimtFwd& f, int chains);
 cudaError_t launch_forward_simt(const KmvArgs& a, const SimtFwd& f, int n_items, cudaStream_t st);
@@ -196,11 +199,11 @@ struct SimtBwd {
   int n_tiles, rows, mp, nz;  // tiles, rows per thread, columns per CTA (the kernel's width), column chunks
   int chunk;                  // columns per chunk (<= mp): W_ij is summed per chunk
   int folds, units;           // folds (512 columns) per J unit, units
-  double* part;               // want_gv and several units or folds: (units, chains, m, N_total) sums
+  double* part;               // want_gv and several units: (units, chains, m, N_total) sums
 };
 int backward_mp(int m);      // columns per backward pass
 SimtBwd simt_bwd_plan(const SimtTiles& T, int n_items, int chains, int64_t n_total, int64_t max_rows, int d, int m,
-                      bool want_gv, int num_sms);
+                      bool want_gv, int num_sms, bool one_unit);
 // The plan of one unit per 128-row item, whose partials are (n_items, chains, n_z, n_theta)
 // and which needs no part (kmv_backward_noalloc).
 SimtBwd simt_bwd_plan_plain(int n_items, int d, int m);
@@ -477,16 +480,20 @@ struct kmv_handle_s {
   bool capturing = false;
   // stream on which the bodies of conditional (WHILE) graph nodes are captured
   cudaStream_t side = nullptr;
-  // FP32 kernels: wide row tiles of the layout; the J units' partial sums and the
-  // zeroed counters, grown on first use (not under capture).  Outgrown buffers are
-  // kept until the handle goes, for graphs captured with them; they at least double,
-  // so all of them together stay below twice the last.
+  // FP32 kernels: wide row tiles of the layout; the J units' partial sums (at most
+  // kSimtPartMax) and the zeroed counters, grown on first use (not under capture).
+  // Outgrown buffers are freed, or, once a graph has been captured with them, kept until
+  // the handle goes; buffers at least double up to kSimtPartMax, so all of them together
+  // stay below twice that.
   kmv::SimtTiles simt_tiles;
   double* simt_part = nullptr;
   size_t simt_part_bytes = 0;
   uint32_t* simt_count = nullptr;
   size_t simt_counters = 0;
   std::vector<void*> simt_retired;
+  size_t simt_retired_bytes = 0;
+  bool simt_captured = false;
+  bool bwd_one_unit = false;   // the FP32 adjoint of the current call takes one unit (take_backward)
   int num_sms = 0;   // of the device
   // kernel timing (kmv_profile_enable): event pairs around the main product kernels
   bool prof = false;

@@ -104,10 +104,10 @@ __global__ void __launch_bounds__(kGradThreads) grad_finalize_kernel(DevLayout L
 
 // Rows per thread and the number of J units: the wide variant once its finest split
 // (units of one fold) gives every SM two CTAs; then about 8 CTAs per SM, and with
-// dL/dV at most 512 MB of partial sums.  N = 20,000, d = 8, m = 16: 4.38 ms with one row
+// dL/dV at most kSimtPartMax bytes of partial sums (a single unit needs none).  N = 20,000, d = 8, m = 16: 4.38 ms with one row
 // per thread and no units, 1.10 ms now, with 0.03 ms for the sums of dL/dV and theta.
 SimtBwd simt_bwd_plan(const SimtTiles& T, int n_items, int chains, int64_t n_total, int64_t max_rows, int d, int m,
-                      bool want_gv, int num_sms) {
+                      bool want_gv, int num_sms, bool one_unit) {
   SimtBwd f = simt_bwd_plan_plain(n_items, d, m);
   const int R = bwd_rows(dim_class(d), f.mp);
   const int64_t fpc = std::max<int64_t>(1, (max_rows + kFoldTiles * kTile - 1) / (kFoldTiles * kTile));
@@ -121,7 +121,8 @@ SimtBwd simt_bwd_plan(const SimtTiles& T, int n_items, int chains, int64_t n_tot
   int64_t units = std::min<int64_t>(fpc, std::max<int64_t>(1, (8 * (int64_t)num_sms + ctas - 1) / std::max<int64_t>(1, ctas)));
   units = std::min<int64_t>(units, std::max(1, 65535 / f.nz));
   const int64_t bytes = want_gv ? (int64_t)sizeof(double) * chains * m * std::max<int64_t>(1, n_total) : 0;
-  while (units > 1 && bytes * units > (int64_t(512) << 20)) --units;
+  while (units > 1 && bytes * units > kSimtPartMax) --units;
+  if (one_unit) units = 1;
   f.folds = (int)((fpc + units - 1) / units);
   f.units = (int)((fpc + f.folds - 1) / f.folds);
   return f;
@@ -144,7 +145,7 @@ size_t simt_bwd_partials(const SimtBwd& f, int n_items, int chains, int n_theta)
   return (size_t)std::max(1, n_items) * chains * f.nz * f.units * n_theta;
 }
 size_t simt_bwd_part_bytes(const SimtBwd& f, int chains, int64_t n_total, int m) {
-  return f.units > 1 || (f.folds > 1 && f.rows > 1) ? sizeof(double) * (size_t)f.units * chains * m * (size_t)n_total : 0;
+  return f.units > 1 ? sizeof(double) * (size_t)f.units * chains * m * (size_t)n_total : 0;
 }
 
 template <int D>

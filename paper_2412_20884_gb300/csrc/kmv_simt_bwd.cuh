@@ -79,11 +79,16 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
   double* sgl = sg_store;
   if constexpr (kLocalG) asm volatile("" : "+l"(sgl));
   bool first_g = true;
-  // those of dL/dV: in registers with one row per thread, else in f.part
-  constexpr int RV = R == 1 ? MP : 1;
+  // those of dL/dV: in registers with one row per thread and few dimensions, else in
+  // local memory likewise
+  constexpr bool kRegV = R == 1 && D < 32;
+  constexpr int RV = kRegV ? MP : 1;
   double svp[RV];
 #pragma unroll
   for (int q = 0; q < RV; ++q) svp[q] = 0.0;
+  double gv_store[kRegV ? 1 : R * MP];
+  double* gv = gv_store;
+  asm volatile("" : "+l"(gv));
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int64_t i = r0 + r * kTile + tid;
@@ -106,11 +111,11 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
   }
 
   const uint32_t inv = dd > 1 ? 0xffffffffu / (uint32_t)dd + 1u : 0u;
-  const bool paired = je - jb > kFoldTiles * kTile;
+  const bool several = je - jb > kFoldTiles * kTile;
   bool first = true;
   // adds the FP32 sums of dL/dV of this thread's rows to the FP64 ones
   auto fold_v = [&]() {
-    if constexpr (R == 1) {
+    if constexpr (kRegV) {
 #pragma unroll
       for (int q = 0; q < RV; ++q) svp[q] += (double)accv_at(0, q);
 #pragma unroll
@@ -118,15 +123,10 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
     } else {
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        const int64_t i = r0 + r * kTile + tid;
-        if (i < o1) {
 #pragma unroll
-          for (int q = 0; q < MP; ++q)
-            if (q < mc) {
-              double* p = &f.part[(((size_t)u * a.chains + c) * a.m + c0 + q) * (size_t)a.n_total + i];
-              const double v = (double)accv_at(r, q);
-              *p = first ? v : *p + v;
-            }
+        for (int q = 0; q < MP; ++q) {
+          const double v = (double)accv_at(r, q);
+          gv[r * MP + q] = first ? v : gv[r * MP + q] + v;
         }
 #pragma unroll
         for (int q = 0; q < MP / 2; ++q) accv[r][q] = 0;
@@ -247,19 +247,29 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
       }
     }
     __syncthreads();
-    if (paired && jt + kJT < je && (step + 1) % (kFoldTiles * kTile / kJT) == 0) {
+    if (several && jt + kJT < je && (step + 1) % (kFoldTiles * kTile / kJT) == 0) {
       fold_g();
       if (want_gv) fold_v();
     }
   }
   fold_g();
   const bool direct = f.units == 1;
-  if (want_gv && (R == 1 || !direct || paired)) fold_v();
-  if (R == 1 && want_gv && !direct && r0 + tid < o1) {
+  // the FP64 sum of an element of dL/dV with the last FP32 sum added
+  auto gv_total = [&](int r, int q) {
+    const double v = (double)accv_at(r, q);
+    if constexpr (kRegV) return svp[q % RV] + v;
+    else return first ? v : gv[r * MP + q] + v;
+  };
+  if (want_gv && !direct) {
 #pragma unroll
-    for (int q = 0; q < RV; ++q)
-      if (q < mc)
-        f.part[(((size_t)u * a.chains + c) * a.m + c0 + q) * (size_t)a.n_total + r0 + tid] = svp[q];
+    for (int r = 0; r < R; ++r) {
+      const int64_t i = r0 + r * kTile + tid;
+      if (i < o1) {
+#pragma unroll
+        for (int q = 0; q < MP; ++q)
+          if (q < mc) f.part[(((size_t)u * a.chains + c) * a.m + c0 + q) * (size_t)a.n_total + i] = gv_total(r, q);
+      }
+    }
   }
 
   // noise gradient and, in a single unit, dL/dV
@@ -275,11 +285,7 @@ __global__ void __launch_bounds__(kTile) bwd_simt_kernel(KmvArgs a, SimtBwd f) {
           const int64_t idx = (vbase + i) * a.m + c0 + q;
           const double g = (double)a.G[idx];
           if (u == 0) noise += g * (double)a.V[idx];
-          if (want_gv && direct) {
-            double v = R == 1 ? svp[q % RV] : (double)accv_at(r, q);
-            if (R > 1 && paired) v = f.part[((size_t)c * a.m + c0 + q) * (size_t)a.n_total + i];
-            a.Y[idx] = (float)(ai * v + as2[1] * g);
-          }
+          if (want_gv && direct) a.Y[idx] = (float)(ai * gv_total(r, q) + as2[1] * g);
         }
       }
     }

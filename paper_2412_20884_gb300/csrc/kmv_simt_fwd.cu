@@ -95,7 +95,7 @@ int forward_jsplit(int n_items, int chains, int m, int64_t max_rows, int num_sms
 // J units in a kernel of its own (now by the last CTA of a tile to arrive, up to two
 // columns; with more columns that CTA's serial share costs more than a launch).
 SimtFwd simt_fwd_plan(const SimtTiles& T, int n_inst, int n_items, int chains, int64_t n_total, int64_t max_rows, int d, int m,
-                      int num_sms) {
+                      int num_sms, bool one_unit) {
   SimtFwd f{};
   const int D = dim_class(d);
   f.n_inst = n_inst;
@@ -113,10 +113,11 @@ SimtFwd simt_fwd_plan(const SimtTiles& T, int n_inst, int n_items, int chains, i
   f.n_tiles = !big ? n_items : R == 4 ? T.n4 : T.n2;
   const int64_t ctas = (int64_t)f.n_tiles * chains * f.nz * f.js;
   // about 8 CTAs per SM (two to four resident, so that the last wave is short), with at
-  // most 512 MB of partial sums
+  // most kSimtPartMax bytes of partial sums; a single unit (upc == 1 == js) needs none
   int64_t upc = std::min<int64_t>(fpc, std::max<int64_t>(1, (8 * (int64_t)num_sms + ctas - 1) / std::max<int64_t>(1, ctas)));
   const int64_t bytes = (int64_t)sizeof(double) * f.js * chains * m * std::max<int64_t>(1, n_total);
-  while (upc > 1 && bytes * upc > (int64_t(512) << 20)) --upc;
+  while (upc > 1 && bytes * upc > kSimtPartMax) --upc;
+  if (one_unit) upc = 1;
   f.folds = (int)((fpc + upc - 1) / upc);
   f.upc = (int)((fpc + f.folds - 1) / f.folds);
   f.max_units = f.js * f.upc;
@@ -125,7 +126,7 @@ SimtFwd simt_fwd_plan(const SimtTiles& T, int n_inst, int n_items, int chains, i
 }
 
 size_t simt_fwd_part_bytes(const SimtFwd& f, int chains, int64_t n_total, int m) {
-  return f.max_units > 1 || f.folds > 1 ? sizeof(double) * (size_t)f.max_units * chains * m * (size_t)n_total : 0;
+  return f.max_units > 1 ? sizeof(double) * (size_t)f.max_units * chains * m * (size_t)n_total : 0;
 }
 size_t simt_fwd_counters(const SimtFwd& f, int chains) { return f.ticket ? (size_t)f.n_tiles * chains * f.nz : 0; }
 

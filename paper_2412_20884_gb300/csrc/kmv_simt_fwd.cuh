@@ -247,22 +247,37 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
       vi[r][q] = (MP <= 2 && q < mc && i < o1) ? a.V[(vbase + i) * a.m + c0 + q] : 0.f;
     }
 
-  const bool paired = je - jb > kFoldTiles * kTile;   // several folds: sums kept in f.part
-  const int unit = jc * f.upc + u;
+  const bool several = je - jb > kFoldTiles * kTile;   // several folds in this unit
   bool first = true;
-  // adds the FP32 sums to the FP64 ones in global memory (this thread's own elements)
+  // The FP64 sums of several folds: in registers with one row per thread, else in the
+  // thread's local memory, since R * MP doubles do not fit beside the loop's registers and
+  // global memory for them (twice the size of V) is not to be asked of a call with one
+  // unit per row.  The pointer is hidden from the compiler, which would put the array
+  // into registers.
+  constexpr bool kInRegs = R == 1 && MP <= 32;
+  double run[kInRegs ? MP : 1], sums_store[kInRegs ? 1 : R * MP];
+  double* sums = sums_store;
+  if constexpr (kInRegs) {
+#pragma unroll
+    for (int q = 0; q < MP; ++q) run[q] = 0.0;
+  } else {
+    asm volatile("" : "+l"(sums));
+  }
+  // the sum of an element so far, with the FP32 sum added
+  auto total = [&](int r, int q) {
+    const double v = (double)acc_at(r, q);
+    if constexpr (kInRegs)
+      return several ? run[q] + v : v;
+    else
+      return first ? v : sums[r * MP + q] + v;
+  };
   auto fold = [&]() {
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      const int64_t i = r0 + r * kTile + tid;
-      if (i < o1) {
 #pragma unroll
-        for (int q = 0; q < MP; ++q)
-          if (q < mc) {
-            double* p = &f.part[simt_part_at(a, unit, c, c0 + q, i)];
-            const double v = (double)acc_at(r, q);
-            *p = first ? v : *p + v;
-          }
+      for (int q = 0; q < MP; ++q) {
+        if constexpr (kInRegs) run[q] = total(r, q);
+        else sums[r * MP + q] = total(r, q);
       }
 #pragma unroll
       for (int q = 0; q < NP; ++q) acc[r][q] = 0;
@@ -349,7 +364,7 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
     }
     if (more) store(buf ^ 1);
     __syncthreads();
-    if (paired && more && (step + 1) % (kFoldTiles * kTile / kJT) == 0) fold();
+    if (several && more && (step + 1) % (kFoldTiles * kTile / kJT) == 0) fold();
   }
 
   const int n_it = min(R, a.L.inst_item0[b + 1] - item0);
@@ -365,9 +380,7 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
 #pragma unroll
         for (int q = 0; q < MP; ++q)
           if (q < mc) {
-            double v = (double)acc_at(r, q);
-            if (paired) v = f.part[simt_part_at(a, 0, c, c0 + q, i)] + v;
-            dots[r] += simt_put_y(a, s, c, i, c0 + q, ai, s2, v,
+            dots[r] += simt_put_y(a, s, c, i, c0 + q, ai, s2, total(r, q),
                                   MP <= 2 ? vi[r][q % PV] : a.V[(vbase + i) * a.m + c0 + q]);
           }
       }
@@ -375,7 +388,16 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
     if (a.dot_partial) simt_put_dots<R>(a, b, c, s, item0, n_it, dots, red, &s_flag);
     return;
   }
-  fold();
+  const int unit = jc * f.upc + u;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int64_t i = r0 + r * kTile + tid;
+    if (i < o1) {
+#pragma unroll
+      for (int q = 0; q < MP; ++q)
+        if (q < mc) f.part[simt_part_at(a, unit, c, c0 + q, i)] = total(r, q);
+    }
+  }
   if (!f.ticket) return;
   // the tile's last unit to finish adds the units in order
   __syncthreads();
