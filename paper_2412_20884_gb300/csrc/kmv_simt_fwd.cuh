@@ -131,8 +131,12 @@ __device__ __forceinline__ void simt_put_dots(const KmvArgs& a, int b, int c, in
   if (*s_flag) cg_finish_pq(a.L, a, b, c, s, red);
 }
 
+// Least CTAs per SM asked of the compiler (0: none): at 3 and 4 dimensions it took 132 and
+// 138 registers, three CTAs, for 16 columns (N = 3000, d = 3, m = 32: 47 against 31 us).
+constexpr int fwd_min_ctas(int D, int MP, int R) { return R == 1 && MP == 16 && (D == 3 || D == 4) ? 4 : 0; }
+
 template <int D, int MP, int R>
-__global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
+__global__ void __launch_bounds__(kTile, fwd_min_ctas(D, MP, R)) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
   chain_trigger();
   if (a.chained == 2) chain_wait();
   const int dd = a.d;   // <= D; the dimensions past it are zero and add nothing
@@ -249,12 +253,13 @@ __global__ void __launch_bounds__(kTile) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
 
   const bool several = je - jb > kFoldTiles * kTile;   // several folds in this unit
   bool first = true;
-  // The FP64 sums of several folds: in registers with one row per thread, else in the
-  // thread's local memory, since R * MP doubles do not fit beside the loop's registers and
-  // global memory for them (twice the size of V) is not to be asked of a call with one
-  // unit per row.  The pointer is hidden from the compiler, which would put the array
-  // into registers.
-  constexpr bool kInRegs = R == 1 && MP <= 32;
+  // The FP64 sums of several folds: in the thread's local memory, since R * MP doubles do
+  // not fit beside the loop's registers and global memory for them (twice the size of V)
+  // is not to be asked of a call with one unit per row.  The pointer is hidden from the
+  // compiler, which would put the array into registers (N = 3000, d = 16, m = 4: 26 against
+  // 20 us).  In registers for one row per thread, wide chunks and few dimensions, where
+  // the loop has room for them (N = 300, d = 16, m = 32: 28 against 44 us).
+  constexpr bool kInRegs = R == 1 && MP >= 16 && 2 * D <= MP;
   double run[kInRegs ? MP : 1], sums_store[kInRegs ? 1 : R * MP];
   double* sums = sums_store;
   if constexpr (kInRegs) {
