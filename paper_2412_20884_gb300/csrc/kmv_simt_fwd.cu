@@ -17,6 +17,7 @@ extern template cudaError_t fwd_launch_d<12>(const KmvArgs&, const SimtFwd&, dim
 extern template cudaError_t fwd_launch_d<16>(const KmvArgs&, const SimtFwd&, dim3, cudaStream_t);
 extern template cudaError_t fwd_launch_d<24>(const KmvArgs&, const SimtFwd&, dim3, cudaStream_t);
 extern template cudaError_t fwd_launch_d<32>(const KmvArgs&, const SimtFwd&, dim3, cudaStream_t);
+extern template cudaError_t fwd_launch_d<48>(const KmvArgs&, const SimtFwd&, dim3, cudaStream_t);
 extern template cudaError_t fwd_launch_d<64>(const KmvArgs&, const SimtFwd&, dim3, cudaStream_t);
 
 // Adds the units' sums and writes Y, 128 rows and kCombineCols columns at a time.
@@ -45,22 +46,26 @@ __global__ void __launch_bounds__(kTile) fwd_simt_combine_kernel(KmvArgs a, Simt
 
 namespace {
 
-constexpr int kDims[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 64};
+constexpr int kDims[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
 int dim_class(int d) {
   for (int v : kDims)
     if (d <= v) return v;
   return 0;
 }
 
-// Columns per CTA: the width with the least time over all chunks.  Per row and pair a
+// Columns per CTA: the width with the least time over all chunks (above 32 dimensions
+// with their number: `row_ctas` CTAs per chunk count as one wave up to two per SM, so that
+// a small set is split over more CTAs: N = 1000, d = 64, m = 64 takes 54 us, 99 us with the
+// widest chunk).  Per row and pair a
 // chunk takes (2 D + mp + 6) / 4 clocks of the SM's FMA pipe (6: the exponential and
 // the loop around it) and its R rows share (D + mp) clocks of shared-memory loads.
-int fwd_width(int D, int m) {
+int fwd_width(int D, int m, double row_ctas, int num_sms) {
   int best = 1;
   double cost = -1.0;
-  for (int mp = 1; mp <= fwd_most_columns(D); mp *= 2) {
+  for (int mp = D > 32 ? std::min(16, pow2ceil(m)) : 1; mp <= fwd_most_columns(D); mp *= 2) {
     const double fma = (2.0 * D + mp + 6.0) / 4.0, lds = (double)(D + mp) / fwd_rows(D, mp);
-    const double c = ((m + mp - 1) / mp) * std::max(fma, lds);
+    const double nz = (m + mp - 1) / mp;
+    const double c = (D > 32 ? std::max(1.0, nz * row_ctas / (2.0 * num_sms)) : nz) * std::max(fma, lds);
     if (cost < 0.0 || c < cost) {
       cost = c;
       best = mp;
@@ -99,9 +104,9 @@ SimtFwd simt_fwd_plan(const SimtTiles& T, int n_inst, int n_items, int chains, i
   SimtFwd f{};
   const int D = dim_class(d);
   f.n_inst = n_inst;
-  f.mp = fwd_width(D, m);
-  f.nz = (m + f.mp - 1) / f.mp;
   f.js = forward_jsplit(n_items, chains, m, max_rows, num_sms);
+  f.mp = fwd_width(D, m, (double)n_items * chains * f.js, num_sms);
+  f.nz = (m + f.mp - 1) / f.mp;
   const int64_t n_jt = (max_rows + kJT - 1) / kJT, per = (n_jt + f.js - 1) / f.js;
   const int64_t fpc = std::max<int64_t>(1, (per * kJT + kFoldTiles * kTile - 1) / (kFoldTiles * kTile));
   const int R = fwd_rows(D, f.mp);
@@ -149,6 +154,7 @@ cudaError_t launch_forward_simt(const KmvArgs& a, const SimtFwd& plan, int n_ite
       case 16: e = fwd_launch_d<16>(a, f, grid, st); break;
       case 24: e = fwd_launch_d<24>(a, f, grid, st); break;
       case 32: e = fwd_launch_d<32>(a, f, grid, st); break;
+      case 48: e = fwd_launch_d<48>(a, f, grid, st); break;
       case 64: e = fwd_launch_d<64>(a, f, grid, st); break;
     }
     if (e != cudaSuccess) return e;

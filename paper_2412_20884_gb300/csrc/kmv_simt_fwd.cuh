@@ -135,6 +135,8 @@ __device__ __forceinline__ void simt_put_dots(const KmvArgs& a, int b, int c, in
 // 138 registers, three CTAs, for 16 columns (N = 3000, d = 3, m = 32: 47 against 31 us).
 constexpr int fwd_min_ctas(int D, int MP, int R) { return R == 1 && MP == 16 && (D == 3 || D == 4) ? 4 : 0; }
 
+__host__ __device__ constexpr int fwd_buffers(int D, int MP) { return 8 * (D * kXS + kJT * MP) <= 47 * 1024 ? 2 : 1; }
+
 template <int D, int MP, int R>
 __global__ void __launch_bounds__(kTile, fwd_min_ctas(D, MP, R)) fwd_simt_kernel(KmvArgs a, SimtFwd f) {
   chain_trigger();
@@ -154,8 +156,10 @@ __global__ void __launch_bounds__(kTile, fwd_min_ctas(D, MP, R)) fwd_simt_kernel
   if (t1 <= t0) return;   // an empty unit: the last ones of a short instance
   const int64_t jb = o0 + (int64_t)t0 * kJT, je = min(o1, o0 + (int64_t)t1 * kJT);
 
-  __shared__ __align__(16) float sx[2][D * kXS];
-  __shared__ __align__(16) float sv[2][kJT * MP];
+  // two buffers where they fit the 48 KB of static shared memory
+  constexpr int NB = fwd_buffers(D, MP);
+  __shared__ __align__(16) float sx[NB][D * kXS];
+  __shared__ __align__(16) float sv[NB][kJT * MP];
   __shared__ float sc[D];
   __shared__ double as2[2];
   __shared__ double red[kTile / 32];
@@ -232,7 +236,7 @@ __global__ void __launch_bounds__(kTile, fwd_min_ctas(D, MP, R)) fwd_simt_kernel
   load_scale(th, dd, a.ard, sc);
   if ((f.max_units == 1 || f.ticket) && tid >= 96 && tid < 98) as2[tid - 96] = exp(th[tid == 96 ? 0 : a.n_theta - 1]);
   if (dd < D)
-    for (int e = tid; e < (D - dd) * kXS; e += kTile) sx[0][dd * kXS + e] = sx[1][dd * kXS + e] = 0.f;
+    for (int e = tid; e < (D - dd) * kXS; e += kTile) sx[0][dd * kXS + e] = sx[NB - 1][dd * kXS + e] = 0.f;
   __syncthreads();
 #pragma unroll
   for (int r = 0; r < R; ++r)
@@ -294,7 +298,7 @@ __global__ void __launch_bounds__(kTile, fwd_min_ctas(D, MP, R)) fwd_simt_kernel
   __syncthreads();
   int step = 0;
   for (int64_t jt = jb; jt < je; jt += kJT, ++step) {
-    const int buf = step & 1;
+    const int buf = NB == 2 ? step & 1 : 0;
     const bool more = jt + kJT < je;
     if (more) {
       fetch_x(jt + kJT);
@@ -367,7 +371,8 @@ __global__ void __launch_bounds__(kTile, fwd_min_ctas(D, MP, R)) fwd_simt_kernel
         }
       }
     }
-    if (more) store(buf ^ 1);
+    if (NB == 1) __syncthreads();   // the one buffer has been read
+    if (more) store(NB == 2 ? buf ^ 1 : 0);
     __syncthreads();
     if (several && more && (step + 1) % (kFoldTiles * kTile / kJT) == 0) fold();
   }
@@ -429,10 +434,11 @@ __global__ void __launch_bounds__(kTile, fwd_min_ctas(D, MP, R)) fwd_simt_kernel
 // the probabilities of four points stay below the 255 of a thread).
 constexpr int fwd_rows(int D, int MP) { return D <= 8 || (D <= 16 && MP <= 16) ? 4 : D <= 32 ? 2 : 1; }
 
-// The widest chunk built: 32 columns where the distances cost as much as they do (and
-// the staged tiles fit 48 KB); below, two 16-column chunks of four rows are cheaper
-// than one of 32 columns and two rows.
-constexpr int fwd_most_columns(int D) { return D >= 16 && D <= 32 ? 32 : 16; }
+// The widest chunk built: 32 columns where the distances cost as much as they do (one
+// chunk of 64 was no faster than two of 32: 1.02 against 0.93 ms at N = 9001, d = 33,
+// m = 64, and four of 16, padded to 64 dimensions, took 3.41 ms); below, two 16-column
+// chunks of four rows are cheaper than one of 32 columns and two rows.
+constexpr int fwd_most_columns(int D) { return D >= 16 ? 32 : 16; }
 
 template <int D, int MP>
 cudaError_t fwd_launch_mp(const KmvArgs& a, const SimtFwd& f, dim3 grid, cudaStream_t st) {
@@ -454,9 +460,10 @@ cudaError_t fwd_launch_d(const KmvArgs& a, const SimtFwd& f, dim3 grid, cudaStre
     case 4: return fwd_launch_mp<D, 4>(a, f, grid, st);
     case 8: return fwd_launch_mp<D, 8>(a, f, grid, st);
     case 16: return fwd_launch_mp<D, 16>(a, f, grid, st);
-    default:
-      if constexpr (fwd_most_columns(D) == 32) return fwd_launch_mp<D, 32>(a, f, grid, st);
+    case 32:
+      if constexpr (fwd_most_columns(D) >= 32) return fwd_launch_mp<D, 32>(a, f, grid, st);
       return cudaErrorInvalidValue;
+    default: return cudaErrorInvalidValue;
   }
 }
 
