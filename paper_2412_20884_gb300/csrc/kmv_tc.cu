@@ -351,6 +351,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) tc_fwd_kernel(TcFwdArgs a) {
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
             two_sum_add(v[q].x, v[q].y, __uint_as_float(o[q]));
+            // a column of V with an infinity: the sum is infinite, its error (inf - inf) not NaN
+            if (isinf(v[q].x)) v[q].y = 0.f;
             if (c0 + q < a.mz) {
               double* pd = &a.part[part_idx(t, a.mz, c0 + q, rowp)];
               if (last && fresh)

@@ -59,3 +59,16 @@ def test_sums_above_fp32_range(kmv_handle, n, chains, d, m):
     one = torch.full_like(V, 1e-35)
     gV = kmv_handle.kmv_backward(pts, theta, one, V, prec="fp32")[1][0, rows].cpu().numpy()
     assert np.max(np.abs(gV - ref) / ref) <= TOL["fp32"][0]
+
+
+def test_infinite_entries_in_the_wide_tensor_core_form(kmv_handle):
+    # 20 columns, 8 chains of 20,000 rows: items of more than 32 J tiles, whose sums over
+    # 4096 columns are folded several times; K0 >= 0.88 keeps every probability positive
+    n, chains, m = 20000, 8, 20
+    rng, _, _, pts, theta = _inputs(n, chains, 3, 0.0, 7200)
+    V = torch.tensor(0.1 + rng.random((chains, n, m)), dtype=torch.float32, device="cuda")
+    V[0, n // 3, 0] = float("inf")
+    Y = kmv_handle.kmv_forward(pts, theta, V, prec="bf16_hilo")
+    assert torch.all(Y[0, :, 0] == float("inf"))
+    Y[0, :, 0] = 0.0
+    assert torch.all(torch.isfinite(Y))
