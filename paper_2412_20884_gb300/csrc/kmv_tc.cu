@@ -1058,7 +1058,10 @@ __global__ void __launch_bounds__(kFmaThreads, 1) tc_fwd_fma_kernel(TcFwdArgs a)
       }
       ++it;
     }
-  fma_exp_out:;
+  fma_exp_out:
+    // a wait that gave up leaves the chunk loaded ahead in flight: the tensor memory is freed
+    // below only when every load from it is done
+    tmem_ld_wait();
   }
 
   tc_fence_before();
