@@ -484,6 +484,20 @@ struct Poll {
     slot ^= 1;
     return KMV_OK;
   }
+  // The count of the last test, before the next one is due.
+  kmv_status look(kmv_handle h) {
+    KMV_CUDA(h, cudaEventSynchronize(h->poll_ev[slot ^ 1]));
+    done = (h->host_flag + 8)[slot ^ 1] == 0;
+    return KMV_OK;
+  }
+  // At the start of iteration `it`.  The first count is looked at after one iteration, not
+  // after kCheckEvery: a solve that starts converged (a zero right-hand side, a good warm
+  // start) then queues one masked iteration, not four, and the GPU has that one to work on
+  // while the host waits.
+  kmv_status test(kmv_handle h, const int32_t* n_active, int it, cudaStream_t st) {
+    if (it % kCheckEvery == 0) return step(h, n_active, st);
+    return it == 1 ? look(h) : KMV_OK;
+  }
 };
 
 struct CgBufs {
@@ -601,10 +615,8 @@ kmv_status run_cg(kmv_handle h, const kmv_points* pts, const double* theta, cons
   } else {
     Poll poll;
     for (int it = 0; it < maxiter; ++it) {
-      if (it % kCheckEvery == 0) {
-        KMV_TRY(poll.step(h, B.n_active, st));
-        if (poll.done) break;
-      }
+      KMV_TRY(poll.test(h, B.n_active, it, st));
+      if (poll.done) break;
       KMV_TRY(iteration(st, (it > 0 || warm) ? 1 : 0));
     }
   }
@@ -722,10 +734,8 @@ kmv_status run_pcg(kmv_handle h, const kmv_points* pts, const double* theta, con
   } else {
     Poll poll;
     for (int it = 0; it < maxiter; ++it) {
-      if (it % kCheckEvery == 0) {
-        KMV_TRY(poll.step(h, B.n_active, st));
-        if (poll.done) break;
-      }
+      KMV_TRY(poll.test(h, B.n_active, it, st));
+      if (poll.done) break;
       KMV_TRY(iteration(st, (it > 0 || warm) ? 1 : 0));
     }
   }
@@ -983,10 +993,8 @@ kmv_status run_mcg(kmv_handle h, const kmv_points* pts, const double* theta, con
   const McgBetaHook hook{B.count + n_sys, B.cols, B.partial, tol, maxiter, B.n_active};
   Poll poll;
   for (int it = 0; it < maxiter; ++it) {
-    if (it % kCheckEvery == 0) {
-      KMV_TRY(poll.step(h, B.n_active, st));
-      if (poll.done) break;
-    }
+    KMV_TRY(poll.test(h, B.n_active, it, st));
+    if (poll.done) break;
     KMV_TRY(run_forward(h, a, prec, st));
     KMV_CUDA(h, launch_mcg_dot(h->dev, L.n_items, L.chains, L.n_total, m, B.p, B.q, B.sys_any, B.partial, B.count,
                                B.cols, pre ? 1 : 0, B.n_active, chained, st));
@@ -1139,10 +1147,8 @@ kmv_status run_mscg(kmv_handle h, const kmv_points* pts, const double* theta, co
   }
   Poll poll;
   for (int it = 0; it < maxiter; ++it) {
-    if (it % kCheckEvery == 0) {
-      KMV_TRY(poll.step(h, B.n_active, st));
-      if (poll.done) break;
-    }
+    KMV_TRY(poll.test(h, B.n_active, it, st));
+    if (poll.done) break;
     a.reuse_prep = it > 0;   // theta is fixed within the solve
     KMV_TRY(run_forward(h, a, prec, st));
     if (fused) {
