@@ -1,7 +1,9 @@
-// Per-system CG steps shared by the CG kernels (kmv_cg.cu) and the products'
-// epilogues when they carry the p.q step of a CG iteration (kmv_tc.cu,
-// kmv_simt_fwd.cu), so that every path takes the same arithmetic in the same
-// order.
+// Per-system CG steps shared by the CG kernels (kmv_cg.cu, kmv_pcg.cu, kmv_mscg.cu) and
+// the products' epilogues when they carry the p.q step of a CG iteration (kmv_tc.cu,
+// kmv_simt_fwd.cuh): every path takes the same steps from the same FP64 partials.  The
+// partials of a system are summed in a fixed order, which differs between the fused
+// paths (by the whole block that arrives last, sys_sum_block) and the separate kernels
+// (by one thread, sys_sum), so these agree to the sums' rounding and not in every bit.
 #pragma once
 
 #include "kmv_internal.cuh"

@@ -15,7 +15,8 @@ namespace kmv {
 // Rows per work item of the SIMT kernels and of the reductions built on them.
 constexpr int kTile = 128;
 constexpr int kMaxD = 64;
-// Columns of V handled by one SIMT pass (forward / backward).
+// Columns per CTA: the width that the FP32 forward's J chunks are counted for
+// (forward_jsplit; its kernel takes 16 to 64, fwd_most_columns) and the adjoint's most.
 constexpr int kMaxMPFwd = 64;
 constexpr int kMaxJSplit = 16;   // J-range chunks of the FP32 forward at small sizes
 constexpr int kMaxMPBwd = 32;
@@ -206,7 +207,7 @@ SimtBwd simt_bwd_plan(const SimtTiles& T, int n_items, int chains, int64_t n_tot
                       bool want_gv, int num_sms, bool one_unit);
 // The plan of one unit per 128-row item, whose partials are (n_items, chains, n_z, n_theta)
 // and which needs no part (kmv_backward_noalloc).
-SimtBwd simt_bwd_plan_plain(int n_items, int d, int m);
+SimtBwd simt_bwd_plan_plain(int n_items, int m);
 // Doubles of the gradient partials: (n_items, chains, nz, units, n_theta), a tile's at its first item.
 size_t simt_bwd_partials(const SimtBwd& f, int n_items, int chains, int n_theta);
 size_t simt_bwd_part_bytes(const SimtBwd& f, int chains, int64_t n_total, int m);

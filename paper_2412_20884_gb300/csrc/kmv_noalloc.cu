@@ -125,7 +125,7 @@ extern "C" kmv_status kmv_backward_noalloc(const kmv_points* pts, int32_t chains
   a.n_z = n_z;
   a.grad_partial = reinterpret_cast<double*>(base + o_part);
   // one unit per item: no scratch beyond the partials
-  const SimtBwd plan = simt_bwd_plan_plain((int)n_items, pts->d, m);
+  const SimtBwd plan = simt_bwd_plan_plain((int)n_items, m);
   if (n_items > 0 && launch_backward_simt(a, plan, (int)n_items, st) != cudaSuccess) return KMV_ECUDA;
   if (launch_grad_finalize(L, plan, pts->n_inst, chains, n_theta, theta, a.grad_partial, grad_theta, false, st) !=
       cudaSuccess)

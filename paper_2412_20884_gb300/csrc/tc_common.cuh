@@ -12,7 +12,7 @@
 
 namespace kmv {
 
-constexpr int kThreads = 320;      // 2 exp warpgroups + MMA warp + producer warp
+// Of the kernels with two exp warpgroups (warps 0-7).
 constexpr int kMmaWarp = 8;
 constexpr int kLoadWarp = 9;
 constexpr int kMaxKX = 112;        // d <= 35 (X operand width, BF16 elements)
