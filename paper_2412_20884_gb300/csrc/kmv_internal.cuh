@@ -184,6 +184,7 @@ struct SimtFwd {
   int max_units;             // js * upc; 1: every CTA writes its rows' Y itself
   int ticket;                // the last unit of a tile adds the units and writes Y; else the combine kernel does
   double* part;              // (max_units, chains, m, N_total) sums, for several units
+                             // (FP32 for a ticket's units of one fold)
   uint32_t* count;           // ticket: one zeroed counter per (tile, chain, column chunk)
 };
 // Most bytes of one call's J-unit sums (js > 1 only at sizes that stay below 20 MB).

@@ -90,6 +90,40 @@ __device__ __forceinline__ double simt_part_sum(const KmvArgs& a, const SimtFwd&
   return s;
 }
 
+// The same for units of one fold, which a product by ticket stores as the FP32 sums that
+// they are.  The FP64 pipe gives 2 lanes per clock and SM: 16 FP64 adds of 128 rows in a
+// small product's last CTA took 1.3 of its 8.7 us.  Here every addition's rounding error is
+// kept, and the errors' own in a third term, which is more than FP64's precision; sums
+// that leave FP32's range (and infinities) are taken again in FP64.
+__device__ __forceinline__ double simt_part_sum_f32(const KmvArgs& a, const SimtFwd& f, const SimtUnits& U, int c,
+                                                    int col, int64_t i) {
+  const size_t step = (size_t)a.chains * a.m * (size_t)a.n_total;
+  const float* p = reinterpret_cast<const float*>(f.part) + simt_part_at(a, 0, c, col, i);
+  const bool one_run = f.upc == 1 || U.in_chunk(0) == (uint32_t)f.upc;
+  const uint32_t runs = one_run ? 1 : U.n_chunks;
+  auto run_of = [&](uint32_t jc) { return f.upc == 1 ? U.n_chunks : one_run ? U.count() : U.in_chunk(jc); };
+  float s = 0.f, e = 0.f, e2 = 0.f;
+  for (uint32_t jc = 0; jc < runs; ++jc) {
+    const uint32_t n = run_of(jc);
+    for (uint32_t u0 = 0; u0 < n; u0 += 8) {
+      float v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = u0 + k < n ? __ldcg(p + (jc * f.upc + u0 + k) * step) : 0.f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        float err = 0.f;
+        two_sum_add(s, err, v[k]);
+        two_sum_add(e, e2, err);
+      }
+    }
+  }
+  if (isfinite(s)) return (double)s + ((double)e + (double)e2);
+  double t = 0.0;
+  for (uint32_t jc = 0; jc < runs; ++jc)
+    for (uint32_t u = 0, n = run_of(jc); u < n; ++u) t += (double)__ldcg(p + (jc * f.upc + u) * step);
+  return t;
+}
+
 // alpha and sigma^2 of a system: two lanes, one exp (an FP64 exp takes some 1100
 // clocks, and 2 lanes per clock and SM: once per CTA, not per thread).
 __device__ __forceinline__ void load_alpha_s2(const KmvArgs& a, int s, double* as2) {
@@ -399,13 +433,17 @@ __global__ void __launch_bounds__(kTile, fwd_min_ctas(D, MP, R)) fwd_simt_kernel
     return;
   }
   const int unit = jc * f.upc + u;
+  const bool f32_parts = f.ticket && f.folds == 1;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int64_t i = r0 + r * kTile + tid;
     if (i < o1) {
 #pragma unroll
       for (int q = 0; q < MP; ++q)
-        if (q < mc) f.part[simt_part_at(a, unit, c, c0 + q, i)] = total(r, q);
+        if (q < mc) {
+          if (MP <= 2 && f32_parts) reinterpret_cast<float*>(f.part)[simt_part_at(a, unit, c, c0 + q, i)] = acc_at(r, q);
+          else f.part[simt_part_at(a, unit, c, c0 + q, i)] = total(r, q);
+        }
     }
   }
   if (!f.ticket) return;
@@ -424,7 +462,10 @@ __global__ void __launch_bounds__(kTile, fwd_min_ctas(D, MP, R)) fwd_simt_kernel
       const double ai = a.amp ? alpha * (double)a.amp[vbase + i] : alpha;
 #pragma unroll
       for (int q = 0; q < PV; ++q)   // (ticket: at most two columns)
-        if (q < mc) dots[r] += simt_put_y(a, s, c, i, c0 + q, ai, s2, simt_part_sum(a, f, U, c, c0 + q, i), vi[r][q]);
+        if (q < mc) dots[r] += simt_put_y(a, s, c, i, c0 + q, ai, s2,
+                                            f32_parts ? simt_part_sum_f32(a, f, U, c, c0 + q, i)
+                                                      : simt_part_sum(a, f, U, c, c0 + q, i),
+                                            vi[r][q]);
     }
   }
   if (a.dot_partial) simt_put_dots<R>(a, b, c, s, item0, n_it, dots, red, &s_flag);
