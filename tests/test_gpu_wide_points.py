@@ -1,4 +1,4 @@
-"""The FP32 product of points with more than 32 dimensions: parity at the edges of its
+"""The FP32 product and adjoint of points with more than 32 dimensions: parity at the edges of its
 dimension classes (48, 64) and column widths (16, 32), and the time of wide V."""
 import numpy as np
 import pytest
@@ -7,7 +7,7 @@ import torch
 import workloads as wl
 from helpers import abs_row_products, componentwise_err, f32, to_dev
 from oracle import se_kernel as sk
-from test_gpu_kmv import TOL, _check_forward
+from test_gpu_kmv import TOL, _check_backward, _check_forward
 
 pytestmark = pytest.mark.gpu
 
@@ -30,6 +30,13 @@ def test_forward_of_large_sets(kmv_handle, d, m):
         ref = sk.kmv(X, w.theta[c], Vh[c], True, rows=rows)
         scale = abs_row_products(X, w.theta[c], Vh[c], True, rows)
         assert componentwise_err(Y[c, rows], ref, scale) <= TOL["fp32"][0]
+
+
+# 1,100 rows: sums over several folds, kept in local memory
+@pytest.mark.parametrize("prec", ["fp32", "bf16_hilo"])
+@pytest.mark.parametrize("d,m", [(33, 2), (33, 40), (48, 17), (64, 5)])
+def test_adjoint(kmv_handle, d, m, prec):
+    _check_backward(kmv_handle, wl.ragged([1100, 65], d=d, chains=1, m=m, seed=9850 + d + m, ell_range=(1.0, 4.0)), prec)
 
 
 def test_many_dimensions_keep_the_wide_chunks(kmv_handle):
