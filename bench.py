@@ -574,6 +574,21 @@ def c5_copy_hmc(h, dev, n=16384, dt=2.5e-4, updates=10, n_int=20, rank=128):
         th = torch.tensor(w.theta, dtype=torch.float64, device=dev)
         acc, dhs, its = [], [], []
         lf_ms = 0.0
+        # every call and torch operation of the loop once, untimed: on a fresh machine their kernels'
+        # first use took 1.4 s of the 2.6 s of the form that runs first
+        gen = torch.Generator(device=dev).manual_seed(1)
+        U, lam, _ = h.nystrom_build(pts, th, torch.randn(8, w.n_total, rank, generator=gen, device=dev), prec="fp32")
+        h.set_preconditioner(pts, U, lam)
+        phi, _, _ = h.phi_refresh(pts, th, torch.randn(8, w.n_total, generator=gen, device=dev), n_poles=15,
+                                  cg_tol=1e-6, cg_maxiter=3000, prec=prec)
+        th_w, pi = th.clone(), torch.zeros_like(th)
+        fail = torch.zeros(8, dtype=torch.int32, device=dev)
+        H0, _, _, _ = h.kmv_energy(pts, y, phi, th_w, pi, cg_maxiter=3000)
+        st, itc, _ = h.leapfrog_step(pts, y, phi, th_w, pi, dt, cg_maxiter=3000, prec=prec)
+        fail |= st
+        torch.stack([itc.float().mean()]).mean().item()
+        ok = accept(H0, H0, torch.ones(8, dtype=torch.float64, device=dev), th, th_w, status=fail)
+        float(ok.float().mean()), (H0 - H0).cpu()
         torch.cuda.synchronize()
         t0 = time.perf_counter()
         for it in range(updates):
@@ -669,6 +684,11 @@ def c1_hmc(h, dev, w, pts, y):
             rng = np.random.default_rng(11)
             th = torch.tensor(w.theta, dtype=torch.float64, device=dev)
             acc, fails = [], 0
+            # one update untimed, from a copy of theta: it loads the kernels of the loop
+            ok, fail = hmc_update(h, pts, y, th.clone(), dt, 10, torch.ones(1, w.n_total, device=dev),
+                                  torch.zeros_like(th), torch.ones(1, dtype=torch.float64, device=dev), prec=prec,
+                                  cg_maxiter=5000)
+            int(ok.item()), int((fail != 0).sum().item())
             torch.cuda.synchronize()
             t0 = time.perf_counter()
             for _ in range(updates):
