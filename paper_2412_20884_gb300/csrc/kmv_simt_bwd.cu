@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kGradThreads) grad_finalize_kernel(DevLayout L
 // Rows per thread and the number of J units: the wide variant once its finest split
 // (units of one fold) gives every SM two CTAs; then about 8 CTAs per SM, and with
 // dL/dV at most kSimtPartMax bytes of partial sums (a single unit needs none).  N = 20,000, d = 8, m = 16: 4.38 ms with one row
-// per thread and no units, 1.10 ms now, with 0.03 ms for the sums of dL/dV and theta.
+// per thread and no units, 1.12 ms now, with 0.03 ms for the sums of dL/dV and theta.
 SimtBwd simt_bwd_plan(const SimtTiles& T, int n_items, int chains, int64_t n_total, int64_t max_rows, int d, int m,
                       bool want_gv, int num_sms, bool one_unit) {
   SimtBwd f = simt_bwd_plan_plain(n_items, m);

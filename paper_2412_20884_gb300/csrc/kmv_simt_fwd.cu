@@ -96,7 +96,7 @@ int forward_jsplit(int n_items, int chains, int m, int64_t max_rows, int num_sms
 // to two CTAs per SM); four rows and units of 512 columns and up take 0.46 ms, with
 // 0.03 ms for their sum.  The wide variant starts where its finest split fills every SM
 // twice: at 2048 rows (d = 1, m = 1) its four tiles of 512 rows would leave most of the
-// chip idle, and the one-row variant takes 7.6 us there against 12 us with the sum of the
+// chip idle, and the one-row variant takes 7.7 us there against 12 us with the sum of the
 // J units in a kernel of its own (now by the last CTA of a tile to arrive, up to two
 // columns; with more columns that CTA's serial share costs more than a launch).
 SimtFwd simt_fwd_plan(const SimtTiles& T, int n_inst, int n_items, int chains, int64_t n_total, int64_t max_rows, int d, int m,
